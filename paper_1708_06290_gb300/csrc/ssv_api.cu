@@ -80,6 +80,7 @@ static void free_handle_buffers(Handle* h) {
   cudaFree(h->Ct);
   cudaFree(h->tauB);
   cudaFree(h->tauA);
+  cudaFree(h->Tq);
   cudaFree(h->hnorm2);
   cudaFree(h->Hhi);
   cudaFree(h->Hlo);
@@ -87,7 +88,7 @@ static void free_handle_buffers(Handle* h) {
 
 static size_t handle_bytes(int n, int m, int p) {
   size_t b = sizeof(double) * ((size_t)n * n + (size_t)n * m + (size_t)(p > 0 ? p : 1) * n +
-                               (size_t)m + (size_t)n + 2) +
+                               (size_t)m + (size_t)n + q_t_count(n, m) + 2) +
              2 * sizeof(float) * (size_t)n * n;
   return b;
 }
@@ -161,6 +162,7 @@ static int make_handle(int n, int m, int p, cudaStream_t st, Handle** out) {
   alloc(&h->Ct, (size_t)ldct * n);
   alloc(&h->tauB, (size_t)m);
   alloc(&h->tauA, (size_t)n);
+  alloc(&h->Tq, q_t_count(n, m));
   alloc(&h->hnorm2, 2);
   if (e == cudaSuccess) e = cudaMalloc((void**)&h->Hhi, sizeof(float) * (size_t)n * n);
   if (e == cudaSuccess) e = cudaMalloc((void**)&h->Hlo, sizeof(float) * (size_t)n * n);

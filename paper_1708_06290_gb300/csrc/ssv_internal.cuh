@@ -68,6 +68,7 @@ struct Handle {
   double* Ct;     // max(p,1) x n, ld max(p,1)
   double* tauB;   // m
   double* tauA;   // n
+  double* Tq;     // T factors of Q's compact WY blocks (q_t_count doubles; empty without Q)
   double* hnorm2; // 2: ||H||_F^2 and trace(H) of the structural part
   float* Hhi;     // n x n: fl32(H) on and above the m-th subdiagonal, 0 below
   float* Hlo;     // n x n: fl32(H - Hhi), 0 below (Hhi + Hlo carries 48 bits of H)
@@ -107,6 +108,7 @@ size_t reduce_tc_scratch_bytes(int n, int p);
 int reduce_fp64(Handle* h, const double* A, long long lda, const double* B, long long ldb,
                 const double* C, long long ldc, int arith, cudaStream_t st);
 // back-transform X = Q Xhat (reduce_fp64.cu)
+size_t q_t_count(int n, int m);
 int apply_q_fp64(const Handle* h, int ncols, const double* Xhat, long long ldx, double* X,
                  long long ldX, cudaStream_t st);
 // load a stored reduced triple with explicit zeros (reduce_fp64.cu)
