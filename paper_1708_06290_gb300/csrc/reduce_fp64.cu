@@ -14,6 +14,7 @@
 // Every kernel is stream-ordered; tau never leaves the device.
 #include <algorithm>
 
+#include "cluster.cuh"
 #include "ssv_internal.cuh"
 
 namespace ssv {
@@ -108,22 +109,6 @@ __device__ __forceinline__ double q_entry(const QBlock& q, int n, int row, int k
   const int d = row - q.pv - k;
   if (k >= q.cnt || row >= n || d < 0) return 0.0;
   return d == 0 ? 1.0 : q.v[row + (size_t)k * n];
-}
-
-__device__ __forceinline__ void cluster_sync_all() {
-  asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
-}
-__device__ __forceinline__ double cluster_ld(const double* p, int rank) {
-  uint32_t a = (uint32_t)__cvta_generic_to_shared(p), r;
-  asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(a), "r"(rank));
-  double v;
-  asm volatile("ld.shared::cluster.f64 %0, [%1];" : "=d"(v) : "r"(r) : "memory");
-  return v;
-}
-__device__ __forceinline__ int cluster_rank() {
-  uint32_t r;
-  asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
-  return (int)r;
 }
 
 // the 32 x 32 tile of V of one row group, staged by its warp (lane = row, so
@@ -306,32 +291,11 @@ constexpr size_t q_apply_smem() {
   return sizeof(double) * (size_t)(kQW * kQB * kQLd + 2 * kQW * 32 * 2 * CC + 4 * kQB * 2 * CC);
 }
 
-template <typename... KArgs, typename... Args>
-cudaError_t launch_cluster(void (*kern)(KArgs...), int grid, int R, size_t smem, cudaStream_t st, Args... args) {
-  cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-  if (e != cudaSuccess) return e;
-  cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3((unsigned)grid);
-  cfg.blockDim = dim3(kQT);
-  cfg.dynamicSmemBytes = smem;
-  cfg.stream = st;
-  cudaLaunchAttribute at[1];
-  at[0].id = cudaLaunchAttributeClusterDimension;
-  at[0].val.clusterDim.x = (unsigned)R;
-  at[0].val.clusterDim.y = 1;
-  at[0].val.clusterDim.z = 1;
-  cfg.attrs = at;
-  cfg.numAttrs = 1;
-  e = cudaLaunchKernelEx(&cfg, kern, args...);
-  if (e == cudaSuccess) count_launch();
-  return e;
-}
-
 template <int CC>
 cudaError_t launch_apply_q(const QSrc& q, int R, const double* T, cd* X, long long ldx, int ncols,
                            cudaStream_t st) {
   const int grid = (ncols + CC - 1) / CC * R;
-  return launch_cluster(apply_q_kernel<CC>, grid, R, q_apply_smem<CC>(), st, q, R, T, X, ldx, ncols);
+  return launch_cluster(apply_q_kernel<CC>, grid, kQT, R, q_apply_smem<CC>(), st, q, R, T, X, ldx, ncols);
 }
 
 __global__ void copy_masked_kernel(const double* __restrict__ src, long long lds, int rows, int cols,
@@ -395,7 +359,7 @@ static int make_q_t(Handle* h, cudaStream_t st) {
   const int nblk = q_blocks(h->kb) + q_blocks(h->ka);
   if (nblk == 0) return SSV_OK;
   constexpr int kR = 4;
-  SSV_CUDA_TRY(launch_cluster(q_t_kernel, nblk * kR, kR, kQTSmem, st, q_src(h), kR, h->Tq));
+  SSV_CUDA_TRY(launch_cluster(q_t_kernel, nblk * kR, kQT, kR, kQTSmem, st, q_src(h), kR, h->Tq));
   return SSV_OK;
 }
 

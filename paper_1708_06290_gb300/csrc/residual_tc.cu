@@ -17,18 +17,26 @@
 //     (the 36 products with k + l <= 9; the dropped ones are below
 //     2^{-56} relative to the row and column scales).
 //
-// Persistent CTAs (two per SM) take work items of 128 rows of H and one
-// shift (N = 32 real columns, 2m of them live).  Per 32-deep K stage the
-// sixteen slice tiles (no-swizzle K-major core-matrix layout, stored tile by
-// tile in global memory) are copied into shared memory by one thread with
-// 1-D TMA bulk copies completing on an mbarrier; four threads (lane 0 of each warp, each owning two of
-// the eight levels) issue the 72 tcgen05.mma (kind::f16, BF16 x BF16 -> FP32,
-// M = 128, N = 32, K = 16) into eight TMEM accumulators (one per level, 32
-// columns each) and commit to their own mbarriers; after every fourth stage
-// the warps read the levels back (tcgen05.ld) and add them, scaled by
-// 2^{-7t}, into double-float accumulators.  The epilogue forms E in FP64.
+// Persistent CTAs (one per SM) take work items of 128 rows of H and one group
+// of shifts (N = 32 real columns: 32 / cs shifts of cs columns, 2m rounded up
+// to a power of two), in three roles that only meet at mbarriers:
+//   * a producer thread copies the sixteen digit tiles of a 32-deep K stage
+//     (no-swizzle K-major core-matrix layout, stored tile by tile in global
+//     memory) into one of two stage buffers with 1-D TMA bulk copies;
+//   * an issuing thread multiplies a stage into one of two TMEM windows: the
+//     eight digit tiles of Xhat lie side by side, so one tcgen05.mma (kind::f16,
+//     BF16 x BF16 -> FP32, M = 128, K = 16) of H digit a against Xhat digits
+//     0 .. 7 - a (N = 32 (8 - a) columns) lands digit b in level a + b; every
+//     fourth stage completes a window;
+//   * four warps read a finished window's levels back (tcgen05.ld) and add
+//     them, scaled by 2^{-7t}, into double-float sums while the other window
+//     multiplies; after an item's last window they form E in FP64.
+// What bounds it: the stage copies from L2 (80 KB a stage) and the products
+// (36 x 32 columns) take about the same time, 1.2 k clocks a stage; the readout
+// of a window (2.2 k clocks of FP32) hides under the next one's products.
 #include <algorithm>
 
+#include "cluster.cuh"
 #include "ssv_internal.cuh"
 #include "tc_common.cuh"
 
@@ -37,65 +45,30 @@ namespace ssv {
 namespace {
 
 constexpr int kM = 128;       // rows of H per tile = TMEM lanes
-constexpr int kN = 32;        // real columns per shift (2m, zero-padded)
-// Tile-shape parameters.  Measured on GB300 at n = 5000, m = 16 (ms per 2000
-// shifts): the products are small (N = 32), so throughput follows the number
-// of threads issuing them: one CTA per SM with two TMEM windows and the next
-// stage prefetched 208; two CTAs per SM, 16-deep stages, prefetched 142; two
-// CTAs per SM, 32-deep stages, one buffer 128, with two issuers 122, with four
-// 112, and staged by TMA bulk copies instead of cp.async 106 (the default);
-// without the products at all 61 (staging by cp.async, and readout).  TMA bulk
-// copies into two buffers: 16-deep stages, two CTAs per SM 136; 32-deep
-// stages, one CTA per SM with two TMEM windows 152 (the N = 32 products, not
-// the copies, set the pace).
-#ifndef SSV_TC_KS
-#define SSV_TC_KS 32          // K per shared-memory stage (16 or 32)
-#endif
-#ifndef SSV_TC_TWO_WINDOWS
-#define SSV_TC_TWO_WINDOWS 0  // 1: two TMEM windows in flight, one CTA per SM
-#endif
-#ifndef SSV_TC_INTERLEAVE
-#define SSV_TC_INTERLEAVE 0   // 1: consecutive products to different levels (one issuer)
-#endif
-#ifndef SSV_TC_ISSUERS
-#define SSV_TC_ISSUERS 4      // threads issuing products, each owning whole levels
-#endif
-#ifndef SSV_TC_BUFFERS
-#define SSV_TC_BUFFERS 1      // 2: the next stage streams in during the products
-#endif
-#ifndef SSV_TC_FUSED
-#define SSV_TC_FUSED 1        // 1: fused-level products in the two-shift kernel (24 per stage)
-#endif
-#ifndef SSV_TC_PAIRS
-#define SSV_TC_PAIRS 1        // 1: two shifts per work item (N = 64, one CTA per SM)
-#endif
-#ifndef SSV_TC_BULK
-#define SSV_TC_BULK 1         // one buffer: stage with 1-D TMA bulk copies (else cp.async)
-#endif
-constexpr int kKS = SSV_TC_KS;  // K per shared-memory stage (16 or 32)
-constexpr bool kPairs = SSV_TC_PAIRS != 0;
+constexpr int kN = 32;        // real columns per group of shifts
+constexpr int kKS = 32;       // K per shared-memory stage
 constexpr int kSl = 8;        // digit slices of H and of Xhat
 constexpr int kLev = 8;       // levels t = 2 .. 9
 constexpr int kWin = 128 / kKS;  // stages per exact accumulation window (K = 128)
 constexpr int kKG = kKS / 8;     // core matrices along K in a tile
 constexpr int kAT = kM * kKS;    // BF16 elements of one H slice tile
 constexpr int kBT = kN * kKS;    // BF16 elements of one Xhat slice tile
-// two accumulation windows in flight (the finished one is read while the next
-// multiplies: all of TMEM, one CTA per SM) or one (two CTAs per SM)
-constexpr bool kTwoWin = SSV_TC_TWO_WINDOWS != 0;
-constexpr int kTmemCols = (kTwoWin ? 2 : 1) * kLev * kN;
-constexpr int kCtasPerSm = kTwoWin ? 1 : 2;
 constexpr uint32_t kStageBytes = (uint32_t)kSl * (kAT + kBT) * 2;
-constexpr int kBuf = SSV_TC_BUFFERS;  // 2: the next stage streams in during the products
-constexpr int kIss = SSV_TC_ISSUERS;  // threads issuing products (lane 0 of warps 0 ..)
-constexpr bool kBulk = SSV_TC_BULK != 0;
-static_assert(kIss == 1 || kIss == 2 || kIss == 4, "issuers");
-constexpr size_t kSmem = kBuf * (size_t)kStageBytes + 64;
-static_assert(kCtasPerSm * kSmem <= 227 * 1024, "shared memory of the resident CTAs");
-static_assert(kCtasPerSm * kTmemCols <= 512, "TMEM columns of the resident CTAs");
+constexpr int kWinCols = kLev * kN;  // TMEM columns of a window; two windows
+constexpr int kDrain = 128;          // readout threads (one per row), warps 0 .. 3
+constexpr int kT = kDrain + 64;      // + the producer's and the issuer's warp
+constexpr size_t kSmem = 2 * (size_t)kStageBytes + 128;
+static_assert(kSmem <= 227 * 1024, "shared memory");
+static_assert(2 * kWinCols == 512, "TMEM columns of the two windows");
 using namespace tcg;
-constexpr uint32_t kIdesc = idesc_bf16(kM, kN);
 static_assert(kSl == kDigits, "eight digit slices");
+
+// column stride of one shift in a group: 2m real columns rounded up to a power of two
+__host__ __device__ inline int group_cols(int m) {
+  int c = 2;
+  while (c < 2 * m) c <<= 1;
+  return c;
+}
 
 // element offset inside a K-major core-matrix tile with kKG core matrices
 // along K: core (row group g, K group kk) at (g * kKG + kk) * 64 elements,
@@ -105,22 +78,32 @@ __host__ __device__ __forceinline__ int tile_off(int row, int k) {
   return (((row >> 3) * kKG + (k >> 3)) * 8 + (row & 7)) * 8 + (k & 7);
 }
 
-__global__ void tc_hrow_kernel(int n, int m, int npad, const double* __restrict__ H,
-                               int* __restrict__ hexp) {
-  const int i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= npad) return;
-  if (i >= n) {
-    hexp[i] = 0;
-    return;
-  }
+// Row exponents of H's structural part: blocks of 128 rows x kHChunk columns
+// (hexp preset to INT_MIN-like bytes, combined by atomicMax).  One thread per
+// row over all n columns took 0.87 ms at n = 4000, a chain of n loads on 32 SMs.
+constexpr int kHChunk = 64;
+__global__ void __launch_bounds__(256) tc_hrow_kernel(int n, int m, const double* __restrict__ H,
+                                                      int* __restrict__ hexp) {
+  __shared__ int part[128];
+  const int row = threadIdx.x & 127, half = threadIdx.x >> 7;
+  const int i = blockIdx.x * 128 + row;
+  const int j0 = blockIdx.y * kHChunk, j1 = min(n, j0 + kHChunk);
+  // the chunk lies left of the structural part of every row of the block
+  if (j1 <= (int)blockIdx.x * 128 - m) return;
   double mx = 0.0;
   bool bad = false;
-  for (int j = max(0, i - m); j < n; ++j) {
-    const double v = fabs(H[i + (size_t)j * n]);
-    if (!(v <= 1.7976931348623157e308)) bad = true;
-    else mx = fmax(mx, v);
+  if (i < n) {
+#pragma unroll 8
+    for (int j = max(j0, i - m) + half; j < j1; j += 2) {
+      const double v = fabs(H[i + (size_t)j * n]);
+      if (!(v <= 1.7976931348623157e308)) bad = true;
+      else mx = fmax(mx, v);
+    }
   }
-  hexp[i] = bad ? kBadExp : scale_exp(mx);
+  int E = i < n ? (bad ? kBadExp : scale_exp(mx)) : 0;  // padding rows: 0
+  if (half == 1) part[row] = E;
+  __syncthreads();
+  if (half == 0) atomicMax(hexp + i, max(E, part[row]));
 }
 
 // items (i, j8): rows i fastest (coalesced reads of column-major H)
@@ -154,82 +137,107 @@ __global__ void tc_hsplit_kernel(int n, int m, int npad, const double* __restric
   }
 }
 
-// one block per active shift: column exponents, then the digit tiles
-__global__ void __launch_bounds__(256) tc_xsplit_kernel(int n, int m, int npad,
+// Digits of Xhat: a cluster of R CTAs per active shift finds the column
+// exponents (each CTA over its share of the K tiles, combined through
+// distributed shared memory), then writes its share of the digit tiles.
+// Bound by memory: reads X twice (16 m bytes a row) and writes 16 digits of
+// 2 m columns.  A warp takes 8 real columns x 32 rows of X, so that a digit
+// plane's store is 512 contiguous bytes (one block per shift, 16-byte pieces
+// 128 bytes apart: 6.4 ms for 2000 shifts at n = 5000, m = 16, and 0.33 ms for
+// 40 at n = 4000).
+// Entry w of the list takes columns (w mod S) cs .. of group w / S (S = 32 / cs).
+__global__ void __launch_bounds__(256) tc_xsplit_kernel(int n, int m, int npad, int cs, int R,
                                                         const int* __restrict__ list,
                                                         const int* __restrict__ count,
                                                         const cd* __restrict__ X, long long ldx,
                                                         uint4* __restrict__ Xs,
                                                         int* __restrict__ xexp) {
-  const int w = blockIdx.x;
-  if (w >= *count) return;
+  const int w = blockIdx.x / R;
+  if (w >= *count) return;  // the whole cluster
   const int sh = list[w];
-  const int tid = threadIdx.x;
+  const int rank = cluster_rank();
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const int KT = npad / kKS;
   const cd* Xh = X + (size_t)sh * m * ldx;
-  __shared__ int sE[kN];
+  const int S = kN / cs, grp = w / S, r0 = (w % S) * cs;  // this shift's rows of the group's tiles
+  __shared__ int sE[kN], tE[kN];
+  if (tid < kN) sE[tid] = tid < 2 * m ? -0x7fffffff : 0;
+  __syncthreads();
+  const int per = (KT + R - 1) / R;
+  const int J0 = min(KT, rank * per), J1 = min(KT, J0 + per);
   {
-    const int c = tid >> 3, part = tid & 7;  // 8 threads per real column
-    double mx = 0.0;
-    bool bad = false;
-    if (c < 2 * m) {
-      const int q = c >> 1;
-      for (int j = part; j < n; j += 8) {
+    // complex column q by `parts` warps, lanes along the rows
+    const int parts = max(1, 8 / m);
+    const int ja = J0 * kKS, jb = min(n, J1 * kKS);
+    for (int u = warp; u < m * parts; u += 8) {
+      const int q = u % m, part = u / m;
+      double mr = 0.0, mi = 0.0;
+      bool br = false, bi = false;
+#pragma unroll 4
+      for (int j = ja + part * 32 + lane; j < jb; j += parts * 32) {
         const cd x = Xh[j + (size_t)q * ldx];
-        const double v = fabs((c & 1) ? x.y : x.x);
-        if (!(v <= 1.7976931348623157e308)) bad = true;
-        else mx = fmax(mx, v);
+        const double vr = fabs(x.x), vi = fabs(x.y);
+        if (!(vr <= 1.7976931348623157e308)) br = true;
+        else mr = fmax(mr, vr);
+        if (!(vi <= 1.7976931348623157e308)) bi = true;
+        else mi = fmax(mi, vi);
       }
-    }
-    for (int o = 4; o > 0; o >>= 1) {
-      mx = fmax(mx, __shfl_xor_sync(0xffffffffu, mx, o));
-      bad = __shfl_xor_sync(0xffffffffu, (int)bad, o) || bad;
-    }
-    if (part == 0) {
-      const int E = bad ? kBadExp : (c < 2 * m ? scale_exp(mx) : 0);
-      sE[c] = E;
-      xexp[(size_t)sh * kN + c] = E;
+      int er = br ? kBadExp : scale_exp(mr), ei = bi ? kBadExp : scale_exp(mi);
+      er = __reduce_max_sync(0xffffffffu, er);
+      ei = __reduce_max_sync(0xffffffffu, ei);
+      if (lane == 0) {
+        atomicMax(&sE[2 * q], er);
+        atomicMax(&sE[2 * q + 1], ei);
+      }
     }
   }
   __syncthreads();
-  const int nj8 = npad / 8;
-  for (int it = tid; it < kN * nj8; it += blockDim.x) {
-    const int c = it / nj8, j8 = it % nj8;
-    const int E = sE[c];
+  if (R > 1) {
+    cluster_sync_all();
+    if (tid < kN) {
+      int E = sE[tid];
+      for (int r = 0; r < R; ++r) E = max(E, cluster_ld(sE + tid, r));
+      tE[tid] = E;
+    }
+  } else if (tid < kN) {
+    tE[tid] = sE[tid];
+  }
+  __syncthreads();
+  if (tid < cs && rank == 0) xexp[(size_t)grp * kN + r0 + tid] = tE[tid];
+  // lane = (real column c0 + lane mod 8, K group lane / 8 of the 32-deep tile)
+  const int cl = lane & 7, kg = lane >> 3;
+  const int nc8 = (cs + 7) / 8;
+  for (int u = warp; u < (J1 - J0) * nc8; u += 8) {
+    const int J = J0 + u / nc8, c = (u % nc8) * 8 + cl;
+    if (c >= cs) continue;
+    const int E = tE[c];
+    const bool act = c < 2 * m;
+    const double* xp = reinterpret_cast<const double*>(Xh + (size_t)(c >> 1) * ldx) + (c & 1);
     unsigned short dg[8][kSl];
+    const int j = J * kKS + kg * 8;
 #pragma unroll
     for (int e = 0; e < 8; ++e) {
-      const int j = j8 * 8 + e;
       double v = 0.0;
-      if (c < 2 * m && j < n) {
-        const cd x = Xh[j + (size_t)(c >> 1) * ldx];
-        v = (c & 1) ? x.y : x.x;
-      }
+      if (act && j + e < n) v = xp[2 * (size_t)(j + e)];
       digits8(v, E, dg[e]);
     }
-    const int J = (j8 * 8) / kKS;
-    const int off = tile_off(c, (j8 * 8) % kKS);
+    const int off = tile_off(r0 + c, kg * 8);
 #pragma unroll
     for (int l = 0; l < kSl; ++l) {
-      uint4 u;
-      u.x = dg[0][l] | ((unsigned)dg[1][l] << 16);
-      u.y = dg[2][l] | ((unsigned)dg[3][l] << 16);
-      u.z = dg[4][l] | ((unsigned)dg[5][l] << 16);
-      u.w = dg[6][l] | ((unsigned)dg[7][l] << 16);
-      const size_t base = ((size_t)(sh * kSl + l) * KT + J) * kBT + off;
-      Xs[base / 8] = u;
+      uint4 o;
+      o.x = dg[0][l] | ((unsigned)dg[1][l] << 16);
+      o.y = dg[2][l] | ((unsigned)dg[3][l] << 16);
+      o.z = dg[4][l] | ((unsigned)dg[5][l] << 16);
+      o.w = dg[6][l] | ((unsigned)dg[7][l] << 16);
+      const size_t base = ((size_t)(grp * kSl + l) * KT + J) * kBT + off;
+      Xs[base / 8] = o;
     }
   }
+  if (R > 1) cluster_sync_all();  // no CTA leaves while its maxima may still be read
 }
 
-// issuer owning level t: whole levels, 9 products per issuer with four
-// ({9, 2}, {8, 3}, {7, 4}, {6, 5}), 18 with two
-__host__ __device__ constexpr int level_owner(int t) {
-  return kIss == 1 ? 0 : kIss == 4 ? (t <= 5 ? t - 2 : 9 - t) : ((t <= 5 ? t - 2 : 9 - t) >= 2 ? 1 : 0);
-}
-
-// Work item = (row block I, active shift w), grouped 16 shifts at a time so
-// that the CTAs resident together share H and Xhat tiles in L2.
+// Work item = (row block I, group g of shifts), 16 groups at a time so that
+// the CTAs resident together share H and Xhat tiles in L2.
 constexpr int kGroup = 16;
 __device__ __forceinline__ void task_coords(long long t, int RB, int cnt, int* I, int* w) {
   const long long full = (long long)(cnt / kGroup) * kGroup * RB;
@@ -245,513 +253,221 @@ __device__ __forceinline__ void task_coords(long long t, int RB, int cnt, int* I
   }
 }
 
-__global__ void __launch_bounds__(kM, kCtasPerSm) tc_residual_kernel(
+// a bounded wait of one role: gives up at the poll limit or when another role
+// has (the block then leaves together)
+__device__ __forceinline__ bool role_wait(uint32_t mbar, uint32_t parity, volatile int* fail) {
+  for (long long it = 0; it < kWaitLimit / 64; ++it) {
+    if (mbar_wait(mbar, parity, 64)) return true;
+    if (*fail) return false;
+  }
+  *fail = 1;
+  return false;
+}
+
+template <int CS>
+__global__ void __launch_bounds__(kT, 1) tc_residual_kernel(
     int n, int m, int npad, const uint4* __restrict__ Hs, const int* __restrict__ hexp,
     const uint4* __restrict__ Xs, const int* __restrict__ xexp, const double* __restrict__ R,
     const cd* __restrict__ shifts, const int* __restrict__ list, const int* __restrict__ count,
     const cd* __restrict__ X, long long ldx, float2* __restrict__ E, double* __restrict__ acc,
     int* __restrict__ err) {
+  constexpr int S = kN / CS;  // shifts of a group
   extern __shared__ __align__(128) unsigned char smem[];
-  // two stage buffers, each: kSl H slice tiles (kAT) then kSl Xhat slice tiles (kBT)
-  unsigned long long* mbar = reinterpret_cast<unsigned long long*>(smem + kBuf * kStageBytes);
-  uint32_t* tslot = reinterpret_cast<uint32_t*>(mbar + kIss + kBuf);  // mbar[kIss + b]: loads of buffer b
-  __shared__ double red[2][kM / 32];
-  const int tid = threadIdx.x, warp = tid >> 5;
+  __shared__ __align__(8) unsigned long long mbar[8];
+  __shared__ uint32_t tslot;
+  __shared__ volatile int fail;
+  __shared__ int issued[2];  // stages copied, stages multiplied (read when a wait gave up)
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const int KT = npad / kKS, RB = npad / kM;
   const int cnt = *count;
-  const uint32_t mb = smem_addr(mbar);
+  const int ngrp = (cnt + S - 1) / S;
+  const long long items = (long long)ngrp * RB;
+  // full[b] / empty[b]: stage buffer b copied / multiplied; tfull[t] / tempty[t]:
+  // TMEM window t complete / read back
+  const uint32_t full = smem_addr(mbar), empty = full + 16, tfull = full + 32, tempty = full + 48;
   const uint32_t sBase = smem_addr(smem);
   if (warp == 0) {
-    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(
-                     smem_addr(tslot)),
-                 "r"(kTmemCols));
+    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_addr(&tslot)),
+                 "r"(512));
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;");
   }
   if (tid == 0) {
-    for (int q = 0; q < kIss + kBuf; ++q) asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(mb + 8u * q));
+    for (int q = 0; q < 8; ++q)
+      asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(full + 8u * q), "r"(q >= 6 ? kDrain / 32 : 1));
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    fail = 0;
+    issued[0] = 0;
+    issued[1] = 0;
   }
   fence_before();
   __syncthreads();
   fence_after();
-  const uint32_t tmem = *tslot;
-  uint32_t phase = 0;
-  uint32_t lphase[2] = {0u, 0u};
-  bool pend[2] = {false, false};  // a bulk copy into buffer b not yet seen complete
-  const uint32_t lmb = mb + 8u * kIss;
-  bool failed = false;
-  float ah[kN], al[kN];
-  // copy the slice tiles of K stage J of (row block I, shift sh) into buffer b
-  auto stage_in = [&](int I, int sh, int J, int b) {
-    const uint32_t dst = sBase + (uint32_t)b * kStageBytes;
-    if constexpr (kBulk) {
-      // sixteen contiguous tiles: one thread, sixteen TMA bulk copies
-      pend[b] = true;
-      if (tid == 0) {
-        const uint32_t lb = lmb + 8u * (uint32_t)b;
-        asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(lb), "r"(kStageBytes)
-                     : "memory");
-        for (int k = 0; k < kSl; ++k)
-          bulk_copy(dst + (uint32_t)(k * kAT * 2), Hs + ((size_t)(k * RB + I) * KT + J) * (kAT / 8),
-                    (uint32_t)(kAT * 2), lb);
-        for (int l = 0; l < kSl; ++l)
-          bulk_copy(dst + (uint32_t)(kSl * kAT * 2 + l * kBT * 2),
-                    Xs + ((size_t)(sh * kSl + l) * KT + J) * (kBT / 8), (uint32_t)(kBT * 2), lb);
-      }
-    } else {
-      for (int v = tid; v < kSl * (kAT + kBT) / 8; v += kM) {
-        const uint4* src;
-        if (v < kSl * kAT / 8) {
-          const int k = v / (kAT / 8), o = v % (kAT / 8);
-          src = Hs + ((size_t)(k * RB + I) * KT + J) * (kAT / 8) + o;
-        } else {
-          const int vb = v - kSl * kAT / 8;
-          const int l = vb / (kBT / 8), o = vb % (kBT / 8);
-          src = Xs + ((size_t)(sh * kSl + l) * KT + J) * (kBT / 8) + o;
-        }
-        cp16(dst + (uint32_t)v * 16u, src);
-      }
-      asm volatile("cp.async.commit_group;" ::: "memory");
-    }
-  };
-  // levels of one accumulation window (TMEM half `half`) into the double-float sums
-  auto read_window = [&](uint32_t half) {
-    float sc = 0.0078125f * 0.0078125f;  // 2^{-7t}, t = 2
-#pragma unroll 1
-    for (int lv = 0; lv < kLev; ++lv) {
-      uint32_t r[32];
-      tmem_ld32(tmem + ((uint32_t)(warp * 32) << 16) + half + (uint32_t)(lv * kN), r);
-#pragma unroll
-      for (int c = 0; c < kN; ++c) {
-        const float p = __uint_as_float(r[c]) * sc;
-        const float s = ah[c] + p;
-        const float bp = s - ah[c];
-        al[c] += (ah[c] - (s - bp)) + (p - bp);
-        ah[c] = s;
-      }
-      sc *= 0.0078125f;
-    }
-  };
-  for (long long t = blockIdx.x; t < (long long)cnt * RB && !failed; t += gridDim.x) {
-    int I, w;
-    task_coords(t, RB, cnt, &I, &w);
-    const int sh = list[w];
-    const int i0 = I * kM;
-    const int J0 = max(0, i0 - m) / kKS;
-    const int nst = KT - J0;
-#pragma unroll
-    for (int c = 0; c < kN; ++c) { ah[c] = 0.f; al[c] = 0.f; }
-    if (kBuf == 2) stage_in(I, sh, J0, 0);
-    for (int st = 0; st < nst; ++st) {
-      const int b = kBuf == 2 ? (st & 1) : 0;
-      if (kBuf == 1) stage_in(I, sh, J0 + st, 0);
-      if constexpr (kBulk) {
-        // the tiles land through the async proxy that the products read
-        const bool lok = mbar_wait(lmb + 8u * (uint32_t)b, lphase[b]);
-        if (__syncthreads_or(!lok)) {
-          failed = true;
-          break;
-        }
-        lphase[b] ^= 1u;
-        pend[b] = false;
-      } else {
-        asm volatile("cp.async.wait_group 0;" ::: "memory");
-        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-        __syncthreads();
-      }
-      const uint32_t half = kTwoWin ? (uint32_t)(((st / kWin) & 1) * kLev * kN) : 0u;
-      const int iss = tid >> 5;
-      if ((tid & 31) == 0 && iss < kIss) {
-        fence_after();
-        const bool fresh = (st % kWin) == 0;
-        const uint32_t aBase = sBase + (uint32_t)b * kStageBytes;
-        const uint32_t bBase = aBase + (uint32_t)(kSl * kAT * 2);
-        constexpr uint32_t kSbo = (uint32_t)kKG * 128u;
-        // slice pair (k, l) into level t = k + l; the first product of each
-        // level in a window overwrites, the rest accumulate
-        auto issue = [&](int k, int l, int ks) {
-          const int lv = k + l;
-          const uint64_t ad = mat_desc(aBase + (uint32_t)((k - 1) * kAT * 2 + ks * 256), 128u, kSbo);
-          const uint64_t bd = mat_desc(bBase + (uint32_t)((l - 1) * kBT * 2 + ks * 256), 128u, kSbo);
-          const bool first = fresh && k == max(1, lv - kSl) && ks == 0;
-          mma_bf16(tmem + half + (uint32_t)((lv - 2) * kN), ad, bd, kIdesc, first ? 0u : 1u);
-        };
-        static_assert(kIss == 1 || SSV_TC_INTERLEAVE == 0, "interleaving needs one issuer");
-        if constexpr (SSV_TC_INTERLEAVE != 0) {
-          // consecutive products go to different levels
-#pragma unroll 1
-          for (int ks = 0; ks < kKS / 16; ++ks)
-#pragma unroll 1
-            for (int k = 1; k <= kSl; ++k)
-#pragma unroll 1
-              for (int l = 1; l <= kSl + 1 - k; ++l) issue(k, l, ks);
-        } else {
-#pragma unroll 1
-          for (int lv = 2; lv <= kSl + 1; ++lv) {
-            if (level_owner(lv) != iss) continue;
-#pragma unroll 1
-            for (int k = max(1, lv - kSl); k <= min(kSl, lv - 1); ++k)
-#pragma unroll
-              for (int ks = 0; ks < kKS / 16; ++ks) issue(k, lv - k, ks);
-          }
-        }
-        mma_commit(mb + 8u * (uint32_t)iss);
-      }
-      // the next stage streams into the other buffer (its MMAs completed
-      // before the previous iteration ended) while these MMAs run
-      if (kBuf == 2 && st + 1 < nst) stage_in(I, sh, J0 + st + 1, b ^ 1);
-      // with two windows, the previous window's levels (the other TMEM half)
-      // are read meanwhile
-      if (kTwoWin && st > 0 && (st % kWin) == 0) {
-        fence_after();
-        read_window(half ^ (uint32_t)(kLev * kN));
-        fence_before();
-      }
+  const uint32_t tmem = tslot;
+  if (warp == 4) {
+    if (lane == 0) {
+      // ---- producer: stage i (counted over all items) into buffer i & 1
+      unsigned i = 0;
       bool ok = true;
-      for (int q = 0; q < kIss; ++q) ok = mbar_wait(mb + 8u * q, phase) && ok;
-      phase ^= 1u;
-      if (__syncthreads_or(!ok)) {
-        failed = true;
-        break;
-      }
-      // with one window, it is read as soon as its last products are done
-      if (!kTwoWin && ((st % kWin) == kWin - 1 || st == nst - 1)) {
-        fence_after();
-        read_window(0u);
-        fence_before();
-        __syncthreads();
-      }
-    }
-    if (failed) break;
-    if (kTwoWin) {
-      fence_after();
-      read_window((uint32_t)((((nst - 1) / kWin) & 1) * kLev * kN));
-      fence_before();
-    }
-    // epilogue: E(i, q) = R(i, q) - (H Xhat)(i, q) + sigma Xhat(i, q)
-    const int i = i0 + tid;
-    double e2 = 0.0, x2 = 0.0;
-    if (i < n) {
-      const cd sigma = shifts[sh];
-      const int Ei = hexp[i];
-      const int* Ec = xexp + (size_t)sh * kN;
-      const cd* Xh = X + (size_t)sh * m * ldx;
-#pragma unroll
-      for (int q = 0; q < kN / 2; ++q) {
-        if (q < m) {
-          const int er_ = Ec[2 * q], ei_ = Ec[2 * q + 1];
-          const bool bad = Ei == kBadExp || er_ == kBadExp || ei_ == kBadExp;
-          const double hxr = ldexp((double)ah[2 * q] + (double)al[2 * q], Ei + er_);
-          const double hxi = ldexp((double)ah[2 * q + 1] + (double)al[2 * q + 1], Ei + ei_);
-          const cd x = Xh[i + (size_t)q * ldx];
-          double vr = -hxr + (sigma.x * x.x - sigma.y * x.y);
-          double vi = -hxi + (sigma.x * x.y + sigma.y * x.x);
-          if (i <= q) vr += R[i + (size_t)q * n];
-          if (bad) vr = __longlong_as_double(0x7ff8000000000000LL);
-          e2 += vr * vr + vi * vi;
-          x2 += x.x * x.x + x.y * x.y;
-          if (E != nullptr) E[(size_t)sh * n * m + i + (size_t)q * n] = make_float2((float)vr, (float)vi);
+      for (long long t = blockIdx.x; t < items && ok; t += gridDim.x) {
+        int I, g;
+        task_coords(t, RB, ngrp, &I, &g);
+        for (int J = max(0, I * kM - m) / kKS; J < KT; ++J, ++i) {
+          const uint32_t b = i & 1u;
+          if (!role_wait(empty + 8u * b, ((i >> 1) & 1u) ^ 1u, &fail)) {
+            ok = false;
+            break;
+          }
+          const uint32_t dst = sBase + b * kStageBytes, lb = full + 8u * b;
+          asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(lb), "r"(kStageBytes)
+                       : "memory");
+          for (int k = 0; k < kSl; ++k)
+            bulk_copy(dst + (uint32_t)(k * kAT * 2), Hs + ((size_t)(k * RB + I) * KT + J) * (kAT / 8),
+                      (uint32_t)(kAT * 2), lb);
+          for (int l = 0; l < kSl; ++l)
+            bulk_copy(dst + (uint32_t)(kSl * kAT * 2 + l * kBT * 2),
+                      Xs + ((size_t)(g * kSl + l) * KT + J) * (kBT / 8), (uint32_t)(kBT * 2), lb);
+          issued[0] = (int)(i + 1);
         }
       }
     }
-    for (int o = 16; o > 0; o >>= 1) {
-      e2 += __shfl_xor_sync(0xffffffffu, e2, o);
-      x2 += __shfl_xor_sync(0xffffffffu, x2, o);
-    }
-    if ((tid & 31) == 0) {
-      red[0][warp] = e2;
-      red[1][warp] = x2;
-    }
-    __syncthreads();
-    if (tid == 0) {
-      double a = 0.0, bsum = 0.0;
-      for (int k = 0; k < kM / 32; ++k) { a += red[0][k]; bsum += red[1][k]; }
-      atomicAdd(acc + 2 * (size_t)sh, a);
-      atomicAdd(acc + 2 * (size_t)sh + 1, bsum);
-    }
-    __syncthreads();
-  }
-  if (failed) {
-    // a tensor-core completion never arrived: record it (every shift then
-    // fails certification), give the MMAs in flight one more bounded wait,
-    // drain this thread's copies, then release TMEM
-    if (tid == 0) {
-      atomicExch(err, 1);
-      for (int q = 0; q < kIss; ++q) mbar_wait(mb + 8u * q, phase ^ 1u);
-      if (kBulk)
-        for (int b = 0; b < kBuf; ++b)
-          if (pend[b]) mbar_wait(lmb + 8u * (uint32_t)b, lphase[b]);
-    }
-    asm volatile("cp.async.wait_group 0;" ::: "memory");
-    __syncthreads();
-  }
-  fence_before();
-  __syncthreads();
-  fence_after();
-  if (warp == 0)
-    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(kTmemCols));
-}
-
-// ---------------------------------------------------------------------------
-// Two shifts per work item: the same digit products with N = 64 (the two
-// shifts' Xhat slice tiles side by side form one 64-row B tile, since a 32-row
-// tile is exactly four core-matrix row groups), so every H tile staged serves
-// two shifts and each product is twice as large.  One CTA per SM (the eight
-// levels x 64 columns fill TMEM), two stage buffers by TMA bulk copies, 256
-// threads: thread (row, half) reads the 32 columns of one shift.
-// ---------------------------------------------------------------------------
-constexpr int kN2 = 64;
-constexpr int kT2 = 2 * kM;
-constexpr uint32_t kIdesc2 = idesc_bf16(kM, kN2);
-constexpr uint32_t kStage2 = (uint32_t)kSl * (kAT + 2 * kBT) * 2;
-constexpr size_t kSmem2 = 2 * (size_t)kStage2 + 128;
-static_assert(kSmem2 <= 227 * 1024, "shared memory of the two-shift residual");
-static_assert(kLev * kN2 <= 512, "TMEM columns of the two-shift residual");
-constexpr int kWaitIss = SSV_TC_FUSED ? 1 : kIss;  // MMA barriers the two-shift kernel commits
-constexpr int kPairGroup = 8;  // pairs that resident CTAs take together (L2 sharing of H tiles)
-
-__device__ __forceinline__ void pair_coords(long long t, int RB, int np, int* I, int* w) {
-  const long long full = (long long)(np / kPairGroup) * kPairGroup * RB;
-  if (t < full) {
-    const long long g = t / ((long long)kPairGroup * RB), r = t % ((long long)kPairGroup * RB);
-    *I = (int)(r / kPairGroup);
-    *w = (int)(g * kPairGroup + r % kPairGroup);
-  } else {
-    const int gl = np - (np / kPairGroup) * kPairGroup;
-    const long long r = t - full;
-    *I = (int)(r / gl);
-    *w = (np / kPairGroup) * kPairGroup + (int)(r % gl);
-  }
-}
-
-__global__ void __launch_bounds__(kT2, 1) tc_residual2_kernel(
-    int n, int m, int npad, const uint4* __restrict__ Hs, const int* __restrict__ hexp,
-    const uint4* __restrict__ Xs, const int* __restrict__ xexp, const double* __restrict__ R,
-    const cd* __restrict__ shifts, const int* __restrict__ list, const int* __restrict__ count,
-    const cd* __restrict__ X, long long ldx, float2* __restrict__ E, double* __restrict__ acc,
-    int* __restrict__ err) {
-  extern __shared__ __align__(128) unsigned char smem[];
-  unsigned long long* mbar = reinterpret_cast<unsigned long long*>(smem + 2 * (size_t)kStage2);
-  uint32_t* tslot = reinterpret_cast<uint32_t*>(mbar + kIss + 2);  // mbar[kIss + b]: loads of buffer b
-  __shared__ double red[2][kT2 / 32];
-  const int tid = threadIdx.x, warp = tid >> 5;
-  const int row = tid & (kM - 1), half = tid >> 7;
-  const int KT = npad / kKS, RB = npad / kM;
-  const int cnt = *count;
-  const int npair = (cnt + 1) / 2;
-  const uint32_t mb = smem_addr(mbar);
-  const uint32_t lmb = mb + 8u * kIss;
-  const uint32_t sBase = smem_addr(smem);
-  if (warp == 0) {
-    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(
-                     smem_addr(tslot)),
-                 "r"(kLev * kN2));
-    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;");
-  }
-  if (tid == 0) {
-    for (int q = 0; q < kIss + 2; ++q) asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(mb + 8u * q));
-    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-  }
-  fence_before();
-  __syncthreads();
-  fence_after();
-  const uint32_t tmem = *tslot;
-  uint32_t phase = 0;
-  uint32_t lphase[2] = {0u, 0u};
-  bool pend[2] = {false, false};
-  bool failed = false;
-  float ah[32], al[32];
-  // K stage J of (row block I, shifts s0, s1 (s1 < 0: none)) into buffer b
-  auto stage_in = [&](int I, int s0, int s1, int J, int b) {
-    pend[b] = true;
-    if (tid != 0) return;
-    const uint32_t dst = sBase + (uint32_t)b * kStage2;
-    const uint32_t lb = lmb + 8u * (uint32_t)b;
-    const uint32_t bytes = (uint32_t)kSl * (kAT + (s1 >= 0 ? 2 : 1) * kBT) * 2;
-    asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(lb), "r"(bytes) : "memory");
-    for (int k = 0; k < kSl; ++k)
-      bulk_copy(dst + (uint32_t)(k * kAT * 2), Hs + ((size_t)(k * RB + I) * KT + J) * (kAT / 8),
-                (uint32_t)(kAT * 2), lb);
-    for (int l = 0; l < kSl; ++l) {
-      const uint32_t xb = dst + (uint32_t)(kSl * kAT * 2 + l * 2 * kBT * 2);
-      bulk_copy(xb, Xs + ((size_t)(s0 * kSl + l) * KT + J) * (kBT / 8), (uint32_t)(kBT * 2), lb);
-      if (s1 >= 0)
-        bulk_copy(xb + (uint32_t)(kBT * 2), Xs + ((size_t)(s1 * kSl + l) * KT + J) * (kBT / 8),
-                  (uint32_t)(kBT * 2), lb);
-    }
-  };
-  // this thread's 32 columns of every level of one window into the double-float sums
-  auto read_window = [&]() {
-    float sc = 0.0078125f * 0.0078125f;  // 2^{-7t}, t = 2
-#pragma unroll 1
-    for (int lv = 0; lv < kLev; ++lv) {
-      uint32_t r[32];
-      tmem_ld32(tmem + ((uint32_t)((warp & 3) * 32) << 16) + (uint32_t)(lv * kN2 + half * 32), r);
+  } else if (warp == 5) {
+    if (lane == 0) {
+      // ---- issuer: window v (counted over all items) into TMEM half v & 1
+      unsigned i = 0, v = 0;
+      bool ok = true;
+      for (long long t = blockIdx.x; t < items && ok; t += gridDim.x) {
+        int I, g;
+        task_coords(t, RB, ngrp, &I, &g);
+        const int nst = KT - max(0, I * kM - m) / kKS;
+        for (int st = 0; st < nst; ++st, ++i) {
+          const uint32_t b = i & 1u, h = v & 1u;
+          const bool fresh = (st % kWin) == 0;
+          if (fresh && !role_wait(tempty + 8u * h, ((v >> 1) & 1u) ^ 1u, &fail)) ok = false;
+          if (ok && !role_wait(full + 8u * b, (i >> 1) & 1u, &fail)) ok = false;
+          if (!ok) break;
+          fence_after();
+          const uint32_t aBase = sBase + b * kStageBytes;
+          const uint32_t bBase = aBase + (uint32_t)(kSl * kAT * 2);
+          const uint32_t d = tmem + h * (uint32_t)kWinCols;
+          constexpr uint32_t kSbo = (uint32_t)kKG * 128u;
 #pragma unroll
-      for (int c = 0; c < 32; ++c) {
-        const float p = __uint_as_float(r[c]) * sc;
-        const float s = ah[c] + p;
-        const float bp = s - ah[c];
-        al[c] += (ah[c] - (s - bp)) + (p - bp);
-        ah[c] = s;
-      }
-      sc *= 0.0078125f;
-    }
-  };
-  for (long long t = blockIdx.x; t < (long long)npair * RB && !failed; t += gridDim.x) {
-    int I, w;
-    pair_coords(t, RB, npair, &I, &w);
-    const int s0 = list[2 * w];
-    const int s1 = 2 * w + 1 < cnt ? list[2 * w + 1] : -1;
-    const int i0 = I * kM;
-    const int J0 = max(0, i0 - m) / kKS;
-    const int nst = KT - J0;
+          for (int ks = 0; ks < kKS / 16; ++ks) {
 #pragma unroll
-    for (int c = 0; c < 32; ++c) { ah[c] = 0.f; al[c] = 0.f; }
-    stage_in(I, s0, s1, J0, 0);
-    for (int st = 0; st < nst; ++st) {
-      const int b = st & 1;
-      const bool lok = mbar_wait(lmb + 8u * (uint32_t)b, lphase[b]);
-      if (__syncthreads_or(!lok)) {
-        failed = true;
-        break;
-      }
-      lphase[b] ^= 1u;
-      pend[b] = false;
-      const int iss = tid >> 5;
-#if SSV_TC_FUSED
-      // fused levels: the B digit tiles of a stage sit side by side (64 rows
-      // each), so one product of H digit a against B digits b0 .. b0 + c - 1
-      // (N = 64 c <= 256) lands digit b in TMEM level a + b; 24 products per
-      // stage instead of 72.  The two products of a = 0 cover all eight
-      // levels and open the window, so one thread issues everything in order.
-      if (tid == 0) {
-        fence_after();
-        const bool fresh = (st % kWin) == 0;
-        const uint32_t aBase = sBase + (uint32_t)b * kStage2;
-        const uint32_t bBase = aBase + (uint32_t)(kSl * kAT * 2);
-        constexpr uint32_t kSbo = (uint32_t)kKG * 128u;
-#pragma unroll
-        for (int ks = 0; ks < kKS / 16; ++ks) {
-#pragma unroll
-          for (int da = 0; da < kSl; ++da) {
-#pragma unroll
-            for (int b0 = 0; b0 < kSl - da; b0 += 4) {
-              const int c = min(4, kSl - da - b0);
+            for (int da = 0; da < kSl; ++da) {
               const uint64_t ad = mat_desc(aBase + (uint32_t)(da * kAT * 2 + ks * 256), 128u, kSbo);
-              const uint64_t bd = mat_desc(bBase + (uint32_t)(b0 * 2 * kBT * 2 + ks * 256), 128u, kSbo);
-              const bool first = fresh && ks == 0 && da == 0;
-              mma_bf16(tmem + (uint32_t)((da + b0) * kN2), ad, bd, idesc_bf16(kM, kN2 * c), first ? 0u : 1u);
+              const uint64_t bd = mat_desc(bBase + (uint32_t)(ks * 256), 128u, kSbo);
+              // a = 0 reaches every level: its first product opens the window
+              mma_bf16(d + (uint32_t)(da * kN), ad, bd, idesc_bf16(kM, kN * (kSl - da)),
+                       (fresh && ks == 0 && da == 0) ? 0u : 1u);
             }
           }
+          mma_commit(empty + 8u * b);
+          issued[1] = (int)(i + 1);
+          if ((st % kWin) == kWin - 1 || st == nst - 1) {
+            mma_commit(tfull + 8u * h);
+            ++v;
+          }
         }
-        mma_commit(mb);
       }
-#else
-      if ((tid & 31) == 0 && iss < kIss) {
-        fence_after();
-        const bool fresh = (st % kWin) == 0;
-        const uint32_t aBase = sBase + (uint32_t)b * kStage2;
-        const uint32_t bBase = aBase + (uint32_t)(kSl * kAT * 2);
-        constexpr uint32_t kSbo = (uint32_t)kKG * 128u;
-#pragma unroll 1
-        for (int lv = 2; lv <= kSl + 1; ++lv) {
-          if (level_owner(lv) != iss) continue;
-#pragma unroll 1
-          for (int k = max(1, lv - kSl); k <= min(kSl, lv - 1); ++k) {
+    }
+  } else {
+    // ---- readout and epilogue: thread = row
+    unsigned v = 0;
+    bool ok = true;
+    for (long long t = blockIdx.x; t < items && ok; t += gridDim.x) {
+      int I, g;
+      task_coords(t, RB, ngrp, &I, &g);
+      const int i0 = I * kM;
+      const int nst = KT - max(0, i0 - m) / kKS;
+      float ah[kN], al[kN];
 #pragma unroll
-            for (int ks = 0; ks < kKS / 16; ++ks) {
-              const uint64_t ad = mat_desc(aBase + (uint32_t)((k - 1) * kAT * 2 + ks * 256), 128u, kSbo);
-              const uint64_t bd =
-                  mat_desc(bBase + (uint32_t)((lv - k - 1) * 2 * kBT * 2 + ks * 256), 128u, kSbo);
-              const bool first = fresh && k == max(1, lv - kSl) && ks == 0;
-              mma_bf16(tmem + (uint32_t)((lv - 2) * kN2), ad, bd, kIdesc2, first ? 0u : 1u);
-            }
-          }
-        }
-        mma_commit(mb + 8u * (uint32_t)iss);
-      }
-#endif
-      (void)iss;
-      // the next stage streams into the other buffer (its products finished
-      // in the previous round)
-      if (st + 1 < nst) stage_in(I, s0, s1, J0 + st + 1, b ^ 1);
-      bool ok = true;
-      for (int q = 0; q < kWaitIss; ++q) ok = mbar_wait(mb + 8u * q, phase) && ok;
-      if (__syncthreads_or(!ok)) {
-        failed = true;
-        break;
-      }
-      phase ^= 1u;
-      if ((st % kWin) == kWin - 1 || st == nst - 1) {
+      for (int c = 0; c < kN; ++c) { ah[c] = 0.f; al[c] = 0.f; }
+      for (int st = 0; st < nst; st += kWin, ++v) {
+        const uint32_t h = v & 1u;
+        // every lane polls; the warp agrees (it reads TMEM together)
+        ok = __all_sync(0xffffffffu, role_wait(tfull + 8u * h, (v >> 1) & 1u, &fail));
+        if (!ok) break;
         fence_after();
-        read_window();
+        float sc = 0.0078125f * 0.0078125f;  // 2^{-7t}, t = 2
+#pragma unroll 1
+        for (int lv = 0; lv < kLev; ++lv) {
+          uint32_t r[32];
+          tmem_ld32(tmem + ((uint32_t)(warp * 32) << 16) + h * (uint32_t)kWinCols + (uint32_t)(lv * kN), r);
+#pragma unroll
+          for (int c = 0; c < kN; ++c) {
+            const float pv = __uint_as_float(r[c]) * sc;
+            const float s = ah[c] + pv;
+            const float bp = s - ah[c];
+            al[c] += (ah[c] - (s - bp)) + (pv - bp);
+            ah[c] = s;
+          }
+          sc *= 0.0078125f;
+        }
         fence_before();
-        __syncthreads();
+        __syncwarp();
+        if (lane == 0)
+          asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(tempty + 8u * h) : "memory");
       }
-    }
-    if (failed) break;
-    // epilogue of this thread's shift: E(i, q) = R(i, q) - (H Xhat)(i, q) + sigma Xhat(i, q)
-    const int sh = half == 0 ? s0 : s1;
-    const int i = i0 + row;
-    double e2 = 0.0, x2 = 0.0;
-    if (sh >= 0 && i < n) {
-      const cd sigma = shifts[sh];
-      const int Ei = hexp[i];
-      const int* Ec = xexp + (size_t)sh * kN;
-      const cd* Xh = X + (size_t)sh * m * ldx;
+      if (!ok) break;
+      // E(i, q) = R(i, q) - (H Xhat)(i, q) + sigma Xhat(i, q) of the group's shifts
+      const int i = i0 + tid;
+      const int Ei = i < n ? hexp[i] : 0;
 #pragma unroll
-      for (int q = 0; q < kN / 2; ++q) {
-        if (q < m) {
-          const int er_ = Ec[2 * q], ei_ = Ec[2 * q + 1];
-          const bool bad = Ei == kBadExp || er_ == kBadExp || ei_ == kBadExp;
-          const double hxr = ldexp((double)ah[2 * q] + (double)al[2 * q], Ei + er_);
-          const double hxi = ldexp((double)ah[2 * q + 1] + (double)al[2 * q + 1], Ei + ei_);
-          const cd x = Xh[i + (size_t)q * ldx];
-          double vr = -hxr + (sigma.x * x.x - sigma.y * x.y);
-          double vi = -hxi + (sigma.x * x.y + sigma.y * x.x);
-          if (i <= q) vr += R[i + (size_t)q * n];
-          if (bad) vr = __longlong_as_double(0x7ff8000000000000LL);
-          e2 += vr * vr + vi * vi;
-          x2 += x.x * x.x + x.y * x.y;
-          if (E != nullptr) E[(size_t)sh * n * m + i + (size_t)q * n] = make_float2((float)vr, (float)vi);
+      for (int l = 0; l < S; ++l) {
+        const int w = g * S + l;
+        if (w >= cnt) continue;
+        const int sh = list[w];
+        double e2 = 0.0, x2 = 0.0;
+        if (i < n) {
+          const cd sigma = shifts[sh];
+          const int* Ec = xexp + (size_t)g * kN + l * CS;
+          const cd* Xh = X + (size_t)sh * m * ldx;
+#pragma unroll
+          for (int q = 0; q < CS / 2; ++q) {
+            if (q < m) {
+              const int c = l * CS + 2 * q;
+              const int er_ = Ec[2 * q], ei_ = Ec[2 * q + 1];
+              const bool bad = Ei == kBadExp || er_ == kBadExp || ei_ == kBadExp;
+              const double hxr = ldexp((double)ah[c] + (double)al[c], Ei + er_);
+              const double hxi = ldexp((double)ah[c + 1] + (double)al[c + 1], Ei + ei_);
+              const cd x = Xh[i + (size_t)q * ldx];
+              double vr = -hxr + (sigma.x * x.x - sigma.y * x.y);
+              const double vi = -hxi + (sigma.x * x.y + sigma.y * x.x);
+              if (i <= q) vr += R[i + (size_t)q * n];
+              if (bad) vr = __longlong_as_double(0x7ff8000000000000LL);
+              e2 += vr * vr + vi * vi;
+              x2 += x.x * x.x + x.y * x.y;
+              if (E != nullptr) E[(size_t)sh * n * m + i + (size_t)q * n] = make_float2((float)vr, (float)vi);
+            }
+          }
+        }
+        for (int o = 16; o > 0; o >>= 1) {
+          e2 += __shfl_xor_sync(0xffffffffu, e2, o);
+          x2 += __shfl_xor_sync(0xffffffffu, x2, o);
+        }
+        if (lane == 0) {
+          atomicAdd(acc + 2 * (size_t)sh, e2);
+          atomicAdd(acc + 2 * (size_t)sh + 1, x2);
         }
       }
     }
-    for (int o = 16; o > 0; o >>= 1) {
-      e2 += __shfl_xor_sync(0xffffffffu, e2, o);
-      x2 += __shfl_xor_sync(0xffffffffu, x2, o);
-    }
-    if ((tid & 31) == 0) {
-      red[0][warp] = e2;
-      red[1][warp] = x2;
-    }
-    __syncthreads();
-    if ((tid & (kM - 1)) == 0 && sh >= 0) {
-      double a = 0.0, bsum = 0.0;
-      for (int k = half * (kM / 32); k < (half + 1) * (kM / 32); ++k) { a += red[0][k]; bsum += red[1][k]; }
-      atomicAdd(acc + 2 * (size_t)sh, a);
-      atomicAdd(acc + 2 * (size_t)sh + 1, bsum);
-    }
-    __syncthreads();
   }
-  if (failed) {
+  __syncwarp();
+  __syncthreads();
+  if (fail != 0 && tid == 0) {
     // a completion never arrived: record it (every shift then fails
-    // certification), give the products and copies in flight one more
-    // bounded wait, then release TMEM
-    if (tid == 0) {
-      atomicExch(err, 1);
-      for (int q = 0; q < kWaitIss; ++q) mbar_wait(mb + 8u * q, phase);
-      for (int b = 0; b < 2; ++b)
-        if (pend[b]) mbar_wait(lmb + 8u * (uint32_t)b, lphase[b]);
-    }
-    __syncthreads();
+    // certification) and give the copies and products in flight one more
+    // bounded wait
+    atomicExch(err, 1);
+    const unsigned nl = (unsigned)issued[0], nm = (unsigned)issued[1];
+    for (unsigned i = nl > 2 ? nl - 2 : 0; i < nl; ++i) mbar_wait(full + 8u * (i & 1u), (i >> 1) & 1u);
+    for (unsigned i = nm > 2 ? nm - 2 : 0; i < nm; ++i) mbar_wait(empty + 8u * (i & 1u), (i >> 1) & 1u);
   }
   fence_before();
   __syncthreads();
   fence_after();
   if (warp == 0)
-    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(kLev * kN2));
+    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(512));
 }
 
 __global__ void tc_identity_list_kernel(int s, int* __restrict__ list, int* __restrict__ count,
@@ -792,10 +508,17 @@ size_t resid_tc_hbytes(int n) {
   return ((size_t)kSl * np * np * 2 + 255) / 256 * 256 + (np * sizeof(int) + 255) / 256 * 256;
 }
 
-size_t resid_tc_xbytes(int n, int s) {
-  const size_t np = (size_t)resid_tc_npad(n);
-  return ((size_t)s * kSl * kN * np * 2 + 255) / 256 * 256 +
-         ((size_t)s * kN * sizeof(int) + 255) / 256 * 256 + 256;
+// bytes of the digit tiles of s shifts in whole groups
+static size_t x_tile_bytes(int n, int m, int s) {
+  const int S = kN / group_cols(m);
+  const size_t G = (size_t)((s + S - 1) / S);
+  return (G * kSl * kN * (size_t)resid_tc_npad(n) * 2 + 255) / 256 * 256;
+}
+
+size_t resid_tc_xbytes(int n, int m, int s) {
+  const int S = kN / group_cols(m);
+  const size_t G = (size_t)((s + S - 1) / S);
+  return x_tile_bytes(n, m, s) + (G * kN * sizeof(int) + 255) / 256 * 256 + 256;
 }
 
 int resid_tc_split_h(const Handle* h, void* hbuf, cudaStream_t st) {
@@ -803,7 +526,9 @@ int resid_tc_split_h(const Handle* h, void* hbuf, cudaStream_t st) {
   unsigned char* b = static_cast<unsigned char*>(hbuf);
   uint4* Hs = reinterpret_cast<uint4*>(b);
   int* hexp = reinterpret_cast<int*>(b + ((size_t)kSl * np * np * 2 + 255) / 256 * 256);
-  tc_hrow_kernel<<<(np + 127) / 128, 128, 0, st>>>(n, m, np, h->H, hexp);
+  SSV_CUDA_TRY(cudaMemsetAsync(hexp, 0x80, sizeof(int) * (size_t)np, st));
+  tc_hrow_kernel<<<dim3((unsigned)(np / 128), (unsigned)((n + kHChunk - 1) / kHChunk)), 256, 0, st>>>(n, m, h->H,
+                                                                                                     hexp);
   count_launch();
   const long long items = (long long)np * (np / 8);
   const int grid = (int)std::min<long long>((items + 255) / 256, (long long)num_sms() * 16);
@@ -824,28 +549,22 @@ int resid_tc_run(const Handle* h, const void* hbuf, void* xbuf, int s, const dou
   const int* hexp = reinterpret_cast<const int*>(hb + ((size_t)kSl * np * np * 2 + 255) / 256 * 256);
   unsigned char* xb = static_cast<unsigned char*>(xbuf);
   uint4* Xs = reinterpret_cast<uint4*>(xb);
-  int* xexp = reinterpret_cast<int*>(xb + ((size_t)s * kSl * kN * np * 2 + 255) / 256 * 256);
+  int* xexp = reinterpret_cast<int*>(xb + x_tile_bytes(n, m, s));
   const cd* X = reinterpret_cast<const cd*>(Xhat);
-  tc_xsplit_kernel<<<s, 256, 0, st>>>(n, m, np, list, count, X, ldx, Xs, xexp);
-  count_launch();
-  if (kPairs) {
-    SSV_CUDA_TRY(cudaFuncSetAttribute(tc_residual2_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                      (int)kSmem2));
-    const long long tasks = (long long)((s + 1) / 2) * (np / kM);
-    const int grid = (int)std::max<long long>(1, std::min<long long>(tasks, (long long)num_sms()));
-    tc_residual2_kernel<<<grid, kT2, kSmem2, st>>>(n, m, np, Hs, hexp, Xs, xexp, h->R,
-                                                   reinterpret_cast<const cd*>(shifts), list, count, X,
-                                                   ldx, static_cast<float2*>(E), acc, err);
-  } else {
-    SSV_CUDA_TRY(cudaFuncSetAttribute(tc_residual_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                      (int)kSmem));
-    const long long tasks = (long long)s * (np / kM);
-    const int grid =
-        (int)std::max<long long>(1, std::min<long long>(tasks, (long long)num_sms() * kCtasPerSm));
-    tc_residual_kernel<<<grid, kM, kSmem, st>>>(n, m, np, Hs, hexp, Xs, xexp, h->R,
-                                                reinterpret_cast<const cd*>(shifts), list, count, X,
-                                                ldx, static_cast<float2*>(E), acc, err);
-  }
+  const int cs = group_cols(m), S = kN / cs;
+  const int xr = cluster_for(s);
+  SSV_CUDA_TRY(launch_cluster(tc_xsplit_kernel, s * xr, 256, xr, 0, st, n, m, np, cs, xr, list, count, X, ldx, Xs,
+                              xexp));
+  auto kern = cs <= 2    ? tc_residual_kernel<2>
+              : cs <= 4  ? tc_residual_kernel<4>
+              : cs <= 8  ? tc_residual_kernel<8>
+              : cs <= 16 ? tc_residual_kernel<16>
+                         : tc_residual_kernel<32>;
+  SSV_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmem));
+  const long long tasks = (long long)((s + S - 1) / S) * (np / kM);
+  const int grid = (int)std::max<long long>(1, std::min<long long>(tasks, (long long)num_sms()));
+  kern<<<grid, kT, kSmem, st>>>(n, m, np, Hs, hexp, Xs, xexp, h->R, reinterpret_cast<const cd*>(shifts), list, count,
+                                X, ldx, reinterpret_cast<float2*>(E), acc, err);
   count_launch();
   SSV_CUDA_TRY(cudaGetLastError());
   return SSV_OK;
@@ -855,7 +574,7 @@ int backward_error_tc(const Handle* h, int s, const double* shifts, const double
                       long long ldx, double* eta, cudaStream_t st) {
   if (s == 0) return SSV_OK;
   if (h->m > kN / 2) return SSV_ENOTSUP;
-  const size_t hb = resid_tc_hbytes(h->n), xb = resid_tc_xbytes(h->n, s);
+  const size_t hb = resid_tc_hbytes(h->n), xb = resid_tc_xbytes(h->n, h->m, s);
   const size_t lb = ((size_t)s * sizeof(int) + 255) / 256 * 256;
   const size_t ab = ((size_t)2 * s * sizeof(double) + 255) / 256 * 256;
   unsigned char* buf = nullptr;

@@ -23,6 +23,7 @@
 // with the FP64 kernel.  Outputs: G = Ct Xhat (FP64) or Xhat.
 #include <algorithm>
 
+#include "cluster.cuh"
 #include "ssv_internal.cuh"
 
 namespace ssv {
@@ -768,17 +769,33 @@ __global__ void __launch_bounds__(1024) mixed_compact_kernel(int s, const int* _
 }
 
 // Outputs of converged shifts (G = +-Ct Xhat in FP64, or Xhat); the others are
-// marked for the FP64 re-solve.
-__global__ void mixed_output_kernel(int n, int m, int p, int s, int mode,
-                                    const double* __restrict__ Ct, int ldct,
-                                    const cd* __restrict__ Xall, const int* __restrict__ flags,
-                                    const double* __restrict__ eta, cd* __restrict__ out,
-                                    long long ldo, int* __restrict__ status,
-                                    double* __restrict__ resid, int* __restrict__ fallback) {
+// marked for the FP64 re-solve.  A cluster of R CTAs takes a shift, each a
+// range of the n rows; G's partial sums meet in distributed shared memory,
+// chunk by chunk of kOutC entries, in rank order.  Bound by the FP64 pipe
+// (2 n p m multiply-adds a shift) once the SMs are filled; with one CTA per
+// shift and one thread per entry of G, 40 shifts at n = 4000, p = m = 16 took
+// 1.45 ms (a chain of n loads on 40 SMs).
+constexpr int kOutC = 256;  // entries of G at a time
+constexpr int kOutT = 32;   // rows of Xhat staged at a time
+constexpr int kOutX = 512, kOutCt = 1024;  // staged entries of Xhat (complex) and Ct
+__global__ void __launch_bounds__(256) mixed_output_kernel(
+    int n, int m, int p, int s, int mode, int R, const double* __restrict__ Ct, int ldct,
+    const cd* __restrict__ Xall, const int* __restrict__ flags, const double* __restrict__ eta,
+    cd* __restrict__ out, long long ldo, int* __restrict__ status, double* __restrict__ resid,
+    int* __restrict__ fallback) {
+  __shared__ double sums[2][2 * kOutC];
+  __shared__ cd xs[kOutX];
+  __shared__ double cs[kOutCt];
   const size_t nm = (size_t)n * m;
-  for (int sh = blockIdx.x; sh < s; sh += gridDim.x) {
+  const int tid = threadIdx.x, rank = cluster_rank();
+  const int per = (n + R - 1) / R;
+  const int t0 = min(n, rank * per), t1 = min(n, t0 + per);
+  // rows staged at a time: all m columns of Xhat and all p rows of Ct when they fit
+  const int T = min(kOutT, min(kOutX / m, kOutCt / max(p, 1)));
+  int par = 0;
+  for (int sh = blockIdx.x / R; sh < s; sh += gridDim.x / R) {
     const bool ok = (flags[sh] & kFlagOk) != 0;
-    if (threadIdx.x == 0) {
+    if (tid == 0 && rank == 0) {
       fallback[sh] = ok ? 0 : 1;
       if (!ok) atomicAdd(&g_refine_counts[1], 1ull);
       if (ok && status) status[sh] = SSV_SHIFT_OK;
@@ -789,24 +806,68 @@ __global__ void mixed_output_kernel(int n, int m, int p, int s, int mode,
     cd* o = out + (size_t)sh * m * ldo;
     if (mode == SSV_G || mode == SSV_TF) {
       const double sg = mode == SSV_TF ? -1.0 : 1.0;
-      for (int idx = threadIdx.x; idx < p * m; idx += blockDim.x) {
-        const int i = idx % p, q = idx / p;
+      for (int e0 = 0; e0 < p * m; e0 += kOutC, par ^= 1) {
+        // tpe threads (a power of two) share an entry, each every tpe-th row
+        const int ne = min(kOutC, p * m - e0);
+        int tpe = 1;
+        while (tpe < 32 && 2 * tpe * ne <= 256) tpe <<= 1;
+        const int el = tid / tpe, sub = tid % tpe;
+        const int i = el < ne ? (e0 + el) % p : 0, q = el < ne ? (e0 + el) / p : 0;
         double ar = 0.0, ai = 0.0;
-        for (int t = 0; t < n; ++t) {
-          const double c = Ct[i + (size_t)t * ldct];
-          const cd x = Xh[t + (size_t)q * n];
-          ar = fma(c, x.x, ar);
-          ai = fma(c, x.y, ai);
+        if (T >= 1) {
+          for (int tb = t0; tb < t1; tb += T) {
+            const int nt = min(T, t1 - tb);
+            __syncthreads();
+            for (int e = tid; e < nt * m; e += 256) xs[(e / nt) * T + e % nt] = Xh[(tb + e % nt) + (size_t)(e / nt) * n];
+            for (int e = tid; e < nt * p; e += 256) cs[e] = Ct[e % p + (size_t)(tb + e / p) * ldct];
+            __syncthreads();
+            if (el < ne) {
+#pragma unroll 4
+              for (int t = sub; t < nt; t += tpe) {
+                const double c = cs[t * p + i];
+                const cd x = xs[q * T + t];
+                ar = fma(c, x.x, ar);
+                ai = fma(c, x.y, ai);
+              }
+            }
+          }
+        } else if (el < ne) {  // very wide systems: straight from global memory
+          for (int t = t0 + sub; t < t1; t += tpe) {
+            const double c = Ct[i + (size_t)t * ldct];
+            const cd x = Xh[t + (size_t)q * n];
+            ar = fma(c, x.x, ar);
+            ai = fma(c, x.y, ai);
+          }
         }
-        o[i + (size_t)q * ldo] = mkcd(sg * ar, sg * ai);
+        for (int w = tpe >> 1; w > 0; w >>= 1) {
+          ar += __shfl_xor_sync(0xffffffffu, ar, w);
+          ai += __shfl_xor_sync(0xffffffffu, ai, w);
+        }
+        if (R > 1) {
+          // a buffer is written again two chunks later, behind the next chunk's
+          // barrier, which every reader of it has passed by then
+          if (el < ne && sub == 0) {
+            sums[par][2 * el] = ar;
+            sums[par][2 * el + 1] = ai;
+          }
+          cluster_sync_all();
+          if (el < ne && sub == 0 && el % R == rank) {
+            ar = 0.0;
+            ai = 0.0;
+            for (int r = 0; r < R; ++r) {
+              ar += cluster_ld(&sums[par][2 * el], r);
+              ai += cluster_ld(&sums[par][2 * el + 1], r);
+            }
+          }
+        }
+        if (el < ne && sub == 0 && el % R == rank) o[i + (size_t)q * ldo] = mkcd(sg * ar, sg * ai);
       }
     } else {
-      for (long long idx = threadIdx.x; idx < (long long)nm; idx += blockDim.x) {
-        const int i = (int)(idx % n), q = (int)(idx / n);
-        o[i + (size_t)q * ldo] = Xh[idx];
-      }
+      for (int q = 0; q < m; ++q)
+        for (int i = t0 + tid; i < t1; i += 256) o[i + (size_t)q * ldo] = Xh[i + (size_t)q * n];
     }
   }
+  if (R > 1) cluster_sync_all();  // no CTA leaves while its sums may still be read
 }
 
 __global__ void mixed_init_kernel(int s, int* __restrict__ flags, double* __restrict__ eta,
@@ -862,7 +923,7 @@ size_t mixed_layout(int n, int m, int s, int grid, size_t slot_bytes, MixedScrat
          oB = take(sizeof(int) * s), oS0 = take(sizeof(int) * s), oC = take(sizeof(int)),
          oR = take(sizeof(int));
   const bool tc = m <= kTcMaxM;
-  const size_t oH = tc ? take(resid_tc_hbytes(n)) : 0, oXs = tc ? take(resid_tc_xbytes(n, s)) : 0;
+  const size_t oH = tc ? take(resid_tc_hbytes(n)) : 0, oXs = tc ? take(resid_tc_xbytes(n, m, s)) : 0;
   if (ms && base) {
     ms->X = reinterpret_cast<cd*>(base + oX);
     ms->E = reinterpret_cast<cf*>(base + oE);
@@ -980,11 +1041,13 @@ int run_mixed(const Handle* h, int s, const double* shifts, int nb, int mode, do
     count_launch();
     trace_end(tr, st);
   }
-  mixed_output_kernel<<<std::min(s, num_sms() * 8), 256, 0, st>>>(
-      n, m, p, s, mode, h->Ct, p > 0 ? p : 1, ms.X, ms.flags, ms.eta,
-      reinterpret_cast<cd*>(out), ldo, status, resid, ms.fallback);
-  count_launch();
-  SSV_CUDA_TRY(cudaGetLastError());
+  const int ro = cluster_for(s);
+  const double* eta = ms.eta;
+  const int* flags = ms.flags;
+  const cd* xall = ms.X;
+  SSV_CUDA_TRY(launch_cluster(mixed_output_kernel, std::min(s, num_sms() * 8) * ro, 256, ro, 0, st, n, m, p, s, mode,
+                              ro, (const double*)h->Ct, p > 0 ? p : 1, xall, flags, eta, reinterpret_cast<cd*>(out),
+                              ldo, status, resid, ms.fallback));
   return SSV_OK;
 }
 

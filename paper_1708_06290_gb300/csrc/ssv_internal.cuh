@@ -47,15 +47,17 @@ __host__ __device__ __forceinline__ cd cdiv(cd a, cd b) {
 // handle
 // --------------------------------------------------------------------------
 // s = s_hi + s_lo accumulates a_hi*b_hi exactly (FMA error term) plus the FP32
-// cross terms a_hi*b_lo + a_lo*b_hi; the high sum is kept with two-sum.
+// cross terms a_hi*b_lo + a_lo*b_hi; the high sum is kept with two-sum.  The
+// product is formed by the intrinsic: contracted into the following addition it
+// would no longer be the p that e completes.
 __device__ __forceinline__ void df_mac(float& s_hi, float& s_lo, float a_hi, float a_lo, float b_hi,
                                        float b_lo) {
-  const float p = a_hi * b_hi;
+  const float p = __fmul_rn(a_hi, b_hi);
   const float e = fmaf(a_hi, b_hi, -p);
   const float t = fmaf(a_hi, b_lo, fmaf(a_lo, b_hi, e));
-  const float s = s_hi + p;
-  const float bp = s - s_hi;
-  const float err = (s_hi - (s - bp)) + (p - bp);
+  const float s = __fadd_rn(s_hi, p);
+  const float bp = __fadd_rn(s, -s_hi);
+  const float err = __fadd_rn(__fadd_rn(s_hi, -__fadd_rn(s, -bp)), __fadd_rn(p, -bp));
   s_hi = s;
   s_lo += err + t;
 }
@@ -165,7 +167,7 @@ int backward_error_fp64_masked(const Handle* h, int s, const double* shifts, con
 constexpr int kTcMaxM = 16;
 int resid_tc_npad(int n);
 size_t resid_tc_hbytes(int n);
-size_t resid_tc_xbytes(int n, int s);
+size_t resid_tc_xbytes(int n, int m, int s);
 int resid_tc_split_h(const Handle* h, void* hbuf, cudaStream_t st);
 // E (complex64, n x m per shift, may be null) and acc += (||E||_F^2, ||Xhat||_F^2)
 // for the shifts list[0 .. *count); Xhat of shift j at Xhat + 2 j m ldx doubles
