@@ -23,7 +23,7 @@ static __device__ __forceinline__ dw dw_add(dw x, dw y) {
   return dw_fast(s, e + (x.lo + y.lo));
 }
 static __device__ __forceinline__ dw dw_mul(dw x, dw y) {
-  const float p = x.hi * y.hi;
+  const float p = __fmul_rn(x.hi, y.hi);  // not contracted into the sum below
   const float e = fmaf(x.hi, y.lo, fmaf(x.lo, y.hi, fmaf(x.hi, y.hi, -p)));
   return dw_fast(p, e);
 }

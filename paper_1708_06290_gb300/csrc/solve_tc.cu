@@ -44,6 +44,7 @@
 #include <algorithm>
 
 #include "dfloat.cuh"
+#include "panel.cuh"
 #include "ssv_internal.cuh"
 #include "tc_common.cuh"
 
@@ -71,11 +72,9 @@ __device__ __forceinline__ size_t bck(long long i, size_t n, int* err) {
 #define BCK(i, n) ((size_t)(i))
 #endif
 
-constexpr int kPT = 256;             // threads of the setup, panel and final kernels
+constexpr int kPT = 256;             // threads of the setup and final kernels
 constexpr int kNBT = 128;            // n_b of the tensor-core sweep (K of the update)
 constexpr int kMaxM = kTcMaxM;       // m <= 16
-constexpr int kSlots = kMaxM + 1;    // m live + the fresh column
-constexpr int kCoefRows = kNBT + kMaxM;
 constexpr int kUM = 128;             // H rows per update item = TMEM lanes
 // real columns per update item (shift group): 64 = one update block per SM with
 // two stage buffers; 32 = two blocks per SM with one stage buffer each, so that
@@ -95,17 +94,12 @@ constexpr int kLev = 8;              // levels k + l = 0 .. 7
 constexpr int kStages = kNBT / kKS;  // stages per block step
 constexpr int kAT = kUM * kKS;       // BF16 elements of one H digit tile
 constexpr int kBT = kUN * kKS;       // BF16 elements of one P1 digit tile
-#ifndef SSV_TCS_FUSED
-#define SSV_TCS_FUSED 1  // 1: Z1 P1 as fused-level products (one per H digit and <= 256 columns)
-#endif
-// a stage: eight H digit tiles, seven P1 digit tiles and (fused form) one tile of
-// zeros standing for P1 digit 7, so that the H digit 0 products reach all levels
-constexpr int kBPlanes = SSV_TCS_FUSED ? kSD + 1 : kSD;
+// a stage: eight H digit tiles, seven P1 digit tiles and one tile of zeros
+// standing for P1 digit 7, so that the H digit 0 products reach all levels
+constexpr int kBPlanes = kSD + 1;
 constexpr uint32_t kStageBytes = (uint32_t)(kSDH * kAT + kBPlanes * kBT) * 2;
 constexpr uint32_t kLoadBytes = (uint32_t)(kSDH * kAT + kSD * kBT) * 2;  // copied per stage
 constexpr uint32_t kZeroOff = kLoadBytes;                                 // the zero tile in a stage
-constexpr int kIss = 4;              // threads issuing products (lane 0 of warps 0..3)
-constexpr uint32_t kIdescU = idesc_bf16(kUM, kUN);
 constexpr int kTmemCols = 8 * kUN;   // 8 levels x kUN columns
 // polls of one mbarrier wait before the update gives up (a stage's copies and
 // products complete within microseconds)
@@ -115,7 +109,7 @@ static_assert(kLev * kUN <= kTmemCols, "TMEM columns of the levels");
 // the group's Z2 and P2 digit tiles); the group's P2 / sigma rows (S * 2 m^2 <=
 // 64 m float4); the column exponents of P1 and of P2's real form (kUN ints
 // each); the row maxima of the quarters (4 x 128 floats); the shifts (at most
-// kUN); kIss + 3 mbarriers; the TMEM address slot
+// kUN); four mbarriers; the TMEM address slot
 constexpr size_t kOffPc = (size_t)kBufU * kStageBytes;
 constexpr size_t kPcF4 = (size_t)kUN * kMaxM;
 constexpr size_t kOffExp = kOffPc + kPcF4 * 16;
@@ -123,7 +117,7 @@ constexpr size_t kOffExp2 = kOffExp + (size_t)kUN * sizeof(int);
 constexpr size_t kOffXmax = kOffExp2 + (size_t)kUN * sizeof(int);
 constexpr size_t kOffSig = kOffXmax + (size_t)4 * kUM * sizeof(float);
 constexpr size_t kOffBar = kOffSig + (size_t)kUN * 16;
-constexpr size_t kOffSlot = kOffBar + (size_t)(kIss + 3) * 8;
+constexpr size_t kOffSlot = kOffBar + 4 * 8;
 constexpr size_t kUpdSmem = kOffSlot + 16;
 static_assert(kOffBar % 8 == 0 && kOffSig % 16 == 0, "alignment of the smem carve-up");
 static_assert(kCtasU * (kUpdSmem + 1024) <= 228 * 1024, "shared memory of the update blocks");
@@ -136,13 +130,6 @@ static_assert(7 * (128 * 16 + 16 * 16) * 2 * (kUN / 16) <= kBufU * (size_t)kStag
 // H digit tiles
 __host__ __device__ __forceinline__ int tile_off(int row, int k) {
   return (((row >> 3) * kKG + (k >> 3)) * 8 + (row & 7)) * 8 + (k & 7);
-}
-
-// products of level t: H digit k, transform digit t - k, k in [max(0, t - 6), min(7, t)]
-// (1, 2, 3, 4, 5, 6, 7, 7 for t = 0 .. 7); issuer owning level t:
-// {7, 1}, {6, 0}, {5, 2}, {4, 3} (9, 8, 9, 9 products)
-__host__ __device__ constexpr int level_owner(int t) {
-  return (t == 7 || t == 1) ? 0 : (t == 6 || t == 0) ? 1 : (t == 5 || t == 2) ? 2 : 3;
 }
 
 // column stride of one shift in a group: 2m real columns rounded up to a power of two
@@ -202,30 +189,26 @@ __device__ void write_z2_digits(const TcsArgs& a, int sh, int i, const float4* Z
   }
   const int E = scale_exp_f(mx);
   a.zexp[BCK((size_t)sh * a.npad + i, (size_t)a.s * a.npad)] = E;
+  const float inv = digit_scale(E);
   const size_t T0 = ((size_t)sh * a.RB + i / 128) * 7 * (128 * cs);
   for (int k8 = 0; k8 < cs; k8 += 8) {
-    unsigned short dg[8][7];
+    float hi[8], lo[8];
 #pragma unroll
     for (int e = 0; e < 8; ++e) {
       const int kk = k8 + e, q = kk >> 1;
-      float hi = 0.f, lo = 0.f;
+      hi[e] = lo[e] = 0.f;
       if (q < m) {
         const float4 z = Z2f[BCK((a.p + i) + (size_t)q * ldz, a.z2_stride)];
-        hi = (kk & 1) ? z.z : z.x;
-        lo = (kk & 1) ? z.w : z.y;
+        hi[e] = (kk & 1) ? z.z : z.x;
+        lo[e] = (kk & 1) ? z.w : z.y;
       }
-      digits7_pair(hi, lo, E, dg[e]);
     }
     const int off = tile_off_kg(i % 128, k8, kg);
+    uint4 dg[7];
+    digits7_oct(hi, lo, inv, dg);
 #pragma unroll
-    for (int l = 0; l < 7; ++l) {
-      uint4 u;
-      u.x = dg[0][l] | ((unsigned)dg[1][l] << 16);
-      u.y = dg[2][l] | ((unsigned)dg[3][l] << 16);
-      u.z = dg[4][l] | ((unsigned)dg[5][l] << 16);
-      u.w = dg[6][l] | ((unsigned)dg[7][l] << 16);
-      *reinterpret_cast<uint4*>(a.Zd + BCK(T0 + (size_t)l * (128 * cs) + off, a.n_zd)) = u;
-    }
+    for (int l = 0; l < 7; ++l)
+      *reinterpret_cast<uint4*>(a.Zd + BCK(T0 + (size_t)l * (128 * cs) + off, a.n_zd)) = dg[l];
   }
 }
 
@@ -255,19 +238,32 @@ __global__ void __launch_bounds__(kPT) tcs_setup_kernel(TcsArgs a) {
 }
 
 // ---- panel of block step `step` (1-based), rows k - nbe .. k - 1 ------------
+constexpr int kCtRows = 16;  // rows of Ct staged at a time
+template <int MAXM>
 struct PanelSmem {
-  float4 cand[kSlots * kNBT];
-  float4 coef[kCoefRows * kSlots];
-  float4 vf[kMaxM + 4];
+  using Panel = pan::Smem<pan::DF32, MAXM, kNBT>;
+  static constexpr int S = Panel::S;
+  Panel p;  // p.W: the coefficients; p.F: later a chunk of Ct rows as FP32 pairs
   int fexp[2 * kMaxM];
   int f2exp[2 * kMaxM];
   int sing;
 };
+// Threads and resident panels per SM.  FEW (no more shifts than SMs, m > 8): one
+// panel per SM with twice the threads for the update of the sub-block's other
+// rows (m = 16: 183 us per block of 128 rows against 191); else two with 256.
+template <int MAXM, bool FEW>
+constexpr int panel_threads() { return MAXM <= 4 ? 128 : MAXM <= 8 || !FEW ? 256 : 512; }
+template <int MAXM, bool FEW>
+constexpr int panel_per_sm() { return MAXM <= 4 ? 5 : MAXM <= 8 ? 3 : FEW ? 1 : 2; }
 
-__global__ void __launch_bounds__(kPT, 3) tcs_panel_kernel(TcsArgs a, int k, int nbe, int step) {
+template <int MAXM, bool FEW>
+__global__ void __launch_bounds__(panel_threads<MAXM, FEW>(), panel_per_sm<MAXM, FEW>())
+    tcs_panel_kernel(TcsArgs a, int k, int nbe, int step) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  PanelSmem& sm = *reinterpret_cast<PanelSmem*>(smem_raw);
-  constexpr int S = kSlots;
+  using PS = PanelSmem<MAXM>;
+  PS& sm = *reinterpret_cast<PS*>(smem_raw);
+  constexpr int S = PS::S;
+  constexpr int T = panel_threads<MAXM, FEW>();
   const int sh = blockIdx.x;
   const int tid = threadIdx.x;
   const int n = a.n, m = a.m, p = a.p, ldz = p + n;
@@ -276,154 +272,36 @@ __global__ void __launch_bounds__(kPT, 3) tcs_panel_kernel(TcsArgs a, int k, int
   const cd sigma = a.shifts[sh];
   float4* Z2f = a.Z2 + (size_t)sh * a.z2_stride;
   const double sing_tol = (double)n * 7.105427357601002e-15 * sqrt(shifted_norm2(a.hnorm, n, sigma));
-  const float sing_tol_f = (float)sing_tol;
-  const float* __restrict__ Hhi = a.Hhi;
-  const float* __restrict__ Hlo = a.Hlo;
-  auto split4 = [](cd z) -> float4 { return df_split(z); };
-  // entry (global row gr, fresh column jc) of H - sigma I as FP32 pairs
-  auto fresh4 = [&](int gr, int jc) -> float4 {
-    const size_t hidx = (size_t)gr + (size_t)jc * n;
-    if (gr == jc) return split4(csub(mkcd((double)Hhi[hidx] + (double)Hlo[hidx], 0.0), sigma));
-    return make_float4(Hhi[hidx], Hlo[hidx], 0.f, 0.f);
-  };
-  float4* cand4 = sm.cand;
-  float4* coef4 = sm.coef;
-  float4* vf = sm.vf;
+  float4* coef4 = sm.p.W;
+  float2* ct = &sm.p.F[0][0];   // kCtRows x (kNBT + 1), after the panel
+  static_assert(sizeof(sm.p.F) >= sizeof(float2) * kCtRows * (kNBT + 1), "staged Ct rows");
   if (tid == 0) sm.sing = 0;
-  for (int idx = tid; idx < m * nbe; idx += kPT) {
-    const int t = idx % nbe, q = idx / nbe;
-    cand4[q * kNBT + t] = Z2f[BCK((r + t) + (size_t)q * ldz, a.z2_stride)];
+  for (int e = tid; e < nbe * m; e += T) {
+    const int row = e % nbe, q = e / nbe;
+    coef4[row * S + q] = Z2f[BCK((r + row) + (size_t)q * ldz, a.z2_stride)];
   }
-  for (int idx = tid; idx < kCoefRows * S; idx += kPT) {
-    const int c = idx / S, slot = idx % S;
-    const bool one = (slot < m && c == kNBT + slot) || (slot == m && c == nbe - 1);
-    coef4[idx] = make_float4(one ? 1.f : 0.f, 0.f, 0.f, 0.f);
-  }
-  {
-    const int c = nbe - 1, jc = j0 + c;
-    for (int t = tid; t <= c; t += kPT) cand4[m * kNBT + t] = fresh4(k - nbe + t, jc);
-  }
-  __syncthreads();
-  for (int c = nbe - 1; c >= 0; --c) {
-    const int fs = m;                         // slot of the fresh column of row c
-    // the next fresh column is read now, its latency hidden behind this row
-    float4 pre = make_float4(0.f, 0.f, 0.f, 0.f);
-    if (c > 0 && tid < c) pre = fresh4(k - nbe + tid, j0 + c - 1);
-    if (tid < 32) {
-      // reflector scalars in double-word arithmetic:
-      //   v = conj(x) + e^{i arg conj(x_f)} ||x|| e_f,  tau = 1 / (||x||^2 + |x_f| ||x||)
-      dw rest2{0.f, 0.f};
-      for (int q = tid; q < m; q += 32) {
-        const float4 x = cand4[q * kNBT + c];
-        df_mac(rest2.hi, rest2.lo, x.x, x.y, x.x, x.y);
-        df_mac(rest2.hi, rest2.lo, x.z, x.w, x.z, x.w);
-        vf[q] = make_float4(x.x, x.y, -x.z, -x.w);
-      }
-      rest2 = dw_fast(rest2.hi, rest2.lo);
-      for (int o = 16; o > 0; o >>= 1)
-        rest2 = dw_add(rest2, dw{__shfl_xor_sync(0xffffffffu, rest2.hi, o),
-                                 __shfl_xor_sync(0xffffffffu, rest2.lo, o)});
-      if (tid == 0) {
-        const float4 xf = cand4[fs * kNBT + c];
-        const dw xr{xf.x, xf.y}, xi{xf.z, xf.w};
-        const dw af2 = dw_add(dw_mul(xr, xr), dw_mul(xi, xi));
-        const dw af = dw_sqrt(af2);
-        const dw nrm2 = dw_add(rest2, af2);
-        const dw nrm = dw_sqrt(nrm2);
-        float4 vfs;
-        if (af.hi > 0.f) {  // conj(x_f) (1 + ||x|| / |x_f|)
-          const dw g = dw_add(dw{1.f, 0.f}, dw_div(nrm, af));
-          const dw vr = dw_mul(xr, g), vi = dw_mul(xi, g);
-          vfs = make_float4(vr.hi, vr.lo, -vi.hi, -vi.lo);
-        } else {
-          vfs = make_float4(nrm.hi, nrm.lo, 0.f, 0.f);
-        }
-        vf[fs] = vfs;
-        const dw tau = rest2.hi > 0.f ? dw_div(dw{1.f, 0.f}, dw_add(nrm2, dw_mul(af, nrm)))
-                                      : dw{0.f, 0.f};
-        vf[kMaxM + 2] = make_float4(tau.hi, tau.lo, 0.f, 0.f);
-        if (nrm.hi <= sing_tol_f) sm.sing = 1;
-      }
-    }
-    __syncthreads();
-    const float4 tauf = vf[kMaxM + 2];
-    {
-      const int nrow = c;
-      const int ncoef = (nbe - c) + m;
-      // nrow + ncoef <= n_b + m < kPT: each thread has at most one row e = tid,
-      // and the thread of window row e < c holds that row's next fresh entry
-      for (int e = tid; e < nrow + ncoef; e += kPT) {
-        float4* base;
-        int stride;
-        if (e < nrow) {
-          base = cand4 + e;
-          stride = kNBT;
-        } else {
-          const int ee = e - nrow;
-          const int crow = ee < nbe - c ? c + ee : kNBT + (ee - (nbe - c));
-          base = coef4 + crow * S;
-          stride = 1;
-        }
-        if (tauf.x != 0.0f) {
-        // w = sum_slot base(slot) v(slot)
-        float wrh = 0.f, wrl = 0.f, wih = 0.f, wil = 0.f;
-        for (int q = 0; q <= m; ++q) {
-          const int slot = q < m ? q : fs;
-          const float4 x = base[slot * stride], v = vf[slot];
-          df_mac(wrh, wrl, x.x, x.y, v.x, v.y);
-          df_mac(wrh, wrl, -x.z, -x.w, v.z, v.w);
-          df_mac(wih, wil, x.x, x.y, v.z, v.w);
-          df_mac(wih, wil, x.z, x.w, v.x, v.y);
-        }
-        float trh = 0.f, trl = 0.f, tih = 0.f, til = 0.f;
-        df_mac(trh, trl, tauf.x, tauf.y, wrh, wrl);
-        df_mac(tih, til, tauf.x, tauf.y, wih, wil);
-        // base(slot) -= t conj(v(slot))
-        for (int q = 0; q <= m; ++q) {
-          const int slot = q < m ? q : fs;
-          float4 x = base[slot * stride];
-          const float4 v = vf[slot];
-          float xrh = x.x, xrl = x.y, xih = x.z, xil = x.w;
-          df_mac(xrh, xrl, -trh, -trl, v.x, v.y);
-          df_mac(xrh, xrl, -tih, -til, v.z, v.w);
-          df_mac(xih, xil, -tih, -til, v.x, v.y);
-          df_mac(xih, xil, trh, trl, v.z, v.w);
-          const float sr = xrh + xrl, si = xih + xil;
-          x = make_float4(sr, xrl - (sr - xrh), si, xil - (si - xih));
-          base[slot * stride] = x;
-        }
-        }
-        // the eliminated column is done with: its slot takes the next fresh
-        // column, whose coefficients are e_{c-1} (row c - 1 is set below; the
-        // rows this loop covers get zero, every other row is zero already)
-        base[fs * stride] = e < nrow ? pre : make_float4(0.f, 0.f, 0.f, 0.f);
-      }
-      if (c > 0 && tid == 0) coef4[(c - 1) * S + fs] = make_float4(1.f, 0.f, 0.f, 0.f);
-    }
-    __syncthreads();
-  }
+  pan::run<pan::DF32, MAXM, kNBT, T, false>(pan::DF32::H{a.Hhi, a.Hlo, n}, k - nbe, j0, sigma, nbe, m, sm.p,
+                                            (pan::SmemR<pan::DF32, MAXM, kNBT>*)nullptr, sing_tol, &sm.sing);
   // coef rows c < nbe hold P1(c, :), rows kNBT + qq hold P2(qq, :) (slots 0..m-1)
 
-  // ---- P1 as BF16 digit tiles: column exponents first (one warp per real column)
+  // ---- P1 as BF16 digit tiles: column exponents first (one warp per complex column)
   const int warp = tid >> 5, lane = tid & 31;
-  for (int cr = warp; cr < 2 * m; cr += kPT / 32) {
-    const int q = cr >> 1;
-    double mx = 0.0;
-    bool bad = false;
+  for (int q = warp; q < m; q += T / 32) {
+    float mr = 0.f, mi = 0.f;
+    bool br = false, bi = false;
     for (int c = lane; c < nbe; c += 32) {
       const float4 w = coef4[c * S + q];
-      const double v = fabs((cr & 1) ? (double)w.z + (double)w.w : (double)w.x + (double)w.y);
-      if (!(v <= 1.7976931348623157e308)) bad = true;
-      else mx = fmax(mx, v);
+      mr = fmaxf(mr, fabsf(w.x));
+      mi = fmaxf(mi, fabsf(w.z));
+      br = br || !(fabsf(w.x) <= 3.4e38f);
+      bi = bi || !(fabsf(w.z) <= 3.4e38f);
     }
-    for (int o = 16; o > 0; o >>= 1) {
-      mx = fmax(mx, __shfl_xor_sync(0xffffffffu, mx, o));
-      bad = __shfl_xor_sync(0xffffffffu, (int)bad, o) || bad;
-    }
-    if (lane == 0) {
-      const int E = bad ? kBadExp : scale_exp(mx);
-      sm.fexp[cr] = E;
-      a.pexp[BCK((size_t)sh * 2 * kMaxM + cr, (size_t)a.s * 2 * kMaxM)] = E;
+    const int er = __reduce_max_sync(0xffffffffu, br ? kBadExp : scale_exp_f(mr));
+    const int ei = __reduce_max_sync(0xffffffffu, bi ? kBadExp : scale_exp_f(mi));
+    if (lane < 2) {
+      const int E = lane ? ei : er;
+      sm.fexp[2 * q + lane] = E;
+      a.pexp[BCK((size_t)sh * 2 * kMaxM + 2 * q + lane, (size_t)a.s * 2 * kMaxM)] = E;
     }
   }
   __syncthreads();
@@ -431,38 +309,34 @@ __global__ void __launch_bounds__(kPT, 3) tcs_panel_kernel(TcsArgs a, int k, int
     // item = (real column cr, 8 consecutive K rows): seven uint4 stores
     const int g = sh / a.S, slot_row = (sh % a.S) * a.cs;
     const size_t Pg0 = (size_t)g * kSD * kStages * kBT;
-    for (int it = tid; it < 2 * m * (kNBT / 8); it += kPT) {
+    for (int it = tid; it < 2 * m * (kNBT / 8); it += T) {
       const int cr = it / (kNBT / 8), c8 = (it % (kNBT / 8)) * 8;
-      const int q = cr >> 1, E = sm.fexp[cr];
-      unsigned short dg[8][kDigits];
+      const int q = cr >> 1;
+      float hi[8], lo[8];
 #pragma unroll
       for (int e = 0; e < 8; ++e) {
         const int c = c8 + e;
-        double v = 0.0;
+        hi[e] = lo[e] = 0.f;
         if (c < nbe) {
           const float4 w = coef4[c * S + q];
-          v = (cr & 1) ? (double)w.z + (double)w.w : (double)w.x + (double)w.y;
+          hi[e] = (cr & 1) ? w.z : w.x;
+          lo[e] = (cr & 1) ? w.w : w.y;
         }
-        digits8(v, E, dg[e]);
       }
+      uint4 dg[7];
+      digits7_oct(hi, lo, digit_scale(sm.fexp[cr]), dg);
       const int J = c8 / kKS;
       const int off = tile_off(slot_row + cr, c8 % kKS);
 #pragma unroll
-      for (int l = 0; l < kSD; ++l) {
-        uint4 u;
-        u.x = dg[0][l] | ((unsigned)dg[1][l] << 16);
-        u.y = dg[2][l] | ((unsigned)dg[3][l] << 16);
-        u.z = dg[4][l] | ((unsigned)dg[5][l] << 16);
-        u.w = dg[6][l] | ((unsigned)dg[7][l] << 16);
-        *reinterpret_cast<uint4*>(a.Pd + BCK(Pg0 + ((size_t)l * kStages + J) * kBT + off, a.n_pd)) = u;
-      }
+      for (int l = 0; l < kSD; ++l)
+        *reinterpret_cast<uint4*>(a.Pd + BCK(Pg0 + ((size_t)l * kStages + J) * kBT + off, a.n_pd)) = dg[l];
     }
   }
   // ---- P2 and the sigma rows for the update's epilogue
   {
     float4* pc = a.pc + (size_t)sh * 2 * kMaxM * kMaxM;
     const int nsig = min(m, nbe);
-    for (int e = tid; e < 2 * m * m; e += kPT) {
+    for (int e = tid; e < 2 * m * m; e += T) {
       const int row = e / m, q = e % m;
       float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
       if (row < m) v = coef4[(kNBT + row) * S + q];
@@ -475,7 +349,7 @@ __global__ void __launch_bounds__(kPT, 3) tcs_panel_kernel(TcsArgs a, int k, int
   //      (0, 1)) as seven-digit tiles, column-scaled
   if (a.tcz) {
     const int cs = a.cs, kg = cs / 8;
-    for (int c = tid; c < cs; c += kPT) {
+    for (int c = tid; c < cs; c += T) {
       const int q = c >> 1;
       float mx = 0.f;
       if (q < m) {
@@ -491,32 +365,27 @@ __global__ void __launch_bounds__(kPT, 3) tcs_panel_kernel(TcsArgs a, int k, int
     }
     __syncthreads();
     const size_t T0 = (size_t)sh * 7 * cs * cs;
-    for (int it = tid; it < cs * (cs / 8); it += kPT) {
+    for (int it = tid; it < cs * (cs / 8); it += T) {
       const int c = it / (cs / 8), k8 = (it % (cs / 8)) * 8;
       const int q = c >> 1, ro = c & 1, E = sm.f2exp[c];
-      unsigned short dg[8][7];
+      float hi[8], lo[8];
 #pragma unroll
       for (int e = 0; e < 8; ++e) {
         const int kk = k8 + e, qq = kk >> 1, ri = kk & 1;
-        float hi = 0.f, lo = 0.f;
+        hi[e] = lo[e] = 0.f;
         if (q < m && qq < m) {
           const float4 w = coef4[(kNBT + qq) * S + q];
-          if (ri == ro) { hi = w.x; lo = w.y; }
-          else if (ri == 1) { hi = -w.z; lo = -w.w; }
-          else { hi = w.z; lo = w.w; }
+          if (ri == ro) { hi[e] = w.x; lo[e] = w.y; }
+          else if (ri == 1) { hi[e] = -w.z; lo[e] = -w.w; }
+          else { hi[e] = w.z; lo[e] = w.w; }
         }
-        digits7_pair(hi, lo, E, dg[e]);
       }
       const int off = tile_off_kg(c, k8, kg);
+      uint4 dg[7];
+      digits7_oct(hi, lo, digit_scale(E), dg);
 #pragma unroll
-      for (int l = 0; l < 7; ++l) {
-        uint4 u;
-        u.x = dg[0][l] | ((unsigned)dg[1][l] << 16);
-        u.y = dg[2][l] | ((unsigned)dg[3][l] << 16);
-        u.z = dg[4][l] | ((unsigned)dg[5][l] << 16);
-        u.w = dg[6][l] | ((unsigned)dg[7][l] << 16);
-        *reinterpret_cast<uint4*>(a.P2d + BCK(T0 + (size_t)l * cs * cs + off, a.n_p2d)) = u;
-      }
+      for (int l = 0; l < 7; ++l)
+        *reinterpret_cast<uint4*>(a.P2d + BCK(T0 + (size_t)l * cs * cs + off, a.n_p2d)) = dg[l];
     }
   }
   // ---- X-hat mode: P1 rows into ZT, P2 parked in this shift's output rows
@@ -524,102 +393,114 @@ __global__ void __launch_bounds__(kPT, 3) tcs_panel_kernel(TcsArgs a, int k, int
   //      writes them, since every later block is at least m rows high)
   if (a.mode == SSV_XHAT) {
     cd* ZT = a.ZT + (size_t)sh * (size_t)n * m;
-    for (int idx = tid; idx < nbe * m; idx += kPT) {
+    for (int idx = tid; idx < nbe * m; idx += T) {
       const int c = idx % nbe, q = idx / nbe;
       ZT[BCK((j0 + c) + (size_t)q * n, (size_t)n * m)] = df_join(coef4[c * S + q]);
     }
     cd* tout = a.out + (size_t)sh * m * a.ldo;
-    for (int idx = tid; idx < m * m; idx += kPT) {
+    for (int idx = tid; idx < m * m; idx += T) {
       const int qq = idx % m, q = idx / m;
       tout[BCK(n - step * m + qq, n) + (size_t)q * a.ldo] = df_join(coef4[(kNBT + qq) * S + q]);
     }
   }
   // ---- the p rows of Ct: Z2(i, :) = Ct(i, fresh) P1 + Z2(i, :) P2, double-float,
-  //      in chunks of whole rows (each entry reads its row's old values)
-  const int rows_per_chunk = max(1, (2 * kPT) / m);
+  //      in chunks of whole rows (each entry reads its row's old values); the
+  //      chunk of Ct is staged once, ks neighbouring lanes share the sum of one
+  //      entry
+  const int rows_per_chunk = min(kCtRows, max(1, T / m));
   for (int i0 = 0; i0 < p; i0 += rows_per_chunk) {
-  const int ic = min(rows_per_chunk, p - i0);
-  float4 nv[2];
-  int nitem = 0;
-  for (int e = tid; e < ic * m && nitem < 2; e += kPT, ++nitem) {
-    const int i = i0 + e / m, q = e % m;
+    const int ic = min(rows_per_chunk, p - i0);
+    for (int e = tid; e < ic * nbe; e += T) {
+      const int i = e % ic, c = e / ic;
+      const double z = a.Ct[(i0 + i) + (size_t)(j0 + c) * a.ldct];
+      const float zh = (float)z;
+      ct[i * (kNBT + 1) + c] = make_float2(zh, (float)(z - (double)zh));
+    }
+    __syncthreads();
+    int ks = 1;
+    while (ks < 32 && 2 * ks * ic * m <= T) ks <<= 1;
+    const int e = tid / ks, sub = tid % ks;
+    const bool act = e < ic * m;
+    const int i = act ? e / m : 0, q = act ? e % m : 0;
     float rh = 0.f, rl = 0.f, ih = 0.f, il = 0.f;
-    for (int c = 0; c < nbe; ++c) {
-      const double z = a.Ct[i + (size_t)(j0 + c) * a.ldct];
-      const float zh = (float)z, zl = (float)(z - (double)zh);
-      const float4 w = coef4[c * S + q];
-      df_mac(rh, rl, zh, zl, w.x, w.y);
-      df_mac(ih, il, zh, zl, w.z, w.w);
+    if (act) {
+#pragma unroll 4
+      for (int c = sub; c < nbe; c += ks) {
+        const float2 z = ct[i * (kNBT + 1) + c];
+        const float4 w = coef4[c * S + q];
+        df_mac(rh, rl, z.x, z.y, w.x, w.y);
+        df_mac(ih, il, z.x, z.y, w.z, w.w);
+      }
+      for (int qq = sub; qq < m; qq += ks) {
+        const float4 zz = Z2f[BCK((i0 + i) + (size_t)qq * ldz, a.z2_stride)];
+        const float4 w = coef4[(kNBT + qq) * S + q];
+        df_mac(rh, rl, zz.x, zz.y, w.x, w.y);
+        df_mac(rh, rl, -zz.z, -zz.w, w.z, w.w);
+        df_mac(ih, il, zz.x, zz.y, w.z, w.w);
+        df_mac(ih, il, zz.z, zz.w, w.x, w.y);
+      }
     }
-    for (int qq = 0; qq < m; ++qq) {
-      const float4 zz = Z2f[BCK(i + (size_t)qq * ldz, a.z2_stride)];
-      const float4 w = coef4[(kNBT + qq) * S + q];
-      df_mac(rh, rl, zz.x, zz.y, w.x, w.y);
-      df_mac(rh, rl, -zz.z, -zz.w, w.z, w.w);
-      df_mac(ih, il, zz.x, zz.y, w.z, w.w);
-      df_mac(ih, il, zz.z, zz.w, w.x, w.y);
+    for (int o = ks >> 1; o > 0; o >>= 1) {
+      const dw x = dw_add(dw{rh, rl}, dw{__shfl_xor_sync(0xffffffffu, rh, o), __shfl_xor_sync(0xffffffffu, rl, o)});
+      const dw y = dw_add(dw{ih, il}, dw{__shfl_xor_sync(0xffffffffu, ih, o), __shfl_xor_sync(0xffffffffu, il, o)});
+      rh = x.hi; rl = x.lo; ih = y.hi; il = y.lo;
     }
-    const float sr = rh + rl, si = ih + il;
-    nv[nitem] = make_float4(sr, rl - (sr - rh), si, il - (si - ih));
-  }
-  __syncthreads();  // every old entry of these rows is read before any is written
-  nitem = 0;
-  for (int e = tid; e < ic * m && nitem < 2; e += kPT, ++nitem) {
-    const int i = i0 + e / m, q = e % m;
-    Z2f[BCK(i + (size_t)q * ldz, a.z2_stride)] = nv[nitem];
-  }
-  __syncthreads();
+    __syncthreads();  // every old entry of these rows is read before any is written
+    if (act && sub == 0) {
+      const float sr = rh + rl, si = ih + il;
+      Z2f[BCK((i0 + i) + (size_t)q * ldz, a.z2_stride)] = make_float4(sr, rl - (sr - rh), si, il - (si - ih));
+    }
   }
   if (tid == 0 && sm.sing) a.flags[sh] = 1;
 }
 
 // ---- update of the H rows above the block: Z2 <- Z1 P1 + Z2 P2 - sigma E P1 --
-// the level sums of one thread's 16 TMEM columns (lane = its row), each level t
-// scaled by 2^{-7 (t + 2)} and added into double-float sums
-static __device__ __forceinline__ void drain_levels(uint32_t tl, int nlev, float (&ah)[16],
-                                                    float (&al)[16], int lstride = kUN) {
-#pragma unroll
-  for (int c = 0; c < 16; ++c) { ah[c] = 0.f; al[c] = 0.f; }
-  float sc = 0.0078125f * 0.0078125f;  // 2^{-7 (t + 2)}, t = 0
-#pragma unroll 1
-  for (int lv = 0; lv < nlev; ++lv) {
-    uint32_t rr[16];
-    tmem_ld16(tl + (uint32_t)(lv * lstride), rr);
-#pragma unroll
-    for (int c = 0; c < 16; ++c) {
-      const float pv = __uint_as_float(rr[c]) * sc;
-      const float s2 = ah[c] + pv;
-      const float bp = s2 - ah[c];
-      al[c] += (ah[c] - (s2 - bp)) + (pv - bp);
-      ah[c] = s2;
-    }
-    sc *= 0.0078125f;
-  }
+// a += b for double-float a and FP32 b (two-sum)
+static __device__ __forceinline__ void add_f(float& hi, float& lo, float b) {
+  const float s = hi + b;
+  const float bp = s - hi;
+  lo += (hi - (s - bp)) + (b - bp);
+  hi = s;
 }
+// 2^e as FP32 for e in [-126, 127]
+static __device__ __forceinline__ float pow2f(int e) { return __int_as_float((e + 127) << 23); }
+// exponents whose pairwise sums, less the levels' 2^-63, stay in FP32's normal
+// range: rows and columns outside take the ldexpf path
+constexpr int kFastExp = 30;
+static __device__ __forceinline__ bool fast_exp(int e) { return e >= -kFastExp && e <= kFastExp; }
 
 constexpr int kUT = (kUN / 16) * kUM;  // update threads: one per H row of the tile and 16 columns
 
-// The update of block step (k, nbe).  TCZ: Z2 P2 as a second round of digit
-// products on the tensor cores (m >= 5); otherwise in double-float in the
-// epilogue.  Per item (row tile I, group g):
+// The update of block step (k, nbe) for shifts of CS real columns (2m rounded
+// up to a power of two).  CS >= 16: Z2 P2 as a second round of digit products
+// on the tensor cores; otherwise in double-float in the epilogue.  Per item
+// (row tile I, group g):
 //   1. the stages of Z1 P1 (H digit tiles x P1 digit tiles) into the eight
-//      TMEM levels, two stage buffers in flight;
-//   2. TCZ: the group's Z2 and P2 digit tiles are copied into the (then free)
-//      stage buffers while the threads drain the Z1 P1 levels into
+//      TMEM levels, the next stage in flight when there are two buffers;
+//   2. CS >= 16: the group's Z2 and P2 digit tiles are copied into the (then
+//      free) stage buffers while the threads drain the Z1 P1 levels into
 //      double-float sums; then the 28 products of Z2 P2 per shift go into
 //      seven TMEM levels, are drained and added;
 //   3. the next item's first stage streams in during the rest of the epilogue:
-//      the shifted-diagonal correction, the new Z2 rows in double-float and
-//      (TCZ) as digit tiles for the next block step.
-template <bool TCZ>
+//      the shifted-diagonal correction and the new rows: as FP32 pairs the 128
+//      that the next panel (or the final block) reads, all others as the digit
+//      tiles of the next block step (CS < 16: every row as pairs).
+//
+// What bounds it: the instructions of the epilogue (drains, scaling, digits),
+// then the stage copies from L2 (H's eight digit planes, 256 KB an item).  So
+// column arithmetic is resolved at compile time (CS), scaling is one multiply
+// by a power of two, and the digits come from FP32 rounding (digits7_oct).
+template <int CS>
 __global__ void __launch_bounds__(kUT, kCtasU) tcs_update_kernel(TcsArgs a, int k, int nbe) {
+  constexpr bool TCZ = CS >= 16;
+  constexpr int S = kUN / CS;             // shifts of a group
   extern __shared__ __align__(128) unsigned char smem[];
   const int n = a.n, m = a.m, p = a.p, ldz = p + n;
   const int hrows = k - nbe;              // H rows above the block
   const int j0 = k - m - nbe;             // first fresh column (a multiple of 32)
   const int nsig = min(m, nbe);
   const int tid = threadIdx.x, warp = tid >> 5;
-  const int S = a.S, cs = a.cs, G = a.ngroups;
+  const int G = a.ngroups;
   // an earlier launch of this solve gave up a wait: its results are void, skip
   // (the flag is read by every thread and combined, so the whole block agrees)
   if (__syncthreads_or(*(volatile int*)a.err != 0)) return;
@@ -634,9 +515,9 @@ __global__ void __launch_bounds__(kUT, kCtasU) tcs_update_kernel(TcsArgs a, int 
   cd* sig = reinterpret_cast<cd*>(smem + kOffSig);                           // <= kUN shifts
   unsigned long long* mbar = reinterpret_cast<unsigned long long*>(smem + kOffBar);
   uint32_t* tslot = reinterpret_cast<uint32_t*>(smem + kOffSlot);
-  const uint32_t mb = smem_addr(mbar);        // kIss MMA barriers, two stage loads, one Z2 / P2 load
-  const uint32_t lmb0 = mb + 8u * kIss;
-  const uint32_t lmb2 = mb + 8u * (kIss + 2);
+  const uint32_t mb = smem_addr(mbar);        // products, two stage loads, one Z2 / P2 load
+  const uint32_t lmb0 = mb + 8u;
+  const uint32_t lmb2 = mb + 24u;
   const uint32_t sBase = smem_addr(smem);
   if (warp == 0) {
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(
@@ -645,12 +526,11 @@ __global__ void __launch_bounds__(kUT, kCtasU) tcs_update_kernel(TcsArgs a, int 
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;");
   }
   if (tid == 0) {
-    for (int q = 0; q < kIss + 3; ++q) asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(mb + 8u * q));
+    for (int q = 0; q < 4; ++q) asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(mb + 8u * q));
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
-  // the zero tiles of the stage buffers (fused form; the copies never write them)
+  // the zero tiles of the stage buffers (the copies never write them)
   auto zero_tile = [&](int b) {
-    if (!SSV_TCS_FUSED) return;
     uint4* zp = reinterpret_cast<uint4*>(smem + (size_t)b * kStageBytes + kZeroOff);
     for (int e = tid; e < kBT * 2 / 16; e += kUT) zp[e] = make_uint4(0u, 0u, 0u, 0u);
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
@@ -666,9 +546,9 @@ __global__ void __launch_bounds__(kUT, kCtasU) tcs_update_kernel(TcsArgs a, int 
   bool pend2 = false;
   bool failed = false;
   // Z2 / P2 digit bytes of one shift
-  const uint32_t zbytes = 7u * 128u * (uint32_t)cs * 2u;
-  const uint32_t pbytes = 7u * (uint32_t)cs * (uint32_t)cs * 2u;
-  const int kgz = cs / 8;
+  constexpr uint32_t zbytes = 7u * 128u * (uint32_t)CS * 2u;
+  constexpr uint32_t pbytes = 7u * (uint32_t)(CS * CS) * 2u;
+  constexpr int kgz = CS >= 8 ? CS / 8 : 1;
 
   // stage st of item (I, g) into buffer b: eight H digit tiles, seven P1 digit tiles
   auto stage_in = [&](int I, int g, int st, int b) {
@@ -692,10 +572,10 @@ __global__ void __launch_bounds__(kUT, kCtasU) tcs_update_kernel(TcsArgs a, int 
                  : "memory");
     for (int l = 0; l < nsh; ++l) {
       const int sh = g * S + l;
-      bulk_copy(sBase + (uint32_t)l * zbytes, a.Zd + BCK(((size_t)sh * a.RB + I) * 7 * (128 * cs), a.n_zd),
+      bulk_copy(sBase + (uint32_t)l * zbytes, a.Zd + BCK(((size_t)sh * a.RB + I) * 7 * (128 * CS), a.n_zd),
                 zbytes, lmb2);
       bulk_copy(sBase + (uint32_t)S * zbytes + (uint32_t)l * pbytes,
-                a.P2d + BCK((size_t)sh * 7 * cs * cs, a.n_p2d), pbytes, lmb2);
+                a.P2d + BCK((size_t)sh * 7 * CS * CS, a.n_p2d), pbytes, lmb2);
     }
   };
 
@@ -707,20 +587,42 @@ __global__ void __launch_bounds__(kUT, kCtasU) tcs_update_kernel(TcsArgs a, int 
   for (; item < items && !failed; item += gridDim.x) {
     const int I = (int)(item / G), g = (int)(item % G);
     const int nsh = min(S, a.s - g * S);  // shifts of this group
+    // rows of this tile that the sigma rows touch (their correction reads pcs)
+    const bool sigtile = I * kUM < j0 + nsig && I * kUM + kUM > j0;
     // the group's sigma rows (and P2 for the double-float epilogue), column
     // exponents and shifts
-    for (int e = tid; e < S * 2 * m * m; e += kUT) {
-      const int l = e / (2 * m * m), o = e % (2 * m * m);
-      const int sh = g * S + l;
-      pcs[e] = sh < a.s ? a.pc[BCK((size_t)sh * 2 * kMaxM * kMaxM + o, a.n_pc)] : make_float4(0.f, 0.f, 0.f, 0.f);
+    if (!TCZ || sigtile) {
+      for (int e = tid; e < S * 2 * m * m; e += kUT) {
+        const int l = e / (2 * m * m), o = e % (2 * m * m);
+        const int sh = g * S + l;
+        pcs[e] = sh < a.s ? a.pc[BCK((size_t)sh * 2 * kMaxM * kMaxM + o, a.n_pc)] : make_float4(0.f, 0.f, 0.f, 0.f);
+      }
     }
-    for (int e = tid; e < S * cs; e += kUT) {
-      const int l = e / cs, c = e % cs;
+    bool cfast = true;
+    for (int e = tid; e < kUN; e += kUT) {
+      const int l = e / CS, c = e % CS;
       const int sh = g * S + l;
-      fexp[e] = (sh < a.s && c < 2 * m) ? a.pexp[(size_t)sh * 2 * kMaxM + c] : 0;
-      if (TCZ) f2exp[e] = (sh < a.s) ? a.p2exp[(size_t)sh * 2 * kMaxM + c] : 0;
+      const bool use = sh < a.s && c < 2 * m;
+      const int E = use ? a.pexp[(size_t)sh * 2 * kMaxM + c] : 0;
+      fexp[e] = E;
+      if (use && !fast_exp(E)) cfast = false;
+      if (TCZ) {
+        const int E2 = use ? a.p2exp[(size_t)sh * 2 * kMaxM + c] : 0;
+        f2exp[e] = E2;
+        if (!fast_exp(E2)) cfast = false;
+      }
     }
     for (int l = tid; l < S; l += kUT) sig[l] = (g * S + l < a.s) ? a.shifts[g * S + l] : mkcd(0.0, 0.0);
+    const bool slowcol = __syncthreads_or(!cfast);
+    // thread (row, quarter) = (tid mod 128, tid / 128) takes one H row and 16 of
+    // the columns; warps w, w + 4, .. read TMEM lanes 32 (w mod 4) ..
+    const int row = tid & (kUM - 1), qt = tid >> 7;
+    const int ih = I * kUM + row;
+    const bool live = ih < hrows;
+    const int Ei = live ? a.hexp[BCK(ih, a.npad)] : 0;
+    const int shq = g * S + (qt * 16) / CS;  // TCZ: the quarter's shift
+    int Ez = 0;
+    if (TCZ && live && shq < a.s) Ez = a.zexp[BCK((size_t)shq * a.npad + ih, (size_t)a.s * a.npad)];
     // ---- 1. Z1 P1: stage st in buffer st & 1
     for (int st = 0; st < nst; ++st) {
       const int buf = kBufU == 2 ? (st & 1) : 0;
@@ -731,15 +633,11 @@ __global__ void __launch_bounds__(kUT, kCtasU) tcs_update_kernel(TcsArgs a, int 
       }
       lphase[buf] ^= 1u;
       pend[buf] = false;
-      const int iss = tid >> 5;
-#if SSV_TCS_FUSED
       // fused levels: the P1 digit tiles sit side by side (kUN rows each, then
       // the zero tile), so one product of H digit kd against P1 digits
       // b0 .. b0 + c - 1 (N = kUN c <= 256) lands digit b in TMEM level kd + b;
       // the kd = 0 products cover every level and open the item, so one thread
-      // issues all of them, and commits to every issuer barrier (their phases
-      // stay in step with the Z2 P2 round)
-      (void)iss;
+      // issues all of them
       if (tid == 0) {
         fence_after();
         const uint32_t aBase = sBase + (uint32_t)buf * kStageBytes;
@@ -761,40 +659,15 @@ __global__ void __launch_bounds__(kUT, kCtasU) tcs_update_kernel(TcsArgs a, int 
             }
           }
         }
-        for (int q = 0; q < kIss; ++q) mma_commit(mb + 8u * (uint32_t)q);
+        mma_commit(mb);
       }
-#else
-      if ((tid & 31) == 0 && iss < kIss) {
-        fence_after();
-        const uint32_t aBase = sBase + (uint32_t)buf * kStageBytes;
-        const uint32_t bBase = aBase + (uint32_t)(kSDH * kAT * 2);
-        constexpr uint32_t kSbo = (uint32_t)kKG * 128u;
-#pragma unroll 1
-        for (int lv = 0; lv < kLev; ++lv) {
-          if (level_owner(lv) != iss) continue;
-#pragma unroll 1
-          for (int kd = max(0, lv - (kSD - 1)); kd <= min(kSDH - 1, lv); ++kd) {
-            const int ld = lv - kd;
-#pragma unroll
-            for (int ks = 0; ks < kKS / 16; ++ks) {
-              const uint64_t ad = mat_desc(aBase + (uint32_t)(kd * kAT * 2 + ks * 256), 128u, kSbo);
-              const uint64_t bd = mat_desc(bBase + (uint32_t)(ld * kBT * 2 + ks * 256), 128u, kSbo);
-              const bool first = st == 0 && kd == max(0, lv - (kSD - 1)) && ks == 0;
-              mma_bf16(tmem + (uint32_t)(lv * kUN), ad, bd, kIdescU, first ? 0u : 1u);
-            }
-          }
-        }
-        mma_commit(mb + 8u * (uint32_t)iss);
-      }
-#endif
       // the next stage streams into the other buffer, whose products finished
       // in the previous round (with one buffer: after these products)
       if (kBufU == 2 && st + 1 < nst) {
         pend[buf ^ 1] = true;
         if (tid == 0) stage_in(I, g, st + 1, buf ^ 1);
       }
-      bool ok = true;
-      for (int q = 0; q < kIss; ++q) ok = mbar_wait(mb + 8u * q, mphase, kUpdWait) && ok;
+      const bool ok = mbar_wait(mb, mphase, kUpdWait);
       if (__syncthreads_or(!ok)) {
         failed = true;
         break;
@@ -806,49 +679,49 @@ __global__ void __launch_bounds__(kUT, kCtasU) tcs_update_kernel(TcsArgs a, int 
       }
     }
     if (failed) break;
-    // both stage buffers are free: TCZ fetches the group's Z2 / P2 tiles into them
+    // the stage buffers are free: TCZ fetches the group's Z2 / P2 tiles into them
     if (TCZ) {
       pend2 = true;
       if (tid == 0) z2_in(I, g, nsh);
     }
-    // ---- epilogue: thread (row, quarter) = (tid mod 128, tid / 128) takes one H
-    //      row and 16 of the 64 columns; warps w, w + 4, w + 8, w + 12 read TMEM
-    //      lanes 32 (w mod 4) ..
+    // ---- epilogue
     fence_after();
-    const int row = tid & (kUM - 1), qt = tid >> 7;
-    const int ih = I * kUM + row;
-    const bool live = ih < hrows;
-    const int Ei = live ? a.hexp[BCK(ih, a.npad)] : 0;
-    const int cdr = ih - j0;  // shifted-diagonal correction row of fresh column cdr
-    const uint32_t tl = tmem + ((uint32_t)((warp & 3) * 32) << 16) + (uint32_t)(qt * 16);
-    float4 acc[8];
-    bool ok_j[8];
-    {
-      float ah[16], al[16];
-      drain_levels(tl, kLev, ah, al);
-      // slot j (0 .. 7) of this quarter = group columns col, col + 1 with
-      // col = 16 qt + 2 j: shift l = col / cs, complex column q = (col mod cs) / 2
+    const uint32_t tl = tmem + ((uint32_t)((warp & 3) * 32) << 16);
+    // the new entries, 16 real columns of the row (Re, Im interleaved), as pairs
+    float ah[16], al[16];
 #pragma unroll
-      for (int j = 0; j < 8; ++j) {
-        const int col = qt * 16 + 2 * j, l = col / cs, q = (col % cs) >> 1;
-        ok_j[j] = live && q < m && l < S && g * S + l < a.s;
-        acc[j] = make_float4(0.f, 0.f, 0.f, 0.f);
-        if (ok_j[j]) {
-          const int er = fexp[col], ei = fexp[col + 1];
-          if (Ei == kBadExp || er == kBadExp || ei == kBadExp) {
-            acc[j] = make_float4(__int_as_float(0x7fc00000), 0.f, __int_as_float(0x7fc00000), 0.f);
-          } else {
-            acc[j] = make_float4(ldexpf(ah[2 * j], Ei + er), ldexpf(al[2 * j], Ei + er),
-                                 ldexpf(ah[2 * j + 1], Ei + ei), ldexpf(al[2 * j + 1], Ei + ei));
-          }
-        }
+    for (int c = 0; c < 16; ++c) { ah[c] = 0.f; al[c] = 0.f; }
+    {
+      float sc = 0.0078125f * 0.0078125f;  // 2^{-7 (t + 2)}, t = 0
+#pragma unroll 1
+      for (int lv = 0; lv < kLev; ++lv) {
+        uint32_t rr[16];
+        tmem_ld16(tl + (uint32_t)(lv * kUN + qt * 16), rr);
+#pragma unroll
+        for (int c = 0; c < 16; ++c) add_f(ah[c], al[c], __uint_as_float(rr[c]) * sc);
+        sc *= 0.0078125f;
+      }
+    }
+    const bool fast = !slowcol && fast_exp(Ei) && (!TCZ || fast_exp(Ez));
+#pragma unroll
+    for (int c = 0; c < 16; ++c) {
+      const int col = qt * 16 + c, Ec = fexp[col];
+      if (fast) {
+        const float f = pow2f(Ei + Ec);
+        ah[c] *= f;
+        al[c] *= f;
+      } else if (Ei == kBadExp || Ec == kBadExp) {
+        ah[c] = __int_as_float(0x7fc00000);
+        al[c] = 0.f;
+      } else {
+        ah[c] = ldexpf(ah[c], Ei + Ec);
+        al[c] = ldexpf(al[c], Ei + Ec);
       }
     }
     if (TCZ) {
       // ---- 2. Z2 P2: the levels of Z1 P1 are read; the same TMEM columns take
       //      the seven levels of the group's Z2 digit tiles x P2 digit tiles
       fence_before();
-      __syncthreads();
       const bool lok = mbar_wait(lmb2, l2phase, kUpdWait);
       if (__syncthreads_or(!lok)) {
         failed = true;
@@ -856,61 +729,30 @@ __global__ void __launch_bounds__(kUT, kCtasU) tcs_update_kernel(TcsArgs a, int 
       }
       l2phase ^= 1u;
       pend2 = false;
-      const int iss = tid >> 5;
-#if SSV_TCS_FUSED
       // fused levels: shift l's seven levels sit side by side in TMEM (columns
-      // 7 cs l + cs lv) and its P2 digit tiles (cs rows each) are stacked, so one
-      // product of Z2 digit kd against P2 digits 0 .. 6 - kd (N = cs (7 - kd))
+      // 7 CS l + CS lv) and its P2 digit tiles (CS rows each) are stacked, so one
+      // product of Z2 digit kd against P2 digits 0 .. 6 - kd (N = CS (7 - kd))
       // lands digit ld in level kd + ld; kd = 0 opens all seven
-      (void)iss;
       if (tid == 0) {
         fence_after();
-        const uint32_t sboz = (uint32_t)kgz * 128u;
+        constexpr uint32_t sboz = (uint32_t)kgz * 128u;
         for (int l = 0; l < nsh; ++l) {
           const uint32_t zb = sBase + (uint32_t)l * zbytes;
           const uint32_t pb = sBase + (uint32_t)S * zbytes + (uint32_t)l * pbytes;
 #pragma unroll 1
-          for (int ks = 0; ks < cs / 16; ++ks) {
+          for (int ks = 0; ks < CS / 16; ++ks) {
 #pragma unroll
             for (int kd = 0; kd < 7; ++kd) {
-              const uint64_t ad = mat_desc(zb + (uint32_t)(kd * 128 * cs * 2 + ks * 256), 128u, sboz);
+              const uint64_t ad = mat_desc(zb + (uint32_t)(kd * 128 * CS * 2 + ks * 256), 128u, sboz);
               const uint64_t bd = mat_desc(pb + (uint32_t)(ks * 256), 128u, sboz);
-              mma_bf16(tmem + (uint32_t)(7 * cs * l + kd * cs), ad, bd, idesc_bf16(kUM, cs * (7 - kd)),
+              mma_bf16(tmem + (uint32_t)(7 * CS * l + kd * CS), ad, bd, idesc_bf16(kUM, CS * (7 - kd)),
                        (kd == 0 && ks == 0) ? 0u : 1u);
             }
           }
         }
-        for (int q = 0; q < kIss; ++q) mma_commit(mb + 8u * (uint32_t)q);
+        mma_commit(mb);
       }
-#else
-      if ((tid & 31) == 0 && iss < kIss) {
-        fence_after();
-        const uint32_t idz = idesc_bf16(kUM, cs);
-        const uint32_t sboz = (uint32_t)kgz * 128u;
-#pragma unroll 1
-        for (int lv = 0; lv < 7; ++lv) {
-          if (level_owner(lv) != iss) continue;
-#pragma unroll 1
-          for (int l = 0; l < nsh; ++l) {
-            const uint32_t zb = sBase + (uint32_t)l * zbytes;
-            const uint32_t pb = sBase + (uint32_t)S * zbytes + (uint32_t)l * pbytes;
-#pragma unroll 1
-            for (int kd = 0; kd <= lv; ++kd) {
-              const int ld = lv - kd;
-#pragma unroll 1
-              for (int ks = 0; ks < cs / 16; ++ks) {
-                const uint64_t ad = mat_desc(zb + (uint32_t)(kd * 128 * cs * 2 + ks * 256), 128u, sboz);
-                const uint64_t bd = mat_desc(pb + (uint32_t)(ld * cs * cs * 2 + ks * 256), 128u, sboz);
-                mma_bf16(tmem + (uint32_t)(lv * kUN + l * cs), ad, bd, idz, (kd == 0 && ks == 0) ? 0u : 1u);
-              }
-            }
-          }
-        }
-        mma_commit(mb + 8u * (uint32_t)iss);
-      }
-#endif
-      bool ok = true;
-      for (int q = 0; q < kIss; ++q) ok = mbar_wait(mb + 8u * q, mphase, kUpdWait) && ok;
+      const bool ok = mbar_wait(mb, mphase, kUpdWait);
       if (__syncthreads_or(!ok)) {
         failed = true;
         break;
@@ -919,6 +761,7 @@ __global__ void __launch_bounds__(kUT, kCtasU) tcs_update_kernel(TcsArgs a, int 
       // the Z2 / P2 tiles covered buffer 0's zero tile: write it again before
       // the next item's first products read it (ordered by the load wait and
       // barrier that precede them)
+#pragma unroll
       for (int b = 0; b < kBufU; ++b)
         if ((size_t)b * kStageBytes + kZeroOff < (size_t)S * (zbytes + pbytes)) zero_tile(b);
     }
@@ -929,132 +772,153 @@ __global__ void __launch_bounds__(kUT, kCtasU) tcs_update_kernel(TcsArgs a, int 
       pend[0] = true;
       if (tid == 0) stage_in((int)(nx / G), (int)(nx % G), 0, 0);
     }
-    if (TCZ) {
+    if constexpr (TCZ) {
       fence_after();
-      float ah[16], al[16];
-#if SSV_TCS_FUSED
-      // shift l = (16 qt) / cs: its levels start at column 7 cs l, this
-      // quarter's columns at (16 qt) mod cs within them
-      drain_levels(tl - (uint32_t)(qt * 16) + (uint32_t)(7 * cs * ((qt * 16) / cs) + (qt * 16) % cs), 7, ah, al,
-                   cs);
-#else
-      drain_levels(tl, 7, ah, al);
-#endif
-      const int l = (qt * 16) / cs;  // one shift per quarter (cs >= 16)
-      const int sh = g * S + l;
-      const int Ez = (live && sh < a.s) ? a.zexp[BCK((size_t)sh * a.npad + ih, (size_t)a.s * a.npad)] : 0;
+      // shift l = (16 qt) / CS: its levels start at column 7 CS l, this
+      // quarter's columns at (16 qt) mod CS within them
+      const uint32_t tz = tl + (uint32_t)(7 * CS * ((qt * 16) / CS) + (qt * 16) % CS);
+      if (fast) {
+        float f[16];
 #pragma unroll
-      for (int j = 0; j < 8; ++j) {
-        if (!ok_j[j]) continue;
-        const int col = qt * 16 + 2 * j;
-        const int fr = f2exp[col], fi = f2exp[col + 1];
-        if (Ez == kBadExp || fr == kBadExp || fi == kBadExp) {
-          acc[j] = make_float4(__int_as_float(0x7fc00000), 0.f, __int_as_float(0x7fc00000), 0.f);
-          continue;
+        for (int c = 0; c < 16; ++c) f[c] = pow2f(Ez + f2exp[qt * 16 + c] - 14);
+#pragma unroll 1
+        for (int lv = 0; lv < 7; ++lv) {
+          uint32_t rr[16];
+          tmem_ld16(tz + (uint32_t)(lv * CS), rr);
+#pragma unroll
+          for (int c = 0; c < 16; ++c) {
+            add_f(ah[c], al[c], __uint_as_float(rr[c]) * f[c]);
+            f[c] *= 0.0078125f;
+          }
         }
-        // acc += level sum, both double-float: two-sum of the high words
-        auto addpair = [](float& h, float& lo, float bh, float bl) {
-          const float s2 = h + bh;
-          const float bp = s2 - h;
-          lo += ((h - (s2 - bp)) + (bh - bp)) + bl;
-          h = s2;
-        };
-        addpair(acc[j].x, acc[j].y, ldexpf(ah[2 * j], Ez + fr), ldexpf(al[2 * j], Ez + fr));
-        addpair(acc[j].z, acc[j].w, ldexpf(ah[2 * j + 1], Ez + fi), ldexpf(al[2 * j + 1], Ez + fi));
+      } else {
+        // one column at a time: its levels into a pair, scaled by ldexpf
+#pragma unroll 1
+        for (int c8 = 0; c8 < 16; c8 += 8) {
+          float bh[8], bl[8];
+#pragma unroll
+          for (int c = 0; c < 8; ++c) { bh[c] = 0.f; bl[c] = 0.f; }
+          float sc = 0.0078125f * 0.0078125f;
+#pragma unroll 1
+          for (int lv = 0; lv < 7; ++lv) {
+            uint32_t rr[8];
+            tmem_ld8(tz + (uint32_t)(lv * CS + c8), rr);
+#pragma unroll
+            for (int c = 0; c < 8; ++c) add_f(bh[c], bl[c], __uint_as_float(rr[c]) * sc);
+            sc *= 0.0078125f;
+          }
+#pragma unroll
+          for (int c = 0; c < 16; ++c) {
+            if ((c & 8) != c8) continue;
+            const int Ec = f2exp[qt * 16 + c];
+            if (Ez == kBadExp || Ec == kBadExp) {
+              ah[c] = __int_as_float(0x7fc00000);
+              al[c] = 0.f;
+            } else {
+              add_f(ah[c], al[c], ldexpf(bh[c & 7], Ez + Ec));
+              al[c] += ldexpf(bl[c & 7], Ez + Ec);
+            }
+          }
+        }
       }
     } else if (live) {
       // several shifts per quarter (m <= 4): + Z2(row, :) P2(:, q) in
       // double-float from the old row of each slot's shift
-#pragma unroll 1
-      for (int qq = 0; qq < m; ++qq) {
-        int lz = -1;
-        float4 zz = make_float4(0.f, 0.f, 0.f, 0.f);
+      constexpr int CC = CS / 2;  // complex columns of a shift
 #pragma unroll
-        for (int j = 0; j < 8; ++j) {
-          if (!ok_j[j]) continue;
-          const int col = qt * 16 + 2 * j, l = col / cs, q = (col % cs) >> 1;
-          if (l != lz) {
-            zz = a.Z2[BCK((size_t)(g * S + l) * a.z2_stride + (p + ih) + (size_t)qq * ldz, a.n_z2)];
-            lz = l;
+      for (int l0 = 0; l0 < 16 / CS; ++l0) {
+        const int l = qt * 16 / CS + l0;
+        if (g * S + l < a.s) {
+          const float4* z = a.Z2 + BCK((size_t)(g * S + l) * a.z2_stride + (p + ih), a.n_z2);
+          float4 zz[CC];
+#pragma unroll
+          for (int qq = 0; qq < CC; ++qq) zz[qq] = qq < m ? z[(size_t)qq * ldz] : make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+          for (int q = 0; q < CC; ++q) {
+            if (q >= m) continue;
+            const int c = l0 * CS + 2 * q;
+#pragma unroll
+            for (int qq = 0; qq < CC; ++qq) {
+              if (qq >= m) continue;
+              const float4 w = pcs[(size_t)l * 2 * m * m + qq * m + q];
+              df_mac(ah[c], al[c], zz[qq].x, zz[qq].y, w.x, w.y);
+              df_mac(ah[c], al[c], -zz[qq].z, -zz[qq].w, w.z, w.w);
+              df_mac(ah[c + 1], al[c + 1], zz[qq].x, zz[qq].y, w.z, w.w);
+              df_mac(ah[c + 1], al[c + 1], zz[qq].z, zz[qq].w, w.x, w.y);
+            }
           }
-          const float4 w = pcs[(size_t)l * 2 * m * m + qq * m + q];
-          df_mac(acc[j].x, acc[j].y, zz.x, zz.y, w.x, w.y);
-          df_mac(acc[j].x, acc[j].y, -zz.z, -zz.w, w.z, w.w);
-          df_mac(acc[j].z, acc[j].w, zz.x, zz.y, w.z, w.w);
-          df_mac(acc[j].z, acc[j].w, zz.z, zz.w, w.x, w.y);
         }
       }
     }
+    const int cdr = ih - j0;  // shifted-diagonal correction row of fresh column cdr
     if (live && cdr >= 0 && cdr < nsig) {
       // - sigma P1(cdr, q)
 #pragma unroll
-      for (int j = 0; j < 8; ++j) {
-        if (!ok_j[j]) continue;
-        const int col = qt * 16 + 2 * j, l = col / cs, q = (col % cs) >> 1;
+      for (int c = 0; c < 16; c += 2) {
+        const int col = qt * 16 + c, l = col / CS, q = (col % CS) >> 1;
+        if (q >= m || g * S + l >= a.s) continue;
         const float4 sgf = df_split(sig[l]);
         const float4 w = pcs[(size_t)l * 2 * m * m + m * m + cdr * m + q];
-        df_mac(acc[j].x, acc[j].y, -sgf.x, -sgf.y, w.x, w.y);
-        df_mac(acc[j].x, acc[j].y, sgf.z, sgf.w, w.z, w.w);
-        df_mac(acc[j].z, acc[j].w, -sgf.x, -sgf.y, w.z, w.w);
-        df_mac(acc[j].z, acc[j].w, -sgf.z, -sgf.w, w.x, w.y);
+        df_mac(ah[c], al[c], -sgf.x, -sgf.y, w.x, w.y);
+        df_mac(ah[c], al[c], sgf.z, sgf.w, w.z, w.w);
+        df_mac(ah[c + 1], al[c + 1], -sgf.x, -sgf.y, w.z, w.w);
+        df_mac(ah[c + 1], al[c + 1], -sgf.z, -sgf.w, w.x, w.y);
       }
     }
     // normalised pairs
 #pragma unroll
-    for (int j = 0; j < 8; ++j) {
-      const float sr = acc[j].x + acc[j].y, si = acc[j].z + acc[j].w;
-      acc[j] = make_float4(sr, acc[j].y - (sr - acc[j].x), si, acc[j].w - (si - acc[j].z));
+    for (int c = 0; c < 16; ++c) {
+      const float s = ah[c] + al[c];
+      al[c] = al[c] - (s - ah[c]);
+      ah[c] = s;
     }
-    float mx = 0.f;
-    if (TCZ) {
-      // the new row's digit exponent: the maximum over the shift's 2m entries,
-      // which two quarters share when cs = 32
+    // the new rows as pairs: those of the next panel or the final block
+    const bool pairs = !TCZ || ih >= hrows - kNBT;
+    if (live && pairs) {
 #pragma unroll
-      for (int j = 0; j < 8; ++j) {
-        if (!ok_j[j]) continue;
-        mx = fmaxf(mx, fmaxf(fabsf(acc[j].x), fabsf(acc[j].z)));
-        if (!(fabsf(acc[j].x) <= 3.4e38f) || !(fabsf(acc[j].z) <= 3.4e38f)) mx = __int_as_float(0x7f800000);
+      for (int c = 0; c < 16; c += 2) {
+        const int col = qt * 16 + c, l = col / CS, q = (col % CS) >> 1;
+        if (q >= m || g * S + l >= a.s) continue;
+        a.Z2[BCK((size_t)(g * S + l) * a.z2_stride + (p + ih) + (size_t)q * ldz, a.n_z2)] =
+            make_float4(ah[c], al[c], ah[c + 1], al[c + 1]);
       }
-      xmax[qt * kUM + row] = mx;
     }
-    // a shift's row may be shared by two quarters: every old entry (double-float
-    // path) and every maximum is read before the writes below
-    __syncthreads();
+    // as digits: the rows above them (none of a tile that lies within the last 128 rows)
+    if (TCZ && I * kUM < hrows - kNBT) {
+      // the row's digit exponent: the maximum over the shift's 2m entries,
+      // which two quarters share when CS = 32
+      float mx = 0.f;
+      bool bad = false;
 #pragma unroll
-    for (int j = 0; j < 8; ++j) {
-      if (!ok_j[j]) continue;
-      const int col = qt * 16 + 2 * j, l = col / cs, q = (col % cs) >> 1;
-      a.Z2[BCK((size_t)(g * S + l) * a.z2_stride + (p + ih) + (size_t)q * ldz, a.n_z2)] = acc[j];
-    }
-    if (TCZ && live) {
-      const int l = (qt * 16) / cs, sh = g * S + l;
-      if (sh < a.s) {
-        if (cs == 32) mx = fmaxf(mx, xmax[(qt ^ 1) * kUM + row]);
+      for (int c = 0; c < 16; ++c) {
+        if ((qt * 16 + c) % CS >= 2 * m) { ah[c] = 0.f; al[c] = 0.f; }
+        mx = fmaxf(mx, fabsf(ah[c]));
+        bad = bad || !(fabsf(ah[c]) <= 3.4e38f);
+      }
+      if (bad) mx = __int_as_float(0x7f800000);
+      if (CS == 32) {
+        xmax[qt * kUM + row] = mx;
+        __syncthreads();
+        mx = fmaxf(mx, xmax[(qt ^ 1) * kUM + row]);
+      }
+      if (live && shq < a.s) {
         const int E = scale_exp_f(mx);
-        const int kb = (qt * 16) % cs;  // this quarter's first K entry of the row
-        if ((qt * 16) % cs == 0) a.zexp[BCK((size_t)sh * a.npad + ih, (size_t)a.s * a.npad)] = E;
-        const size_t T0 = ((size_t)sh * a.RB + I) * 7 * (128 * cs);
+        constexpr int kbm = CS - 1;
+        const int kb = (qt * 16) & kbm;  // this quarter's first K entry of the row
+        if (kb == 0) a.zexp[BCK((size_t)shq * a.npad + ih, (size_t)a.s * a.npad)] = E;
+        const float inv = digit_scale(E);
+        const size_t T0 = ((size_t)shq * a.RB + I) * 7 * (128 * CS);
 #pragma unroll
         for (int h = 0; h < 2; ++h) {
-          unsigned short dg[8][7];
+          float hi[8], lo[8];
 #pragma unroll
-          for (int e = 0; e < 8; ++e) {
-            const int j = h * 4 + (e >> 1);
-            const bool use = ok_j[j];
-            const float hi = use ? ((e & 1) ? acc[j].z : acc[j].x) : 0.f;
-            const float lo = use ? ((e & 1) ? acc[j].w : acc[j].y) : 0.f;
-            digits7_pair(hi, lo, E, dg[e]);
-          }
+          for (int e = 0; e < 8; ++e) { hi[e] = ah[h * 8 + e]; lo[e] = al[h * 8 + e]; }
+          uint4 dg[7];
+          digits7_oct(hi, lo, inv, dg);
           const int off = tile_off_kg(row, kb + h * 8, kgz);
 #pragma unroll
-          for (int l2 = 0; l2 < 7; ++l2) {
-            uint4 u;
-            u.x = dg[0][l2] | ((unsigned)dg[1][l2] << 16);
-            u.y = dg[2][l2] | ((unsigned)dg[3][l2] << 16);
-            u.z = dg[4][l2] | ((unsigned)dg[5][l2] << 16);
-            u.w = dg[6][l2] | ((unsigned)dg[7][l2] << 16);
-            *reinterpret_cast<uint4*>(a.Zd + BCK(T0 + (size_t)l2 * (128 * cs) + off, a.n_zd)) = u;
-          }
+          for (int l2 = 0; l2 < 7; ++l2)
+            *reinterpret_cast<uint4*>(a.Zd + BCK(T0 + (size_t)l2 * (128 * CS) + off, a.n_zd)) = dg[l2];
         }
       }
     }
@@ -1066,7 +930,7 @@ __global__ void __launch_bounds__(kUT, kCtasU) tcs_update_kernel(TcsArgs a, int 
     // flight one more bounded wait, then release TMEM
     if (tid == 0) {
       atomicExch(a.err, 1);
-      for (int q = 0; q < kIss; ++q) mbar_wait(mb + 8u * q, mphase, kUpdWait);
+      mbar_wait(mb, mphase, kUpdWait);
       for (int b = 0; b < 2; ++b)
         if (pend[b]) mbar_wait(lmb0 + 8u * (uint32_t)b, lphase[b], kUpdWait);
       if (pend2) mbar_wait(lmb2, l2phase, kUpdWait);
@@ -1089,7 +953,7 @@ __global__ void tcs_canary_kernel(const unsigned char* c, size_t nbytes, int* er
 #endif
 
 // ---- final m x m block, G or the X-hat back pass ----------------------------
-__global__ void __launch_bounds__(kPT) tcs_final_kernel(TcsArgs a, int nsteps, int nbe_first) {
+__global__ void __launch_bounds__(kPT) tcs_final_kernel(TcsArgs a, int nsteps) {
   __shared__ cd Wm[kMaxM * 2 * kMaxM];
   __shared__ cd lmul[kMaxM];
   __shared__ cd Yb[kMaxM * kMaxM];
@@ -1171,24 +1035,20 @@ __global__ void __launch_bounds__(kPT) tcs_final_kernel(TcsArgs a, int nsteps, i
       tout[BCK(i, p) + (size_t)q * a.ldo] = mkcd(sgn * acc.x, sgn * acc.y);
     }
   } else {
-    // backward pass: z = Y; per step b = B .. 1: X-hat rows of b = P1_b z,
-    // then z = P2_b z; the initial live rows n - m .. n - 1 take the last z.
-    // Step b covers the fresh columns j0_b = (B - b) n_b .. + nbe_b - 1.
-    const cd* ZT = a.ZT + (size_t)sh * (size_t)n * m;
+    // backward pass: z_B = Y; per step b = B .. 1: X-hat rows of b = P1_b z_b,
+    // then z_{b-1} = P2_b z_b; the initial live rows n - m .. n - 1 take the
+    // last z.  Only the chain of the z_b runs here: they go into the shift's
+    // window state (dead by now; nsteps m <= n), and tcs_back_kernel forms the
+    // X-hat rows of all blocks at once.
+    cd* zb = reinterpret_cast<cd*>(a.Z2 + (size_t)sh * a.z2_stride);
     for (int e = tid; e < m * m; e += kPT) zs[(e % m) + (e / m) * kMaxM] = Yb[(e % m) + (e / m) * kMaxM];
     __syncthreads();
     for (int b = nsteps; b >= 1; --b) {
-      const int nbe_b = b == 1 ? nbe_first : kNBT;
-      const int j0b = (nsteps - b) * kNBT;
-      for (int e = tid; e < m * m; e += kPT)
+      for (int e = tid; e < m * m; e += kPT) {
         p2s[(e % m) + (e / m) * kMaxM] = tout[BCK(n - b * m + e % m, n) + (size_t)(e / m) * a.ldo];
-      __syncthreads();
-      for (int idx = tid; idx < nbe_b * m; idx += kPT) {
-        const int i = j0b + idx % nbe_b, q = idx / nbe_b;
-        cd acc = mkcd(0.0, 0.0);
-        for (int t = 0; t < m; ++t) acc = cfma(ZT[BCK(i + (size_t)t * n, (size_t)n * m)], zs[t + q * kMaxM], acc);
-        tout[BCK(i, n) + (size_t)q * a.ldo] = bad ? mkcd(nanv, nanv) : acc;
+        zb[BCK((size_t)(b - 1) * m * m + e, a.z2_stride)] = zs[(e % m) + (e / m) * kMaxM];
       }
+      __syncthreads();
       for (int e = tid; e < m * m; e += kPT) {
         const int rr = e % m, q = e / m;
         cd acc = mkcd(0.0, 0.0);
@@ -1203,6 +1063,7 @@ __global__ void __launch_bounds__(kPT) tcs_final_kernel(TcsArgs a, int nsteps, i
       const int rr = e % m, q = e / m;
       tout[(n - m + rr) + (size_t)q * a.ldo] = bad ? mkcd(nanv, nanv) : zs[rr + q * kMaxM];
     }
+    if (tid == 0) a.flags[sh] = bad ? 1 : 0;
   }
   if (a.status != nullptr && tid == 0) {
     bool fin = true;
@@ -1212,6 +1073,59 @@ __global__ void __launch_bounds__(kPT) tcs_final_kernel(TcsArgs a, int nsteps, i
     }
     a.status[sh] = sing ? SSV_SHIFT_SINGULAR : ((fin && !failed) ? SSV_SHIFT_OK : SSV_SHIFT_NONFINITE);
   }
+}
+
+// X-hat rows of block step b = blockIdx.x mod B + 1 (fresh columns j0_b = (B - b) n_b
+// .. + nbe_b - 1): P1_b z_b, FP64.  One CTA per (block, shift); two threads per
+// row, each half of the m columns.  Bound by the FP64 pipe (4 n m^2
+// multiply-adds a shift); inside the serial chain of the z_b, on one SM per
+// shift, it took 1.34 ms for 40 shifts at n = 4000, m = 16.
+__global__ void __launch_bounds__(kPT) tcs_back_kernel(TcsArgs a, int nsteps, int nbe_first) {
+  __shared__ cd zs[kMaxM * kMaxM];
+  const int b = blockIdx.x % nsteps + 1, sh = blockIdx.x / nsteps, tid = threadIdx.x;
+  const int n = a.n, m = a.m;
+  const int nbe_b = b == 1 ? nbe_first : kNBT;
+  const int j0b = (nsteps - b) * kNBT;
+  const cd* zb = reinterpret_cast<const cd*>(a.Z2 + (size_t)sh * a.z2_stride) + (size_t)(b - 1) * m * m;
+  for (int e = tid; e < m * m; e += kPT) zs[e] = zb[BCK(e, a.z2_stride)];
+  const bool bad = a.flags[sh] != 0 || *a.err != 0;
+  __syncthreads();
+  const int i = j0b + (tid & (kNBT - 1)), half = tid / kNBT;
+  if (i >= j0b + nbe_b) return;
+  const cd* ZT = a.ZT + (size_t)sh * (size_t)n * m;
+  cd* tout = a.out + (size_t)sh * m * a.ldo;
+  const double nanv = __longlong_as_double(0x7ff8000000000000LL);
+  const int qh = (m + 1) / 2, q0 = half * qh, q1 = min(m, q0 + qh);
+  cd acc[kMaxM / 2];
+#pragma unroll
+  for (int u = 0; u < kMaxM / 2; ++u) acc[u] = mkcd(0.0, 0.0);
+#pragma unroll 4
+  for (int t = 0; t < m; ++t) {
+    const cd x = ZT[BCK(i + (size_t)t * n, (size_t)n * m)];
+#pragma unroll
+    for (int u = 0; u < kMaxM / 2; ++u)
+      if (q0 + u < q1) acc[u] = cfma(x, zs[t + (q0 + u) * m], acc[u]);
+  }
+#pragma unroll
+  for (int u = 0; u < kMaxM / 2; ++u)
+    if (q0 + u < q1) tout[BCK(i, n) + (size_t)(q0 + u) * a.ldo] = bad ? mkcd(nanv, nanv) : acc[u];
+}
+
+// the panel kernel for up to MAXM live columns
+struct PanelLaunch {
+  void (*kern)(TcsArgs, int, int, int);
+  int threads;
+  size_t smem;
+};
+template <int MAXM, bool FEW = false>
+PanelLaunch panel_config(cudaError_t* e) {
+  PanelLaunch l{tcs_panel_kernel<MAXM, FEW>, panel_threads<MAXM, FEW>(), sizeof(PanelSmem<MAXM>)};
+  if (*e == cudaSuccess)
+    *e = cudaFuncSetAttribute(l.kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)l.smem);
+  if (*e == cudaSuccess)
+    *e = cudaFuncSetAttribute(l.kern, cudaFuncAttributePreferredSharedMemoryCarveout,
+                              (int)cudaSharedmemCarveoutMaxShared);
+  return l;
 }
 
 }  // namespace
@@ -1314,18 +1228,18 @@ int solve_tc(const Handle* h, int s, const double* shifts, int mode, double* out
     const unsigned char* hb = static_cast<const unsigned char*>(hdig);
     a.Hs = reinterpret_cast<const uint4*>(hb);
     a.hexp = reinterpret_cast<const int*>(hb + ((size_t)kDigits * np * np * 2 + 255) / 256 * 256);
-    const size_t psm = sizeof(PanelSmem);
-    e = cudaFuncSetAttribute(tcs_panel_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)psm);
-    // three panels per SM (74 KB of shared memory each)
-    if (e == cudaSuccess)
-      e = cudaFuncSetAttribute(tcs_panel_kernel, cudaFuncAttributePreferredSharedMemoryCarveout,
-                               (int)cudaSharedmemCarveoutMaxShared);
-    if (e == cudaSuccess)
-      e = cudaFuncSetAttribute(tcs_update_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                               (int)kUpdSmem);
-    if (e == cudaSuccess)
-      e = cudaFuncSetAttribute(tcs_update_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                               (int)kUpdSmem);
+    PanelLaunch panel = m <= 1   ? panel_config<1>(&e)
+                        : m <= 2 ? panel_config<2>(&e)
+                        : m <= 4 ? panel_config<4>(&e)
+                        : m <= 8 ? panel_config<8>(&e)
+                        : s <= num_sms() ? panel_config<16, true>(&e)
+                                         : panel_config<16>(&e);
+    void (*upd)(TcsArgs, int, int) = cs <= 2    ? tcs_update_kernel<2>
+                                     : cs <= 4  ? tcs_update_kernel<4>
+                                     : cs <= 8  ? tcs_update_kernel<8>
+                                     : cs <= 16 ? tcs_update_kernel<16>
+                                                : tcs_update_kernel<32>;
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(upd, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kUpdSmem);
     if (e == cudaSuccess) {
       tcs_setup_kernel<<<s, kPT, 0, st>>>(a);
       count_launch();
@@ -1335,7 +1249,7 @@ int solve_tc(const Handle* h, int s, const double* shifts, int mode, double* out
       while (k > m) {
         const int nbe = step == 0 ? nbe_first : kNBT;
         ++step;
-        tcs_panel_kernel<<<s, kPT, psm, st>>>(a, k, nbe, step);
+        panel.kern<<<s, panel.threads, panel.smem, st>>>(a, k, nbe, step);
         count_launch();
         const int hrows = k - nbe;
         if (hrows > 0) {
@@ -1343,8 +1257,7 @@ int solve_tc(const Handle* h, int s, const double* shifts, int mode, double* out
           const int grid =
               (int)std::max<long long>(1, std::min<long long>(items, (long long)num_sms() * kCtasU));
           void* tru = trace_begin("tcs_update", st);  // per-launch span when tracing is on
-          if (tcz) tcs_update_kernel<true><<<grid, kUT, kUpdSmem, st>>>(a, k, nbe);
-          else tcs_update_kernel<false><<<grid, kUT, kUpdSmem, st>>>(a, k, nbe);
+          upd<<<grid, kUT, kUpdSmem, st>>>(a, k, nbe);
           count_launch();
           trace_end(tru, st);
         }
@@ -1354,8 +1267,12 @@ int solve_tc(const Handle* h, int s, const double* shifts, int mode, double* out
       tcs_canary_kernel<<<1, 256, 0, st>>>(buf + total, kCanary, a.err);
       count_launch();
 #endif
-      tcs_final_kernel<<<s, kPT, 0, st>>>(a, step, nbe_first);
+      tcs_final_kernel<<<s, kPT, 0, st>>>(a, step);
       count_launch();
+      if (mode == SSV_XHAT) {
+        tcs_back_kernel<<<(unsigned)((long long)s * step), kPT, 0, st>>>(a, step, nbe_first);
+        count_launch();
+      }
       e = cudaGetLastError();
     }
   }

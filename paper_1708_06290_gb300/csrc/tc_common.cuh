@@ -56,28 +56,55 @@ static __device__ __forceinline__ int scale_exp_f(float maxabs) {
   return eb == 0 ? -126 : eb - 126;
 }
 
-// the seven 7-bit digits of x = hi + lo (a double-float value, |x| < 2^E)
-// relative to 2^E, as BF16 bit patterns: each word's 24-bit significand is
-// shifted to units of 2^{E - 56} (truncated toward zero) from its bit fields,
-// the low word with its own sign, so no FP64 arithmetic is involved
-static __device__ __forceinline__ void digits7_pair(float hi, float lo, int E, unsigned short (&d)[7]) {
-  auto part = [E](float f) -> long long {
-    const unsigned b = __float_as_uint(f);
-    const int eb = (int)((b >> 23) & 0xffu);
-    const long long mi = (long long)(b & 0x7fffffu) | (eb ? (1ll << 23) : 0ll);
-    const int sh = (eb ? eb : 1) - 94 - E;
-    const long long v = sh >= 0 ? (mi << sh) : (sh > -64 ? (mi >> (-sh)) : 0ll);
-    return (b >> 31) ? -v : v;
-  };
-  const long long M = (E == kBadExp) ? 0ll : part(hi) + part(lo);
-  const unsigned short sgn = M < 0 ? (unsigned short)0x8000u : (unsigned short)0u;
-  const unsigned long long U = (unsigned long long)(M < 0 ? -M : M);
+// 2^{-E} for digits7_oct (0 for a non-finite row: all its digits are zero)
+static __device__ __forceinline__ float digit_scale(int E) { return E == kBadExp ? 0.f : ldexpf(1.0f, -E); }
+
+// Seven digits of eight double-float values x = hi + lo, |x| < 2^E, relative to
+// 2^E (inv = 2^{-E}): x 2^{-E} = sum_l d_l 2^{-7 (l + 1)} + r, |r| <= 2^{-50},
+// d_l the nearest integer of what is left at each step (|d_0| <= 128, the others
+// <= 80), exact in BF16.  out[l] holds digit l of the eight values as packed
+// BF16.  FP32 rounding forms the digits: adding 1.5 2^23 rounds to an integer,
+// the remainder is exact by FMA; the low word joins after three digits by an
+// exact two-sum, its rounding error before the last one.  (Shifting 64-bit
+// integers took about twice the instructions.)
+static __device__ __forceinline__ void digits7_oct(const float (&hi)[8], const float (&lo)[8], float inv,
+                                                   uint4 (&out)[7]) {
+  constexpr float kMagic = 12582912.0f;  // 1.5 * 2^23
+  unsigned pk[7][4];
 #pragma unroll
-  for (int l = 0; l < 7; ++l) {
-    const unsigned int dig = (unsigned int)(U >> (49 - 7 * l)) & 127u;
-    const float f = __uint_as_float(0x4B000000u | dig) - 8388608.0f;
-    d[l] = (unsigned short)(__float_as_uint(f) >> 16) | sgn;
+  for (int e = 0; e < 8; e += 2) {
+    float y[2], er[2];
+    // a non-finite value (inv = 0) gives zero digits
+#pragma unroll
+    for (int u = 0; u < 2; ++u) y[u] = inv != 0.f ? hi[e + u] * inv : 0.f;
+#pragma unroll
+    for (int l = 0; l < 7; ++l) {
+      if (l == 3) {
+#pragma unroll
+        for (int u = 0; u < 2; ++u) {
+          const float r = inv != 0.f ? (lo[e + u] * inv) * 2097152.0f : 0.f;  // 2^21
+          const float s = y[u] + r;
+          const float bp = s - y[u];
+          er[u] = (y[u] - (s - bp)) + (r - bp);
+          y[u] = s;
+        }
+      }
+      if (l == 6) {
+#pragma unroll
+        for (int u = 0; u < 2; ++u) y[u] = fmaf(er[u], 2097152.0f, y[u]);
+      }
+      float d[2];
+#pragma unroll
+      for (int u = 0; u < 2; ++u) {
+        d[u] = fmaf(y[u], 128.0f, kMagic) - kMagic;
+        if (l < 6) y[u] = fmaf(y[u], 128.0f, -d[u]);
+      }
+      // the top halves of the two FP32 patterns
+      pk[l][e >> 1] = __byte_perm(__float_as_uint(d[0]), __float_as_uint(d[1]), 0x7632);
+    }
   }
+#pragma unroll
+  for (int l = 0; l < 7; ++l) out[l] = make_uint4(pk[l][0], pk[l][1], pk[l][2], pk[l][3]);
 }
 
 // element offset in a K-major core-matrix tile with kg core matrices along K
