@@ -26,7 +26,12 @@
 // Look-ahead: in phase C block 0 owns exactly the columns of the NEXT panel;
 // after updating them it factors that panel while the other blocks finish
 // their strips, so each mini-block costs two grid barriers (after phase B and
-// after phase C + panel).
+// after phase C + panel).  One SM's FP64 pipe (2 multiply-adds a clock) is what
+// block 0 has for that, so phase B already does two thirds of the panel's
+// update where the rows are spread over all blocks: each block applies the
+// right update to its rows of the panel columns and forms its part of W =
+// V^T A for them.  Block 0 adds the parts, applies the left update and factors
+// the panel in shared memory (up to kPanelCap entries).
 //
 // The barrier is the library's own: it spins with a bounded iteration count
 // and, if the count runs out, raises an error flag so every block returns and
@@ -54,7 +59,9 @@ constexpr int kRS = 64;          // maximum rows per phase-B sub-strip
 constexpr int kSCmax = 32;       // strip columns per phase-C sub-chunk
 constexpr int kTR = 64;          // rows of a phase-C top tile
 constexpr int kTC = 64;          // columns of a phase-C top tile
-constexpr int kMaxDots = 16;     // dot products reduced together in the panel QR (>= 2 kW - 1)
+constexpr int kMaxDots = 16;     // dot products reduced together in the panel QR (>= 2 kW)
+constexpr int kDT = 128;         // threads that form the dots (their sums cost as much as rows)
+constexpr int kPanelCap = 22272; // entries of a panel kept in shared memory (174 KB)
 constexpr unsigned long long kBarrierSpins = 1ull << 28;  // ~10 s of 32 ns naps
 
 // shared-memory layout (doubles)
@@ -67,7 +74,7 @@ constexpr int kSmVs = kSCmax * kVLD;            // phase C: V rows of the sub-ch
 constexpr int kSmWs = kW * kSCmax;              // phase C: W, then Z = T^T W
 constexpr int kSmC = kSmVs + 2 * kSmWs + kSmVc;   // + staged V rows (pass 2)
 constexpr int kSmTop = (kTR + kTC) * kVLD;       // phase C top tile: Y and V rows
-constexpr int kSmQ = kWarps * kMaxDots + kMaxDots + kSmT + 8;   // panel QR
+constexpr int kSmQ = kDT * kMaxDots + 2 * kMaxDots + kSmT + 8 + kW + 2 * kW * kW;   // panel QR
 constexpr int kSmDoubles = kSmT + std::max(std::max(kSmB, kSmTop), std::max(kSmC, kSmQ));
 
 struct RedArgs {
@@ -82,6 +89,7 @@ struct RedArgs {
   double* VA;      // 2 x (n x kW): rows of the current / next mini-block's V
   double* TA;      // 2 x (kW x kW)
   double* Y;       // (n + p) x kW
+  double* WP;      // gridDim x (kW x kW): the blocks' parts of W for the next panel
   unsigned* bar;   // [0] arrivals, [1] generation
   int* err;        // 1 after a barrier timed out
 };
@@ -118,149 +126,151 @@ __device__ bool grid_barrier(unsigned* bar, int* err, unsigned long long limit) 
   return s_ok != 0;
 }
 
-// Sum of `cnt` (<= kMaxDots) per-thread values over the block -> out[0..cnt).
-__device__ void block_sum_vec(const double* acc, int cnt, double* red, double* out) {
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-#pragma unroll
-  for (int q = 0; q < kMaxDots; ++q) {
-    if (q < cnt) {
-      double v = acc[q];
-      for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-      if (lane == 0) red[warp * kMaxDots + q] = v;
-    }
-  }
-  __syncthreads();
-  if (threadIdx.x < cnt) {
-    double s = 0.0;
-    for (int w = 0; w < kWarps; ++w) s += red[w * kMaxDots + threadIdx.x];
-    out[threadIdx.x] = s;
-  }
-  __syncthreads();
-}
-
 // Householder QR of the L x wc panel P (column-major, leading dimension ld)
 // with wp <= wc reflectors (the columns wp .. wc-1 only receive them),
 // L - k >= 2 for every reflector k < wp.  Reflector k: beta on the diagonal,
 // v(k+1:) below it (v(k) = 1), tau[k]; the rows of V (unit lower trapezoidal,
 // explicit ones and zeros) go to Vout (row-major, ld ldv) and the triangular
 // factor of each group of wg consecutive reflectors to Tout (kW x kW blocks,
-// row-major).  Rows are owned by thread (row mod kT) throughout.
+// row-major).  SM: P is in shared memory (else global, read through L2).
+//
+// One reduction per reflector: with x = P(k:, k), alpha = x(0), v = (1, scal
+// x(1:)), the sums d_q = sum_{i > k} x_i P(i, q) of the later columns (and, for
+// T, of the group's earlier reflectors) are formed together with the norm,
+// before scal is known; v^T P(:, q) = P(k, q) + scal d_q.  A block's FP64 pipe
+// does two multiply-adds a clock, so kDT threads suffice and every partial sum
+// saved is a row's worth of work.
+template <bool SM>
 __device__ void panel_qr(double* P, size_t ld, int L, int wp, int wc, int wg, double* tau,
                          double* Vout, int ldv, double* Tout, double* sm) {
-  double* red = sm;                          // kWarps x kMaxDots
-  double* dots = red + kWarps * kMaxDots;    // kMaxDots
+  double* red = sm;                          // kMaxDots x kDT
+  double* dots = red + kDT * kMaxDots;       // kMaxDots
   double* Tl = dots + kMaxDots;              // kW x kW
-  double* misc = Tl + kSmT;                  // [0] scal, [1] tau
-  const int tid = threadIdx.x;
+  double* misc = Tl + kSmT;                  // [0] scal, [1] tau, [2] beta
+  double* tss = misc + 8;                    // kMaxDots: tau scal (v^T P(:, q))
+  double* zs = tss + kMaxDots;               // kW
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  auto rd = [](const double* q) { return SM ? *q : __ldcg(q); };
   for (int k = 0; k < wp; ++k) {
     double* x = P + (size_t)k * ld;
     const int g0 = (k / wg) * wg;
     const int jj = k - g0;
-    // (a) norm of x(k+1:L) and the reflector
-    {
-      double ss = 0.0;
-      for (int i = k + 1 + ((tid - (k + 1)) % kT + kT) % kT; i < L; i += kT) {
-        const double xi = __ldcg(x + i);
-        ss = fma(xi, xi, ss);
-      }
-      for (int o = 16; o > 0; o >>= 1) ss += __shfl_xor_sync(0xffffffffu, ss, o);
-      if ((tid & 31) == 0) red[tid >> 5] = ss;
-      __syncthreads();
-      if (tid == 0) {
-        double t = 0.0;
-        for (int w = 0; w < kWarps; ++w) t += red[w];
-        dots[0] = t;
-      }
-      __syncthreads();
-    }
-    if (tid == 0) {
-      const double v = dots[0];
-      const double alpha = __ldcg(x + k);
-      double tk = 0.0, scal = 0.0;
-      if (v != 0.0) {
-        const double nrm = sqrt(fma(alpha, alpha, v));
-        const double beta = alpha >= 0.0 ? -nrm : nrm;
-        tk = (beta - alpha) / beta;
-        scal = 1.0 / (alpha - beta);
-        x[k] = beta;
-      }
-      tau[k] = tk;
-      misc[0] = scal;
-      misc[1] = tk;
-    }
-    __syncthreads();
-    const double scal = misc[0], tk = misc[1];
-    // (b) v(k+1:) = x(k+1:) * scal   (own rows)
-    const int ifirst = k + ((tid - k) % kT + kT) % kT;  // first own row >= k
-    if (scal != 0.0)
-      for (int i = ifirst; i < L; i += kT)
-        if (i > k) x[i] = __ldcg(x + i) * scal;
-    // (c) dots: d_q = v^T P(:, q) for q = k+1 .. wc-1, then z_j = V(:, j)^T v
-    //     for j = g0 .. jj-1 (same group), in batches of kMaxDots
+    // columns k (the norm), k + 1 .. wc - 1, then g0 .. k - 1 (reflectors)
     const int nrest = wc - 1 - k;
-    const int nd = nrest + jj;
-    double zloc[kW];
+    const int nd = 1 + nrest + jj;
+    auto col_of = [&](int e) { return e <= nrest ? k + e : g0 + (e - nrest - 1); };
     for (int b0 = 0; b0 < nd; b0 += kMaxDots) {
       const int cnt = min(kMaxDots, nd - b0);
-      double acc[kMaxDots];
+      if (tid < kDT) {
+        double acc[kMaxDots];
 #pragma unroll
-      for (int q = 0; q < kMaxDots; ++q) acc[q] = 0.0;
-      for (int i = ifirst; i < L; i += kT) {
-        const double vi = i == k ? 1.0 : __ldcg(x + i);
+        for (int q = 0; q < kMaxDots; ++q) acc[q] = 0.0;
+        for (int i = k + 1 + tid; i < L; i += kDT) {
+          const double xi = rd(x + i);
 #pragma unroll
-        for (int q = 0; q < kMaxDots; ++q) {
-          if (q < cnt) {
-            const int e = b0 + q;
-            const int col = e < nrest ? k + 1 + e : g0 + (e - nrest);
-            acc[q] = fma(vi, __ldcg(P + i + (size_t)col * ld), acc[q]);
-          }
+          for (int q = 0; q < kMaxDots; ++q)
+            if (q < cnt) acc[q] = fma(xi, rd(P + i + (size_t)col_of(b0 + q) * ld), acc[q]);
         }
+#pragma unroll
+        for (int q = 0; q < kMaxDots; ++q)
+          if (q < cnt) red[q * kDT + tid] = acc[q];
       }
-      block_sum_vec(acc, cnt, red, dots);
-      // (d) update the remaining panel columns of this batch; keep the z's
-      for (int q = 0; q < cnt; ++q) {
-        const int e = b0 + q;
-        if (e < nrest) {
-          const int col = k + 1 + e;
-          const double td = tk * dots[q];
-          if (td != 0.0) {
-            double* pc = P + (size_t)col * ld;
-            for (int i = ifirst; i < L; i += kT) {
-              const double vi = i == k ? 1.0 : __ldcg(x + i);
-              pc[i] = fma(-td, vi, __ldcg(pc + i));
-            }
+      __syncthreads();
+      for (int q = warp; q < cnt; q += kWarps) {
+        const double* r = red + q * kDT + lane;
+        double v = (r[0] + r[32]) + (r[64] + r[96]);
+        for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+        if (lane == 0) dots[q] = v;
+      }
+      __syncthreads();
+      if (b0 == 0) {
+        if (tid == 0) {
+          const double ss = dots[0], alpha = rd(x + k);
+          double tk = 0.0, scal = 0.0, beta = alpha;
+          if (ss != 0.0) {
+            const double nrm = sqrt(fma(alpha, alpha, ss));
+            beta = alpha >= 0.0 ? -nrm : nrm;
+            tk = (beta - alpha) / beta;
+            scal = 1.0 / (alpha - beta);
           }
-        } else if (tid == 0) {
-          zloc[e - nrest] = dots[q];
+          tau[k] = tk;
+          misc[0] = scal;
+          misc[1] = tk;
+          misc[2] = beta;
+        }
+        __syncthreads();
+      }
+      const double scal = misc[0], tk = misc[1];
+      // thread q: v^T of its column; row k of a later column, z of a reflector
+      if (tid < cnt && b0 + tid > 0) {
+        const int e = b0 + tid;
+        double* pk = P + k + (size_t)col_of(e) * ld;
+        const double vp = fma(scal, dots[tid], rd(pk));
+        if (e <= nrest) {
+          const double td = tk * vp;
+          tss[tid] = td * scal;
+          if (tk != 0.0) *pk = rd(pk) - td;
+        } else {
+          zs[e - nrest - 1] = vp;
         }
       }
       __syncthreads();
-    }
-    // (e) T(0:jj, jj) = -tau T(0:jj, 0:jj) z,  T(jj, jj) = tau
-    if (tid == 0) {
-      for (int r = 0; r < jj; ++r) {
-        double s = 0.0;
-        for (int c = r; c < jj; ++c) s = fma(Tl[r * kW + c], zloc[c], s);
-        Tl[r * kW + jj] = -tk * s;
-      }
-      for (int r = jj + 1; r < kW; ++r) Tl[r * kW + jj] = 0.0;
-      Tl[jj * kW + jj] = tk;
-      if (jj == wg - 1 || k == wp - 1) {
-        double* To = Tout + (size_t)(k / wg) * kSmT;
-        for (int e = 0; e < kSmT; ++e) {
-          const int r = e / kW, c = e % kW;
-          To[e] = (r <= jj && c <= jj) ? Tl[e] : 0.0;
+      // later columns of this batch: P(:, q) -= tau (v^T P(:, q)) v below row k
+      const int qn = min(cnt, nrest + 1 - b0);
+      if (tk != 0.0) {
+        for (int i = k + 1 + tid; i < L; i += kT) {
+          const double xi = rd(x + i);
+          for (int q = b0 == 0 ? 1 : 0; q < qn; ++q) {
+            double* pc = P + i + (size_t)(k + b0 + q) * ld;
+            *pc = fma(-tss[q], xi, rd(pc));
+          }
         }
       }
     }
+    const double scal = misc[0], tk = misc[1];
+    // v(k+1:) = scal x(k+1:) (every thread its rows), beta on the diagonal
+    if (tk != 0.0) {
+      for (int i = k + 1 + tid; i < L; i += kT) x[i] = rd(x + i) * scal;
+      if (tid == 0) x[k] = misc[2];
+    }
+    // T(r, jj) = -tau T(r, r:jj) z,  T(jj, jj) = tau: thread r a row
+    if (tid < kW) {
+      double s = 0.0;
+#pragma unroll
+      for (int c = 0; c < kW; ++c)
+        if (c >= tid && c < jj) s = fma(Tl[tid * kW + c], zs[c], s);
+      Tl[tid * kW + jj] = tid < jj ? -tk * s : tid == jj ? tk : 0.0;
+    }
     __syncthreads();
+    if (jj == wg - 1 || k == wp - 1) {
+      double* To = Tout + (size_t)(k / wg) * kSmT;
+      for (int e = tid; e < kSmT; e += kT) {
+        const int r = e / kW, c = e % kW;
+        To[e] = (r <= jj && c <= jj) ? Tl[e] : 0.0;
+      }
+      __syncthreads();
+    }
   }
   // dense rows of V
   for (long long o = tid; o < (long long)L * wp; o += kT) {
     const int i = (int)(o / wp), k = (int)(o % wp);
-    const double v = i < k ? 0.0 : (i == k ? 1.0 : __ldcg(P + i + (size_t)k * ld));
+    const double v = i < k ? 0.0 : (i == k ? 1.0 : rd(P + i + (size_t)k * ld));
     Vout[(size_t)i * ldv + k] = v;
   }
+  __syncthreads();
+}
+
+// The same on a panel in global memory, staged in shared memory when it fits.
+__device__ void panel_qr_any(double* P, size_t ld, int L, int wp, int wc, int wg, double* tau,
+                             double* Vout, int ldv, double* Tout, double* sm, double* pan) {
+  if ((long long)L * wc > kPanelCap) {
+    panel_qr<false>(P, ld, L, wp, wc, wg, tau, Vout, ldv, Tout, sm);
+    return;
+  }
+  for (int e = threadIdx.x; e < L * wc; e += kT) pan[e] = __ldcg(P + e % L + (size_t)(e / L) * ld);
+  __syncthreads();
+  panel_qr<true>(pan, (size_t)L, L, wp, wc, wg, tau, Vout, ldv, Tout, sm);
+  for (int e = threadIdx.x; e < L * wc; e += kT) P[e % L + (size_t)(e / L) * ld] = pan[e];
   __syncthreads();
 }
 
@@ -275,10 +285,12 @@ __device__ __forceinline__ double* ext_row(const RedArgs& a, int i, size_t* ld) 
 }
 
 // Phase B, rows [i0, i1) of A_ext: Y = A_ext(rows, r0:n) V T.  W >= w is the
-// compile-time width (V and T are zero beyond w).
+// compile-time width (V and T are zero beyond w).  For the columns pc .. pc +
+// wn - 1 of the next panel (rows r0 .. n - 1) also the right update, and this
+// block's part of V^T A(r0:, pc:pc+wn) after it.
 template <int W>
 __device__ void phase_b(const RedArgs& a, int r0, int w, const double* __restrict__ V, int ldv,
-                        const double* __restrict__ Ts, double* sm) {
+                        const double* __restrict__ Ts, int pc, int wn, double* sm) {
   constexpr int VC = kVCW / W, VLD = W == 1 ? 1 : W + 1;
   const int n = a.n, np = a.n + a.p;
   double* Vc = sm;
@@ -287,6 +299,7 @@ __device__ void phase_b(const RedArgs& a, int r0, int w, const double* __restric
   const int tid = threadIdx.x;
   const int i0 = (int)(((long long)np * blockIdx.x) / gridDim.x);
   const int i1 = (int)(((long long)np * (blockIdx.x + 1)) / gridDim.x);
+  double wpart = 0.0;  // thread k * wn + q < w * wn: entry (k, q) of this block's part of W
   for (int rs0 = i0; rs0 < i1; rs0 += kRS) {
     const int RS = min(kRS, i1 - rs0);
     const int CG = kT / RS;
@@ -331,9 +344,111 @@ __device__ void phase_b(const RedArgs& a, int r0, int w, const double* __restric
       double s = 0.0;
       for (int j = 0; j <= k; ++j) s = fma(AV[rr * W + j], Ts[j * kW + k], s);
       a.Y[(size_t)(rs0 + rr) * kW + k] = s;
+      part[rr * W + k] = s;
     }
     __syncthreads();
+    if (wn > 0) {
+      // the next panel's columns: rows r0 .. n - 1 of this sub-strip
+      double* xs = AV;                 // RS x wn (wn <= kW = the width AV is sized for)
+      double* vs = part + kRS * kW;    // RS x W: the rows of V
+      for (int e = tid; e < RS * W; e += kT) {
+        const int i = rs0 + e / W, k = e % W;
+        vs[e] = (i >= r0 && i < n && k < w) ? __ldcg(V + (size_t)(i - r0) * ldv + k) : 0.0;
+      }
+      for (int e = tid; e < RS * wn; e += kT) {
+        const int rr = e % RS, q = e / RS;
+        const int i = rs0 + rr, c = pc + q;
+        double x = 0.0;
+        if (i >= r0 && i < n) {
+          double* px = a.H + i + (size_t)c * n;
+          x = __ldcg(px);
+          if (c >= r0) {
+            const double* vc = V + (size_t)(c - r0) * ldv;
+#pragma unroll
+            for (int k = 0; k < W; ++k)
+              if (k < w) x = fma(-part[rr * W + k], __ldcg(vc + k), x);
+            *px = x;
+          }
+        }
+        xs[rr * wn + q] = x;
+      }
+      __syncthreads();
+      if (tid < w * wn) {
+        const int k = tid / wn, q = tid % wn;
+        double s0 = 0.0, s1 = 0.0;
+        for (int rr = 0; rr + 1 < RS; rr += 2) {
+          s0 = fma(vs[rr * W + k], xs[rr * wn + q], s0);
+          s1 = fma(vs[(rr + 1) * W + k], xs[(rr + 1) * wn + q], s1);
+        }
+        if (RS & 1) s0 = fma(vs[(RS - 1) * W + k], xs[(RS - 1) * wn + q], s0);
+        wpart += s0 + s1;
+      }
+      __syncthreads();
+    }
   }
+  if (wn > 0 && tid < w * wn) a.WP[(size_t)blockIdx.x * kW * kW + tid] = wpart;
+}
+
+// The next panel after phase B (block 0): W from the blocks' parts, the left
+// update A(r0:, pc:pc+wn) -= V T^T W, then the QR of its rows rn .. n - 1.
+template <int W>
+__device__ void panel_step(const RedArgs& a, int r0, int w, const double* __restrict__ V, int ldv,
+                           const double* __restrict__ Ts, int pc, int wn, int tn, double* sm, double* pan) {
+  const int n = a.n, m = a.m, L = n - r0, rn = pc + m, Lq = n - rn;
+  double* Ws = sm + kDT * kMaxDots + 2 * kMaxDots + kSmT + 8 + kW;  // behind the QR's areas
+  double* Zs = Ws + kW * kW;
+  const int tid = threadIdx.x;
+  {
+    // eight lanes a sum, in a fixed order
+    const int e = tid / 8, sub = tid % 8;
+    double s = 0.0;
+    if (e < w * wn)
+      for (int g = sub; g < (int)gridDim.x; g += 8) s += __ldcg(a.WP + (size_t)g * kW * kW + e);
+    for (int o = 4; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+    if (e < w * wn && sub == 0) Ws[e] = s;
+  }
+  __syncthreads();
+  if (tid < w * wn) {
+    const int k = tid / wn, q = tid % wn;
+    double s = 0.0;
+    for (int j = 0; j <= k; ++j) s = fma(Ts[j * kW + k], Ws[j * wn + q], s);
+    Zs[k * wn + q] = s;
+  }
+  __syncthreads();
+  const bool fits = (long long)Lq * wn <= kPanelCap;
+  for (int i = r0 + tid; i < n; i += kT) {
+    double v[W];
+    const double* vr = V + (size_t)(i - r0) * ldv;
+#pragma unroll
+    for (int k = 0; k < W; ++k) v[k] = k < w ? __ldcg(vr + k) : 0.0;
+    double x[kW];
+#pragma unroll
+    for (int q = 0; q < kW; ++q) x[q] = q < wn ? __ldcg(a.H + i + (size_t)(pc + q) * n) : 0.0;
+#pragma unroll
+    for (int k = 0; k < W; ++k) {
+#pragma unroll
+      for (int q = 0; q < kW; ++q)
+        if (q < wn) x[q] = fma(-v[k], k < w ? Zs[k * wn + q] : 0.0, x[q]);
+    }
+#pragma unroll
+    for (int q = 0; q < kW; ++q) {
+      if (q >= wn) continue;
+      if (fits && i >= rn) pan[(size_t)q * Lq + (i - rn)] = x[q];
+      else a.H[i + (size_t)(pc + q) * n] = x[q];
+    }
+  }
+  __syncthreads();
+  (void)L;
+  double* P = a.H + rn + (size_t)pc * n;
+  double* Vout = a.VA + (size_t)(tn & 1) * n * kW;
+  double* Tout = a.TA + (size_t)(tn & 1) * kSmT;
+  if (fits) {
+    panel_qr<true>(pan, (size_t)Lq, Lq, wn, wn, wn, a.tauA + pc, Vout, kW, Tout, sm);
+    for (int e = tid; e < Lq * wn; e += kT) P[e % Lq + (size_t)(e / Lq) * n] = pan[e];
+  } else {
+    panel_qr<false>(P, (size_t)n, Lq, wn, wn, wn, a.tauA + pc, Vout, kW, Tout, sm);
+  }
+  __syncthreads();
 }
 
 // Columns per phase-C sub-chunk: two per warp in pass 2.
@@ -518,17 +633,12 @@ __device__ void top_tile(const RedArgs& a, int r0, int w, const double* __restri
 template <int W>
 __device__ void block_step(const RedArgs& a, int r0, int lc, int w, const double* V, int ldv,
                            const double* Ts, int wn, int tn, double* work, bool* ok) {
-  const int n = a.n, m = a.m, p = a.p;
-  phase_b<W>(a, r0, w, V, ldv, Ts, work);
+  const int n = a.n, p = a.p;
+  phase_b<W>(a, r0, w, V, ldv, Ts, lc, wn, work);
   if (!grid_barrier(a.bar, a.err, kBarrierSpins)) { *ok = false; return; }
   if (blockIdx.x == 0) {
     // look-ahead: the next panel's columns (rows r0 .. n-1), then its QR
-    if (wn > 0) {
-      phase_c_bottom<W>(a, r0, w, V, ldv, Ts, lc, lc + wn, work);
-      const int rn = lc + m;
-      panel_qr(a.H + rn + (size_t)lc * n, (size_t)n, n - rn, wn, wn, wn, a.tauA + lc,
-               a.VA + (size_t)(tn & 1) * n * kW, kW, a.TA + (size_t)(tn & 1) * kSmT, work);
-    }
+    if (wn > 0) panel_step<W>(a, r0, w, V, ldv, Ts, lc, wn, tn, work, work + kSmDoubles - kSmT);
   } else {
     // the other blocks split, by multiply-add count, the bottom columns
     // [lc + wn, n) (3 (n - r0) w each) followed by the top tiles
@@ -560,17 +670,18 @@ __global__ void __launch_bounds__(kT, 1) reduce_blocked_kernel(RedArgs a) {
   extern __shared__ double sm[];
   double* Ts = sm;              // T of the current step
   double* work = sm + kSmT;
+  double* pan = sm + kSmDoubles;  // a panel (kPanelCap)
   const int n = a.n, m = a.m;
   // Step 1 of Algorithm 1: QR of B (block 0), reflectors grouped by kW
   if (blockIdx.x == 0 && a.kb > 0)
-    panel_qr(a.R, (size_t)n, n, a.kb, m, kW, a.tauB, a.VB, a.kb, a.TB, work);
+    panel_qr_any(a.R, (size_t)n, n, a.kb, m, kW, a.tauB, a.VB, a.kb, a.TB, work, pan);
   const int nbB = (a.kb + kW - 1) / kW;
   const int naA = a.ka > 0 ? (a.ka + a.wa - 1) / a.wa : 0;
   const int nsteps = nbB + naA;
   // the first A panel, when there is no B step to look ahead from
   if (nbB == 0 && naA > 0 && blockIdx.x == 0) {
     const int w1 = min(a.wa, a.ka);
-    panel_qr(a.H + m, (size_t)n, n - m, w1, w1, w1, a.tauA, a.VA, kW, a.TA, work);
+    panel_qr_any(a.H + m, (size_t)n, n - m, w1, w1, w1, a.tauA, a.VA, kW, a.TA, work, pan);
   }
   if (!grid_barrier(a.bar, a.err, kBarrierSpins)) return;
   for (int s = 0; s < nsteps; ++s) {
@@ -628,7 +739,7 @@ int reduce_persistent(Handle* h, cudaStream_t st) {
   const int kb = std::max(h->kb, 0);
   const int nbB = (kb + kW - 1) / kW;
   const size_t ndbl = (size_t)n * kb + (size_t)nbB * kSmT + 2 * (size_t)n * kW + 2 * (size_t)kSmT +
-                      (size_t)np * kW;
+                      (size_t)np * kW + (size_t)std::max(2, num_sms()) * kW * kW;
   const size_t bytes = sizeof(double) * ndbl + 4 * sizeof(unsigned) + 16;
   unsigned char* wsp = nullptr;
   SSV_CUDA_TRY(pool_alloc((void**)&wsp, bytes, st));
@@ -642,11 +753,13 @@ int reduce_persistent(Handle* h, cudaStream_t st) {
   a.VA = a.TB + (size_t)nbB * kSmT;
   a.TA = a.VA + 2 * (size_t)n * kW;
   a.Y = a.TA + 2 * (size_t)kSmT;
+  a.WP = a.Y + (size_t)np * kW;
   a.bar = reinterpret_cast<unsigned*>(d + ndbl);
   a.err = reinterpret_cast<int*>(a.bar + 2);
   int rc = SSV_OK;
   cudaError_t e = cudaMemsetAsync(a.bar, 0, 4 * sizeof(unsigned), st);
-  const size_t smem = sizeof(double) * kSmDoubles;
+  const size_t smem = sizeof(double) * (size_t)(kSmDoubles + kPanelCap);
+  static_assert(sizeof(double) * (kSmDoubles + kPanelCap) <= 227 * 1024, "shared memory of the reduction");
   if (e == cudaSuccess)
     e = cudaFuncSetAttribute(reduce_blocked_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
                              (int)smem);
