@@ -15,14 +15,14 @@
 //      rows of Ct (small), writes P1 as BF16 digit tiles, and keeps the P1
 //      rows and P2 that the X-hat back pass needs;
 //   2. update (persistent, one thread block per SM): work items of 128 rows
-//      of H x one group of shifts (N = 64 real columns: each shift's m complex
+//      of H x one group of shifts (N = 32 real columns: each shift's m complex
 //      columns as 2m real ones, padded to a power of two).  Z1 P1 is formed
 //      exactly as in the tensor-core residual (error-free splitting after
 //      Ozaki, Ogita, Oishi and Rump): H's rows and P1's real columns are
 //      written as 7-bit digits relative to a power-of-two scale (eight for a
 //      row of H, seven for a column of P1), each digit exact in BF16, and the
 //      35 digit products H_k P_l with k + l <= 7 run as tcgen05.mma (BF16 x
-//      BF16 -> FP32, M = 128, N = 64, K = 16) into eight TMEM accumulators, one
+//      BF16 -> FP32, M = 128, K = 16, seven digits of P1 per product) into eight TMEM accumulators, one
 //      per level k + l, where every partial sum is an integer below
 //      7 * 128 * 127^2 < 2^24 and therefore exact.  The
 //      digit tiles reach shared memory by 1-D TMA bulk copies on an mbarrier,
@@ -76,16 +76,7 @@ constexpr int kPT = 256;             // threads of the setup and final kernels
 constexpr int kNBT = 128;            // n_b of the tensor-core sweep (K of the update)
 constexpr int kMaxM = kTcMaxM;       // m <= 16
 constexpr int kUM = 128;             // H rows per update item = TMEM lanes
-// real columns per update item (shift group): 64 = one update block per SM with
-// two stage buffers; 32 = two blocks per SM with one stage buffer each, so that
-// one block's epilogue runs under the other's products
-#ifndef SSV_TCS_N
-#define SSV_TCS_N 64
-#endif
-constexpr int kUN = SSV_TCS_N;
-static_assert(kUN == 32 || kUN == 64, "update item width");
-constexpr int kBufU = kUN == 64 ? 2 : 1;   // stage buffers of an update block
-constexpr int kCtasU = kUN == 64 ? 1 : 2;  // update blocks per SM
+constexpr int kUN = 32;              // real columns per update item (a group of shifts)
 constexpr int kKS = 32;              // K per shared-memory stage
 constexpr int kKG = kKS / 8;         // core matrices along K in a tile
 constexpr int kSDH = 8;              // digits of H (all eight slices of its digit tiles)
@@ -94,36 +85,17 @@ constexpr int kLev = 8;              // levels k + l = 0 .. 7
 constexpr int kStages = kNBT / kKS;  // stages per block step
 constexpr int kAT = kUM * kKS;       // BF16 elements of one H digit tile
 constexpr int kBT = kUN * kKS;       // BF16 elements of one P1 digit tile
-// a stage: eight H digit tiles, seven P1 digit tiles and one tile of zeros
-// standing for P1 digit 7, so that the H digit 0 products reach all levels
-constexpr int kBPlanes = kSD + 1;
-constexpr uint32_t kStageBytes = (uint32_t)(kSDH * kAT + kBPlanes * kBT) * 2;
-constexpr uint32_t kLoadBytes = (uint32_t)(kSDH * kAT + kSD * kBT) * 2;  // copied per stage
-constexpr uint32_t kZeroOff = kLoadBytes;                                 // the zero tile in a stage
-constexpr int kTmemCols = 8 * kUN;   // 8 levels x kUN columns
+constexpr uint32_t kStageBytes = (uint32_t)(kSDH * kAT + kSD * kBT) * 2;  // H and P1 digit tiles
+constexpr int kWinCols = kLev * kUN;  // TMEM columns of an item; two items in flight
 // polls of one mbarrier wait before the update gives up (a stage's copies and
 // products complete within microseconds)
 constexpr long long kUpdWait = 1LL << 22;
-static_assert(kLev * kUN <= kTmemCols, "TMEM columns of the levels");
-// dynamic shared memory of the update, in this order: two stage buffers (later
-// the group's Z2 and P2 digit tiles); the group's P2 / sigma rows (S * 2 m^2 <=
-// 64 m float4); the column exponents of P1 and of P2's real form (kUN ints
-// each); the row maxima of the quarters (4 x 128 floats); the shifts (at most
-// kUN); four mbarriers; the TMEM address slot
-constexpr size_t kOffPc = (size_t)kBufU * kStageBytes;
-constexpr size_t kPcF4 = (size_t)kUN * kMaxM;
-constexpr size_t kOffExp = kOffPc + kPcF4 * 16;
-constexpr size_t kOffExp2 = kOffExp + (size_t)kUN * sizeof(int);
-constexpr size_t kOffXmax = kOffExp2 + (size_t)kUN * sizeof(int);
-constexpr size_t kOffSig = kOffXmax + (size_t)4 * kUM * sizeof(float);
-constexpr size_t kOffBar = kOffSig + (size_t)kUN * 16;
-constexpr size_t kOffSlot = kOffBar + 4 * 8;
-constexpr size_t kUpdSmem = kOffSlot + 16;
-static_assert(kOffBar % 8 == 0 && kOffSig % 16 == 0, "alignment of the smem carve-up");
-static_assert(kCtasU * (kUpdSmem + 1024) <= 228 * 1024, "shared memory of the update blocks");
-// the Z2 / P2 digit tiles of a group (S shifts, 7 digits, 128 x cs and cs x cs) reuse the stage buffers
-static_assert(7 * (128 * 32 + 32 * 32) * 2 * (kUN / 32) <= kBufU * (size_t)kStageBytes, "Z2 P2 tiles");
-static_assert(7 * (128 * 16 + 16 * 16) * 2 * (kUN / 16) <= kBufU * (size_t)kStageBytes, "Z2 P2 tiles");
+static_assert(2 * kWinCols == 512, "TMEM columns of the two items");
+// shared memory of the update: two stage buffers, then the Z2 and P2 digit tiles
+// of one item (S shifts: 7 digits of 128 x cs and of cs x cs; S cs = kUN)
+constexpr size_t kOffZ = 2 * (size_t)kStageBytes;
+constexpr size_t kUpdSmem = kOffZ + (size_t)7 * (128 * kUN + kUN * 32) * 2;
+static_assert(kUpdSmem + 1024 <= 227 * 1024, "shared memory of the update");
 
 // element offset in a K-major core-matrix tile (8 rows x 8 K per 128 bytes;
 // byte strides 128 along K, kKG * 128 along rows): the layout of the residual's
@@ -176,6 +148,10 @@ struct TcsArgs {
   size_t n_z2, n_zt, n_pd, n_zd, n_p2d, n_pc, n_hs, n_out;
 };
 
+// exponent 0 for a zero (or denormal) row or column: its digits are zero at any
+// scale, and the update's fast path takes moderate exponents only
+__device__ __forceinline__ int col_exp(int E) { return E <= -126 ? 0 : E; }
+
 // digit tiles of window row p + i (H row i) of shift sh, from the double-float
 // values Z2f(p + i, q): the row exponent over the 2m real entries, seven
 // digits of each entry at K = 2q (Re), 2q + 1 (Im), zero up to cs
@@ -187,7 +163,7 @@ __device__ void write_z2_digits(const TcsArgs& a, int sh, int i, const float4* Z
     mx = fmaxf(mx, fmaxf(fabsf(z.x), fabsf(z.z)));
     if (!(fabsf(z.x) <= 3.4e38f) || !(fabsf(z.z) <= 3.4e38f)) mx = __int_as_float(0x7f800000);
   }
-  const int E = scale_exp_f(mx);
+  const int E = col_exp(scale_exp_f(mx));
   a.zexp[BCK((size_t)sh * a.npad + i, (size_t)a.s * a.npad)] = E;
   const float inv = digit_scale(E);
   const size_t T0 = ((size_t)sh * a.RB + i / 128) * 7 * (128 * cs);
@@ -299,7 +275,7 @@ __global__ void __launch_bounds__(panel_threads<MAXM, FEW>(), panel_per_sm<MAXM,
     const int er = __reduce_max_sync(0xffffffffu, br ? kBadExp : scale_exp_f(mr));
     const int ei = __reduce_max_sync(0xffffffffu, bi ? kBadExp : scale_exp_f(mi));
     if (lane < 2) {
-      const int E = lane ? ei : er;
+      const int E = col_exp(lane ? ei : er);
       sm.fexp[2 * q + lane] = E;
       a.pexp[BCK((size_t)sh * 2 * kMaxM + 2 * q + lane, (size_t)a.s * 2 * kMaxM)] = E;
     }
@@ -359,7 +335,7 @@ __global__ void __launch_bounds__(panel_threads<MAXM, FEW>(), panel_per_sm<MAXM,
           if (!(fabsf(w.x) <= 3.4e38f) || !(fabsf(w.z) <= 3.4e38f)) mx = __int_as_float(0x7f800000);
         }
       }
-      const int E = scale_exp_f(mx);
+      const int E = col_exp(scale_exp_f(mx));
       sm.f2exp[c] = E;
       a.p2exp[BCK((size_t)sh * 2 * kMaxM + c, (size_t)a.s * 2 * kMaxM)] = E;
     }
@@ -469,37 +445,55 @@ static __device__ __forceinline__ float pow2f(int e) { return __int_as_float((e 
 constexpr int kFastExp = 30;
 static __device__ __forceinline__ bool fast_exp(int e) { return e >= -kFastExp && e <= kFastExp; }
 
-constexpr int kUT = (kUN / 16) * kUM;  // update threads: one per H row of the tile and 16 columns
+constexpr int kUT = 2 * kUM + 64;  // update threads: two epilogue groups, the producer's and the issuer's warp
+
+// a bounded wait of one role: gives up at the poll limit or when another role
+// has (the block then leaves together)
+static __device__ __forceinline__ bool role_wait(uint32_t mbar, uint32_t parity, volatile int* fail) {
+  for (long long it = 0; it < kUpdWait / 64; ++it) {
+    if (mbar_wait(mbar, parity, 64)) return true;
+    if (*fail) return false;
+  }
+  *fail = 1;
+  return false;
+}
 
 // The update of block step (k, nbe) for shifts of CS real columns (2m rounded
-// up to a power of two).  CS >= 16: Z2 P2 as a second round of digit products
-// on the tensor cores; otherwise in double-float in the epilogue.  Per item
-// (row tile I, group g):
-//   1. the stages of Z1 P1 (H digit tiles x P1 digit tiles) into the eight
-//      TMEM levels, the next stage in flight when there are two buffers;
-//   2. CS >= 16: the group's Z2 and P2 digit tiles are copied into the (then
-//      free) stage buffers while the threads drain the Z1 P1 levels into
-//      double-float sums; then the 28 products of Z2 P2 per shift go into
-//      seven TMEM levels, are drained and added;
-//   3. the next item's first stage streams in during the rest of the epilogue:
-//      the shifted-diagonal correction and the new rows: as FP32 pairs the 128
-//      that the next panel (or the final block) reads, all others as the digit
-//      tiles of the next block step (CS < 16: every row as pairs).
+// up to a power of two).  An item is 128 rows of H x one group of S = 32 / CS
+// shifts; a persistent block works on two at a time, in roles that only meet at
+// mbarriers:
+//   * a producer thread copies the K stages of Z1 P1 (H digit tiles x P1 digit
+//     tiles) into two stage buffers and, CS >= 16, the group's Z2 and P2 digit
+//     tiles into a third;
+//   * an issuing thread multiplies: item v's Z1 P1 into the eight levels of TMEM
+//     window v mod 2, then, once these are read, its Z2 P2 into seven levels of
+//     the same window, one item behind;
+//   * two groups of four warps take alternate items (thread = row, 32 columns):
+//     levels into double-float sums, scaling, the shifted-diagonal correction,
+//     and the new rows: as FP32 pairs the 128 that the next panel (or the final
+//     block) reads, all others as the digit tiles of the next block step (CS <
+//     16: Z2 P2 in double-float here, and every row as pairs).
 //
-// What bounds it: the instructions of the epilogue (drains, scaling, digits),
-// then the stage copies from L2 (H's eight digit planes, 256 KB an item).  So
-// column arithmetic is resolved at compile time (CS), scaling is one multiply
-// by a power of two, and the digits come from FP32 rounding (digits7_oct).
+// What bounds it, per item at CS = 32: the copies from L2 (392 KB, about 6.5 k
+// clocks), the epilogue's instructions (5.3 k issue slots a scheduler) and the
+// products (5.5 k clocks), which run side by side.  One item at a time, each
+// phase after the other, took 6.0 ms a launch at the start of the sweep of 2000
+// shifts at n = 5000, m = 16 (114 ms for the 39 launches).
 template <int CS>
-__global__ void __launch_bounds__(kUT, kCtasU) tcs_update_kernel(TcsArgs a, int k, int nbe) {
+__global__ void __launch_bounds__(kUT, 1) tcs_update_kernel(TcsArgs a, int k, int nbe) {
   constexpr bool TCZ = CS >= 16;
   constexpr int S = kUN / CS;             // shifts of a group
   extern __shared__ __align__(128) unsigned char smem[];
+  __shared__ __align__(8) unsigned long long mbar[14];
+  __shared__ uint32_t tslot;
+  __shared__ volatile int fail;
+  // stages copied / multiplied, Z2 tiles copied / multiplied (read when a wait gave up)
+  __shared__ int issued[4];
   const int n = a.n, m = a.m, p = a.p, ldz = p + n;
   const int hrows = k - nbe;              // H rows above the block
   const int j0 = k - m - nbe;             // first fresh column (a multiple of 32)
   const int nsig = min(m, nbe);
-  const int tid = threadIdx.x, warp = tid >> 5;
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const int G = a.ngroups;
   // an earlier launch of this solve gave up a wait: its results are void, skip
   // (the flag is read by every thread and combined, so the whole block agrees)
@@ -508,440 +502,406 @@ __global__ void __launch_bounds__(kUT, kCtasU) tcs_update_kernel(TcsArgs a, int 
   const long long items = (long long)RT * G;
   const int nst = (nbe + kKS - 1) / kKS;
   const int JH0 = j0 / kKS;
-  float4* pcs = reinterpret_cast<float4*>(smem + kOffPc);                   // S x 2 m m
-  int* fexp = reinterpret_cast<int*>(smem + kOffExp);                        // kUN
-  int* f2exp = reinterpret_cast<int*>(smem + kOffExp2);                      // kUN
-  float* xmax = reinterpret_cast<float*>(smem + kOffXmax);                   // 4 x 128
-  cd* sig = reinterpret_cast<cd*>(smem + kOffSig);                           // <= kUN shifts
-  unsigned long long* mbar = reinterpret_cast<unsigned long long*>(smem + kOffBar);
-  uint32_t* tslot = reinterpret_cast<uint32_t*>(smem + kOffSlot);
-  const uint32_t mb = smem_addr(mbar);        // products, two stage loads, one Z2 / P2 load
-  const uint32_t lmb0 = mb + 8u;
-  const uint32_t lmb2 = mb + 24u;
-  const uint32_t sBase = smem_addr(smem);
+  // full / empty[2]: a stage buffer copied / multiplied; zfull / zempty: the Z2
+  // buffer; pfull / pread[2]: window's Z1 P1 levels complete / read; qfull /
+  // qread[2]: its Z2 P2 levels
+  const uint32_t full = smem_addr(mbar), empty = full + 16, zfull = full + 32, zempty = full + 40;
+  const uint32_t pfull = full + 48, pread = full + 64, qfull = full + 80, qread = full + 96;
+  const uint32_t sBase = smem_addr(smem), sZ = sBase + (uint32_t)kOffZ;
   if (warp == 0) {
-    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(
-                     smem_addr(tslot)),
-                 "r"(kTmemCols));
+    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_addr(&tslot)),
+                 "r"(2 * kWinCols));
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;");
   }
   if (tid == 0) {
-    for (int q = 0; q < 4; ++q) asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(mb + 8u * q));
+    for (int q = 0; q < 14; ++q)  // pread and qread: one arrival per warp of the group
+      asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(full + 8u * q),
+                   "r"(q == 8 || q == 9 || q >= 12 ? kUM / 32 : 1));
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    fail = 0;
+    for (int q = 0; q < 4; ++q) issued[q] = 0;
   }
-  // the zero tiles of the stage buffers (the copies never write them)
-  auto zero_tile = [&](int b) {
-    uint4* zp = reinterpret_cast<uint4*>(smem + (size_t)b * kStageBytes + kZeroOff);
-    for (int e = tid; e < kBT * 2 / 16; e += kUT) zp[e] = make_uint4(0u, 0u, 0u, 0u);
-    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-  };
-  for (int b = 0; b < kBufU; ++b) zero_tile(b);
   fence_before();
   __syncthreads();
   fence_after();
-  const uint32_t tmem = *tslot;
-  uint32_t mphase = 0, l2phase = 0;
-  uint32_t lphase[2] = {0u, 0u};
-  bool pend[2] = {false, false};  // a stage copy into buffer b not yet seen complete
-  bool pend2 = false;
-  bool failed = false;
+  const uint32_t tmem = tslot;
   // Z2 / P2 digit bytes of one shift
   constexpr uint32_t zbytes = 7u * 128u * (uint32_t)CS * 2u;
   constexpr uint32_t pbytes = 7u * (uint32_t)(CS * CS) * 2u;
   constexpr int kgz = CS >= 8 ? CS / 8 : 1;
+  const long long mine = blockIdx.x < items ? (items - blockIdx.x + gridDim.x - 1) / gridDim.x : 0;
 
-  // stage st of item (I, g) into buffer b: eight H digit tiles, seven P1 digit tiles
-  auto stage_in = [&](int I, int g, int st, int b) {
-    const uint32_t dst = sBase + (uint32_t)b * kStageBytes;
-    const uint32_t lmb = lmb0 + 8u * (uint32_t)b;
-    asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(lmb), "r"(kLoadBytes)
-                 : "memory");
-    for (int l = 0; l < kSDH; ++l)
-      bulk_copy(dst + (uint32_t)(l * kAT * 2),
-                a.Hs + BCK(((size_t)(l * a.RB + I) * a.KT + (JH0 + st)) * (kAT / 8), a.n_hs),
-                (uint32_t)(kAT * 2), lmb);
-    const size_t Pg0 = (size_t)g * kSD * kStages * kBT;
-    for (int l = 0; l < kSD; ++l)
-      bulk_copy(dst + (uint32_t)(kSDH * kAT * 2 + l * kBT * 2),
-                a.Pd + BCK(Pg0 + ((size_t)l * kStages + st) * kBT, a.n_pd), (uint32_t)(kBT * 2), lmb);
-  };
-  // the group's Z2 digit tiles of row tile I, then its P2 digit tiles
-  auto z2_in = [&](int I, int g, int nsh) {
-    asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(lmb2),
-                 "r"((uint32_t)nsh * (zbytes + pbytes))
-                 : "memory");
-    for (int l = 0; l < nsh; ++l) {
-      const int sh = g * S + l;
-      bulk_copy(sBase + (uint32_t)l * zbytes, a.Zd + BCK(((size_t)sh * a.RB + I) * 7 * (128 * CS), a.n_zd),
-                zbytes, lmb2);
-      bulk_copy(sBase + (uint32_t)S * zbytes + (uint32_t)l * pbytes,
-                a.P2d + BCK((size_t)sh * 7 * CS * CS, a.n_p2d), pbytes, lmb2);
-    }
-  };
-
-  long long item = blockIdx.x;
-  if (item < items) {
-    pend[0] = true;
-    if (tid == 0) stage_in((int)(item / G), (int)(item % G), 0, 0);
-  }
-  for (; item < items && !failed; item += gridDim.x) {
-    const int I = (int)(item / G), g = (int)(item % G);
-    const int nsh = min(S, a.s - g * S);  // shifts of this group
-    // rows of this tile that the sigma rows touch (their correction reads pcs)
-    const bool sigtile = I * kUM < j0 + nsig && I * kUM + kUM > j0;
-    // the group's sigma rows (and P2 for the double-float epilogue), column
-    // exponents and shifts
-    if (!TCZ || sigtile) {
-      for (int e = tid; e < S * 2 * m * m; e += kUT) {
-        const int l = e / (2 * m * m), o = e % (2 * m * m);
-        const int sh = g * S + l;
-        pcs[e] = sh < a.s ? a.pc[BCK((size_t)sh * 2 * kMaxM * kMaxM + o, a.n_pc)] : make_float4(0.f, 0.f, 0.f, 0.f);
+  if (warp == 2 * kUM / 32) {
+    if (lane == 0) {
+      // ---- producer
+      unsigned i = 0;
+      bool ok = true;
+      auto stages = [&](long long v) {
+        const long long item = blockIdx.x + v * gridDim.x;
+        const int I = (int)(item / G), g = (int)(item % G);
+        const size_t Pg0 = (size_t)g * kSD * kStages * kBT;
+        for (int st = 0; st < nst && ok; ++st, ++i) {
+          const uint32_t b = i & 1u;
+          if (!role_wait(empty + 8u * b, ((i >> 1) & 1u) ^ 1u, &fail)) {
+            ok = false;
+            return;
+          }
+          const uint32_t dst = sBase + b * kStageBytes, lb = full + 8u * b;
+          asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(lb), "r"(kStageBytes)
+                       : "memory");
+          for (int l = 0; l < kSDH; ++l)
+            bulk_copy(dst + (uint32_t)(l * kAT * 2),
+                      a.Hs + BCK(((size_t)(l * a.RB + I) * a.KT + (JH0 + st)) * (kAT / 8), a.n_hs),
+                      (uint32_t)(kAT * 2), lb);
+          for (int l = 0; l < kSD; ++l)
+            bulk_copy(dst + (uint32_t)(kSDH * kAT * 2 + l * kBT * 2),
+                      a.Pd + BCK(Pg0 + ((size_t)l * kStages + st) * kBT, a.n_pd), (uint32_t)(kBT * 2), lb);
+          issued[0] = (int)(i + 1);
+        }
+      };
+      auto ztiles = [&](long long v) {
+        const long long item = blockIdx.x + v * gridDim.x;
+        const int I = (int)(item / G), g = (int)(item % G);
+        if (!role_wait(zempty, ((unsigned)v & 1u) ^ 1u, &fail)) {
+          ok = false;
+          return;
+        }
+        const int nsh = min(S, a.s - g * S);
+        asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(zfull),
+                     "r"((uint32_t)nsh * (zbytes + pbytes))
+                     : "memory");
+        for (int l = 0; l < nsh; ++l) {
+          const int sh = g * S + l;
+          bulk_copy(sZ + (uint32_t)l * zbytes, a.Zd + BCK(((size_t)sh * a.RB + I) * 7 * (128 * CS), a.n_zd), zbytes,
+                    zfull);
+          bulk_copy(sZ + (uint32_t)S * zbytes + (uint32_t)l * pbytes, a.P2d + BCK((size_t)sh * 7 * CS * CS, a.n_p2d),
+                    pbytes, zfull);
+        }
+        issued[2] = (int)(v + 1);
+      };
+      // in the issuer's order: Z1 P1 of item v + 1 before Z2 P2 of item v
+      for (long long v = 0; v < mine + (TCZ ? 1 : 0) && ok; ++v) {
+        if (v < mine) stages(v);
+        if (TCZ && v > 0 && ok) ztiles(v - 1);
       }
     }
-    bool cfast = true;
-    for (int e = tid; e < kUN; e += kUT) {
-      const int l = e / CS, c = e % CS;
-      const int sh = g * S + l;
-      const bool use = sh < a.s && c < 2 * m;
-      const int E = use ? a.pexp[(size_t)sh * 2 * kMaxM + c] : 0;
-      fexp[e] = E;
-      if (use && !fast_exp(E)) cfast = false;
-      if (TCZ) {
-        const int E2 = use ? a.p2exp[(size_t)sh * 2 * kMaxM + c] : 0;
-        f2exp[e] = E2;
-        if (!fast_exp(E2)) cfast = false;
-      }
-    }
-    for (int l = tid; l < S; l += kUT) sig[l] = (g * S + l < a.s) ? a.shifts[g * S + l] : mkcd(0.0, 0.0);
-    const bool slowcol = __syncthreads_or(!cfast);
-    // thread (row, quarter) = (tid mod 128, tid / 128) takes one H row and 16 of
-    // the columns; warps w, w + 4, .. read TMEM lanes 32 (w mod 4) ..
-    const int row = tid & (kUM - 1), qt = tid >> 7;
-    const int ih = I * kUM + row;
-    const bool live = ih < hrows;
-    const int Ei = live ? a.hexp[BCK(ih, a.npad)] : 0;
-    const int shq = g * S + (qt * 16) / CS;  // TCZ: the quarter's shift
-    int Ez = 0;
-    if (TCZ && live && shq < a.s) Ez = a.zexp[BCK((size_t)shq * a.npad + ih, (size_t)a.s * a.npad)];
-    // ---- 1. Z1 P1: stage st in buffer st & 1
-    for (int st = 0; st < nst; ++st) {
-      const int buf = kBufU == 2 ? (st & 1) : 0;
-      const bool lok = mbar_wait(lmb0 + 8u * (uint32_t)buf, lphase[buf], kUpdWait);
-      if (__syncthreads_or(!lok)) {
-        failed = true;
-        break;
-      }
-      lphase[buf] ^= 1u;
-      pend[buf] = false;
-      // fused levels: the P1 digit tiles sit side by side (kUN rows each, then
-      // the zero tile), so one product of H digit kd against P1 digits
-      // b0 .. b0 + c - 1 (N = kUN c <= 256) lands digit b in TMEM level kd + b;
-      // the kd = 0 products cover every level and open the item, so one thread
-      // issues all of them
-      if (tid == 0) {
-        fence_after();
-        const uint32_t aBase = sBase + (uint32_t)buf * kStageBytes;
-        const uint32_t bBase = aBase + (uint32_t)(kSDH * kAT * 2);
-        constexpr uint32_t kSbo = (uint32_t)kKG * 128u;
-        constexpr int kMaxC = 256 / kUN;
+  } else if (warp == 2 * kUM / 32 + 1) {
+    if (lane == 0) {
+      // ---- issuer
+      unsigned i = 0;
+      bool ok = true;
+      // fused levels: the P1 digit tiles sit side by side (kUN rows each), so one
+      // product of H digit kd against P1 digits 0 .. c - 1 (N = kUN c) lands digit
+      // b in level kd + b.  The first products of an item open the levels: those
+      // of kd = 0 levels 0 .. 6, digit 6 of kd = 1 level 7.
+      auto z1p1 = [&](long long v) {
+        const uint32_t h = (unsigned)v & 1u, u = (unsigned)(v >> 1);
+        const uint32_t d = tmem + h * (uint32_t)kWinCols;
+        if (!role_wait((TCZ ? qread : pread) + 8u * h, (u & 1u) ^ 1u, &fail)) ok = false;
+        for (int st = 0; st < nst && ok; ++st, ++i) {
+          const uint32_t b = i & 1u;
+          if (!role_wait(full + 8u * b, (i >> 1) & 1u, &fail)) {
+            ok = false;
+            return;
+          }
+          fence_after();
+          const uint32_t aBase = sBase + b * kStageBytes;
+          const uint32_t bBase = aBase + (uint32_t)(kSDH * kAT * 2);
+          constexpr uint32_t kSbo = (uint32_t)kKG * 128u;
 #pragma unroll
-        for (int ks = 0; ks < kKS / 16; ++ks) {
+          for (int ks = 0; ks < kKS / 16; ++ks) {
+            const bool first = st == 0 && ks == 0;
 #pragma unroll
-          for (int kd = 0; kd < kSDH; ++kd) {
-            const int nb = kd == 0 ? kLev : min(kSD, kLev - kd);  // P1 digits (7: the zero tile)
-#pragma unroll
-            for (int b0 = 0; b0 < nb; b0 += kMaxC) {
-              const int c = min(kMaxC, nb - b0);
+            for (int kd = 0; kd < kSDH; ++kd) {
               const uint64_t ad = mat_desc(aBase + (uint32_t)(kd * kAT * 2 + ks * 256), 128u, kSbo);
-              const uint64_t bd = mat_desc(bBase + (uint32_t)(b0 * kBT * 2 + ks * 256), 128u, kSbo);
-              const bool first = st == 0 && ks == 0 && kd == 0;
-              mma_bf16(tmem + (uint32_t)((kd + b0) * kUN), ad, bd, idesc_bf16(kUM, kUN * c), first ? 0u : 1u);
+              const uint64_t bd = mat_desc(bBase + (uint32_t)(ks * 256), 128u, kSbo);
+              constexpr int kOpen = kSD - 1;  // the digit of kd = 1 that opens the last level
+              if (kd == 1 && first) {
+                mma_bf16(d + (uint32_t)kUN, ad, bd, idesc_bf16(kUM, kUN * kOpen), 1u);
+                const uint64_t b6 = mat_desc(bBase + (uint32_t)(kOpen * kBT * 2 + ks * 256), 128u, kSbo);
+                mma_bf16(d + (uint32_t)((kOpen + 1) * kUN), ad, b6, idesc_bf16(kUM, kUN), 0u);
+              } else {
+                const int c = kd == 0 ? kSD : kLev - kd;
+                mma_bf16(d + (uint32_t)(kd * kUN), ad, bd, idesc_bf16(kUM, kUN * c), (first && kd == 0) ? 0u : 1u);
+              }
             }
           }
+          mma_commit(empty + 8u * b);
+          issued[1] = (int)(i + 1);
         }
-        mma_commit(mb);
-      }
-      // the next stage streams into the other buffer, whose products finished
-      // in the previous round (with one buffer: after these products)
-      if (kBufU == 2 && st + 1 < nst) {
-        pend[buf ^ 1] = true;
-        if (tid == 0) stage_in(I, g, st + 1, buf ^ 1);
-      }
-      const bool ok = mbar_wait(mb, mphase, kUpdWait);
-      if (__syncthreads_or(!ok)) {
-        failed = true;
-        break;
-      }
-      mphase ^= 1u;
-      if (kBufU == 1 && st + 1 < nst) {
-        pend[0] = true;
-        if (tid == 0) stage_in(I, g, st + 1, 0);
-      }
-    }
-    if (failed) break;
-    // the stage buffers are free: TCZ fetches the group's Z2 / P2 tiles into them
-    if (TCZ) {
-      pend2 = true;
-      if (tid == 0) z2_in(I, g, nsh);
-    }
-    // ---- epilogue
-    fence_after();
-    const uint32_t tl = tmem + ((uint32_t)((warp & 3) * 32) << 16);
-    // the new entries, 16 real columns of the row (Re, Im interleaved), as pairs
-    float ah[16], al[16];
-#pragma unroll
-    for (int c = 0; c < 16; ++c) { ah[c] = 0.f; al[c] = 0.f; }
-    {
-      float sc = 0.0078125f * 0.0078125f;  // 2^{-7 (t + 2)}, t = 0
-#pragma unroll 1
-      for (int lv = 0; lv < kLev; ++lv) {
-        uint32_t rr[16];
-        tmem_ld16(tl + (uint32_t)(lv * kUN + qt * 16), rr);
-#pragma unroll
-        for (int c = 0; c < 16; ++c) add_f(ah[c], al[c], __uint_as_float(rr[c]) * sc);
-        sc *= 0.0078125f;
-      }
-    }
-    const bool fast = !slowcol && fast_exp(Ei) && (!TCZ || fast_exp(Ez));
-#pragma unroll
-    for (int c = 0; c < 16; ++c) {
-      const int col = qt * 16 + c, Ec = fexp[col];
-      if (fast) {
-        const float f = pow2f(Ei + Ec);
-        ah[c] *= f;
-        al[c] *= f;
-      } else if (Ei == kBadExp || Ec == kBadExp) {
-        ah[c] = __int_as_float(0x7fc00000);
-        al[c] = 0.f;
-      } else {
-        ah[c] = ldexpf(ah[c], Ei + Ec);
-        al[c] = ldexpf(al[c], Ei + Ec);
-      }
-    }
-    if (TCZ) {
-      // ---- 2. Z2 P2: the levels of Z1 P1 are read; the same TMEM columns take
-      //      the seven levels of the group's Z2 digit tiles x P2 digit tiles
-      fence_before();
-      const bool lok = mbar_wait(lmb2, l2phase, kUpdWait);
-      if (__syncthreads_or(!lok)) {
-        failed = true;
-        break;
-      }
-      l2phase ^= 1u;
-      pend2 = false;
-      // fused levels: shift l's seven levels sit side by side in TMEM (columns
-      // 7 CS l + CS lv) and its P2 digit tiles (CS rows each) are stacked, so one
-      // product of Z2 digit kd against P2 digits 0 .. 6 - kd (N = CS (7 - kd))
-      // lands digit ld in level kd + ld; kd = 0 opens all seven
-      if (tid == 0) {
+        if (ok) mma_commit(pfull + 8u * h);
+      };
+      // shift l's seven levels sit side by side (columns 7 CS l + CS lv) and its
+      // P2 digit tiles (CS rows each) are stacked: one product of Z2 digit kd
+      // against P2 digits 0 .. 6 - kd lands digit ld in level kd + ld
+      auto z2p2 = [&](long long v) {
+        const uint32_t h = (unsigned)v & 1u, u = (unsigned)(v >> 1);
+        const uint32_t d = tmem + h * (uint32_t)kWinCols;
+        const int g = (int)((blockIdx.x + v * gridDim.x) % G), nsh = min(S, a.s - g * S);
+        if (!role_wait(pread + 8u * h, u & 1u, &fail) || !role_wait(zfull, (unsigned)v & 1u, &fail)) {
+          ok = false;
+          return;
+        }
         fence_after();
         constexpr uint32_t sboz = (uint32_t)kgz * 128u;
         for (int l = 0; l < nsh; ++l) {
-          const uint32_t zb = sBase + (uint32_t)l * zbytes;
-          const uint32_t pb = sBase + (uint32_t)S * zbytes + (uint32_t)l * pbytes;
-#pragma unroll 1
+          const uint32_t zb = sZ + (uint32_t)l * zbytes;
+          const uint32_t pb = sZ + (uint32_t)S * zbytes + (uint32_t)l * pbytes;
+#pragma unroll
           for (int ks = 0; ks < CS / 16; ++ks) {
 #pragma unroll
             for (int kd = 0; kd < 7; ++kd) {
               const uint64_t ad = mat_desc(zb + (uint32_t)(kd * 128 * CS * 2 + ks * 256), 128u, sboz);
               const uint64_t bd = mat_desc(pb + (uint32_t)(ks * 256), 128u, sboz);
-              mma_bf16(tmem + (uint32_t)(7 * CS * l + kd * CS), ad, bd, idesc_bf16(kUM, CS * (7 - kd)),
+              mma_bf16(d + (uint32_t)(7 * CS * l + kd * CS), ad, bd, idesc_bf16(kUM, CS * (7 - kd)),
                        (kd == 0 && ks == 0) ? 0u : 1u);
             }
           }
         }
-        mma_commit(mb);
+        mma_commit(zempty);
+        mma_commit(qfull + 8u * h);
+        issued[3] = (int)(v + 1);
+      };
+      for (long long v = 0; v < mine + (TCZ ? 1 : 0) && ok; ++v) {
+        if (v < mine) z1p1(v);
+        if (TCZ && v > 0 && ok) z2p2(v - 1);
       }
-      const bool ok = mbar_wait(mb, mphase, kUpdWait);
-      if (__syncthreads_or(!ok)) {
-        failed = true;
-        break;
+    }
+  } else {
+    // ---- epilogue: group h = warp / 4 takes items v = h, h + 2, ..
+    const uint32_t h = (uint32_t)(warp >> 2);
+    const int row = tid & (kUM - 1);
+    const uint32_t tl = tmem + h * (uint32_t)kWinCols + ((uint32_t)((warp & 3) * 32) << 16);
+    auto arrive = [&](uint32_t b) {
+      fence_before();
+      __syncwarp();
+      if (lane == 0) asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(b) : "memory");
+    };
+    for (long long v = h; v < mine; v += 2) {
+      const uint32_t par = (unsigned)(v >> 1) & 1u;
+      const long long item = blockIdx.x + v * gridDim.x;
+      const int I = (int)(item / G), g = (int)(item % G);
+      const int ih = I * kUM + row;
+      const bool live = ih < hrows;
+      // exponents: of the row, of this lane's column (P1's, P2's), of the row's Z2
+      const int Ei = live ? a.hexp[BCK(ih, a.npad)] : 0;
+      int E1 = 0, E2 = 0;
+      {
+        const int sh = g * S + lane / CS, c = lane % CS;
+        if (sh < a.s && c < 2 * m) {
+          E1 = a.pexp[(size_t)sh * 2 * kMaxM + c];
+          if (TCZ) E2 = a.p2exp[(size_t)sh * 2 * kMaxM + c];
+        }
       }
-      mphase ^= 1u;
-      // the Z2 / P2 tiles covered buffer 0's zero tile: write it again before
-      // the next item's first products read it (ordered by the load wait and
-      // barrier that precede them)
+      int Ez[TCZ ? S : 1];
+      bool fast = fast_exp(Ei);
+      if constexpr (TCZ) {
 #pragma unroll
-      for (int b = 0; b < kBufU; ++b)
-        if ((size_t)b * kStageBytes + kZeroOff < (size_t)S * (zbytes + pbytes)) zero_tile(b);
-    }
-    // ---- 3. the stage buffers are free again: the next item's first stage
-    //      streams in during the rest of the epilogue
-    if (item + gridDim.x < items) {
-      const long long nx = item + gridDim.x;
-      pend[0] = true;
-      if (tid == 0) stage_in((int)(nx / G), (int)(nx % G), 0, 0);
-    }
-    if constexpr (TCZ) {
+        for (int l = 0; l < S; ++l) {
+          Ez[l] = (live && g * S + l < a.s) ? a.zexp[BCK((size_t)(g * S + l) * a.npad + ih, (size_t)a.s * a.npad)] : 0;
+          fast = fast && fast_exp(Ez[l]);
+        }
+      }
+      // the row exponents of a warp and the column exponents: one path per warp
+      fast = __all_sync(0xffffffffu, fast && fast_exp(E1) && fast_exp(E2));
+      if (!__all_sync(0xffffffffu, role_wait(pfull + 8u * h, par, &fail))) break;
       fence_after();
-      // shift l = (16 qt) / CS: its levels start at column 7 CS l, this
-      // quarter's columns at (16 qt) mod CS within them
-      const uint32_t tz = tl + (uint32_t)(7 * CS * ((qt * 16) / CS) + (qt * 16) % CS);
-      if (fast) {
-        float f[16];
+      // the new entries, 32 real columns of the row (Re, Im interleaved), as pairs
+      float ah[kUN], al[kUN];
 #pragma unroll
-        for (int c = 0; c < 16; ++c) f[c] = pow2f(Ez + f2exp[qt * 16 + c] - 14);
+      for (int c = 0; c < kUN; ++c) { ah[c] = 0.f; al[c] = 0.f; }
+      {
+        float sc = 0.0078125f * 0.0078125f;  // 2^{-7 (t + 2)}, t = 0
 #pragma unroll 1
-        for (int lv = 0; lv < 7; ++lv) {
-          uint32_t rr[16];
-          tmem_ld16(tz + (uint32_t)(lv * CS), rr);
+        for (int lv = 0; lv < kLev; ++lv) {
+          uint32_t rr[32];
+          tmem_ld32(tl + (uint32_t)(lv * kUN), rr);
 #pragma unroll
-          for (int c = 0; c < 16; ++c) {
-            add_f(ah[c], al[c], __uint_as_float(rr[c]) * f[c]);
-            f[c] *= 0.0078125f;
+          for (int c = 0; c < kUN; ++c) add_f(ah[c], al[c], __uint_as_float(rr[c]) * sc);
+          sc *= 0.0078125f;
+        }
+      }
+      arrive(pread + 8u * h);
+#pragma unroll
+      for (int c = 0; c < kUN; ++c) {
+        const int Ec = __shfl_sync(0xffffffffu, E1, c);
+        if (fast) {
+          const float f = pow2f(Ei + Ec);
+          ah[c] *= f;
+          al[c] *= f;
+        } else if (Ei == kBadExp || Ec == kBadExp) {
+          ah[c] = __int_as_float(0x7fc00000);
+          al[c] = 0.f;
+        } else {
+          ah[c] = ldexpf(ah[c], Ei + Ec);
+          al[c] = ldexpf(al[c], Ei + Ec);
+        }
+      }
+      if constexpr (TCZ) {
+        if (!__all_sync(0xffffffffu, role_wait(qfull + 8u * h, par, &fail))) break;
+        fence_after();
+        // 16 columns at a time: shift l's levels start at column 7 CS l
+#pragma unroll
+        for (int c0 = 0; c0 < kUN; c0 += 16) {
+          const uint32_t tz = tl + (uint32_t)(7 * CS * (c0 / CS) + c0 % CS);
+          const int ez = Ez[c0 / CS];
+          if (fast) {
+            float f[16];
+#pragma unroll
+            for (int c = 0; c < 16; ++c) f[c] = pow2f(ez + __shfl_sync(0xffffffffu, E2, c0 + c) - 14);
+#pragma unroll 1
+            for (int lv = 0; lv < 7; ++lv) {
+              uint32_t rr[16];
+              tmem_ld16(tz + (uint32_t)(lv * CS), rr);
+#pragma unroll
+              for (int c = 0; c < 16; ++c) {
+                add_f(ah[c0 + c], al[c0 + c], __uint_as_float(rr[c]) * f[c]);
+                f[c] *= 0.0078125f;
+              }
+            }
+          } else {
+            float bh[16], bl[16];
+#pragma unroll
+            for (int c = 0; c < 16; ++c) { bh[c] = 0.f; bl[c] = 0.f; }
+            float sc = 0.0078125f * 0.0078125f;
+#pragma unroll 1
+            for (int lv = 0; lv < 7; ++lv) {
+              uint32_t rr[16];
+              tmem_ld16(tz + (uint32_t)(lv * CS), rr);
+#pragma unroll
+              for (int c = 0; c < 16; ++c) add_f(bh[c], bl[c], __uint_as_float(rr[c]) * sc);
+              sc *= 0.0078125f;
+            }
+#pragma unroll
+            for (int c = 0; c < 16; ++c) {
+              const int Ec = __shfl_sync(0xffffffffu, E2, c0 + c);
+              if (ez == kBadExp || Ec == kBadExp) {
+                ah[c0 + c] = __int_as_float(0x7fc00000);
+                al[c0 + c] = 0.f;
+              } else {
+                add_f(ah[c0 + c], al[c0 + c], ldexpf(bh[c], ez + Ec));
+                al[c0 + c] += ldexpf(bl[c], ez + Ec);
+              }
+            }
           }
         }
-      } else {
-        // one column at a time: its levels into a pair, scaled by ldexpf
-#pragma unroll 1
-        for (int c8 = 0; c8 < 16; c8 += 8) {
-          float bh[8], bl[8];
+        arrive(qread + 8u * h);
+      } else if (live) {
+        // several shifts (m <= 4): + Z2(row, :) P2(:, q) in double-float from the
+        // old row of each shift
+        constexpr int CC = CS / 2;  // complex columns of a shift
 #pragma unroll
-          for (int c = 0; c < 8; ++c) { bh[c] = 0.f; bl[c] = 0.f; }
-          float sc = 0.0078125f * 0.0078125f;
-#pragma unroll 1
-          for (int lv = 0; lv < 7; ++lv) {
-            uint32_t rr[8];
-            tmem_ld8(tz + (uint32_t)(lv * CS + c8), rr);
+        for (int l = 0; l < S; ++l) {
+          if (g * S + l < a.s) {
+            const float4* z = a.Z2 + BCK((size_t)(g * S + l) * a.z2_stride + (p + ih), a.n_z2);
+            const float4* pc = a.pc + BCK((size_t)(g * S + l) * 2 * kMaxM * kMaxM, a.n_pc);
+            float4 zz[CC];
 #pragma unroll
-            for (int c = 0; c < 8; ++c) add_f(bh[c], bl[c], __uint_as_float(rr[c]) * sc);
-            sc *= 0.0078125f;
-          }
+            for (int qq = 0; qq < CC; ++qq) zz[qq] = qq < m ? z[(size_t)qq * ldz] : make_float4(0.f, 0.f, 0.f, 0.f);
 #pragma unroll
-          for (int c = 0; c < 16; ++c) {
-            if ((c & 8) != c8) continue;
-            const int Ec = f2exp[qt * 16 + c];
-            if (Ez == kBadExp || Ec == kBadExp) {
-              ah[c] = __int_as_float(0x7fc00000);
-              al[c] = 0.f;
-            } else {
-              add_f(ah[c], al[c], ldexpf(bh[c & 7], Ez + Ec));
-              al[c] += ldexpf(bl[c & 7], Ez + Ec);
+            for (int q = 0; q < CC; ++q) {
+              if (q >= m) continue;
+              const int c = l * CS + 2 * q;
+#pragma unroll
+              for (int qq = 0; qq < CC; ++qq) {
+                if (qq >= m) continue;
+                const float4 w = pc[qq * m + q];
+                df_mac(ah[c], al[c], zz[qq].x, zz[qq].y, w.x, w.y);
+                df_mac(ah[c], al[c], -zz[qq].z, -zz[qq].w, w.z, w.w);
+                df_mac(ah[c + 1], al[c + 1], zz[qq].x, zz[qq].y, w.z, w.w);
+                df_mac(ah[c + 1], al[c + 1], zz[qq].z, zz[qq].w, w.x, w.y);
+              }
             }
           }
         }
       }
-    } else if (live) {
-      // several shifts per quarter (m <= 4): + Z2(row, :) P2(:, q) in
-      // double-float from the old row of each slot's shift
-      constexpr int CC = CS / 2;  // complex columns of a shift
+      const int cdr = ih - j0;  // shifted-diagonal correction row of fresh column cdr
+      if (live && cdr >= 0 && cdr < nsig) {
+        // - sigma P1(cdr, q)
 #pragma unroll
-      for (int l0 = 0; l0 < 16 / CS; ++l0) {
-        const int l = qt * 16 / CS + l0;
-        if (g * S + l < a.s) {
-          const float4* z = a.Z2 + BCK((size_t)(g * S + l) * a.z2_stride + (p + ih), a.n_z2);
-          float4 zz[CC];
+        for (int c = 0; c < kUN; c += 2) {
+          const int l = c / CS, q = (c % CS) >> 1, sh = g * S + l;
+          if (q >= m || sh >= a.s) continue;
+          const float4 sgf = df_split(a.shifts[sh]);
+          const float4 w = a.pc[BCK((size_t)sh * 2 * kMaxM * kMaxM + m * m + cdr * m + q, a.n_pc)];
+          df_mac(ah[c], al[c], -sgf.x, -sgf.y, w.x, w.y);
+          df_mac(ah[c], al[c], sgf.z, sgf.w, w.z, w.w);
+          df_mac(ah[c + 1], al[c + 1], -sgf.x, -sgf.y, w.z, w.w);
+          df_mac(ah[c + 1], al[c + 1], -sgf.z, -sgf.w, w.x, w.y);
+        }
+      }
+      // normalised pairs
 #pragma unroll
-          for (int qq = 0; qq < CC; ++qq) zz[qq] = qq < m ? z[(size_t)qq * ldz] : make_float4(0.f, 0.f, 0.f, 0.f);
+      for (int c = 0; c < kUN; ++c) {
+        const float s = ah[c] + al[c];
+        al[c] = al[c] - (s - ah[c]);
+        ah[c] = s;
+      }
+      // as pairs: the rows of the next panel or the final block
+      if (live && (!TCZ || ih >= hrows - kNBT)) {
 #pragma unroll
-          for (int q = 0; q < CC; ++q) {
-            if (q >= m) continue;
-            const int c = l0 * CS + 2 * q;
+        for (int c = 0; c < kUN; c += 2) {
+          const int l = c / CS, q = (c % CS) >> 1;
+          if (q >= m || g * S + l >= a.s) continue;
+          a.Z2[BCK((size_t)(g * S + l) * a.z2_stride + (p + ih) + (size_t)q * ldz, a.n_z2)] =
+              make_float4(ah[c], al[c], ah[c + 1], al[c + 1]);
+        }
+      }
+      // as digits: the rows above them (none of a tile that lies within the last 128 rows)
+      if constexpr (TCZ) {
+        if (live && I * kUM < hrows - kNBT) {
 #pragma unroll
-            for (int qq = 0; qq < CC; ++qq) {
-              if (qq >= m) continue;
-              const float4 w = pcs[(size_t)l * 2 * m * m + qq * m + q];
-              df_mac(ah[c], al[c], zz[qq].x, zz[qq].y, w.x, w.y);
-              df_mac(ah[c], al[c], -zz[qq].z, -zz[qq].w, w.z, w.w);
-              df_mac(ah[c + 1], al[c + 1], zz[qq].x, zz[qq].y, w.z, w.w);
-              df_mac(ah[c + 1], al[c + 1], zz[qq].z, zz[qq].w, w.x, w.y);
+          for (int l = 0; l < S; ++l) {
+            const int sh = g * S + l;
+            if (sh >= a.s) continue;
+            // the row's digit exponent: the maximum over the shift's 2m entries
+            float mx = 0.f;
+            bool bad = false;
+#pragma unroll
+            for (int c = l * CS; c < (l + 1) * CS; ++c) {
+              if (c % CS >= 2 * m) { ah[c] = 0.f; al[c] = 0.f; }
+              mx = fmaxf(mx, fabsf(ah[c]));
+              bad = bad || !(fabsf(ah[c]) <= 3.4e38f);
+            }
+            if (bad) mx = __int_as_float(0x7f800000);
+            const int E = col_exp(scale_exp_f(mx));
+            a.zexp[BCK((size_t)sh * a.npad + ih, (size_t)a.s * a.npad)] = E;
+            const float inv = digit_scale(E);
+            const size_t T0 = ((size_t)sh * a.RB + I) * 7 * (128 * CS);
+#pragma unroll
+            for (int k8 = 0; k8 < CS; k8 += 8) {
+              float hi[8], lo[8];
+#pragma unroll
+              for (int e = 0; e < 8; ++e) { hi[e] = ah[l * CS + k8 + e]; lo[e] = al[l * CS + k8 + e]; }
+              uint4 dg[7];
+              digits7_oct(hi, lo, inv, dg);
+              const int off = tile_off_kg(row, k8, kgz);
+#pragma unroll
+              for (int l2 = 0; l2 < 7; ++l2)
+                *reinterpret_cast<uint4*>(a.Zd + BCK(T0 + (size_t)l2 * (128 * CS) + off, a.n_zd)) = dg[l2];
             }
           }
         }
       }
     }
-    const int cdr = ih - j0;  // shifted-diagonal correction row of fresh column cdr
-    if (live && cdr >= 0 && cdr < nsig) {
-      // - sigma P1(cdr, q)
-#pragma unroll
-      for (int c = 0; c < 16; c += 2) {
-        const int col = qt * 16 + c, l = col / CS, q = (col % CS) >> 1;
-        if (q >= m || g * S + l >= a.s) continue;
-        const float4 sgf = df_split(sig[l]);
-        const float4 w = pcs[(size_t)l * 2 * m * m + m * m + cdr * m + q];
-        df_mac(ah[c], al[c], -sgf.x, -sgf.y, w.x, w.y);
-        df_mac(ah[c], al[c], sgf.z, sgf.w, w.z, w.w);
-        df_mac(ah[c + 1], al[c + 1], -sgf.x, -sgf.y, w.z, w.w);
-        df_mac(ah[c + 1], al[c + 1], -sgf.z, -sgf.w, w.x, w.y);
-      }
-    }
-    // normalised pairs
-#pragma unroll
-    for (int c = 0; c < 16; ++c) {
-      const float s = ah[c] + al[c];
-      al[c] = al[c] - (s - ah[c]);
-      ah[c] = s;
-    }
-    // the new rows as pairs: those of the next panel or the final block
-    const bool pairs = !TCZ || ih >= hrows - kNBT;
-    if (live && pairs) {
-#pragma unroll
-      for (int c = 0; c < 16; c += 2) {
-        const int col = qt * 16 + c, l = col / CS, q = (col % CS) >> 1;
-        if (q >= m || g * S + l >= a.s) continue;
-        a.Z2[BCK((size_t)(g * S + l) * a.z2_stride + (p + ih) + (size_t)q * ldz, a.n_z2)] =
-            make_float4(ah[c], al[c], ah[c + 1], al[c + 1]);
-      }
-    }
-    // as digits: the rows above them (none of a tile that lies within the last 128 rows)
-    if (TCZ && I * kUM < hrows - kNBT) {
-      // the row's digit exponent: the maximum over the shift's 2m entries,
-      // which two quarters share when CS = 32
-      float mx = 0.f;
-      bool bad = false;
-#pragma unroll
-      for (int c = 0; c < 16; ++c) {
-        if ((qt * 16 + c) % CS >= 2 * m) { ah[c] = 0.f; al[c] = 0.f; }
-        mx = fmaxf(mx, fabsf(ah[c]));
-        bad = bad || !(fabsf(ah[c]) <= 3.4e38f);
-      }
-      if (bad) mx = __int_as_float(0x7f800000);
-      if (CS == 32) {
-        xmax[qt * kUM + row] = mx;
-        __syncthreads();
-        mx = fmaxf(mx, xmax[(qt ^ 1) * kUM + row]);
-      }
-      if (live && shq < a.s) {
-        const int E = scale_exp_f(mx);
-        constexpr int kbm = CS - 1;
-        const int kb = (qt * 16) & kbm;  // this quarter's first K entry of the row
-        if (kb == 0) a.zexp[BCK((size_t)shq * a.npad + ih, (size_t)a.s * a.npad)] = E;
-        const float inv = digit_scale(E);
-        const size_t T0 = ((size_t)shq * a.RB + I) * 7 * (128 * CS);
-#pragma unroll
-        for (int h = 0; h < 2; ++h) {
-          float hi[8], lo[8];
-#pragma unroll
-          for (int e = 0; e < 8; ++e) { hi[e] = ah[h * 8 + e]; lo[e] = al[h * 8 + e]; }
-          uint4 dg[7];
-          digits7_oct(hi, lo, inv, dg);
-          const int off = tile_off_kg(row, kb + h * 8, kgz);
-#pragma unroll
-          for (int l2 = 0; l2 < 7; ++l2)
-            *reinterpret_cast<uint4*>(a.Zd + BCK(T0 + (size_t)l2 * (128 * CS) + off, a.n_zd)) = dg[l2];
-        }
-      }
-    }
-    fence_before();
-    __syncthreads();
   }
-  if (failed) {
-    // a completion never arrived: record it, give the products and copies in
-    // flight one more bounded wait, then release TMEM
-    if (tid == 0) {
-      atomicExch(a.err, 1);
-      mbar_wait(mb, mphase, kUpdWait);
-      for (int b = 0; b < 2; ++b)
-        if (pend[b]) mbar_wait(lmb0 + 8u * (uint32_t)b, lphase[b], kUpdWait);
-      if (pend2) mbar_wait(lmb2, l2phase, kUpdWait);
-    }
-    __syncthreads();
+  __syncwarp();
+  __syncthreads();
+  if (fail != 0 && tid == 0) {
+    // a completion never arrived: record it and give the copies and products in
+    // flight one more bounded wait
+    atomicExch(a.err, 1);
+    const unsigned nl = (unsigned)issued[0], nm = (unsigned)issued[1];
+    for (unsigned i = nl > 2 ? nl - 2 : 0; i < nl; ++i) mbar_wait(full + 8u * (i & 1u), (i >> 1) & 1u, kUpdWait);
+    for (unsigned i = nm > 2 ? nm - 2 : 0; i < nm; ++i) mbar_wait(empty + 8u * (i & 1u), (i >> 1) & 1u, kUpdWait);
+    if (issued[2] > 0) mbar_wait(zfull, (unsigned)(issued[2] - 1) & 1u, kUpdWait);
+    if (issued[3] > 0) mbar_wait(zempty, (unsigned)(issued[3] - 1) & 1u, kUpdWait);
   }
   fence_before();
   __syncthreads();
   fence_after();
   if (warp == 0)
-    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(kTmemCols));
+    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(2 * kWinCols));
 }
 
 #ifdef SSV_BOUNDS_CHECK
@@ -1080,6 +1040,10 @@ __global__ void __launch_bounds__(kPT) tcs_final_kernel(TcsArgs a, int nsteps) {
 // row, each half of the m columns.  Bound by the FP64 pipe (4 n m^2
 // multiply-adds a shift); inside the serial chain of the z_b, on one SM per
 // shift, it took 1.34 ms for 40 shifts at n = 4000, m = 16.
+// QH: columns of a thread, ceil(m / 2) rounded up to a power of two (an inactive
+// column costs its FP64 issue slots all the same: 0.96 ms with eight for m = 4,
+// 2000 shifts at n = 1000).
+template <int QH>
 __global__ void __launch_bounds__(kPT) tcs_back_kernel(TcsArgs a, int nsteps, int nbe_first) {
   __shared__ cd zs[kMaxM * kMaxM];
   const int b = blockIdx.x % nsteps + 1, sh = blockIdx.x / nsteps, tid = threadIdx.x;
@@ -1096,18 +1060,18 @@ __global__ void __launch_bounds__(kPT) tcs_back_kernel(TcsArgs a, int nsteps, in
   cd* tout = a.out + (size_t)sh * m * a.ldo;
   const double nanv = __longlong_as_double(0x7ff8000000000000LL);
   const int qh = (m + 1) / 2, q0 = half * qh, q1 = min(m, q0 + qh);
-  cd acc[kMaxM / 2];
+  cd acc[QH];
 #pragma unroll
-  for (int u = 0; u < kMaxM / 2; ++u) acc[u] = mkcd(0.0, 0.0);
+  for (int u = 0; u < QH; ++u) acc[u] = mkcd(0.0, 0.0);
 #pragma unroll 4
   for (int t = 0; t < m; ++t) {
     const cd x = ZT[BCK(i + (size_t)t * n, (size_t)n * m)];
 #pragma unroll
-    for (int u = 0; u < kMaxM / 2; ++u)
+    for (int u = 0; u < QH; ++u)
       if (q0 + u < q1) acc[u] = cfma(x, zs[t + (q0 + u) * m], acc[u]);
   }
 #pragma unroll
-  for (int u = 0; u < kMaxM / 2; ++u)
+  for (int u = 0; u < QH; ++u)
     if (q0 + u < q1) tout[BCK(i, n) + (size_t)(q0 + u) * a.ldo] = bad ? mkcd(nanv, nanv) : acc[u];
 }
 
@@ -1255,7 +1219,7 @@ int solve_tc(const Handle* h, int s, const double* shifts, int mode, double* out
         if (hrows > 0) {
           const long long items = (long long)((hrows + kUM - 1) / kUM) * G;
           const int grid =
-              (int)std::max<long long>(1, std::min<long long>(items, (long long)num_sms() * kCtasU));
+              (int)std::max<long long>(1, std::min<long long>(items, (long long)num_sms()));
           void* tru = trace_begin("tcs_update", st);  // per-launch span when tracing is on
           upd<<<grid, kUT, kUpdSmem, st>>>(a, k, nbe);
           count_launch();
@@ -1270,7 +1234,9 @@ int solve_tc(const Handle* h, int s, const double* shifts, int mode, double* out
       tcs_final_kernel<<<s, kPT, 0, st>>>(a, step);
       count_launch();
       if (mode == SSV_XHAT) {
-        tcs_back_kernel<<<(unsigned)((long long)s * step), kPT, 0, st>>>(a, step, nbe_first);
+        auto back = m <= 2 ? tcs_back_kernel<1> : m <= 4 ? tcs_back_kernel<2> : m <= 8 ? tcs_back_kernel<4>
+                                                                              : tcs_back_kernel<8>;
+        back<<<(unsigned)((long long)s * step), kPT, 0, st>>>(a, step, nbe_first);
         count_launch();
       }
       e = cudaGetLastError();
