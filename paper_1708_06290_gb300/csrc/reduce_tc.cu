@@ -64,8 +64,8 @@ constexpr int kD = kDigits;              // digits per operand value
 constexpr int kBmax = 128;               // reflectors per block at most
 constexpr int kMaxW = 64;                // mini-block width (m) at most
 constexpr int kWinTiles = 4;             // K tiles per exact window (4 x 32 = 128)
-constexpr int kGT = 256;                 // threads of the product kernel
-constexpr int kIssuers = 1;              // MMA completion barriers (one issuing thread)
+constexpr int kDrainT = 256;             // readout and epilogue threads of the product kernel
+constexpr int kGT = kDrainT + 64;        // + the producer's and the issuer's warp
 constexpr unsigned long long kSpin = 1ull << 26;  // grid barrier naps before giving up
 
 // Debug builds (-DSSV_BOUNDS_CHECK): every global index of these kernels is
@@ -116,27 +116,33 @@ __host__ __device__ __forceinline__ size_t tile_index(const DigitMat& M, int dig
 __device__ __forceinline__ void digits_of(double x, int E, unsigned short (&d)[kD]) { digits8(x, E, d); }
 
 // ---------------------------------------------------------------------------
-// Splitting.  Element (r, k) of the source is src[r * sr + k * sk]; rows
+// Splitting.  Element (r, k) of the source is src[off(r) + k * sk]; rows
 // [r_lo, r_hi) and K [k_lo, k_hi) are taken, everything else of a tile is 0.
+// off(r) = r * sr, and for r >= wrap the imaginary part of row r - wrap: the
+// real form of a complex operand (sr and sk counted in doubles).
 // ---------------------------------------------------------------------------
+__device__ __forceinline__ long long row_off(int r, long long sr, int wrap) {
+  return r < wrap ? (long long)r * sr : 1 + (long long)(r - wrap) * sr;
+}
+
 
 // exponent pass: ex[r] = max over the K range of scale_exp(|x|) (ex preset to INT_MIN)
 __global__ void __launch_bounds__(256) split_exp_kernel(const double* __restrict__ src, long long sr,
                                                         long long sk, int r_lo, int r_hi, int k_lo,
-                                                        int k_hi, int kchunk, int* __restrict__ ex,
+                                                        int k_hi, int kchunk, int wrap, int* __restrict__ ex,
                                                         size_t nsrc, size_t nex, int* err) {
   const int tid = threadIdx.x;
   const int rb = r_lo + blockIdx.x * 64;
   const int kb = k_lo + blockIdx.y * kchunk;
   const int ke = min(k_hi, kb + kchunk);
-  if (sk == 1) {
-    // K contiguous: a warp per row, lanes along K
+  if (sk <= 2) {
+    // K (nearly) contiguous: a warp per row, lanes along K
     const int lane = tid & 31, wp = tid >> 5;
     for (int rr = wp; rr < 64; rr += 8) {
       const int r = rb + rr;
       if (r >= r_hi) break;
       double mx = 0.0;
-      for (int k = kb + lane; k < ke; k += 32) mx = fmax(mx, fabs(src[RBCK((size_t)r * sr + k, nsrc, err)]));
+      for (int k = kb + lane; k < ke; k += 32) mx = fmax(mx, fabs(src[RBCK(row_off(r, sr, wrap) + (long long)k * sk, nsrc, err)]));
       for (int o = 16; o > 0; o >>= 1) mx = fmax(mx, __shfl_xor_sync(0xffffffffu, mx, o));
       if (lane == 0) atomicMax(ex + RBCK(r, nex, err), scale_exp(mx));
     }
@@ -148,7 +154,7 @@ __global__ void __launch_bounds__(256) split_exp_kernel(const double* __restrict
     double mx = 0.0;
     if (r < r_hi)
       for (int k = kb + g; k < ke; k += 4)
-        mx = fmax(mx, fabs(src[RBCK((size_t)r * sr + (size_t)k * sk, nsrc, err)]));
+        mx = fmax(mx, fabs(src[RBCK(row_off(r, sr, wrap) + (long long)k * sk, nsrc, err)]));
     part[g][rr] = mx;
     __syncthreads();
     if (g == 0 && r < r_hi) {
@@ -161,19 +167,19 @@ __global__ void __launch_bounds__(256) split_exp_kernel(const double* __restrict
 // digit pass: one CTA per tile (I, J) of [I0, I0 + gridDim.x) x [J0, J0 + gridDim.y)
 __global__ void __launch_bounds__(256) split_dig_kernel(const double* __restrict__ src, long long sr,
                                                         long long sk, int r_lo, int r_hi, int k_lo,
-                                                        int k_hi, DigitMat M, int I0, int J0, size_t nsrc,
-                                                        size_t nex, int* err) {
+                                                        int k_hi, int wrap, DigitMat M, int I0, int J0,
+                                                        size_t nsrc, size_t nex, int* err) {
   __shared__ double t[kTR][kTK + 1];
   const int tid = threadIdx.x;
   const int I = I0 + blockIdx.x, J = J0 + blockIdx.y;
   const int rb = I * kTR, kb = J * kTK;
   for (int e = tid; e < kTileEl; e += 256) {
     int rr, kk;
-    if (sk == 1) { rr = e / kTK; kk = e % kTK; }
+    if (sk <= 2) { rr = e / kTK; kk = e % kTK; }
     else { rr = e % kTR; kk = e / kTR; }
     const int r = rb + rr, k = kb + kk;
     double v = 0.0;
-    if (r >= r_lo && r < r_hi && k >= k_lo && k < k_hi) v = src[RBCK((size_t)r * sr + (size_t)k * sk, nsrc, err)];
+    if (r >= r_lo && r < r_hi && k >= k_lo && k < k_hi) v = src[RBCK(row_off(r, sr, wrap) + (long long)k * sk, nsrc, err)];
     t[rr][kk] = v;
   }
   __syncthreads();
@@ -217,6 +223,8 @@ struct GArgs {
   int sub;
   int ksplit;
   long long kstride;
+  int rs = 1;          // row stride of C in doubles (2: one part of a complex matrix)
+  int wrap = INT_MAX;  // columns from here on: the imaginary parts of columns 0 ..
   int* err;
 };
 
@@ -231,7 +239,11 @@ struct GCfg {
   static constexpr int kNS = 3 * (size_t)kStage + 256 <= 227 * 1024 ? 3 : 2;
   static constexpr size_t kSmem = kNS * (size_t)kStage + 256;
   static constexpr uint32_t kUsed = (uint32_t)LV * NT;
-  static constexpr uint32_t kCols = kUsed <= 32 ? 32 : kUsed <= 64 ? 64 : kUsed <= 128 ? 128 : kUsed <= 256 ? 256 : 512;
+  // TMEM windows: two when they fit (N = 16), so that one is read back while the
+  // next one multiplies
+  static constexpr int kTW = 2 * kUsed <= 512 ? 2 : 1;
+  static constexpr uint32_t kNeed = (uint32_t)kTW * kUsed;
+  static constexpr uint32_t kCols = kNeed <= 32 ? 32 : kNeed <= 64 ? 64 : kNeed <= 128 ? 128 : kNeed <= 256 ? 256 : 512;
   static_assert(kSmem <= 227 * 1024, "shared memory of the digit product");
   static_assert(kUsed <= 512, "TMEM columns");
   static_assert(LV == 8 || LV == 9, "levels");
@@ -250,27 +262,51 @@ __device__ __forceinline__ double pow2(int e) {
   return ldexp(1.0, e);
 }
 
+// a bounded wait of one role: gives up at the poll limit or when another role
+// has (the CTA then leaves together)
+__device__ __forceinline__ bool role_wait(uint32_t mbar, uint32_t parity, volatile int* fail) {
+  for (long long it = 0; it < kWaitLimit / 64; ++it) {
+    if (mbar_wait(mbar, parity, 64)) return true;
+    if (*fail) return false;
+  }
+  *fail = 1;
+  return false;
+}
+
+// Three roles that only meet at mbarriers: a producer thread copies K stages
+// into the stage buffers, an issuing thread multiplies them into a TMEM window,
+// eight warps read finished windows back and write the tile.  So the next
+// stages' copies and products run under the readout and the FP64 epilogue, which
+// had alternated with them (one stage in flight, block barriers around each).
 template <int NT, int LV>
 __global__ void __launch_bounds__(kGT, 1) tc_gemm_kernel(GArgs g) {
   using Cfg = GCfg<NT, LV>;
   constexpr int CPT = NT / 2;
   extern __shared__ __align__(128) unsigned char smem[];
-  constexpr int NS = Cfg::kNS;
-  unsigned long long* mbar = reinterpret_cast<unsigned long long*>(smem + NS * (size_t)Cfg::kStage);
-  uint32_t* tslot = reinterpret_cast<uint32_t*>(mbar + kIssuers + NS);
+  constexpr int NS = Cfg::kNS, TW = Cfg::kTW;
+  // full[NS], empty[NS]: stage buffer copied / multiplied; tfull[TW], tempty[TW]:
+  // TMEM window complete / read back
+  __shared__ __align__(8) unsigned long long mbar[2 * NS + 2 * TW];
+  __shared__ uint32_t tslot;
+  __shared__ volatile int fail;
+  __shared__ int issued[2];  // stages copied, stages multiplied (read when a wait gave up)
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const int quarter = warp & 3, half = warp >> 2;
-  const uint32_t mb = smem_addr(mbar);
-  const uint32_t lmb = mb + 8u * kIssuers;  // lmb + 8 b: loads of stage buffer b
+  const uint32_t full = smem_addr(mbar), empty = full + 8u * NS, tfull = empty + 8u * NS, tempty = tfull + 8u * TW;
   const uint32_t sBase = smem_addr(smem);
   if (warp == 0) {
-    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_addr(tslot)),
+    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_addr(&tslot)),
                  "r"(Cfg::kCols));
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;");
   }
   if (tid == 0) {
-    for (int q = 0; q < kIssuers + NS; ++q) asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(mb + 8u * q));
+    for (int q = 0; q < 2 * NS + 2 * TW; ++q)
+      asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(full + 8u * q),
+                   "r"(q >= 2 * NS + TW ? kDrainT / 32 : 1));
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    fail = 0;
+    issued[0] = 0;
+    issued[1] = 0;
   }
   for (int bq = 0; bq < NS; ++bq) {
     uint4* zp = reinterpret_cast<uint4*>(smem + (size_t)bq * Cfg::kStage + kD * (Cfg::kABytes + Cfg::kBBytes));
@@ -280,11 +316,7 @@ __global__ void __launch_bounds__(kGT, 1) tc_gemm_kernel(GArgs g) {
   fence_before();
   __syncthreads();
   fence_after();
-  const uint32_t tmem = *tslot;
-  uint32_t phase = 0;
-  uint32_t lphase[3] = {0u, 0u, 0u};
-  bool pend[3] = {false, false, false};
-  bool failed = false;
+  const uint32_t tmem = tslot;
   const int iI0 = g.M0 / 128, iI1 = (g.M1 + 127) / 128;
   const int iN0 = g.N0 / NT, iN1 = (g.N1 + NT - 1) / NT;
   const int nI = max(0, iI1 - iI0), nN = max(0, iN1 - iN0);
@@ -311,159 +343,167 @@ __global__ void __launch_bounds__(kGT, 1) tc_gemm_kernel(GArgs g) {
     t.nst = max(0, jhi - jlo);
     return t;
   };
-  // stage st of tile t into buffer b
-  auto stage_in = [&](const Tile& t, int st, int b) {
-    pend[b] = true;
-    if (tid != 0) return;
-    const int J = t.jlo + st;
-    const uint32_t dst = sBase + (uint32_t)b * Cfg::kStage;
-    const uint32_t lb = lmb + 8u * (uint32_t)b;
-    asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(lb),
-                 "r"(Cfg::kStage - Cfg::kBBytes)
-                 : "memory");
-    for (int d = 0; d < kD; ++d)
-      bulk_copy(dst + (uint32_t)d * Cfg::kABytes,
-                A.d + RBCR(tile_index(A, d, J, 2 * t.iI), 2 * kTileEl, A.nd, g.err), Cfg::kABytes, lb);
-    for (int d = 0; d < kD; ++d)
-      bulk_copy(dst + kD * Cfg::kABytes + (uint32_t)d * Cfg::kBBytes,
-                B.d + RBCR(tile_index(B, d, J, t.n0 / kTR) + (size_t)(t.n0 % kTR) * kTK, NT * kTK, B.nd, g.err),
-                Cfg::kBBytes, lb);
-  };
-  bool prefetched = false;  // the first stages of this CTA's next tile are already in flight
-  for (long long tt = blockIdx.x; tt < ntile && !failed; tt += gridDim.x) {
-    const Tile cur = tile_of(tt);
-    const int i0 = cur.iI * 128, n0 = cur.n0, ks = cur.ks;
-    const int nst = cur.nst;
-    // exact level sums of every window, in 64-bit words: word w holds levels
-    // 4w .. 4w + 3, level L at bit 21 - 7 (L - 4 w); a window adds less than
-    // 2^46 to a word, so 2^17 windows (K up to 16 M) cannot overflow it
-    long long wacc[NW][CPT];
-#pragma unroll
-    for (int w = 0; w < NW; ++w)
-#pragma unroll
-      for (int c = 0; c < CPT; ++c) wacc[w][c] = 0;
-    if (!prefetched)
-      for (int q = 0; q < NS - 1 && q < nst; ++q) stage_in(cur, q, q);
-    prefetched = false;
-    for (int st = 0; st < nst; ++st) {
-      const int b = st % NS;
-      const bool lok = mbar_wait(lmb + 8u * (uint32_t)b, lphase[b]);
-      if (__syncthreads_or(!lok)) {
-        failed = true;
-        break;
+  if (warp == kDrainT / 32) {
+    if (lane == 0) {
+      // ---- producer: stage i (counted over all tiles) into buffer i mod NS
+      unsigned i = 0;
+      bool ok = true;
+      for (long long tt = blockIdx.x; tt < ntile && ok; tt += gridDim.x) {
+        const Tile t = tile_of(tt);
+        for (int st = 0; st < t.nst; ++st, ++i) {
+          const uint32_t b = i % NS;
+          if (!role_wait(empty + 8u * b, ((i / NS) & 1u) ^ 1u, &fail)) {
+            ok = false;
+            break;
+          }
+          const int J = t.jlo + st;
+          const uint32_t dst = sBase + b * Cfg::kStage, lb = full + 8u * b;
+          asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(lb),
+                       "r"(Cfg::kStage - Cfg::kBBytes)
+                       : "memory");
+          for (int d = 0; d < kD; ++d)
+            bulk_copy(dst + (uint32_t)d * Cfg::kABytes,
+                      A.d + RBCR(tile_index(A, d, J, 2 * t.iI), 2 * kTileEl, A.nd, g.err), Cfg::kABytes, lb);
+          for (int d = 0; d < kD; ++d)
+            bulk_copy(dst + kD * Cfg::kABytes + (uint32_t)d * Cfg::kBBytes,
+                      B.d + RBCR(tile_index(B, d, J, t.n0 / kTR) + (size_t)(t.n0 % kTR) * kTK, NT * kTK, B.nd, g.err),
+                      Cfg::kBBytes, lb);
+          issued[0] = (int)(i + 1);
+        }
       }
-      lphase[b] ^= 1u;
-      pend[b] = false;
-      if (tid == 0) {
-        // fused levels: the B digit planes of a stage sit side by side (NT rows
-        // each, then the zero plane), so one product of A digit a against B
-        // digits b0 .. b0 + c - 1 (N = NT c <= 256) lands digit b in TMEM level
-        // a + b; the products of a = 0 reach every level (the zero plane stands
-        // for B digit 8) and open the window, so one thread issues them all
-        fence_after();
-        const bool fresh = (st % kWinTiles) == 0;
-        const uint32_t aBase = sBase + (uint32_t)b * Cfg::kStage;
-        const uint32_t bBase = aBase + kD * Cfg::kABytes;
-        constexpr int kMaxC = 256 / NT;
+    }
+  } else if (warp == kDrainT / 32 + 1) {
+    if (lane == 0) {
+      // ---- issuer: window v (counted over all tiles) into TMEM window v mod TW
+      unsigned i = 0, v = 0;
+      bool ok = true;
+      for (long long tt = blockIdx.x; tt < ntile && ok; tt += gridDim.x) {
+        const int nst = tile_of(tt).nst;
+        for (int st = 0; st < nst; ++st, ++i) {
+          const uint32_t b = i % NS, h = v % TW;
+          const bool fresh = (st % kWinTiles) == 0;
+          if (fresh && !role_wait(tempty + 8u * h, ((v / TW) & 1u) ^ 1u, &fail)) ok = false;
+          if (ok && !role_wait(full + 8u * b, (i / NS) & 1u, &fail)) ok = false;
+          if (!ok) break;
+          // fused levels: the B digit planes of a stage sit side by side (NT rows
+          // each, then the zero plane), so one product of A digit a against B
+          // digits b0 .. b0 + c - 1 (N = NT c <= 256) lands digit b in TMEM level
+          // a + b; the products of a = 0 reach every level (the zero plane stands
+          // for B digit 8) and open the window, so one thread issues them all
+          fence_after();
+          const uint32_t aBase = sBase + b * Cfg::kStage;
+          const uint32_t bBase = aBase + kD * Cfg::kABytes;
+          const uint32_t dt = tmem + h * Cfg::kUsed;
+          constexpr int kMaxC = 256 / NT;
 #pragma unroll
-        for (int kk = 0; kk < kTK / 16; ++kk) {
+          for (int kk = 0; kk < kTK / 16; ++kk) {
 #pragma unroll
-          for (int a = 0; a < kD; ++a) {
-            const int nb = a == 0 ? LV : LV - a;  // B digits 0 .. nb - 1 (digit 8: the zero plane)
+            for (int a = 0; a < kD; ++a) {
+              const int nb = a == 0 ? LV : LV - a;  // B digits 0 .. nb - 1 (digit 8: the zero plane)
 #pragma unroll
-            for (int b0 = 0; b0 < nb; b0 += kMaxC) {
-              const int c = min(kMaxC, nb - b0);
-              const uint64_t ad = mat_desc(aBase + (uint32_t)a * Cfg::kABytes + (uint32_t)kk * 256u, 128u, 512u);
-              const uint64_t bd = mat_desc(bBase + (uint32_t)b0 * Cfg::kBBytes + (uint32_t)kk * 256u, 128u, 512u);
-              mma_bf16(tmem + (uint32_t)((a + b0) * NT), ad, bd, idesc_bf16(128, NT * c),
-                       (fresh && kk == 0 && a == 0) ? 0u : 1u);
+              for (int b0 = 0; b0 < nb; b0 += kMaxC) {
+                const int c = min(kMaxC, nb - b0);
+                const uint64_t ad = mat_desc(aBase + (uint32_t)a * Cfg::kABytes + (uint32_t)kk * 256u, 128u, 512u);
+                const uint64_t bd = mat_desc(bBase + (uint32_t)b0 * Cfg::kBBytes + (uint32_t)kk * 256u, 128u, 512u);
+                mma_bf16(dt + (uint32_t)((a + b0) * NT), ad, bd, idesc_bf16(128, NT * c),
+                         (fresh && kk == 0 && a == 0) ? 0u : 1u);
+              }
             }
           }
+          mma_commit(empty + 8u * b);
+          issued[1] = (int)(i + 1);
+          if ((st % kWinTiles) == kWinTiles - 1 || st == nst - 1) {
+            mma_commit(tfull + 8u * h);
+            ++v;
+          }
         }
-        mma_commit(mb);
       }
-      // the buffer of stage st - 1 (its products finished last round) takes stage st + NS - 1
-      if (st + NS - 1 < nst) stage_in(cur, st + NS - 1, (st + NS - 1) % NS);
-      const bool ok = mbar_wait(mb, phase);
-      if (__syncthreads_or(!ok)) {
-        failed = true;
-        break;
-      }
-      phase ^= 1u;
-      if (st == nst - 1 && tt + gridDim.x < ntile) {
-        // every buffer is free: the next tile's first stages stream in during
-        // the drain and the epilogue of this one
-        const Tile nx = tile_of(tt + gridDim.x);
-        for (int q = 0; q < NS - 1 && q < nx.nst; ++q) stage_in(nx, q, q);
-        prefetched = true;
-      }
-      if ((st % kWinTiles) == kWinTiles - 1 || st == nst - 1) {
+    }
+  } else {
+    // ---- readout and epilogue: thread = (row, half of the columns)
+    unsigned v = 0;
+    bool ok = true;
+    for (long long tt = blockIdx.x; tt < ntile && ok; tt += gridDim.x) {
+      const Tile cur = tile_of(tt);
+      const int i0 = cur.iI * 128, n0 = cur.n0, ks = cur.ks;
+      // exact level sums of every window, in 64-bit words: word w holds levels
+      // 4w .. 4w + 3, level L at bit 21 - 7 (L - 4 w); a window adds less than
+      // 2^46 to a word, so 2^17 windows (K up to 16 M) cannot overflow it
+      long long wacc[NW][CPT];
+#pragma unroll
+      for (int w = 0; w < NW; ++w)
+#pragma unroll
+        for (int c = 0; c < CPT; ++c) wacc[w][c] = 0;
+      for (int st = 0; st < cur.nst; st += kWinTiles, ++v) {
+        const uint32_t h = v % TW;
+        ok = __all_sync(0xffffffffu, role_wait(tfull + 8u * h, (v / TW) & 1u, &fail));
+        if (!ok) break;
         fence_after();
 #pragma unroll
         for (int w = 0; w < NW; ++w) {
 #pragma unroll 1
           for (int L = 4 * w; L < min(LV, 4 * w + 4); ++L) {
             uint32_t rv[CPT];
-            tmem_ld_cols<CPT>(tmem + ((uint32_t)(quarter * 32) << 16) + (uint32_t)(L * NT + half * CPT), rv);
+            tmem_ld_cols<CPT>(tmem + h * Cfg::kUsed + ((uint32_t)(quarter * 32) << 16) +
+                                  (uint32_t)(L * NT + half * CPT),
+                              rv);
             const int sh = 21 - 7 * (L - 4 * w);
 #pragma unroll
             for (int c = 0; c < CPT; ++c) wacc[w][c] += (long long)__float2int_rn(__uint_as_float(rv[c])) << sh;
           }
         }
         fence_before();
-        __syncthreads();
+        __syncwarp();
+        if (lane == 0)
+          asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(tempty + 8u * h) : "memory");
       }
-    }
-    if (failed) break;
-    // epilogue: word w weighs 2^{Ea + Eb - 35 - 28 w}; all loads of C first
-    const int r = i0 + quarter * 32 + lane;
-    if (r >= g.M0 && r < g.M1) {
-      const int Ea = A.ex ? A.ex[RBCK(r, (size_t)A.RT * kTR, g.err)] : 1;
-      const size_t c0 = (size_t)ks * g.kstride + (size_t)(r + g.roff);  // C offset of column 0
-      double x[CPT];
+      if (!ok) break;
+      // word w weighs 2^{Ea + Eb - 35 - 28 w}
+      const int r = i0 + quarter * 32 + lane;
+      if (r >= g.M0 && r < g.M1) {
+        const int Ea = A.ex ? A.ex[RBCK(r, (size_t)A.RT * kTR, g.err)] : 1;
+        const size_t c0 = (size_t)ks * g.kstride + (size_t)(r + g.roff) * g.rs;  // C offset of column 0
+        auto cidx = [&](int col) { return RBCK(c0 + row_off(col + g.coff, g.ldc, g.wrap), g.nc, g.err); };
+        // eight columns at a time, their loads of C in flight together
 #pragma unroll
-      for (int c = 0; c < CPT; ++c) {
-        const int col = n0 + half * CPT + c;
-        const int Eb = (col >= g.N0 && col < g.N1) ? (B.ex ? B.ex[RBCK(col, (size_t)B.RT * kTR, g.err)] : 1) : 0;
-        double v = 0.0;
-        if (Ea == kBadExp || Eb == kBadExp) {
-          v = __longlong_as_double(0x7ff8000000000000LL);
-        } else if (Ea > -4000 && Eb > -4000) {
+        for (int cb = 0; cb < CPT; cb += 8) {
+          double x[8], old[8];
 #pragma unroll
-          for (int w = NW - 1; w >= 0; --w) v = fma((double)wacc[w][c], pow2(Ea + Eb - 35 - 28 * w), v);
-        }
-        x[c] = v;
-      }
-      auto cidx = [&](int col) { return RBCK(c0 + (long long)(col + g.coff) * g.ldc, g.nc, g.err); };
-      if (g.sub) {
-        double old[CPT];
+          for (int c = 0; c < 8; ++c) {
+            const int col = n0 + half * CPT + cb + c;
+            old[c] = (g.sub && col >= g.N0 && col < g.N1) ? g.C[cidx(col)] : 0.0;
+          }
 #pragma unroll
-        for (int c = 0; c < CPT; ++c) {
-          const int col = n0 + half * CPT + c;
-          old[c] = (col >= g.N0 && col < g.N1) ? g.C[cidx(col)] : 0.0;
-        }
+          for (int c = 0; c < 8; ++c) {
+            const int col = n0 + half * CPT + cb + c;
+            const int Eb = (col >= g.N0 && col < g.N1) ? (B.ex ? B.ex[RBCK(col, (size_t)B.RT * kTR, g.err)] : 1) : 0;
+            double xv = 0.0;
+            if (Ea == kBadExp || Eb == kBadExp) {
+              xv = __longlong_as_double(0x7ff8000000000000LL);
+            } else if (Ea > -4000 && Eb > -4000) {
 #pragma unroll
-        for (int c = 0; c < CPT; ++c) {
-          const int col = n0 + half * CPT + c;
-          if (col >= g.N0 && col < g.N1) g.C[cidx(col)] = old[c] - x[c];
-        }
-      } else {
+              for (int w = NW - 1; w >= 0; --w) xv = fma((double)wacc[w][cb + c], pow2(Ea + Eb - 35 - 28 * w), xv);
+            }
+            x[c] = xv;
+          }
 #pragma unroll
-        for (int c = 0; c < CPT; ++c) {
-          const int col = n0 + half * CPT + c;
-          if (col >= g.N0 && col < g.N1) g.C[cidx(col)] = x[c];
+          for (int c = 0; c < 8; ++c) {
+            const int col = n0 + half * CPT + cb + c;
+            if (col >= g.N0 && col < g.N1) g.C[cidx(col)] = g.sub ? old[c] - x[c] : x[c];
+          }
         }
       }
     }
   }
-  if (failed) {
-    if (tid == 0) {
-      atomicExch(g.err, 1);
-      mbar_wait(mb, phase);
-      for (int b = 0; b < NS; ++b)
-        if (pend[b]) mbar_wait(lmb + 8u * (uint32_t)b, lphase[b]);
-    }
-    __syncthreads();
+  __syncwarp();
+  __syncthreads();
+  if (fail != 0 && tid == 0) {
+    // a completion never arrived: record it and give the copies and products in
+    // flight one more bounded wait
+    atomicExch(g.err, 1);
+    const unsigned nl = (unsigned)issued[0], nm = (unsigned)issued[1];
+    for (unsigned i = nl > NS ? nl - NS : 0; i < nl; ++i) mbar_wait(full + 8u * (i % NS), (i / NS) & 1u);
+    for (unsigned i = nm > NS ? nm - NS : 0; i < nm; ++i) mbar_wait(empty + 8u * (i % NS), (i / NS) & 1u);
   }
   fence_before();
   __syncthreads();
@@ -487,6 +527,7 @@ constexpr int kRedPiv = 8192;            // pivot rows of the QR (two slots of 6
 constexpr int kRedS = 8192 + 128;        // S = V^T V_s ((j + wp) x wp)
 constexpr int kRedTotal = kRedS + 8192;
 constexpr size_t kPanFixed = 4096 + 4096 + 256 + 64 * 3 + 8 + 8 * kBmax;  // doubles besides the panel
+constexpr size_t kPanSmem = 200 * 1024;  // with the staged rows of V and Y at most
 
 struct PanArgs {
   double* P;          // panel column t, matrix row r: P[r + t * ldp]
@@ -505,6 +546,7 @@ struct PanArgs {
   double* tau;        // tau of reflector t at tau[t]
   DigitMat vcol;      // V's digits, operand row = reflector, K = r (exponent 1: the unit pivot is
                       // every reflector's largest entry)
+  int staged;         // the CTA's rows of V and Y (j columns) go to shared memory
   double* part;       // [3][G][kPartW]
   double* red;        // kRedTotal
   unsigned* bar;      // this launch's arrival counter (zero at its start)
@@ -515,27 +557,26 @@ struct PanArgs {
 
 // Grid-wide barrier with a bounded wait: false once any CTA has given up.
 // *bar counts this launch's arrivals (every panel launch has a counter of its
-// own, zeroed at the start of the reduction); the k-th barrier completes when
-// it reaches k * gridDim.x, so a CTA waits for the multiple of gridDim.x at or
-// above its own arrival.
-__device__ bool grid_sync(unsigned* bar, int* err) {
+// own, zeroed at the start of the reduction); the k-th barrier (k from 1) of
+// the launch completes when it reaches k * gridDim.x.  The arrival returns
+// nothing: it and the first poll are on their way together.
+__device__ bool grid_sync(unsigned* bar, int* err, unsigned k) {
   __shared__ int s_ok;
   __syncthreads();
   if (threadIdx.x == 0) {
-    __threadfence();
-    const unsigned arrived = atomicAdd(bar, 1u) + 1u;
-    const unsigned target = (arrived + gridDim.x - 1) / gridDim.x * gridDim.x;
+    const unsigned target = k * gridDim.x;
+    asm volatile("fence.acq_rel.gpu;\n\tred.release.gpu.global.add.u32 [%0], 1;" ::"l"(bar) : "memory");
     unsigned long long spins = 0;
     for (;;) {
       unsigned now;
       asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(now) : "l"(bar) : "memory");
       if ((int)(now - target) >= 0) break;
-      if (*(volatile int*)err != 0) break;
+      if ((spins & 15) == 15 && *(volatile int*)err != 0) break;
       if (++spins > kSpin) {
         atomicExch(err, 1);
         break;
       }
-      if (spins > 64) __nanosleep(32);
+      if (spins > 4096) __nanosleep(32);
     }
     __threadfence();
     s_ok = (*(volatile int*)err == 0);
@@ -546,8 +587,9 @@ __device__ bool grid_sync(unsigned* bar, int* err) {
 
 // Sums with every thread of the CTA: out(e) = sum_k term(e, k) for e in
 // [e0, e1), k < count(e); tpe threads (a power of two <= 32, the largest with
-// tpe (e1 - e0) <= kPT) share an output, each taking every tpe-th k eight at
-// a time, then a shuffle tree.  The order is fixed, so every CTA that forms the
+// tpe (e1 - e0) <= kPT) share an output, each taking every tpe-th k sixteen at
+// a time (all loads of a panel's cross-CTA sums in flight at once), then a
+// shuffle tree.  The order is fixed, so every CTA that forms the
 // same sums gets the same bits.
 template <typename Count, typename Term, typename Store>
 __device__ __forceinline__ void block_sums(int e0, int e1, Count count, Term term, Store store) {
@@ -564,14 +606,17 @@ __device__ __forceinline__ void block_sums(int e0, int e1, Count count, Term ter
     double acc = 0.0;
     if (act) {
       const int K = count(e);
-      int k = sub;
-      for (; k + 7 * tpe < K; k += 8 * tpe) {
-        double v[8];
+      for (int k = sub; k < K; k += 16 * tpe) {
+        double v[16];
 #pragma unroll
-        for (int q = 0; q < 8; ++q) v[q] = term(e, k + q * tpe);
-        acc += ((v[0] + v[1]) + (v[2] + v[3])) + ((v[4] + v[5]) + (v[6] + v[7]));
+        for (int q = 0; q < 16; ++q) v[q] = k + q * tpe < K ? term(e, k + q * tpe) : 0.0;
+#pragma unroll
+        for (int h = 8; h > 0; h >>= 1)
+#pragma unroll
+          for (int q = 0; q < 8; ++q)
+            if (q < h) v[q] += v[q + h];
+        acc += v[0];
       }
-      for (; k < K; k += tpe) acc += term(e, k);
     }
     for (int o = tpe >> 1; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
     if (act && sub == 0) store(e, acc);
@@ -605,6 +650,9 @@ __global__ void __launch_bounds__(kPT, 1) panel_kernel(PanArgs a) {
   double* taus = piv + 64;
   double* misc = taus + 64;
   double* tw = misc + 8;                 // 8 warps x kBmax: a row of T
+  double* Vb = tw + 8 * kBmax;           // staged: V(ra + rl, i) at Vb[i * rpc + rl]
+  double* Yb = Vb + (size_t)rpc * j;     // staged: Y of the same rows
+  unsigned nbar = 0;                     // grid barriers so far
   auto slot = [&](int q, int gg) { return a.part + RBCR(((size_t)q * G + gg) * kPartW, kPartW, a.npart, a.err); };
   // checked element accesses (plain indexing in normal builds)
   auto Pi = [&](long long i) -> double& { return a.P[RBCK(i, a.np, a.err)]; };
@@ -614,57 +662,85 @@ __global__ void __launch_bounds__(kPT, 1) panel_kernel(PanArgs a) {
   // partial e of CTA gg in slot q
   auto Pt = [&](int q, int gg, int e) { return a.part + RBCK(((size_t)q * G + gg) * kPartW + e, a.npart, a.err); };
 
+  // Everything the panel reads of earlier results starts at once: its columns,
+  // the rows of V that carry the right update's coefficients, and (staged) this
+  // CTA's rows of V and Y.  Read in the loops that use them they cost an L2
+  // round trip every few multiply-adds.
+  auto cp8 = [](double* dst, const double* src) {
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" ::"r"(smem_addr(dst)), "l"(src) : "memory");
+  };
   for (int e = tid; e < nr * w; e += kPT) {
     const int rl = e % nr, t = e / nr;
-    Ps[t * rpc + rl] = Pi((size_t)(ra + rl) + (size_t)t * a.ldp);
+    cp8(Ps + t * rpc + rl, &Pi((size_t)(ra + rl) + (size_t)t * a.ldp));
   }
+  for (int e = tid; e < w * j; e += kPT) {
+    const int t = e % w, i = e / w;
+    cp8(Vc + t * j + i, &Vi((size_t)(a.c0 + t) + (size_t)i * a.ldv));
+  }
+  if (a.staged) {
+    for (int e = tid; e < nr * j; e += kPT) {
+      const int rl = e % nr, i = e / nr;
+      cp8(Vb + i * rpc + rl, &Vi((size_t)(ra + rl) + (size_t)i * a.ldv));
+      cp8(Yb + i * rpc + rl, a.Y + RBCK((size_t)a.yoff + ra + rl + (size_t)i * a.ldy, a.ny, a.err));
+    }
+  }
+  asm volatile("cp.async.commit_group;\n\tcp.async.wait_group 0;" ::: "memory");
+  __syncthreads();
+  // V and Y of this CTA's rows (reflector i < j)
+  auto vr = [&](int rl, int i) -> double {
+    return a.staged ? Vb[i * rpc + rl] : Vi((size_t)(ra + rl) + (size_t)i * a.ldv);
+  };
+  auto yr = [&](int rl, int i) -> double {
+    return a.staged ? Yb[i * rpc + rl] : a.Y[RBCK((size_t)a.yoff + ra + rl + (size_t)i * a.ldy, a.ny, a.err)];
+  };
+  // P(rl, t) -= sum_{i < j} f(rl, i) g(i, t): tpe lanes share an entry
+  auto rank_update = [&](auto f, auto gq) {
+    const int nE = nr * w;
+    int tpe = 8;
+    while (tpe > 1 && tpe * nE > kPT) tpe >>= 1;
+    const int per = kPT / tpe, sub = tid % tpe;
+    for (int c0 = 0; c0 < nE; c0 += per) {
+      const int e = c0 + tid / tpe;
+      const bool act = e < nE;
+      const int rl = act ? e % nr : 0, t = act ? e / nr : 0;
+      double acc = 0.0;
+      if (act) {
+#pragma unroll 8
+        for (int i = sub; i < j; i += tpe) acc = fma(f(rl, i), gq(i, t), acc);
+      }
+      for (int o = tpe >> 1; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
+      if (act && sub == 0) Ps[t * rpc + rl] -= acc;
+    }
+    __syncthreads();
+  };
   if (j > 0) {
     // from the right: P -= Y(rows, 0:j) V(c0:c0+w, 0:j)^T
-    for (int e = tid; e < w * j; e += kPT) {
-      const int t = e % w, i = e / w;
-      Vc[t * j + i] = Vi((size_t)(a.c0 + t) + (size_t)i * a.ldv);
-    }
-    __syncthreads();
-    for (int e = tid; e < nr * w; e += kPT) {
-      const int rl = e % nr, t = e / nr;
-      const size_t y0 = (size_t)a.yoff + ra + rl;
-      double acc = Ps[t * rpc + rl];
-      for (int i = 0; i < j; ++i) acc = fma(-a.Y[RBCK(y0 + (size_t)i * a.ldy, a.ny, a.err)], Vc[t * j + i], acc);
-      Ps[t * rpc + rl] = acc;
-    }
-    __syncthreads();
+    rank_update(yr, [&](int i, int t) { return Vc[t * j + i]; });
     // from the left: W = V^T P, Z = T^T W, P -= V Z
     double* my = slot(0, g);
     for (int e = tid; e < j * w; e += kPT) {
       const int i = e / w, t = e % w;
-      const size_t v0 = (size_t)ra + (size_t)i * a.ldv;
       double acc = 0.0;
-      for (int rl = 0; rl < nr; ++rl) acc = fma(Vi(v0 + rl), Ps[t * rpc + rl], acc);
+#pragma unroll 8
+      for (int rl = 0; rl < nr; ++rl) acc = fma(vr(rl, i), Ps[t * rpc + rl], acc);
       my[RBCK(e, kPartW, a.err)] = acc;
     }
-    if (!grid_sync(a.bar, a.err)) return;
+    if (!grid_sync(a.bar, a.err, ++nbar)) return;
     const int ch = (j * w + G - 1) / G;
     const int e0 = min(j * w, g * ch), e1 = min(j * w, (g + 1) * ch);
     block_sums(
         e0, e1, [&](int) { return G; }, [&](int e, int gg) { return __ldcg(Pt(0, gg, e)); },
         [&](int e, double v) { *Ri(kRedW + e) = v; });
-    if (!grid_sync(a.bar, a.err)) return;
+    if (!grid_sync(a.bar, a.err, ++nbar)) return;
     block_sums(
         e0, e1, [&](int e) { return e / w + 1; },
         [&](int e, int k) { return Ti(k + (size_t)(e / w) * kBmax) * __ldcg(Ri(kRedW + k * w + e % w)); },
         [&](int e, double v) { *Ri(kRedZ + e) = v; });
-    if (!grid_sync(a.bar, a.err)) return;
+    if (!grid_sync(a.bar, a.err, ++nbar)) return;
     for (int e = tid; e < j * w; e += kPT) Zs[e] = __ldcg(Ri(kRedZ + e));
     __syncthreads();
-    for (int e = tid; e < nr * w; e += kPT) {
-      const int rl = e % nr, t = e / nr;
-      const size_t v0 = (size_t)ra + rl;
-      double acc = Ps[t * rpc + rl];
-      for (int i = 0; i < j; ++i) acc = fma(-Vi(v0 + (size_t)i * a.ldv), Zs[i * w + t], acc);
-      Ps[t * rpc + rl] = acc;
-    }
+    rank_update(vr, [&](int i, int t) { return Zs[i * w + t]; });
   }
-  __syncthreads();
   // Householder QR of the mini-block: reflector t zeroes rows > pv0 + t of column t
   for (int t = 0; t < wp; ++t) {
     const int pr = a.pv0 + t;
@@ -683,7 +759,7 @@ __global__ void __launch_bounds__(kPT, 1) panel_kernel(PanArgs a) {
       if (tid < nk) slot(t & 1, g)[tid] = rs[tid] + rs[64 + tid] + rs[128 + tid] + rs[192 + tid];
       if (pr >= ra && pr < ra + nr && tid < nk) *Ri(kRedPiv + (t & 1) * 64 + tid) = Ps[(size_t)(t + tid) * rpc + (pr - ra)];
     }
-    if (!grid_sync(a.bar, a.err)) return;
+    if (!grid_sync(a.bar, a.err, ++nbar)) return;
     {
       const int q = t & 1;
       block_sums(
@@ -750,14 +826,14 @@ __global__ void __launch_bounds__(kPT, 1) panel_kernel(PanArgs a) {
     const int i = e / wp, t = e % wp;
     double acc = 0.0;
     if (i < j) {
-      const size_t v0 = (size_t)ra + (size_t)i * a.ldv;
-      for (int rl = 0; rl < nr; ++rl) acc = fma(Vi(v0 + rl), vt(rl, t), acc);
+#pragma unroll 8
+      for (int rl = 0; rl < nr; ++rl) acc = fma(vr(rl, i), vt(rl, t), acc);
     } else {
       for (int rl = 0; rl < nr; ++rl) acc = fma(vt(rl, i - j), vt(rl, t), acc);
     }
     slot(2, g)[RBCK(e, kPartW, a.err)] = acc;
   }
-  if (!grid_sync(a.bar, a.err)) return;
+  if (!grid_sync(a.bar, a.err, ++nbar)) return;
   {
     const int ch = (ns + G - 1) / G;
     block_sums(
@@ -765,7 +841,7 @@ __global__ void __launch_bounds__(kPT, 1) panel_kernel(PanArgs a) {
         [&](int e, int gg) { return __ldcg(Pt(2, gg, e)); },
         [&](int e, double v) { *Ri(kRedS + e) = v; });
   }
-  if (!grid_sync(a.bar, a.err)) return;
+  if (!grid_sync(a.bar, a.err, ++nbar)) return;
   // T's new columns (Eq. for T, one reflector at a time): row i of CTA i mod G,
   // a warp per row, lanes along k; S and the row staged in shared memory
   double* Ss = Vc;  // ns <= 8192 doubles over Vc and Zs
@@ -798,7 +874,11 @@ __global__ void __launch_bounds__(kPT, 1) panel_kernel(PanArgs a) {
 }
 
 // Y's new columns (Eq. for Y): Y(:, j + t) = sum_{t' <= t} (A V_s - Y V^T V_s)(:, t') T_s(t', t)
-// for every row of E; A V_s arrives as `ks` partial sums.
+// for every row of E; A V_s arrives as `ks` partial sums. Bound by the latency
+// of a thread's sum over the j <= 128 columns: kYfixSplit lanes share it, which
+// also makes four times the blocks (47 at 3000 rows of 4 columns otherwise).
+constexpr int kYfixSplit = 4;
+static_assert(kYfixSplit * kMaxW <= 256, "a row of Y to a block at least");
 __global__ void __launch_bounds__(256) yfix_kernel(const double* __restrict__ AV, int ks, long long kstride,
                                                    long long ldav, int rows, double* __restrict__ Y,
                                                    long long ldy, int j, int wp, const double* __restrict__ S,
@@ -807,26 +887,33 @@ __global__ void __launch_bounds__(256) yfix_kernel(const double* __restrict__ AV
   extern __shared__ double ysm[];
   double* Ss = ysm;              // S(i, t) for i < j
   double* Tt = Ss + j * wp;      // Tt[t' + t * wp] = T(j + t', j + t)
-  const int R = 256 / wp;        // rows per CTA
-  double* us = Tt + wp * wp;     // us[t' * R + rl]
+  const int R = 256 / (kYfixSplit * wp);  // rows per CTA
+  double* us = Tt + wp * wp;              // us[(kq * wp + t') * R + rl]
   const int tid = threadIdx.x;
   for (int e = tid; e < j * wp; e += 256) Ss[e] = S[RBCK(e, 8192, err)];
   for (int e = tid; e < wp * wp; e += 256)
     Tt[e] = T[RBCK((size_t)(j + e % wp) + (size_t)(j + e / wp) * kBmax, (size_t)kBmax * kBmax, err)];
   __syncthreads();
-  const int rl = tid % R, tp = tid / R;
+  const int rl = tid % R, tq = tid / R, tp = tq % wp, kq = tq / wp;
   const int e = blockIdx.x * R + rl;
-  const bool act = tp < wp && e < rows;
+  const bool act = kq < kYfixSplit && e < rows;
   if (act) {
     double u = 0.0;
-    for (int q = 0; q < ks; ++q) u += AV[RBCK((size_t)q * kstride + e + (size_t)tp * ldav, nav, err)];
-    for (int i = 0; i < j; ++i) u = fma(-Y[RBCK(e + (size_t)i * ldy, ny, err)], Ss[i * wp + tp], u);
-    us[tp * R + rl] = u;
+    for (int q = kq; q < ks; q += kYfixSplit) u += AV[RBCK((size_t)q * kstride + e + (size_t)tp * ldav, nav, err)];
+#pragma unroll 4
+    for (int i = kq; i < j; i += kYfixSplit)
+      u = fma(-Y[RBCK(e + (size_t)i * ldy, ny, err)], Ss[i * wp + tp], u);
+    us[tq * R + rl] = u;
   }
   __syncthreads();
-  if (act) {
+  if (act && kq == 0) {
     double y = 0.0;
-    for (int q = 0; q <= tp; ++q) y = fma(us[q * R + rl], Tt[q + tp * wp], y);
+    for (int q = 0; q <= tp; ++q) {
+      double u = us[q * R + rl];
+#pragma unroll
+      for (int k = 1; k < kYfixSplit; ++k) u += us[(k * wp + q) * R + rl];
+      y = fma(u, Tt[q + tp * wp], y);
+    }
     Y[RBCK(e + (size_t)(j + tp) * ldy, ny, err)] = y;
   }
 }
@@ -975,21 +1062,21 @@ size_t rtc_layout(int n, int p, unsigned char* base, RtcScratch* S) {
 
 // rows [r_lo, r_hi) x K [k_lo, k_hi) of src into M (tiles of whole 128-row pairs)
 int split_into(const double* src, long long sr, long long sk, int r_lo, int r_hi, int k_lo, int k_hi,
-               const DigitMat& M, size_t nsrc, int* err, cudaStream_t st) {
+               const DigitMat& M, size_t nsrc, int* err, cudaStream_t st, int wrap = INT_MAX) {
   const size_t nex = (size_t)M.RT * kTR;
   if (r_hi <= r_lo || k_hi <= k_lo) return SSV_OK;
   if (M.ex) {
     SSV_CUDA_TRY(cudaMemsetAsync(M.ex, 0x80, sizeof(int) * (size_t)M.RT * kTR, st));
     const int kchunk = 512;
     dim3 grid((unsigned)((r_hi - r_lo + 63) / 64), (unsigned)((k_hi - k_lo + kchunk - 1) / kchunk));
-    split_exp_kernel<<<grid, 256, 0, st>>>(src, sr, sk, r_lo, r_hi, k_lo, k_hi, kchunk, M.ex, nsrc, nex, err);
+    split_exp_kernel<<<grid, 256, 0, st>>>(src, sr, sk, r_lo, r_hi, k_lo, k_hi, kchunk, wrap, M.ex, nsrc, nex, err);
     count_launch();
     SSV_CUDA_TRY(cudaGetLastError());
   }
   const int I0 = 2 * (r_lo / 128), I1 = 2 * ((r_hi + 127) / 128);
   const int J0 = k_lo / kTK, J1 = (k_hi + kTK - 1) / kTK;
-  split_dig_kernel<<<dim3((unsigned)(I1 - I0), (unsigned)(J1 - J0)), 256, 0, st>>>(src, sr, sk, r_lo, r_hi, k_lo,
-                                                                                 k_hi, M, I0, J0, nsrc, nex, err);
+  split_dig_kernel<<<dim3((unsigned)(I1 - I0), (unsigned)(J1 - J0)), 256, 0, st>>>(src, sr, sk, r_lo, r_hi, k_lo, k_hi,
+                                                                                 wrap, M, I0, J0, nsrc, nex, err);
   count_launch();
   SSV_CUDA_TRY(cudaGetLastError());
   return SSV_OK;
@@ -1075,7 +1162,10 @@ int run_panel(RtcScratch& S, int n, int p, double* P, size_t np, long long ldp, 
   a.ny = S.nY;
   a.ntau = ntau;
   a.npart = S.npart;
-  const size_t smem = sizeof(double) * ((size_t)rpc * w + kPanFixed);
+  size_t smem = sizeof(double) * ((size_t)rpc * w + kPanFixed);
+  const size_t rows = sizeof(double) * 2 * (size_t)rpc * j;
+  a.staged = smem + rows <= kPanSmem ? 1 : 0;
+  if (a.staged) smem += rows;
   SSV_CUDA_TRY(cudaFuncSetAttribute(panel_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
   void* args[] = {&a};
   SSV_CUDA_TRY(cudaLaunchCooperativeKernel((const void*)panel_kernel, dim3(G), dim3(kPT), args, smem, st));
@@ -1091,7 +1181,7 @@ int run_panel(RtcScratch& S, int n, int p, double* P, size_t np, long long ldp, 
   g.kstride = S.ldE * kMaxW;
   int rc = gemm_long(wp, g, st);
   if (rc != SSV_OK) return rc;
-  const int R = 256 / wp;
+  const int R = 256 / (kYfixSplit * wp);
   const size_t ysm = sizeof(double) * ((size_t)j * wp + (size_t)wp * wp + 256);
   SSV_CUDA_TRY(cudaFuncSetAttribute(yfix_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)ysm));
   yfix_kernel<<<(rowsE + R - 1) / R, 256, ysm, st>>>(S.AV, g.ksplit, g.kstride, S.ldE, rowsE, S.Y, S.ldE, j, wp,
