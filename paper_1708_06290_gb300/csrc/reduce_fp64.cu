@@ -389,8 +389,8 @@ int reduce_fp64(Handle* h, const double* A, long long lda, const double* B, long
   return SSV_OK;
 }
 
-int apply_q_fp64(const Handle* h, int ncols, const double* Xhat, long long ldx, double* X,
-                 long long ldX, cudaStream_t st) {
+int apply_q(const Handle* h, int ncols, const double* Xhat, long long ldx, double* X, long long ldX,
+            bool digits, cudaStream_t st) {
   const int n = h->n;
   if (ncols == 0) return SSV_OK;
   cd* Xc = reinterpret_cast<cd*>(X);
@@ -403,6 +403,11 @@ int apply_q_fp64(const Handle* h, int ncols, const double* Xhat, long long ldx, 
   }
   const int nblk = q_blocks(h->kb) + q_blocks(h->ka);
   if (nblk == 0) return SSV_OK;
+  if (digits && apply_q_tc_supported(h->n, ncols)) {
+    const int rc = apply_q_tc(h, ncols, Xc, ldX, st);
+    if (rc != SSV_ENOMEM) return rc;
+    cudaGetLastError();  // no room for its scratch (nothing written yet): the FP64 path needs none
+  }
   const QSrc q = q_src(h);
   const double* T = h->Tq;
   // Columns per cluster: the fewest columns on the busiest SM, then the widest

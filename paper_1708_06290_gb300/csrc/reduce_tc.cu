@@ -1344,4 +1344,230 @@ int reduce_tc(Handle* h, cudaStream_t st) {
   return rc;
 }
 
+
+// ---------------------------------------------------------------------------
+// X <- Q X for many columns: the reflectors in blocks of kBmax, Q_b = I - V T V^T,
+// with W = V^T X and X -= V Z as digit products.  Z = T W is a triangular solve,
+// T^{-1} = striu(V^T V) + diag(1 / tau) (Joffrain, Low, Quintana-Orti, van de
+// Geijn and Van Zee 2006), so no T is formed.  X enters as its real form, the
+// real parts of all columns, then the imaginary parts.
+// ---------------------------------------------------------------------------
+namespace {
+
+// V(r, k), explicit zeros and unit pivots, of reflectors 0 .. cnt - 1 with pivot
+// rows pv + k, from their packed storage; rows r0 .. n - 1, columns 0 .. kBmax - 1
+__global__ void __launch_bounds__(256) qv_kernel(const double* __restrict__ src, int n, int r0, int pv, int cnt,
+                                                 double* __restrict__ V, long long ldv) {
+  const int r = r0 + blockIdx.x * 256 + threadIdx.x, k = blockIdx.y;
+  if (r >= n) return;
+  const int d = r - pv - k;
+  V[r + (size_t)k * ldv] = (k >= cnt || d < 0) ? 0.0 : d == 0 ? 1.0 : src[r + (size_t)k * n];
+}
+
+// Z = T W for 8 real columns per CTA, a warp each: lane l holds the rows l, l +
+// 32, ..; back substitution from the last reflector, then Z's digits with the
+// column's exponent.  W and S = V^T V arrive as partial sums.
+__global__ void __launch_bounds__(256) qz_kernel(const double* __restrict__ Wp, int ksw, long long wstride,
+                                                 const double* __restrict__ Sp, int kss, int cnt, int ncol,
+                                                 const double* __restrict__ tau, DigitMat Z) {
+  extern __shared__ double S[];  // kBmax x kBmax
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  for (int e = tid; e < cnt * kBmax; e += 256) {
+    double v = 0.0;
+    for (int q = 0; q < kss; ++q) v += Sp[(size_t)q * kBmax * kBmax + e];
+    S[e] = v;
+  }
+  __syncthreads();
+  const int c = blockIdx.x * 8 + warp;
+  if (c >= ncol) return;
+  double w[kBmax / 32];
+#pragma unroll
+  for (int u = 0; u < kBmax / 32; ++u) {
+    const int i = lane + 32 * u;
+    double v = 0.0;
+    if (i < cnt)
+      for (int q = 0; q < ksw; ++q) v += Wp[(size_t)q * wstride + i + (size_t)c * kBmax];
+    w[u] = v;
+  }
+#pragma unroll
+  for (int uk = kBmax / 32 - 1; uk >= 0; --uk) {
+    for (int lk = 31; lk >= 0; --lk) {
+      const int k = 32 * uk + lk;
+      if (k >= cnt) continue;
+      const double z = __shfl_sync(0xffffffffu, w[uk], lk) * __ldg(tau + k);
+      if (lane == lk) w[uk] = z;
+#pragma unroll
+      for (int u = 0; u < kBmax / 32; ++u)
+        if (u < uk || (u == uk && lane < lk)) w[u] = fma(-S[lane + 32 * u + k * kBmax], z, w[u]);
+    }
+  }
+  double mx = 0.0;
+#pragma unroll
+  for (int u = 0; u < kBmax / 32; ++u) mx = fmax(mx, w[u] == w[u] ? fabs(w[u]) : INFINITY);
+  for (int o = 16; o > 0; o >>= 1) mx = fmax(mx, __shfl_xor_sync(0xffffffffu, mx, o));
+  const int E = scale_exp(mx);
+  if (lane == 0) Z.ex[c] = E;
+#pragma unroll
+  for (int u = 0; u < kBmax / 32; ++u) {
+    unsigned short d[kD];
+    digits_of(w[u], E, d);
+    const size_t off = (size_t)tile_off_kg(c % kTR, lane, kTK / 8);
+#pragma unroll
+    for (int l = 0; l < kD; ++l) Z.d[tile_index(Z, l, u, c / kTR) + off] = d[l];
+  }
+}
+
+// every entry NaN when a wait gave up
+__global__ void q_fail_kernel(const int* err, cd* X, long long ldx, int n, int ncols) {
+  if (*err == 0) return;
+  const double nanv = __longlong_as_double(0x7ff8000000000000LL);
+  for (long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x; e < (long long)n * ncols;
+       e += (long long)gridDim.x * blockDim.x)
+    X[e % n + (size_t)(e / n) * ldx] = mkcd(nanv, nanv);
+}
+
+constexpr int kQCols = 1024;  // complex columns at a time (bounds the digit scratch)
+
+struct QtcScratch {
+  double *V, *W, *S;
+  long long ldv;
+  DigitMat vrow, vcol, xcol, zcol;
+  int* err;
+  size_t nV, nW;
+};
+
+size_t qtc_layout(int n, int nc, unsigned char* base, QtcScratch* Q) {
+  size_t off = 0;
+  auto take = [&](size_t bytes) {
+    unsigned char* q = base ? base + off : nullptr;
+    off += rup((long long)bytes, 256);
+    return q;
+  };
+  QtcScratch s;
+  const int RTn = 2 * ((n + 127) / 128), KTn = (n + kTK - 1) / kTK, KTb = kBmax / kTK;
+  const int RTc = 2 * ((2 * nc + 127) / 128);
+  s.ldv = rup(n, 32);
+  s.nV = (size_t)s.ldv * kBmax;
+  s.nW = (size_t)8 * kBmax * 2 * nc;
+  s.V = (double*)take(sizeof(double) * s.nV);
+  s.W = (double*)take(sizeof(double) * s.nW);
+  s.S = (double*)take(sizeof(double) * 8 * kBmax * kBmax);
+  s.err = (int*)take(sizeof(int));
+  auto dm = [&](int RT, int KT, bool ex) {
+    DigitMat M;
+    M.RT = RT;
+    M.KT = KT;
+    M.nd = digit_bytes(RT, KT) / sizeof(unsigned short);
+    M.d = (unsigned short*)take(digit_bytes(RT, KT));
+    M.ex = ex ? (int*)take(sizeof(int) * (size_t)RT * kTR) : nullptr;
+    return M;
+  };
+  s.vrow = dm(RTn, KTb, true);
+  s.vcol = dm(2, KTn, false);
+  s.xcol = dm(RTc, KTn, true);
+  s.zcol = dm(RTc, KTb, true);
+  if (Q) *Q = s;
+  return off;
+}
+
+}  // namespace
+
+// Where the digit products win over the FP64 pipe: that path grows with n^2 ncols,
+// this one up to some 256 columns with the number of blocks alone (2.1 us a
+// reflector before its sums were read in one trip).  FP64 / digit products measured
+// at n ncols = 262144: n = 1024, 256 columns 1.99 / 2.09 ms; n = 2048, 128 columns
+// 5.1 / 4.2; n = 4096, 64 columns 13.2 / 8.9; below: n = 1536, 128 columns 3.0 / 3.2;
+// n = 384, 640 columns 0.96 / 0.99; far above, n = 4096, 640 columns 82.7 / 15.2.
+bool apply_q_tc_supported(int n, int ncols) { return n >= 384 && (long long)n * ncols >= 275000; }
+
+size_t apply_q_tc_scratch_bytes(int n, int ncols) {
+  return apply_q_tc_supported(n, ncols) ? qtc_layout(n, std::min(ncols, kQCols), nullptr, nullptr) : 0;
+}
+
+int apply_q_tc(const Handle* h, int ncols, cd* X, long long ldX, cudaStream_t st) {
+  const int n = h->n, m = h->m, sms = std::max(1, num_sms());
+  const int ncm = std::min(ncols, kQCols);
+  unsigned char* base = nullptr;
+  const size_t bytes = qtc_layout(n, ncm, nullptr, nullptr);
+  SSV_CUDA_TRY(pool_alloc((void**)&base, bytes, st));
+  QtcScratch Q;
+  qtc_layout(n, ncm, base, &Q);
+  int rc = SSV_OK;
+  auto step = [&](int r) {
+    if (rc == SSV_OK) rc = r;
+  };
+  auto cu = [&](cudaError_t e) {
+    if (rc == SSV_OK && e != cudaSuccess) {
+      set_cuda_error(e);
+      rc = SSV_ECUDA;
+    }
+  };
+  cu(cudaMemsetAsync(Q.err, 0, sizeof(int), st));
+  cu(cudaFuncSetAttribute(qz_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                          (int)(sizeof(double) * kBmax * kBmax)));
+  const int nbA = (h->ka + kBmax - 1) / kBmax, nbB = (h->kb + kBmax - 1) / kBmax;
+  const int KTn = (n + kTK - 1) / kTK;
+  auto args = [&](const DigitMat& A, const DigitMat& B, int J0, int J1, int M0, int M1, int N1, double* C, size_t nc,
+                  long long ldc) {
+    GArgs g;
+    g.seg = GSeg{A, B, J0, J1};
+    g.M0 = M0; g.M1 = M1; g.N0 = 0; g.N1 = N1;
+    g.roff = 0; g.coff = 0;
+    g.C = C; g.nc = nc; g.ldc = ldc;
+    g.sub = 0; g.ksplit = 1; g.kstride = 0;
+    g.err = Q.err;
+    return g;
+  };
+  for (int b = nbA + nbB - 1; b >= 0 && rc == SSV_OK; --b) {
+    const bool isA = b >= nbB;
+    const int j = (isA ? b - nbB : b) * kBmax;
+    const int cnt = std::min(kBmax, (isA ? h->ka : h->kb) - j), pv = isA ? m + j : j;
+    const double* src = isA ? h->H + (size_t)j * n : h->R + (size_t)j * n;
+    const double* tau = isA ? h->tauA + j : h->tauB + j;
+    qv_kernel<<<dim3((unsigned)((n - pv + 255) / 256), kBmax), 256, 0, st>>>(src, n, pv, pv, cnt, Q.V, Q.ldv);
+    count_launch();
+    cu(cudaGetLastError());
+    step(split_into(Q.V, 1, Q.ldv, pv, n, 0, cnt, Q.vrow, Q.nV, Q.err, st));
+    step(split_into(Q.V, Q.ldv, 1, 0, cnt, pv, n, Q.vcol, Q.nV, Q.err, st));
+    // S = V^T V
+    const int J0 = pv / kTK, nst = KTn - J0;
+    GArgs gs = args(Q.vcol, Q.vcol, J0, KTn, 0, cnt, cnt, Q.S, (size_t)8 * kBmax * kBmax, kBmax);
+    gs.ksplit = std::max(1, std::min(8, nst / 4));
+    gs.kstride = (long long)kBmax * kBmax;
+    if (rc == SSV_OK) step(gemm_launch<32, 9>(gs, st));
+    for (int c0 = 0; c0 < ncols && rc == SSV_OK; c0 += ncm) {
+      const int nc = std::min(ncm, ncols - c0);
+      double* Xd = reinterpret_cast<double*>(X + (size_t)c0 * ldX);
+      const size_t nX = 2 * ((size_t)ldX * (nc - 1) + n);
+      step(split_into(Xd, 2 * ldX, 2, 0, 2 * nc, pv, n, Q.xcol, nX, Q.err, st, nc));
+      GArgs gw = args(Q.vcol, Q.xcol, J0, KTn, 0, cnt, 2 * nc, Q.W, Q.nW, kBmax);
+      const int nN = (2 * nc + 31) / 32;
+      gw.ksplit = std::max(1, std::min({8, sms / nN, std::max(1, nst / 4)}));
+      gw.kstride = (long long)kBmax * 2 * nc;
+      if (rc == SSV_OK) step(gemm_launch<32, 9>(gw, st));
+      qz_kernel<<<(2 * nc + 7) / 8, 256, sizeof(double) * kBmax * kBmax, st>>>(
+          Q.W, gw.ksplit, gw.kstride, Q.S, gs.ksplit, cnt, 2 * nc, tau, Q.zcol);
+      count_launch();
+      cu(cudaGetLastError());
+      GArgs gx = args(Q.vrow, Q.zcol, 0, (cnt + kTK - 1) / kTK, pv, n, 2 * nc, Xd, nX, 2 * ldX);
+      gx.sub = 1;
+      gx.rs = 2;
+      gx.wrap = nc;
+      if (rc == SSV_OK) step(gemm_launch<64, 8>(gx, st));
+    }
+  }
+  if (rc == SSV_OK) {
+    q_fail_kernel<<<256, 256, 0, st>>>(Q.err, X, ldX, n, ncols);
+    count_launch();
+    cu(cudaGetLastError());
+  }
+  if (rc == SSV_ENOMEM) rc = SSV_ECUDA;  // X may have changed: not for another path to redo
+  cudaError_t e2 = cudaFreeAsync(base, st);
+  if (e2 != cudaSuccess && rc == SSV_OK) {
+    set_cuda_error(e2);
+    rc = SSV_ECUDA;
+  }
+  return rc;
+}
+
 }  // namespace ssv

@@ -264,7 +264,7 @@ int ssv_solve(ssv_handle hh, int s, const double* shifts, const ssv_opts* o_in, 
     rc = solve_fp64(h, s, shifts, &o, out, ldo, status, resid, st);
     trace_end(tr, st);
   }
-  if (rc == SSV_OK && o.mode == SSV_X) rc = apply_q_fp64(h, s * h->m, out, ldo, out, ldo, st);
+  if (rc == SSV_OK && o.mode == SSV_X) rc = apply_q(h, s * h->m, out, ldo, out, ldo, o.precision != SSV_FP64, st);
   return rc;
 }
 
@@ -287,7 +287,7 @@ int ssv_solve_rhs(ssv_handle hh, int s, const double* shifts, const double* bhat
   void* tr = trace_begin("solve_rhs", st);
   rc = solve_fp64_rhs(h, s, shifts, bhat, ldb, &o, out, ldo, status, st);
   trace_end(tr, st);
-  if (rc == SSV_OK && o.mode == SSV_X) rc = apply_q_fp64(h, s, out, ldo, out, ldo, st);
+  if (rc == SSV_OK && o.mode == SSV_X) rc = apply_q(h, s, out, ldo, out, ldo, false, st);
   return rc;
 }
 
@@ -309,7 +309,7 @@ int ssv_solve_trans(ssv_handle hh, int s, const double* shifts, const double* ch
   void* tr = trace_begin("solve_trans", st);
   rc = solve_fp64_trans(h, s, shifts, chat, ldc, &o, out, ldo, status, st);
   trace_end(tr, st);
-  if (rc == SSV_OK && o.mode == SSV_X) rc = apply_q_fp64(h, s, out, ldo, out, ldo, st);
+  if (rc == SSV_OK && o.mode == SSV_X) rc = apply_q(h, s, out, ldo, out, ldo, false, st);
   return rc;
 }
 
@@ -489,7 +489,7 @@ int ssv_apply_q(ssv_handle hh, int ncols, const double* Xhat, long long ldx, dou
   if (ncols == 0) return SSV_OK;
   if (!Xhat || !X || ldx < h->n || ldX < h->n) return SSV_EINVAL;
   if (!h->has_q) return SSV_ENOTSUP;
-  return apply_q_fp64(h, ncols, Xhat, ldx, X, ldX, (cudaStream_t)stream);
+  return apply_q(h, ncols, Xhat, ldx, X, ldX, true, (cudaStream_t)stream);
 }
 
 int ssv_get_reduced(ssv_handle hh, double* H, long long ldh, double* R, long long ldr, double* Ct,
@@ -521,6 +521,9 @@ int ssv_footprint(int n, int m, int p, int s, const ssv_opts* o_in, size_t* byte
   else
     *bytes = o.precision == SSV_MIXED ? solve_mixed_scratch_bytes(n, m, p, s, &o)
                                       : solve_fp64_scratch_bytes(n, m, p, s, &o);
+  // the back-transform runs once the solve's scratch has gone back
+  if (o.mode == SSV_X && o.precision != SSV_FP64)
+    *bytes = std::max(*bytes, apply_q_tc_scratch_bytes(n, s * m));
   return SSV_OK;
 }
 

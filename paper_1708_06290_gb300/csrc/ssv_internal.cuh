@@ -111,8 +111,13 @@ int reduce_fp64(Handle* h, const double* A, long long lda, const double* B, long
                 const double* C, long long ldc, int arith, cudaStream_t st);
 // back-transform X = Q Xhat (reduce_fp64.cu)
 size_t q_t_count(int n, int m);
-int apply_q_fp64(const Handle* h, int ncols, const double* Xhat, long long ldx, double* X,
-                 long long ldX, cudaStream_t st);
+// X = Q Xhat; digits: many columns may go through apply_q_tc
+int apply_q(const Handle* h, int ncols, const double* Xhat, long long ldx, double* X, long long ldX,
+            bool digits, cudaStream_t st);
+// the same for many columns, with digit products on the tensor cores (reduce_tc.cu)
+bool apply_q_tc_supported(int n, int ncols);
+size_t apply_q_tc_scratch_bytes(int n, int ncols);
+int apply_q_tc(const Handle* h, int ncols, cd* X, long long ldX, cudaStream_t st);
 // load a stored reduced triple with explicit zeros (reduce_fp64.cu)
 int load_reduced(Handle* h, const double* H, long long ldh, const double* R, long long ldr,
                  const double* Ct, long long ldc, cudaStream_t st);

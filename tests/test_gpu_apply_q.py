@@ -1,7 +1,8 @@
-"""Back-transform X = Q Xhat in blocks of 32 reflectors: every grouping of
-columns and rows (1-4 columns per cluster, 1-8 CTAs per cluster, ragged last
-block, more and fewer reflectors of Q_B than a block) against the definition
-of Q: Q^T Q = I, B = Q R, A Q = Q H.
+"""Back-transform X = Q Xhat in blocks of reflectors: on the FP64 pipe every
+grouping of columns and rows (1-4 columns per cluster, 1-8 CTAs per cluster),
+on the tensor cores several column chunks, in both a ragged last block and more
+and fewer reflectors of Q_B than a block, against the definition of Q: Q^T Q = I,
+B = Q R, A Q = Q H.
 
 Tolerance: a product of n Householder reflectors in compact WY form has a
 backward error of a small multiple of n eps per column; 50 n eps as for the
@@ -19,7 +20,10 @@ pytestmark = pytest.mark.gpu
 
 @pytest.mark.parametrize("n,m,ncols,pad", [(2, 1, 1, 0), (33, 1, 1, 0), (34, 2, 3, 1), (97, 32, 5, 0),
                                            (65, 40, 2, 3), (300, 5, 40, 0), (300, 3, 153, 0), (290, 16, 305, 7),
-                                           (1100, 4, 24, 0), (2300, 2, 2, 5), (700, 8, 620, 0)])
+                                           (1100, 4, 24, 0), (2300, 2, 2, 5), (700, 8, 620, 0),
+                                           # wide: digit products on the tensor cores
+                                           (384, 1, 720, 0), (769, 3, 365, 2), (1153, 130, 240, 0),
+                                           (800, 2, 1100, 1), (1500, 16, 330, 0)])
 def test_apply_q_definition(n, m, ncols, pad):
     from paper_1708_06290_gb300 import ssv
     sysr = W.random_system(n, m, 1, seed=5200 + n + m + ncols)
