@@ -30,7 +30,12 @@ static __device__ __forceinline__ int cluster_ld(const int* p, int rank) {
   return v;
 }
 
-// launch `grid` blocks in clusters of R (grid a multiple of R, R <= 8)
+static __device__ __forceinline__ void cluster_st(double* p, int rank, double v) {
+  asm volatile("st.shared::cluster.f64 [%0], %1;" ::"r"(cluster_map(p, rank)), "d"(v) : "memory");
+}
+
+// launch `grid` blocks in clusters of R (grid a multiple of R;
+// R > 8 needs cudaFuncAttributeNonPortableClusterSizeAllowed set on the kernel)
 template <typename... KArgs, typename... Args>
 cudaError_t launch_cluster(void (*kern)(KArgs...), int grid, int threads, int R, size_t smem, cudaStream_t st,
                            Args... args) {

@@ -23,17 +23,18 @@
 //
 // A column of the V factor of a block's reflectors has entries of magnitude
 // <= 1 with a unit pivot (|v_r| <= 1 because |alpha - beta| >= |beta| >=
-// |x_r|), so V by columns uses the fixed exponent 1 and the panel kernel
+// |x_r|), so V by columns uses the fixed exponent 1 and the QR kernel
 // writes those digits as the reflectors appear; V by rows (mostly far below
 // 1) is split with per-row exponents at the end of the block.
 //
 // Per block of jb reflectors (rows r0 = z + m .. n-1, trailing columns
 // z + b ..):
-//   per mini-block (panel kernel, cooperative, FP64):
+//   per mini-block (FP64):
 //     P <- P - Y V(cols, :)^T  (from the right),  P <- P - V T^T V^T P  (left),
-//     Householder QR of the mini-block, T's new columns (Eq. for T),
-//   then Y's new columns (Eq. for Y): Y_s = (A V_s - Y V^T V_s) T_s, with
-//     A V_s on the tensor cores (A = the matrix at the start of the block);
+//     one cooperative launch; Householder QR of the mini-block, one cluster;
+//   then A V_s and V^T V_s in one product on the tensor cores (A = the matrix at
+//     the start of the block), and the new columns of Y (Eq. for Y),
+//     Y_s = (A V_s - Y V^T V_s) T_s, and of T (Eq. for T);
 //   block end (Algorithm 3, all on the tensor cores but the T^T product):
 //     A(:, z+m:) -= Y V^T  (rows above r0 and C: from column z + m; rows r0..:
 //                           from column z + b),
@@ -49,6 +50,7 @@
 #include <algorithm>
 #include <climits>
 
+#include "cluster.cuh"
 #include "tc_common.cuh"
 
 namespace ssv {
@@ -225,6 +227,11 @@ struct GArgs {
   long long kstride;
   int rs = 1;          // row stride of C in doubles (2: one part of a complex matrix)
   int wrap = INT_MAX;  // columns from here on: the imaginary parts of columns 0 ..
+  // with C2: one more row tile, B's first 128 rows in A's place, rows < N1 written
+  // to C2 (leading dimension kBmax, partial sums kstride2 apart): V^T V_s beside A V_s
+  double* C2 = nullptr;
+  size_t nc2 = 0;
+  long long kstride2 = 0;
   int* err;
 };
 
@@ -347,18 +354,21 @@ __global__ void __launch_bounds__(kGT, 1) tc_gemm_kernel(GArgs g) {
   const uint32_t tmem = tslot;
   const int iI0 = g.M0 / 128, iI1 = (g.M1 + 127) / 128;
   const int iN0 = g.N0 / NT, iN1 = (g.N1 + NT - 1) / NT;
-  const int nI = max(0, iI1 - iI0), nN = max(0, iN1 - iN0);
+  const int nA = max(0, iI1 - iI0), nN = max(0, iN1 - iN0);
+  const int nI = nA + (LV == 9 && g.C2 != nullptr ? 1 : 0);
   const long long ntile = (long long)nI * nN * g.ksplit;
-  const DigitMat& A = g.seg.A;
   const DigitMat& B = g.seg.B;
   constexpr int NW = (LV + 3) / 4;  // 64-bit words of the level sums
   struct Tile {
     int iI, n0, ks, jlo, nst;
+    bool vv;  // B against itself
   };
   auto tile_of = [&](long long tt) {
     Tile t;
     t.n0 = (iN0 + (int)(tt % nN)) * NT;
-    t.iI = iI0 + (int)((tt / nN) % nI);
+    const int it = (int)((tt / nN) % nI);
+    t.vv = LV == 9 && it >= nA;
+    t.iI = t.vv ? 0 : iI0 + it;
     t.ks = (int)(tt / ((long long)nN * nI));
     int jlo = g.seg.J0, jhi = g.seg.J1;
     if (g.ksplit > 1) {
@@ -378,6 +388,7 @@ __global__ void __launch_bounds__(kGT, 1) tc_gemm_kernel(GArgs g) {
       bool ok = true;
       for (long long tt = blockIdx.x; tt < ntile && ok; tt += gridDim.x) {
         const Tile t = tile_of(tt);
+        const DigitMat& A = LV == 9 && t.vv ? g.seg.B : g.seg.A;
         for (int st = 0; st < t.nst; ++st, ++i) {
           const uint32_t b = i % NS;
           if (!role_wait(empty + 8u * b, ((i / NS) & 1u) ^ 1u, &fail)) {
@@ -488,10 +499,16 @@ __global__ void __launch_bounds__(kGT, 1) tc_gemm_kernel(GArgs g) {
       if (!ok) break;
       // word w weighs 2^{Ea + Eb - 35 - 28 w}
       const int r = i0 + quarter * 32 + lane;
-      if (r >= g.M0 && r < g.M1) {
+      if (LV == 9 && cur.vv ? r < g.N1 : (r >= g.M0 && r < g.M1)) {
+        const DigitMat& A = LV == 9 && cur.vv ? g.seg.B : g.seg.A;
+        double* const C = LV == 9 && cur.vv ? g.C2 : g.C;
         const int Ea = A.ex ? A.ex[RBCK(r, (size_t)A.RT * kTR, g.err)] : 1;
-        const size_t c0 = (size_t)ks * g.kstride + (size_t)(r + g.roff) * g.rs;  // C offset of column 0
-        auto cidx = [&](int col) { return RBCK(c0 + row_off(col + g.coff, g.ldc, g.wrap), g.nc, g.err); };
+        const long long ldc = LV == 9 && cur.vv ? kBmax : g.ldc;
+        // C offset of column 0
+        const size_t c0 = LV == 9 && cur.vv ? (size_t)ks * g.kstride2 + r : (size_t)ks * g.kstride + (size_t)(r + g.roff) * g.rs;
+        auto cidx = [&](int col) {
+          return RBCK(c0 + row_off(col + g.coff, ldc, g.wrap), LV == 9 && cur.vv ? g.nc2 : g.nc, g.err);
+        };
         // eight columns at a time, their loads of C in flight together
 #pragma unroll
         for (int cb = 0; cb < CPT; cb += 8) {
@@ -499,7 +516,7 @@ __global__ void __launch_bounds__(kGT, 1) tc_gemm_kernel(GArgs g) {
 #pragma unroll
           for (int c = 0; c < 8; ++c) {
             const int col = n0 + half * CPT + cb + c;
-            old[c] = (g.sub && col >= g.N0 && col < g.N1) ? g.C[cidx(col)] : 0.0;
+            old[c] = (g.sub && col >= g.N0 && col < g.N1) ? C[cidx(col)] : 0.0;
           }
 #pragma unroll
           for (int c = 0; c < 8; ++c) {
@@ -519,7 +536,7 @@ __global__ void __launch_bounds__(kGT, 1) tc_gemm_kernel(GArgs g) {
 #pragma unroll
           for (int c = 0; c < 8; ++c) {
             const int col = n0 + half * CPT + cb + c;
-            if (col >= g.N0 && col < g.N1) g.C[cidx(col)] = g.sub ? old[c] - x[c] : x[c];
+            if (col >= g.N0 && col < g.N1) C[cidx(col)] = g.sub ? old[c] - x[c] : x[c];
           }
         }
       }
@@ -543,46 +560,42 @@ __global__ void __launch_bounds__(kGT, 1) tc_gemm_kernel(GArgs g) {
 }
 
 // ---------------------------------------------------------------------------
-// Panel of one mini-block (Algorithm 2 between two updates of Y), one
-// cooperative launch: CTA g owns a contiguous range of the panel rows
-// r0 .. n-1, kept in shared memory (column-major per CTA); cross-CTA sums go
-// through per-CTA partial slots and a bounded grid barrier.
+// Panel of one mini-block (Algorithm 2 between two updates of Y).  First its
+// columns receive the block's reflectors so far (panel_update_kernel, one
+// cooperative launch): CTA g owns a contiguous range of the panel rows r0 .. n-1,
+// kept in shared memory (column-major per CTA); cross-CTA sums go through
+// per-CTA partial slots and a bounded grid barrier.  Then one cluster factors
+// them (panel_qr_kernel).
 // ---------------------------------------------------------------------------
 constexpr int kPT = 256;
-constexpr int kPartW = 8192;             // partial-sum slot per CTA (doubles)
+constexpr int kPartW = 4096;             // partial-sum slot per CTA (doubles)
 constexpr int kPanRowsW = 8192;          // rows x columns of the panel per CTA at most
 constexpr int kRedW = 0;                 // W = V^T P (j x w)
 constexpr int kRedZ = 4096;              // Z = T^T W
-constexpr int kRedPiv = 8192;            // pivot rows of the QR (two slots of 64)
-constexpr int kRedS = 8192 + 128;        // S = V^T V_s ((j + wp) x wp)
-constexpr int kRedTotal = kRedS + 8192;
-constexpr size_t kPanFixed = 4096 + 4096 + 256 + 64 * 3 + 8 + 8 * kBmax;  // doubles besides the panel
+constexpr int kRedTotal = 8192;
+constexpr size_t kPanFixed = 4096 + 4096;  // doubles besides the panel
 constexpr size_t kPanSmem = 200 * 1024;  // with the staged rows of V and Y at most
 
 struct PanArgs {
   double* P;          // panel column t, matrix row r: P[r + t * ldp]
   long long ldp;
   int r0, n;          // panel rows [r0, n)
-  int w, wp;          // panel columns; reflectors generated (wp <= w)
-  int pv0;            // pivot row of reflector t: pv0 + t
+  int w;              // panel columns
   int j;              // reflectors of the block before this mini-block
   int c0;             // matrix column of panel column 0 (rows c0.. of V: the right update)
-  double* V;          // V(r, i) = V[r + i * ldv], explicit zeros and unit pivots
+  const double* V;    // V(r, i) = V[r + i * ldv], explicit zeros and unit pivots
   long long ldv;
-  double* T;          // T(i, k) = T[i + k * kBmax], upper triangular
+  const double* T;    // T(i, k) = T[i + k * kBmax], upper triangular
   const double* Y;    // Y(matrix row r, i) = Y[yoff + r + i * ldy]
   long long ldy;
   int yoff;
-  double* tau;        // tau of reflector t at tau[t]
-  DigitMat vcol;      // V's digits, operand row = reflector, K = r (exponent 1: the unit pivot is
-                      // every reflector's largest entry)
   int staged;         // the CTA's rows of V and Y (j columns) go to shared memory
-  double* part;       // [3][G][kPartW]
+  double* part;       // [G][kPartW]
   double* red;        // kRedTotal
   unsigned* bar;      // this launch's arrival counter (zero at its start)
   int* err;
   // extents (doubles from each pointer on) the debug build checks
-  size_t np, nv, ny, ntau, npart;
+  size_t np, nv, ny, npart;
 };
 
 // Grid-wide barrier with a bounded wait: false once any CTA has given up.
@@ -662,11 +675,10 @@ __device__ __forceinline__ void put_digits_v(const DigitMat& M, int row, int k, 
   (void)err;
 }
 
-__global__ void __launch_bounds__(kPT, 1) panel_kernel(PanArgs a) {
+__global__ void __launch_bounds__(kPT, 1) panel_update_kernel(PanArgs a) {
   extern __shared__ double psm[];
   const int G = gridDim.x, g = blockIdx.x, tid = threadIdx.x;
-  const int warp = tid >> 5, lane = tid & 31;
-  const int w = a.w, wp = a.wp, j = a.j;
+  const int w = a.w, j = a.j;
   const int L = a.n - a.r0;
   const int rpc = (L + G - 1) / G;
   const int ra = a.r0 + g * rpc;
@@ -674,23 +686,16 @@ __global__ void __launch_bounds__(kPT, 1) panel_kernel(PanArgs a) {
   double* Ps = psm;                      // Ps[t * rpc + rl]
   double* Vc = Ps + (size_t)rpc * w;     // Vc[t * j + i] = V(c0 + t, i)
   double* Zs = Vc + 4096;                // Zs[i * w + t]
-  double* rs = Zs + 4096;                // 4 x 64 block partials
-  double* dots = rs + 256;
-  double* piv = dots + 64;
-  double* taus = piv + 64;
-  double* misc = taus + 64;
-  double* tw = misc + 8;                 // 8 warps x kBmax: a row of T
-  double* Vb = tw + 8 * kBmax;           // staged: V(ra + rl, i) at Vb[i * rpc + rl]
+  double* Vb = Zs + 4096;                // staged: V(ra + rl, i) at Vb[i * rpc + rl]
   double* Yb = Vb + (size_t)rpc * j;     // staged: Y of the same rows
   unsigned nbar = 0;                     // grid barriers so far
-  auto slot = [&](int q, int gg) { return a.part + RBCR(((size_t)q * G + gg) * kPartW, kPartW, a.npart, a.err); };
   // checked element accesses (plain indexing in normal builds)
   auto Pi = [&](long long i) -> double& { return a.P[RBCK(i, a.np, a.err)]; };
-  auto Vi = [&](long long i) -> double& { return a.V[RBCK(i, a.nv, a.err)]; };
-  auto Ti = [&](long long i) -> double& { return a.T[RBCK(i, (size_t)kBmax * kBmax, a.err)]; };
+  auto Vi = [&](long long i) -> const double& { return a.V[RBCK(i, a.nv, a.err)]; };
+  auto Ti = [&](long long i) -> const double& { return a.T[RBCK(i, (size_t)kBmax * kBmax, a.err)]; };
   auto Ri = [&](long long i) { return a.red + RBCK(i, (size_t)kRedTotal, a.err); };
-  // partial e of CTA gg in slot q
-  auto Pt = [&](int q, int gg, int e) { return a.part + RBCK(((size_t)q * G + gg) * kPartW + e, a.npart, a.err); };
+  // partial e of CTA gg
+  auto Pt = [&](int gg, int e) { return a.part + RBCK((size_t)gg * kPartW + e, a.npart, a.err); };
 
   // Everything the panel reads of earlier results starts at once: its columns,
   // the rows of V that carry the right update's coefficients, and (staged) this
@@ -743,209 +748,256 @@ __global__ void __launch_bounds__(kPT, 1) panel_kernel(PanArgs a) {
     }
     __syncthreads();
   };
-  if (j > 0) {
-    // from the right: P -= Y(rows, 0:j) V(c0:c0+w, 0:j)^T
-    rank_update(yr, [&](int i, int t) { return Vc[t * j + i]; });
-    // from the left: W = V^T P, Z = T^T W, P -= V Z
-    double* my = slot(0, g);
-    for (int e = tid; e < j * w; e += kPT) {
-      const int i = e / w, t = e % w;
-      double acc = 0.0;
+  // from the right: P -= Y(rows, 0:j) V(c0:c0+w, 0:j)^T
+  rank_update(yr, [&](int i, int t) { return Vc[t * j + i]; });
+  // from the left: W = V^T P, Z = T^T W, P -= V Z
+  for (int e = tid; e < j * w; e += kPT) {
+    const int i = e / w, t = e % w;
+    double acc = 0.0;
 #pragma unroll 8
-      for (int rl = 0; rl < nr; ++rl) acc = fma(vr(rl, i), Ps[t * rpc + rl], acc);
-      my[RBCK(e, kPartW, a.err)] = acc;
-    }
-    if (!grid_sync(a.bar, a.err, ++nbar)) return;
-    const int ch = (j * w + G - 1) / G;
-    const int e0 = min(j * w, g * ch), e1 = min(j * w, (g + 1) * ch);
-    block_sums(
-        e0, e1, [&](int) { return G; }, [&](int e, int gg) { return __ldcg(Pt(0, gg, e)); },
-        [&](int e, double v) { *Ri(kRedW + e) = v; });
-    if (!grid_sync(a.bar, a.err, ++nbar)) return;
-    block_sums(
-        e0, e1, [&](int e) { return e / w + 1; },
-        [&](int e, int k) { return Ti(k + (size_t)(e / w) * kBmax) * __ldcg(Ri(kRedW + k * w + e % w)); },
-        [&](int e, double v) { *Ri(kRedZ + e) = v; });
-    if (!grid_sync(a.bar, a.err, ++nbar)) return;
-    for (int e = tid; e < j * w; e += kPT) Zs[e] = __ldcg(Ri(kRedZ + e));
-    __syncthreads();
-    rank_update(vr, [&](int i, int t) { return Zs[i * w + t]; });
+    for (int rl = 0; rl < nr; ++rl) acc = fma(vr(rl, i), Ps[t * rpc + rl], acc);
+    *Pt(g, RBCK(e, kPartW, a.err)) = acc;
   }
-  // Householder QR of the mini-block: reflector t zeroes rows > pv0 + t of column t
-  for (int t = 0; t < wp; ++t) {
-    const int pr = a.pv0 + t;
-    const int nk = w - t;  // columns t .. w-1 (k = t: the squared norm below the pivot)
-    {
-      const int kk = tid & 63, grp = tid >> 6;
-      double acc = 0.0;
-      if (kk < nk) {
-        const double* ck = Ps + (size_t)(t + kk) * rpc;
-        const double* ct = Ps + (size_t)t * rpc;
-        for (int rl = grp; rl < nr; rl += 4)
-          if (ra + rl > pr) acc = fma(ck[rl], ct[rl], acc);
-      }
-      rs[grp * 64 + kk] = acc;
-      __syncthreads();
-      if (tid < nk) slot(t & 1, g)[tid] = rs[tid] + rs[64 + tid] + rs[128 + tid] + rs[192 + tid];
-      if (pr >= ra && pr < ra + nr && tid < nk) *Ri(kRedPiv + (t & 1) * 64 + tid) = Ps[(size_t)(t + tid) * rpc + (pr - ra)];
-    }
-    if (!grid_sync(a.bar, a.err, ++nbar)) return;
-    {
-      const int q = t & 1;
-      block_sums(
-          0, nk, [&](int) { return G; }, [&](int e, int gg) { return __ldcg(Pt(q, gg, e)); },
-          [&](int e, double v) { dots[e] = v; });
-      if (tid < nk) piv[tid] = __ldcg(Ri(kRedPiv + (t & 1) * 64 + tid));
-    }
-    __syncthreads();
-    if (tid == 0) {
-      const double sig = dots[0], alpha = piv[0];
-      double tk = 0.0, scal = 0.0, beta = alpha;
-      if (sig != 0.0) {
-        const double nrm = sqrt(fma(alpha, alpha, sig));
-        beta = alpha >= 0.0 ? -nrm : nrm;
-        tk = (beta - alpha) / beta;
-        scal = 1.0 / (alpha - beta);
-      }
-      misc[0] = tk;
-      misc[1] = scal;
-      misc[2] = beta;
-      taus[t] = tk;
-      if (g == 0) a.tau[RBCK(t, a.ntau, a.err)] = tk;
-    }
-    __syncthreads();
-    const double tk = misc[0], scal = misc[1], beta = misc[2];
-    if (tk != 0.0) {
-      // columns k > t: P(:, k) -= tau v (v^T P(:, k)),  v^T P(:, k) = P(pr, k) + scal d_k
-      for (int e = tid; e < nr * (nk - 1); e += kPT) {
-        const int rl = e % nr, kq = 1 + e / nr;
-        const int r = ra + rl;
-        const double wk = fma(scal, dots[kq], piv[kq]);
-        double* pk = Ps + (size_t)(t + kq) * rpc + rl;
-        if (r > pr) *pk = fma(-tk * wk, Ps[(size_t)t * rpc + rl] * scal, *pk);
-        else if (r == pr) *pk = fma(-tk, wk, *pk);
-      }
-      __syncthreads();
-      for (int rl = tid; rl < nr; rl += kPT) {
-        const int r = ra + rl;
-        double* pt = Ps + (size_t)t * rpc + rl;
-        if (r > pr) *pt *= scal;
-        else if (r == pr) *pt = beta;
-      }
-    }
-    __syncthreads();
-  }
-  // the panel back, the new columns of V (values and digits)
+  if (!grid_sync(a.bar, a.err, ++nbar)) return;
+  const int ch = (j * w + G - 1) / G;
+  const int e0 = min(j * w, g * ch), e1 = min(j * w, (g + 1) * ch);
+  block_sums(
+      e0, e1, [&](int) { return G; }, [&](int e, int gg) { return __ldcg(Pt(gg, e)); },
+      [&](int e, double v) { *Ri(kRedW + e) = v; });
+  if (!grid_sync(a.bar, a.err, ++nbar)) return;
+  block_sums(
+      e0, e1, [&](int e) { return e / w + 1; },
+      [&](int e, int k) { return Ti(k + (size_t)(e / w) * kBmax) * __ldcg(Ri(kRedW + k * w + e % w)); },
+      [&](int e, double v) { *Ri(kRedZ + e) = v; });
+  if (!grid_sync(a.bar, a.err, ++nbar)) return;
+  for (int e = tid; e < j * w; e += kPT) Zs[e] = __ldcg(Ri(kRedZ + e));
+  __syncthreads();
+  rank_update(vr, [&](int i, int t) { return Zs[i * w + t]; });
   for (int e = tid; e < nr * w; e += kPT) {
     const int rl = e % nr, t = e / nr;
     Pi((size_t)(ra + rl) + (size_t)t * a.ldp) = Ps[t * rpc + rl];
   }
-  auto vt = [&](int rl, int t) -> double {
-    const int r = ra + rl, pr = a.pv0 + t;
-    return r < pr ? 0.0 : (r == pr ? 1.0 : Ps[(size_t)t * rpc + rl]);
-  };
-  for (int e = tid; e < nr * wp; e += kPT) {
-    const int rl = e % nr, t = e / nr;
-    const double v = vt(rl, t);
-    Vi((size_t)(ra + rl) + (size_t)(j + t) * a.ldv) = v;
-    if (v != 0.0) put_digits_v(a.vcol, j + t, ra + rl, v, a.err);
-  }
-  // S = V(:, 0:j+wp)^T V_s over the panel rows
-  const int ns = (j + wp) * wp;
-  for (int e = tid; e < ns; e += kPT) {
-    const int i = e / wp, t = e % wp;
-    double acc = 0.0;
-    if (i < j) {
-#pragma unroll 8
-      for (int rl = 0; rl < nr; ++rl) acc = fma(vr(rl, i), vt(rl, t), acc);
-    } else {
-      for (int rl = 0; rl < nr; ++rl) acc = fma(vt(rl, i - j), vt(rl, t), acc);
-    }
-    slot(2, g)[RBCK(e, kPartW, a.err)] = acc;
-  }
-  if (!grid_sync(a.bar, a.err, ++nbar)) return;
-  {
-    const int ch = (ns + G - 1) / G;
-    block_sums(
-        min(ns, g * ch), min(ns, (g + 1) * ch), [&](int) { return G; },
-        [&](int e, int gg) { return __ldcg(Pt(2, gg, e)); },
-        [&](int e, double v) { *Ri(kRedS + e) = v; });
-  }
-  if (!grid_sync(a.bar, a.err, ++nbar)) return;
-  // T's new columns (Eq. for T, one reflector at a time): row i of CTA i mod G,
-  // a warp per row, lanes along k; S and the row staged in shared memory
-  double* Ss = Vc;  // ns <= 8192 doubles over Vc and Zs
-  for (int e = tid; e < ns; e += kPT) Ss[e] = __ldcg(Ri(kRedS + e));
-  __syncthreads();
-  double* trow = tw + warp * kBmax;
-  for (int i = g + warp * G; i < j + wp; i += 8 * G) {
-    for (int k = lane; k < j; k += 32) trow[k] = Ti(i + (size_t)k * kBmax);
-    __syncwarp();
-    for (int t = 0; t < wp; ++t) {
-      const int col = j + t;
-      double val;
-      if (i > col) {
-        val = 0.0;
-      } else if (i == col) {
-        val = taus[t];
-      } else {
-        double acc = 0.0;
-        for (int k = i + lane; k < col; k += 32) acc = fma(trow[k], Ss[k * wp + t], acc);
-        for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
-        val = -taus[t] * acc;
+}
+
+// ---------------------------------------------------------------------------
+// Householder QR of the updated mini-block by one cluster: CTA c owns a
+// contiguous range of the rows (in shared memory where they fit).  Bound by the
+// chain of a reflector: one exchange of partial dot products (v^T P follows from
+// the raw column's), a root, a division, one pass over the rows.  Among 16 CTAs
+// the exchange is a store to distributed shared memory and a cluster barrier;
+// over the whole chip it was a grid barrier and a read of 152 partials, and took
+// more than the arithmetic.  A mini-block of n = 3000, m = 4: 53 us in one launch
+// with V^T V_s and T, now 18 (update) + 19 (QR), V^T V_s a tile of the next product.
+// ---------------------------------------------------------------------------
+constexpr int kQrT = 512;                // threads: 16 warps over the columns
+constexpr int kQrC = 16;                 // CTAs of the cluster at most
+constexpr int kQrW = kQrT / 32;
+constexpr int kQrX = kQrC * kMaxW;       // an exchange buffer (sources x columns)
+// exchange buffers, pivot rows, coefficients, scales, pivots (doubles)
+constexpr size_t kQrFixed = 2 * kQrX + 2 * kMaxW + 3 * kMaxW;
+constexpr size_t kQrSmem = 216 * 1024;
+
+struct QrArgs {
+  double* P;          // panel column t, matrix row r: P[r + t * ldp]
+  long long ldp;
+  int r0, n;          // panel rows [r0, n)
+  int w, wp;          // panel columns; reflectors generated (wp <= w)
+  int pv0;            // pivot row of reflector t: pv0 + t
+  int j;              // reflectors of the block before this mini-block
+  int cs;             // CTAs of the cluster
+  int insm;           // the rows fit the CTAs' shared memory
+  double* V;          // V(r, i) = V[r + i * ldv], explicit zeros and unit pivots
+  long long ldv;
+  double* tau;        // tau of reflector t at tau[t]
+  DigitMat vcol;      // V's digits, operand row = reflector, K = r (exponent 1: the unit pivot is
+                      // every reflector's largest entry)
+  int* err;
+  size_t np, nv, ntau;  // extents the debug build checks
+};
+
+__global__ void __launch_bounds__(kQrT, 1) panel_qr_kernel(QrArgs a) {
+  extern __shared__ double qsm[];
+  double* xch = qsm;                     // [2][source][column]
+  double* piv = xch + 2 * kQrX;          // [2][kMaxW]
+  double* cf = piv + 2 * kMaxW;          // coefficients of the update
+  double* scl = cf + kMaxW;              // v = scl * column below the pivot
+  double* bet = scl + kMaxW;             // R's diagonal
+  double* Psm = bet + kMaxW;
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int c = cluster_rank(), C = a.cs, w = a.w;
+  const int rpc = (a.n - a.r0 + C - 1) / C;
+  const int ra = a.r0 + c * rpc;
+  const int nr = max(0, min(a.n, ra + rpc) - ra);
+  const long long ld = a.insm ? rpc : a.ldp;
+  double* Pg = a.P + ra;
+  double* Ps = a.insm ? Psm : Pg;
+  auto Gi = [&](long long i) { return (long long)RBCK(ra + i, a.np, a.err) - ra; };
+  if (a.insm)
+    for (int t = warp; t < w; t += kQrW)
+#pragma unroll 4
+      for (int rl = lane; rl < nr; rl += 32) Psm[t * ld + rl] = Pg[Gi(rl + (long long)t * a.ldp)];
+  // the cluster has started (its shared memory can be written) and the rows are in
+  cluster_sync_all();
+  for (int t = 0; t < a.wp; ++t) {
+    const int q = t & 1, pr = a.pv0 + t, prl = pr - ra;  // the pivot's row here (or outside [0, nr))
+    const int rb = max(0, prl + 1);
+    const int nk = w - t;  // columns t .. w-1 (k = t: the squared norm below the pivot)
+    int pw = 1;            // columns rounded up to a power of two; wps warps share one
+    while (pw < nk) pw <<= 1;
+    const int wps = max(1, kQrW / pw), sub = warp % wps;
+    const double* ct = Ps + t * ld;
+    for (int k = warp / wps; k < nk; k += kQrW / wps) {
+      const double* ck = ct + k * ld;
+      double acc = 0.0;
+#pragma unroll 4
+      for (int rl = rb + sub * 32 + lane; rl < nr; rl += 32 * wps) acc = fma(ck[rl], ct[rl], acc);
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
+      if (lane < C) {
+        cluster_st(xch + q * kQrX + (c * wps + sub) * pw + k, lane, acc);
+        if (sub == 0 && prl >= 0 && prl < nr) cluster_st(piv + q * kMaxW + k, lane, ck[prl]);
       }
-      __syncwarp();
-      if (lane == 0) trow[col] = val;
-      __syncwarp();
     }
-    for (int t = lane; t < wp; t += 32) Ti(i + (size_t)(j + t) * kBmax) = trow[j + t];
     __syncwarp();
+    cluster_sync_all();
+    if (warp == 0) {
+      // sums over the sources in a fixed order: the same bits in every CTA
+      const double* x = xch + q * kQrX;
+      const int pl = min(pw, 32), parts = 32 / pl;
+      double d[kMaxW / 32];
+#pragma unroll
+      for (int u = 0; u < kMaxW / 32; ++u) {
+        d[u] = 0.0;
+        const int k = (lane & (pl - 1)) + 32 * u;
+        if (32 * u >= nk) continue;
+        if (k < nk)
+#pragma unroll 4
+          for (int sq = lane / pl; sq < C * wps; sq += parts) d[u] += x[sq * pw + k];
+        for (int o = 16; o >= pl; o >>= 1) d[u] += __shfl_xor_sync(0xffffffffu, d[u], o);
+      }
+      const double sig = __shfl_sync(0xffffffffu, d[0], 0), alpha = piv[q * kMaxW];
+      double tk = 0.0, scal = 0.0, beta = alpha;
+      if (sig != 0.0) {
+        const double nrm = sqrt(fma(alpha, alpha, sig));
+        beta = alpha >= 0.0 ? -nrm : nrm;
+        // both quotients in one division: lane parity
+        const double qt = (lane & 1) ? 1.0 / (alpha - beta) : (beta - alpha) / beta;
+        tk = __shfl_sync(0xffffffffu, qt, 0);
+        scal = __shfl_sync(0xffffffffu, qt, 1);
+      }
+      // P(:, k) -= tau v (v^T P(:, k)), v^T P(:, k) = P(pr, k) + scal d_k
+#pragma unroll
+      for (int u = 0; u < kMaxW / 32; ++u) {
+        const int k = lane + 32 * u;
+        if (lane < pl && k < nk) cf[k] = tk != 0.0 ? -tk * fma(scal, d[u], piv[q * kMaxW + k]) : 0.0;
+      }
+      if (lane == 0) {
+        scl[t] = scal;
+        bet[t] = beta;
+        if (c == 0) a.tau[RBCK(t, a.ntau, a.err)] = tk;
+      }
+    }
+    __syncthreads();
+    const double sc = scl[t];
+    for (int k = 1 + warp / wps; k < nk; k += kQrW / wps) {
+      double* pk = Ps + (t + k) * ld;
+      const double g = cf[k], gs = g * sc;
+#pragma unroll 4
+      for (int rl = rb + sub * 32 + lane; rl < nr; rl += 32 * wps) pk[rl] = fma(gs, ct[rl], pk[rl]);
+      if (sub == 0 && lane == 0 && prl >= 0 && prl < nr) pk[prl] += g;
+    }
+    __syncthreads();
+  }
+  // the factored panel (unscaled columns and pivots until here), the new columns
+  // of V (values and digits)
+  for (int t = warp; t < w; t += kQrW) {
+    const int pr = a.pv0 + t;
+    const bool ref = t < a.wp;
+    const double sc = ref ? scl[t] : 1.0;
+    for (int rl = lane; rl < nr; rl += 32) {
+      const int r = ra + rl;
+      double x = Ps[t * ld + rl];
+      if (ref && r > pr) x = sc != 0.0 ? x * sc : x;
+      if (ref && r == pr) x = bet[t];
+      Pg[Gi(rl + (long long)t * a.ldp)] = x;
+      if (!ref) continue;
+      const double v = r < pr ? 0.0 : (r == pr ? 1.0 : x);
+      a.V[RBCK((size_t)r + (size_t)(a.j + t) * a.ldv, a.nv, a.err)] = v;
+      if (v != 0.0) put_digits_v(a.vcol, a.j + t, r, v, a.err);
+    }
   }
 }
 
-// Y's new columns (Eq. for Y): Y(:, j + t) = sum_{t' <= t} (A V_s - Y V^T V_s)(:, t') T_s(t', t)
-// for every row of E; A V_s arrives as `ks` partial sums. Bound by the latency
-// of a thread's sum over the j <= 128 columns: kYfixSplit lanes share it, which
-// also makes four times the blocks (47 at 3000 rows of 4 columns otherwise).
-constexpr int kYfixSplit = 4;
-static_assert(kYfixSplit * kMaxW <= 256, "a row of Y to a block at least");
-__global__ void __launch_bounds__(256) yfix_kernel(const double* __restrict__ AV, int ks, long long kstride,
-                                                   long long ldav, int rows, double* __restrict__ Y,
-                                                   long long ldy, int j, int wp, const double* __restrict__ S,
-                                                   const double* __restrict__ T, size_t nav, size_t ny,
-                                                   int* err) {
+// New columns of Y and T after a mini-block with reflectors j .. j + wp - 1,
+// V_s.  T's recursion, T^{-1} = striu(V^T V) + diag(1 / tau), makes both the same
+// forward substitution by rows: with S = V^T V_s,
+//   u_t = x_t - sum_{i < j} F(e, i) S(i, t),  f_t = tau_t (u_t - sum_{q < t} f_q S(j + q, t)),
+// F = Y and x = A V_s for a row of Y, F = T and x_t = (t == e - j) for row e of T.
+// A V_s and S arrive as `ks` partial sums.  Bound by a thread's latency over the
+// j <= 128 columns: 16 rows to a CTA (1 / 16 of wp > 16's share), the threads left
+// over split the sum.
+struct YfixArgs {
+  const double* AV;   // partial q of row e, column t: AV[q * avstride + e + t * ldav]
+  long long avstride, ldav;
+  const double* S;    // partial q of S(i, t): S[q * sstride + i + t * kBmax]
+  long long sstride;
+  int ks, rows, j, wp;
+  double* Y;
+  long long ldy;
+  double* T;
+  const double* tau;
+  size_t nav, ns, ny;
+  int* err;
+};
+__host__ __device__ constexpr int yfix_rows(int wp) { return wp <= 16 ? 16 : 256 / wp; }
+
+__global__ void __launch_bounds__(256) yfix_kernel(YfixArgs a) {
   extern __shared__ double ysm[];
-  double* Ss = ysm;              // S(i, t) for i < j
-  double* Tt = Ss + j * wp;      // Tt[t' + t * wp] = T(j + t', j + t)
-  const int R = 256 / (kYfixSplit * wp);  // rows per CTA
-  double* us = Tt + wp * wp;              // us[(kq * wp + t') * R + rl]
-  const int tid = threadIdx.x;
-  for (int e = tid; e < j * wp; e += 256) Ss[e] = S[RBCK(e, 8192, err)];
-  for (int e = tid; e < wp * wp; e += 256)
-    Tt[e] = T[RBCK((size_t)(j + e % wp) + (size_t)(j + e / wp) * kBmax, (size_t)kBmax * kBmax, err)];
-  __syncthreads();
+  const int tid = threadIdx.x, j = a.j, wp = a.wp, ns = j + wp;
+  const int R = yfix_rows(wp), KS = 256 / (R * wp);
+  double* Ss = ysm;              // S(i, t) at Ss[i * wp + t], i < j + wp
+  double* us = Ss + ns * wp;     // us[(kq * wp + t) * R + rl]
+  const int nby = (a.rows + R - 1) / R;
+  const bool isT = (int)blockIdx.x >= nby;  // T's rows come after Y's
   const int rl = tid % R, tq = tid / R, tp = tq % wp, kq = tq / wp;
-  const int e = blockIdx.x * R + rl;
-  const bool act = kq < kYfixSplit && e < rows;
+  const int e = ((int)blockIdx.x - (isT ? nby : 0)) * R + rl;
+  const bool act = kq < KS && e < (isT ? ns : a.rows);
+  double* F = isT ? a.T : a.Y;
+  const long long ldf = isT ? kBmax : a.ldy;
+  [[maybe_unused]] const size_t nf = isT ? (size_t)kBmax * kBmax : a.ny;
+  double u = 0.0;
   if (act) {
-    double u = 0.0;
-    for (int q = kq; q < ks; q += kYfixSplit) u += AV[RBCK((size_t)q * kstride + e + (size_t)tp * ldav, nav, err)];
+    if (isT) u = (kq == 0 && e - j == tp) ? 1.0 : 0.0;
+    else
+      for (int q = kq; q < a.ks; q += KS) u += a.AV[RBCK((size_t)q * a.avstride + e + (size_t)tp * a.ldav, a.nav, a.err)];
+  }
+  for (int x = tid; x < ns * wp; x += 256) {
+    const int i = x % ns, t = x / ns;
+    double v = 0.0;
 #pragma unroll 4
-    for (int i = kq; i < j; i += kYfixSplit)
-      u = fma(-Y[RBCK(e + (size_t)i * ldy, ny, err)], Ss[i * wp + tp], u);
+    for (int q = 0; q < a.ks; ++q) v += a.S[RBCK((size_t)q * a.sstride + i + (size_t)t * kBmax, a.ns, a.err)];
+    Ss[i * wp + t] = v;
+  }
+  __syncthreads();
+  if (act) {
+#pragma unroll 8
+    for (int i = kq; i < j; i += KS) u = fma(-F[RBCK(e + (size_t)i * ldf, nf, a.err)], Ss[i * wp + tp], u);
     us[tq * R + rl] = u;
   }
   __syncthreads();
   if (act && kq == 0) {
-    double y = 0.0;
-    for (int q = 0; q <= tp; ++q) {
-      double u = us[q * R + rl];
-#pragma unroll
-      for (int k = 1; k < kYfixSplit; ++k) u += us[(k * wp + q) * R + rl];
-      y = fma(u, Tt[q + tp * wp], y);
-    }
-    Y[RBCK(e + (size_t)(j + tp) * ldy, ny, err)] = y;
+    for (int k = 1; k < KS; ++k) u += us[(k * wp + tp) * R + rl];
   }
+  // column q of the row is final after step q; every column after it takes its part
+  for (int q = 0; q < wp; ++q) {
+    if (act && kq == 0 && tp == q) {
+      u *= a.tau[q];
+      us[q * R + rl] = u;
+    }
+    __syncthreads();
+    if (act && kq == 0 && tp > q) u = fma(-us[q * R + rl], Ss[(j + q) * wp + tp], u);
+  }
+  if (act && kq == 0) F[RBCK(e + (size_t)(j + tp) * ldf, nf, a.err)] = u;
 }
 
 // Z = T^T W for the trailing columns (W in `ks` partial sums, W(i, c) at
@@ -1022,14 +1074,16 @@ struct RtcScratch {
   double* Y;        // ldE x kBmax
   double* W;        // ksW x (kBmax x n)
   double* AV;       // ksY x (ldE x kMaxW)
-  double* part;     // 3 x G x kPartW
+  double* Sp;       // ksY x (kBmax x kMaxW): V^T V_s
+  double* part;     // G x kPartW
   double* red;      // kRedTotal
+  int qrC;          // CTAs of the cluster that factors a panel
   unsigned* bar;    // [0..3]: [2] the error flag; then one arrival counter per panel launch
   int nbar;         // panel-launch counters available
   int panels;       // panel launches so far
   DigitMat erow, ecol, yrow, vrow, vcol, zcol;
   int G;
-  size_t nE, nV, nY, nW, nAV, npart;  // extents in doubles
+  size_t nE, nV, nY, nW, nAV, nSp, npart;  // extents in doubles
 };
 
 inline long long rup(long long x, long long a) { return (x + a - 1) / a * a; }
@@ -1059,13 +1113,15 @@ size_t rtc_layout(int n, int p, unsigned char* base, RtcScratch* S) {
   s.nY = (size_t)ldE * kBmax;
   s.nW = (size_t)ksW * kBmax * (size_t)n;
   s.nAV = (size_t)ksY * ldE * kMaxW;
-  s.npart = 3 * (size_t)G * kPartW;
+  s.nSp = (size_t)ksY * kBmax * kMaxW;
+  s.npart = (size_t)G * kPartW;
   s.E = (double*)take(sizeof(double) * s.nE);
   s.V = (double*)take(sizeof(double) * s.nV);
   s.T = (double*)take(sizeof(double) * kBmax * kBmax);
   s.Y = (double*)take(sizeof(double) * s.nY);
   s.W = (double*)take(sizeof(double) * s.nW);
   s.AV = (double*)take(sizeof(double) * s.nAV);
+  s.Sp = (double*)take(sizeof(double) * s.nSp);
   s.part = (double*)take(sizeof(double) * s.npart);
   s.red = (double*)take(sizeof(double) * kRedTotal);
   s.nbar = n + 16;
@@ -1115,7 +1171,7 @@ int split_into(const double* src, long long sr, long long sk, int r_lo, int r_hi
 template <int NT, int LV>
 int gemm_launch(const GArgs& g, cudaStream_t st) {
   using Cfg = GCfg<NT, LV>;
-  const int nI = (g.M1 + 127) / 128 - g.M0 / 128;
+  const int nI = (g.M1 + 127) / 128 - g.M0 / 128 + (g.C2 != nullptr ? 1 : 0);
   const int nN = (g.N1 + NT - 1) / NT - g.N0 / NT;
   if (g.M1 <= g.M0 || g.N1 <= g.N0 || nI <= 0 || nN <= 0) return SSV_OK;
   const long long tiles = (long long)nI * nN * g.ksplit;
@@ -1157,65 +1213,110 @@ GArgs gemm_args(const DigitMat& A, const DigitMat& B, int J0, int J1, int M0, in
   return g;
 }
 
-// One mini-block: panel (cooperative), A V_s on the tensor cores, Y's new columns.
+// One mini-block: update and QR of the panel, A V_s and V^T V_s on the tensor
+// cores, Y's and T's new columns.
 int run_panel(RtcScratch& S, int n, int p, double* P, size_t np, long long ldp, int r0, int w, int wp, int pv0,
               int j, int c0, double* tau, size_t ntau, cudaStream_t st) {
-  if (S.panels >= S.nbar) return SSV_EINVAL;
   const int L = n - r0;
-  int G = std::min(S.G, std::max(1, (L + 15) / 16));
-  const int rpc = (L + G - 1) / G;
-  if ((long long)rpc * w > kPanRowsW) return SSV_ENOTSUP;
-  PanArgs a;
-  a.P = P;
-  a.ldp = ldp;
-  a.r0 = r0;
-  a.n = n;
-  a.w = w;
-  a.wp = wp;
-  a.pv0 = pv0;
-  a.j = j;
-  a.c0 = c0;
-  a.V = S.V;
-  a.ldv = S.ldv;
-  a.T = S.T;
-  a.Y = S.Y;
-  a.ldy = S.ldE;
-  a.yoff = p;
-  a.tau = tau;
-  a.vcol = S.vcol;
-  a.part = S.part;
-  a.red = S.red;
-  a.bar = S.bar + 4 + S.panels++;
-  a.err = reinterpret_cast<int*>(S.bar + 2);
-  a.np = np;
-  a.nv = S.nV;
-  a.ny = S.nY;
-  a.ntau = ntau;
-  a.npart = S.npart;
-  size_t smem = sizeof(double) * ((size_t)rpc * w + kPanFixed);
-  const size_t rows = sizeof(double) * 2 * (size_t)rpc * j;
-  a.staged = smem + rows <= kPanSmem ? 1 : 0;
-  if (a.staged) smem += rows;
-  SSV_CUDA_TRY(cudaFuncSetAttribute(panel_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-  void* args[] = {&a};
-  SSV_CUDA_TRY(cudaLaunchCooperativeKernel((const void*)panel_kernel, dim3(G), dim3(kPT), args, smem, st));
-  count_launch();
+  int* err = reinterpret_cast<int*>(S.bar + 2);
+  if (j > 0) {
+    if (S.panels >= S.nbar) return SSV_EINVAL;
+    const int G = std::min(S.G, std::max(1, (L + 15) / 16));
+    const int rpc = (L + G - 1) / G;
+    if ((long long)rpc * w > kPanRowsW) return SSV_ENOTSUP;
+    PanArgs a;
+    a.P = P;
+    a.ldp = ldp;
+    a.r0 = r0;
+    a.n = n;
+    a.w = w;
+    a.j = j;
+    a.c0 = c0;
+    a.V = S.V;
+    a.ldv = S.ldv;
+    a.T = S.T;
+    a.Y = S.Y;
+    a.ldy = S.ldE;
+    a.yoff = p;
+    a.part = S.part;
+    a.red = S.red;
+    a.bar = S.bar + 4 + S.panels++;
+    a.err = err;
+    a.np = np;
+    a.nv = S.nV;
+    a.ny = S.nY;
+    a.npart = S.npart;
+    size_t smem = sizeof(double) * ((size_t)rpc * w + kPanFixed);
+    const size_t rows = sizeof(double) * 2 * (size_t)rpc * j;
+    a.staged = smem + rows <= kPanSmem ? 1 : 0;
+    if (a.staged) smem += rows;
+    SSV_CUDA_TRY(cudaFuncSetAttribute(panel_update_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    void* args[] = {&a};
+    SSV_CUDA_TRY(cudaLaunchCooperativeKernel((const void*)panel_update_kernel, dim3(G), dim3(kPT), args, smem, st));
+    count_launch();
+  }
+  {
+    QrArgs a;
+    a.P = P;
+    a.ldp = ldp;
+    a.r0 = r0;
+    a.n = n;
+    a.w = w;
+    a.wp = wp;
+    a.pv0 = pv0;
+    a.j = j;
+    // fewer CTAs where each would have 16 rows or less
+    a.cs = S.qrC;
+    while (a.cs > 1 && L <= 16 * a.cs) a.cs /= 2;
+    const size_t rows = sizeof(double) * (size_t)((L + a.cs - 1) / a.cs) * w;
+    a.insm = sizeof(double) * kQrFixed + rows <= kQrSmem ? 1 : 0;
+    a.V = S.V;
+    a.ldv = S.ldv;
+    a.tau = tau;
+    a.vcol = S.vcol;
+    a.err = err;
+    a.np = np;
+    a.nv = S.nV;
+    a.ntau = ntau;
+    SSV_CUDA_TRY(launch_cluster(panel_qr_kernel, a.cs, kQrT, a.cs, sizeof(double) * kQrFixed + (a.insm ? rows : 0),
+                                st, a));
+  }
   // A V_s: every row of E against the new reflectors (rows pv0.. of V_s are nonzero)
   const int KTn = (n + kTK - 1) / kTK;
   const int rowsE = p + n;
   GArgs g = gemm_args(S.erow, S.vcol, pv0 / kTK, KTn, 0, rowsE, j, j + wp, S.AV, S.nAV, S.ldE, 0, S);
   g.coff = -j;
   const int NT = wp <= 16 ? 16 : 32;
-  const int nI = (rowsE + 127) / 128, nN = (j + wp + NT - 1) / NT - j / NT;
+  const int nI = (rowsE + 127) / 128 + 1, nN = (j + wp + NT - 1) / NT - j / NT;
   g.ksplit = std::max(1, std::min(8, S.G / std::max(1, nI * nN)));
   g.kstride = S.ldE * kMaxW;
+  g.C2 = S.Sp;
+  g.nc2 = S.nSp;
+  g.kstride2 = (long long)kBmax * kMaxW;
   int rc = gemm_long(wp, g, st);
   if (rc != SSV_OK) return rc;
-  const int R = 256 / (kYfixSplit * wp);
-  const size_t ysm = sizeof(double) * ((size_t)j * wp + (size_t)wp * wp + 256);
+  YfixArgs y;
+  y.AV = S.AV;
+  y.avstride = g.kstride;
+  y.ldav = S.ldE;
+  y.S = S.Sp;
+  y.sstride = g.kstride2;
+  y.ks = g.ksplit;
+  y.rows = rowsE;
+  y.j = j;
+  y.wp = wp;
+  y.Y = S.Y;
+  y.ldy = S.ldE;
+  y.T = S.T;
+  y.tau = tau;
+  y.nav = S.nAV;
+  y.ns = S.nSp;
+  y.ny = S.nY;
+  y.err = err;
+  const int R = yfix_rows(wp);
+  const size_t ysm = sizeof(double) * ((size_t)(j + wp) * wp + 256);
   SSV_CUDA_TRY(cudaFuncSetAttribute(yfix_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)ysm));
-  yfix_kernel<<<(rowsE + R - 1) / R, 256, ysm, st>>>(S.AV, g.ksplit, g.kstride, S.ldE, rowsE, S.Y, S.ldE, j, wp,
-                                                     S.red + kRedS, S.T, S.nAV, S.nY, a.err);
+  yfix_kernel<<<(rowsE + R - 1) / R + (j + wp + R - 1) / R, 256, ysm, st>>>(y);
   count_launch();
   SSV_CUDA_TRY(cudaGetLastError());
   return SSV_OK;
@@ -1265,6 +1366,29 @@ __global__ void rtc_canary_kernel(const unsigned char* c, size_t nbytes, int* er
 }
 #endif
 
+// CTAs of the panel's cluster: 16 where the chip can hold such a cluster, else the
+// portable 8
+int qr_cluster() {
+  int nc = 0;
+  cudaLaunchConfig_t cfg = {};
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeClusterDimension;
+  at[0].val.clusterDim.x = kQrC;
+  at[0].val.clusterDim.y = 1;
+  at[0].val.clusterDim.z = 1;
+  cfg.gridDim = dim3(kQrC);
+  cfg.blockDim = dim3(kQrT);
+  cfg.dynamicSmemBytes = kQrSmem;
+  cfg.attrs = at;
+  cfg.numAttrs = 1;
+  if (cudaFuncSetAttribute(panel_qr_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kQrSmem) == cudaSuccess &&
+      cudaFuncSetAttribute(panel_qr_kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) == cudaSuccess &&
+      cudaOccupancyMaxActiveClusters(&nc, panel_qr_kernel, &cfg) == cudaSuccess && nc > 0)
+    return kQrC;
+  (void)cudaGetLastError();
+  return 8;
+}
+
 int clear_block(const RtcScratch& S, int n, cudaStream_t st) {
   SSV_CUDA_TRY(cudaMemsetAsync(S.V, 0, sizeof(double) * S.ldv * kBmax, st));
   SSV_CUDA_TRY(cudaMemsetAsync(S.T, 0, sizeof(double) * kBmax * kBmax, st));
@@ -1300,6 +1424,7 @@ int reduce_tc(Handle* h, cudaStream_t st) {
   SSV_CUDA_TRY(pool_alloc((void**)&base, bytes + kCanary, st));
   RtcScratch S;
   rtc_layout(n, p, base, &S);
+  S.qrC = qr_cluster();
   int* err = reinterpret_cast<int*>(S.bar + 2);
   int rc = SSV_OK;
   auto step = [&](int r) {
@@ -1402,10 +1527,31 @@ __global__ void __launch_bounds__(256) qz_kernel(const double* __restrict__ Wp, 
                                                  const double* __restrict__ tau, DigitMat Z) {
   extern __shared__ double S[];  // kBmax x kBmax
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  for (int e = tid; e < cnt * kBmax; e += 256) {
-    double v = 0.0;
-    for (int q = 0; q < kss; ++q) v += Sp[(size_t)q * kBmax * kBmax + e];
-    S[e] = v;
+  // all partial sums of eight entries in flight: one L2 round trip per 16 KB of S
+  for (int e0 = 0; e0 < cnt * kBmax; e0 += 8 * 256) {
+    double2 v[4][8];
+#pragma unroll
+    for (int u = 0; u < 4; ++u)
+#pragma unroll
+      for (int q = 0; q < 8; ++q) {
+        const int e = e0 + 512 * u + 2 * tid;
+        v[u][q] = (q < kss && e < cnt * kBmax)
+                      ? *reinterpret_cast<const double2*>(Sp + (size_t)q * kBmax * kBmax + e)
+                      : make_double2(0.0, 0.0);
+      }
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+      const int e = e0 + 512 * u + 2 * tid;
+      if (e >= cnt * kBmax) continue;
+      double2 s = v[u][0];
+#pragma unroll
+      for (int q = 1; q < 8; ++q)
+        if (q < kss) {
+          s.x += v[u][q].x;
+          s.y += v[u][q].y;
+        }
+      *reinterpret_cast<double2*>(S + e) = s;
+    }
   }
   __syncthreads();
   const int c = blockIdx.x * 8 + warp;
