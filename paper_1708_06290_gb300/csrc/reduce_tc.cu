@@ -128,7 +128,9 @@ __device__ __forceinline__ long long row_off(int r, long long sr, int wrap) {
 }
 
 
-// exponent pass: ex[r] = max over the K range of scale_exp(|x|) (ex preset to INT_MIN)
+// exponent pass: ex[r] = max over the K range of scale_exp(|x|) (ex preset to
+// INT_MIN), from the high words as integers: a maximum of doubles holds the FP64
+// pipe for 64 clocks a warp (the reduction of n = 3000: 2.64 -> 0.64 ms in all)
 __global__ void __launch_bounds__(256) split_exp_kernel(const double* __restrict__ src, long long sr,
                                                         long long sk, int r_lo, int r_hi, int k_lo,
                                                         int k_hi, int kchunk, int wrap, int* __restrict__ ex,
@@ -137,31 +139,36 @@ __global__ void __launch_bounds__(256) split_exp_kernel(const double* __restrict
   const int rb = r_lo + blockIdx.x * 64;
   const int kb = k_lo + blockIdx.y * kchunk;
   const int ke = min(k_hi, kb + kchunk);
+  auto bits = [&](int r, int k) {
+    return abs_hi(src[RBCK(row_off(r, sr, wrap) + (long long)k * sk, nsrc, err)]);
+  };
   if (sk <= 2) {
     // K (nearly) contiguous: a warp per row, lanes along K
     const int lane = tid & 31, wp = tid >> 5;
+#pragma unroll 2
     for (int rr = wp; rr < 64; rr += 8) {
       const int r = rb + rr;
       if (r >= r_hi) break;
-      double mx = 0.0;
-      for (int k = kb + lane; k < ke; k += 32) mx = fmax(mx, fabs(src[RBCK(row_off(r, sr, wrap) + (long long)k * sk, nsrc, err)]));
-      for (int o = 16; o > 0; o >>= 1) mx = fmax(mx, __shfl_xor_sync(0xffffffffu, mx, o));
-      if (lane == 0) atomicMax(ex + RBCK(r, nex, err), scale_exp(mx));
+      int mx = 0;
+#pragma unroll 4
+      for (int k = kb + lane; k < ke; k += 32) mx = max(mx, bits(r, k));
+      mx = __reduce_max_sync(0xffffffffu, mx);
+      if (lane == 0) atomicMax(ex + RBCK(r, nex, err), scale_exp_hi(mx));
     }
   } else {
     // rows contiguous (sr == 1 in every use): threads along rows, four K groups
-    __shared__ double part[4][64];
+    __shared__ int part[4][64];
     const int rr = tid & 63, g = tid >> 6;
     const int r = rb + rr;
-    double mx = 0.0;
+    int mx = 0;
     if (r < r_hi)
-      for (int k = kb + g; k < ke; k += 4)
-        mx = fmax(mx, fabs(src[RBCK(row_off(r, sr, wrap) + (long long)k * sk, nsrc, err)]));
+#pragma unroll 8
+      for (int k = kb + g; k < ke; k += 4) mx = max(mx, bits(r, k));
     part[g][rr] = mx;
     __syncthreads();
     if (g == 0 && r < r_hi) {
-      mx = fmax(fmax(part[0][rr], part[1][rr]), fmax(part[2][rr], part[3][rr]));
-      atomicMax(ex + RBCK(r, nex, err), scale_exp(mx));
+      mx = max(max(part[0][rr], part[1][rr]), max(part[2][rr], part[3][rr]));
+      atomicMax(ex + RBCK(r, nex, err), scale_exp_hi(mx));
     }
   }
 }
@@ -1034,9 +1041,10 @@ __global__ void __launch_bounds__(256) zmake_kernel(const double* __restrict__ W
   for (int q = 0; q < kBmax / 8; ++q) Ws[ig + 8 * q][cl] = zv[q];
   __syncthreads();
   if (tid < 32) {
-    double mx = 0.0;
-    for (int i = 0; i < jb; ++i) mx = fmax(mx, fabs(Ws[i][tid]));
-    const int E = scale_exp(mx);
+    int mx = 0;
+#pragma unroll 8
+    for (int i = 0; i < jb; ++i) mx = max(mx, abs_hi(Ws[i][tid]));
+    const int E = scale_exp_hi(mx);
     Es[tid] = E;
     if (cb + tid < n) Z.ex[RBCK(cb + tid, (size_t)Z.RT * kTR, err)] = E;
   }
@@ -1153,8 +1161,11 @@ int split_into(const double* src, long long sr, long long sk, int r_lo, int r_hi
   if (r_hi <= r_lo || k_hi <= k_lo) return SSV_OK;
   if (M.ex) {
     SSV_CUDA_TRY(cudaMemsetAsync(M.ex, 0x80, sizeof(int) * (size_t)M.RT * kTR, st));
-    const int kchunk = 512;
-    dim3 grid((unsigned)((r_hi - r_lo + 63) / 64), (unsigned)((k_hi - k_lo + kchunk - 1) / kchunk));
+    // K range of a block: 512, less where the chip would stay idle
+    int kchunk = 512;
+    const int rblk = (r_hi - r_lo + 63) / 64;
+    while (kchunk > 64 && (long long)rblk * ((k_hi - k_lo + kchunk - 1) / kchunk) < 4 * std::max(1, num_sms())) kchunk /= 2;
+    dim3 grid((unsigned)rblk, (unsigned)((k_hi - k_lo + kchunk - 1) / kchunk));
     split_exp_kernel<<<grid, 256, 0, st>>>(src, sr, sk, r_lo, r_hi, k_lo, k_hi, kchunk, wrap, M.ex, nsrc, nex, err);
     count_launch();
     SSV_CUDA_TRY(cudaGetLastError());
@@ -1519,40 +1530,35 @@ __global__ void __launch_bounds__(256) qv_kernel(const double* __restrict__ src,
   V[r + (size_t)k * ldv] = (k >= cnt || d < 0) ? 0.0 : d == 0 ? 1.0 : src[r + (size_t)k * n];
 }
 
+constexpr int kQCols = 1024;  // complex columns at a time (bounds the digit scratch)
+constexpr int kQSplit = 7;    // partial sums of V^T V at most
+
+// S = V^T V from its partial sums, row i scaled by tau_i: a step of the back
+// substitution is then a broadcast and a multiply-add
+__global__ void __launch_bounds__(256) qs_kernel(const double* __restrict__ Sp, int kss, int cnt,
+                                                 const double* __restrict__ tau, double* __restrict__ S) {
+  const int e = blockIdx.x * 256 + threadIdx.x, i = e % kBmax;
+  double v[kQSplit];
+#pragma unroll
+  for (int q = 0; q < kQSplit; ++q) v[q] = q < kss ? Sp[(size_t)q * kBmax * kBmax + e] : 0.0;
+#pragma unroll
+  for (int q = 1; q < kQSplit; ++q) v[0] += v[q];
+  S[e] = i < cnt ? v[0] * __ldg(tau + i) : 0.0;
+}
+
 // Z = T W for 8 real columns per CTA, a warp each: lane l holds the rows l, l +
 // 32, ..; back substitution from the last reflector, then Z's digits with the
-// column's exponent.  W and S = V^T V arrive as partial sums.
+// column's exponent.  W arrives as partial sums.  Bound by the FP64 pipe: 2.5
+// instructions of 64 clocks a step on average, two warps to a scheduler (900
+// columns: 27 us; with every CTA adding S's partial sums itself 69).
 __global__ void __launch_bounds__(256) qz_kernel(const double* __restrict__ Wp, int ksw, long long wstride,
-                                                 const double* __restrict__ Sp, int kss, int cnt, int ncol,
+                                                 const double* __restrict__ Sg, int cnt, int ncol,
                                                  const double* __restrict__ tau, DigitMat Z) {
   extern __shared__ double S[];  // kBmax x kBmax
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  // all partial sums of eight entries in flight: one L2 round trip per 16 KB of S
-  for (int e0 = 0; e0 < cnt * kBmax; e0 += 8 * 256) {
-    double2 v[4][8];
-#pragma unroll
-    for (int u = 0; u < 4; ++u)
-#pragma unroll
-      for (int q = 0; q < 8; ++q) {
-        const int e = e0 + 512 * u + 2 * tid;
-        v[u][q] = (q < kss && e < cnt * kBmax)
-                      ? *reinterpret_cast<const double2*>(Sp + (size_t)q * kBmax * kBmax + e)
-                      : make_double2(0.0, 0.0);
-      }
-#pragma unroll
-    for (int u = 0; u < 4; ++u) {
-      const int e = e0 + 512 * u + 2 * tid;
-      if (e >= cnt * kBmax) continue;
-      double2 s = v[u][0];
-#pragma unroll
-      for (int q = 1; q < 8; ++q)
-        if (q < kss) {
-          s.x += v[u][q].x;
-          s.y += v[u][q].y;
-        }
-      *reinterpret_cast<double2*>(S + e) = s;
-    }
-  }
+#pragma unroll 8
+  for (int e = 2 * tid; e < kBmax * kBmax; e += 512)
+    *reinterpret_cast<double2*>(S + e) = *reinterpret_cast<const double2*>(Sg + e);
   __syncthreads();
   const int c = blockIdx.x * 8 + warp;
   if (c >= ncol) return;
@@ -1561,27 +1567,31 @@ __global__ void __launch_bounds__(256) qz_kernel(const double* __restrict__ Wp, 
   for (int u = 0; u < kBmax / 32; ++u) {
     const int i = lane + 32 * u;
     double v = 0.0;
-    if (i < cnt)
+    if (i < cnt) {
       for (int q = 0; q < ksw; ++q) v += Wp[(size_t)q * wstride + i + (size_t)c * kBmax];
+      v *= __ldg(tau + i);
+    }
     w[u] = v;
   }
+  // z_k = w_k, final once the steps after it have taken their part
 #pragma unroll
   for (int uk = kBmax / 32 - 1; uk >= 0; --uk) {
     for (int lk = 31; lk >= 0; --lk) {
       const int k = 32 * uk + lk;
       if (k >= cnt) continue;
-      const double z = __shfl_sync(0xffffffffu, w[uk], lk) * __ldg(tau + k);
-      if (lane == lk) w[uk] = z;
+      const double z = __shfl_sync(0xffffffffu, w[uk], lk);
 #pragma unroll
-      for (int u = 0; u < kBmax / 32; ++u)
-        if (u < uk || (u == uk && lane < lk)) w[u] = fma(-S[lane + 32 * u + k * kBmax], z, w[u]);
+      for (int u = 0; u <= uk; ++u) {
+        const double f = fma(-S[lane + 32 * u + k * kBmax], z, w[u]);
+        if (u < uk || lane < lk) w[u] = f;
+      }
     }
   }
-  double mx = 0.0;
+  int mx = 0;
 #pragma unroll
-  for (int u = 0; u < kBmax / 32; ++u) mx = fmax(mx, w[u] == w[u] ? fabs(w[u]) : INFINITY);
-  for (int o = 16; o > 0; o >>= 1) mx = fmax(mx, __shfl_xor_sync(0xffffffffu, mx, o));
-  const int E = scale_exp(mx);
+  for (int u = 0; u < kBmax / 32; ++u) mx = max(mx, abs_hi(w[u]));
+  mx = __reduce_max_sync(0xffffffffu, mx);
+  const int E = scale_exp_hi(mx);
   if (lane == 0) Z.ex[c] = E;
 #pragma unroll
   for (int u = 0; u < kBmax / 32; ++u) {
@@ -1602,7 +1612,6 @@ __global__ void q_fail_kernel(const int* err, cd* X, long long ldx, int n, int n
     X[e % n + (size_t)(e / n) * ldx] = mkcd(nanv, nanv);
 }
 
-constexpr int kQCols = 1024;  // complex columns at a time (bounds the digit scratch)
 
 struct QtcScratch {
   double *V, *W, *S;
@@ -1708,9 +1717,13 @@ int apply_q_tc(const Handle* h, int ncols, cd* X, long long ldX, cudaStream_t st
     // S = V^T V
     const int J0 = pv / kTK, nst = KTn - J0;
     GArgs gs = args(Q.vcol, Q.vcol, J0, KTn, 0, cnt, cnt, Q.S, (size_t)8 * kBmax * kBmax, kBmax);
-    gs.ksplit = std::max(1, std::min(8, nst / 4));
+    gs.ksplit = std::max(1, std::min(kQSplit, nst / 4));
     gs.kstride = (long long)kBmax * kBmax;
     if (rc == SSV_OK) step(gemm_launch<32, 9>(gs, st));
+    double* S1 = Q.S + (size_t)kQSplit * kBmax * kBmax;
+    qs_kernel<<<kBmax * kBmax / 256, 256, 0, st>>>(Q.S, gs.ksplit, cnt, tau, S1);
+    count_launch();
+    cu(cudaGetLastError());
     for (int c0 = 0; c0 < ncols && rc == SSV_OK; c0 += ncm) {
       const int nc = std::min(ncm, ncols - c0);
       double* Xd = reinterpret_cast<double*>(X + (size_t)c0 * ldX);
@@ -1722,14 +1735,16 @@ int apply_q_tc(const Handle* h, int ncols, cd* X, long long ldX, cudaStream_t st
       gw.kstride = (long long)kBmax * 2 * nc;
       if (rc == SSV_OK) step(gemm_launch<32, 9>(gw, st));
       qz_kernel<<<(2 * nc + 7) / 8, 256, sizeof(double) * kBmax * kBmax, st>>>(
-          Q.W, gw.ksplit, gw.kstride, Q.S, gs.ksplit, cnt, 2 * nc, tau, Q.zcol);
+          Q.W, gw.ksplit, gw.kstride, S1, cnt, 2 * nc, tau, Q.zcol);
       count_launch();
       cu(cudaGetLastError());
       GArgs gx = args(Q.vrow, Q.zcol, 0, (cnt + kTK - 1) / kTK, pv, n, 2 * nc, Xd, nX, 2 * ldX);
       gx.sub = 1;
       gx.rs = 2;
       gx.wrap = nc;
-      if (rc == SSV_OK) step(gemm_launch<64, 8>(gx, st));
+      // nine levels: the pairs eight leave out all have the sign of the product,
+      // and X lost 1e-15 of its norm over 1000 reflectors (2e-16 with nine)
+      if (rc == SSV_OK) step(gemm_launch<32, 9>(gx, st));
     }
   }
   if (rc == SSV_OK) {

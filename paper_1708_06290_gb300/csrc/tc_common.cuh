@@ -21,7 +21,15 @@ static __device__ __forceinline__ int scale_exp(double maxabs) {
   return ef == 0 ? -1022 : ef - 1022;
 }
 
-// the eight 7-bit digits of x relative to 2^E, as BF16 bit patterns
+// |x|'s high word, ordered as |x| is (NaN above Inf above all), and the same
+// exponent from the largest one
+static __device__ __forceinline__ int abs_hi(double x) { return __double2hiint(x) & 0x7fffffff; }
+static __device__ __forceinline__ int scale_exp_hi(int hi) {
+  const int ef = hi >> 20;
+  return ef == 0x7ff ? kBadExp : ef == 0 ? -1022 : ef - 1022;
+}
+
+// the eight 7-bit digits of x (to nearest) relative to 2^E, as BF16 bit patterns
 static __device__ __forceinline__ void digits8(double x, int E, unsigned short (&d)[kDigits]) {
   const unsigned long long b = (unsigned long long)__double_as_longlong(x);
   const unsigned short sgn = (unsigned short)((b >> 63) << 15);
@@ -35,7 +43,8 @@ static __device__ __forceinline__ void digits8(double x, int E, unsigned short (
   unsigned long long M = 0;
   if (E != kBadExp) {
     if (sh >= 0) M = mant << sh;  // sh <= 3 because |x| < 2^E
-    else if (sh > -64) M = mant >> (-sh);
+    // to nearest: with the rest cut off every product comes out small
+    else if (sh > -64) M = (mant + (1ull << (-sh - 1))) >> (-sh);
   }
 #pragma unroll
   for (int l = 0; l < kDigits; ++l) {
