@@ -55,7 +55,8 @@ constexpr int kAT = kM * kKS;    // BF16 elements of one H slice tile
 constexpr int kBT = kN * kKS;    // BF16 elements of one Xhat slice tile
 constexpr uint32_t kStageBytes = (uint32_t)kSl * (kAT + kBT) * 2;
 constexpr int kWinCols = kLev * kN;  // TMEM columns of a window; two windows
-constexpr int kDrain = 128;          // readout threads (one per row), warps 0 .. 3
+constexpr int kDrain = 256;          // readout threads (row x half of the columns), warps 0 .. 7
+constexpr int kH = kN * kM / kDrain;  // columns of a readout thread
 constexpr int kT = kDrain + 64;      // + the producer's and the issuer's warp
 constexpr size_t kSmem = 2 * (size_t)kStageBytes + 128;
 static_assert(kSmem <= 227 * 1024, "shared memory");
@@ -90,17 +91,12 @@ __global__ void __launch_bounds__(256) tc_hrow_kernel(int n, int m, const double
   const int j0 = blockIdx.y * kHChunk, j1 = min(n, j0 + kHChunk);
   // the chunk lies left of the structural part of every row of the block
   if (j1 <= (int)blockIdx.x * 128 - m) return;
-  double mx = 0.0;
-  bool bad = false;
+  int mx = 0;  // as integers: a maximum of doubles holds the FP64 pipe
   if (i < n) {
 #pragma unroll 8
-    for (int j = max(j0, i - m) + half; j < j1; j += 2) {
-      const double v = fabs(H[i + (size_t)j * n]);
-      if (!(v <= 1.7976931348623157e308)) bad = true;
-      else mx = fmax(mx, v);
-    }
+    for (int j = max(j0, i - m) + half; j < j1; j += 2) mx = max(mx, abs_hi(H[i + (size_t)j * n]));
   }
-  int E = i < n ? (bad ? kBadExp : scale_exp(mx)) : 0;  // padding rows: 0
+  int E = i < n ? scale_exp_hi(mx) : 0;  // padding rows: 0
   if (half == 1) part[row] = E;
   __syncthreads();
   if (half == 0) atomicMax(hexp + i, max(E, part[row]));
@@ -171,20 +167,15 @@ __global__ void __launch_bounds__(256) tc_xsplit_kernel(int n, int m, int npad, 
     const int ja = J0 * kKS, jb = min(n, J1 * kKS);
     for (int u = warp; u < m * parts; u += 8) {
       const int q = u % m, part = u / m;
-      double mr = 0.0, mi = 0.0;
-      bool br = false, bi = false;
+      int mr = 0, mi = 0;
 #pragma unroll 4
       for (int j = ja + part * 32 + lane; j < jb; j += parts * 32) {
         const cd x = Xh[j + (size_t)q * ldx];
-        const double vr = fabs(x.x), vi = fabs(x.y);
-        if (!(vr <= 1.7976931348623157e308)) br = true;
-        else mr = fmax(mr, vr);
-        if (!(vi <= 1.7976931348623157e308)) bi = true;
-        else mi = fmax(mi, vi);
+        mr = max(mr, abs_hi(x.x));
+        mi = max(mi, abs_hi(x.y));
       }
-      int er = br ? kBadExp : scale_exp(mr), ei = bi ? kBadExp : scale_exp(mi);
-      er = __reduce_max_sync(0xffffffffu, er);
-      ei = __reduce_max_sync(0xffffffffu, ei);
+      const int er = scale_exp_hi(__reduce_max_sync(0xffffffffu, mr));
+      const int ei = scale_exp_hi(__reduce_max_sync(0xffffffffu, mi));
       if (lane == 0) {
         atomicMax(&sE[2 * q], er);
         atomicMax(&sE[2 * q + 1], ei);
@@ -303,7 +294,7 @@ __global__ void __launch_bounds__(kT, 1) tc_residual_kernel(
   __syncthreads();
   fence_after();
   const uint32_t tmem = tslot;
-  if (warp == 4) {
+  if (warp == kDrain / 32) {
     if (lane == 0) {
       // ---- producer: stage i (counted over all items) into buffer i & 1
       unsigned i = 0;
@@ -330,7 +321,7 @@ __global__ void __launch_bounds__(kT, 1) tc_residual_kernel(
         }
       }
     }
-  } else if (warp == 5) {
+  } else if (warp == kDrain / 32 + 1) {
     if (lane == 0) {
       // ---- issuer: window v (counted over all items) into TMEM half v & 1
       unsigned i = 0, v = 0;
@@ -371,7 +362,12 @@ __global__ void __launch_bounds__(kT, 1) tc_residual_kernel(
       }
     }
   } else {
-    // ---- readout and epilogue: thread = row
+    // ---- readout and epilogue: thread = (row, half of the columns).  Two warps to
+    // a scheduler: with one, 2000 shifts at n = 5000, m = 16 took 60.3 ms (55.1)
+    const int hf = warp >> 2, cb = kH * hf;
+    // shifts of this half: lb .. lb + SH - 1 of the group, CL columns each from cz on
+    constexpr int SH = CS >= kH ? 1 : kH / CS, CL = CS < kH ? CS : kH;
+    const int lb = cb / CS, cz = cb % CS;
     unsigned v = 0;
     bool ok = true;
     for (long long t = blockIdx.x; t < items && ok; t += gridDim.x) {
@@ -379,9 +375,9 @@ __global__ void __launch_bounds__(kT, 1) tc_residual_kernel(
       task_coords(t, RB, ngrp, &I, &g);
       const int i0 = I * kM;
       const int nst = KT - max(0, i0 - m) / kKS;
-      float ah[kN], al[kN];
+      float ah[kH], al[kH];
 #pragma unroll
-      for (int c = 0; c < kN; ++c) { ah[c] = 0.f; al[c] = 0.f; }
+      for (int c = 0; c < kH; ++c) { ah[c] = 0.f; al[c] = 0.f; }
       for (int st = 0; st < nst; st += kWin, ++v) {
         const uint32_t h = v & 1u;
         // every lane polls; the warp agrees (it reads TMEM together)
@@ -391,10 +387,10 @@ __global__ void __launch_bounds__(kT, 1) tc_residual_kernel(
         float sc = 0.0078125f * 0.0078125f;  // 2^{-7t}, t = 2
 #pragma unroll 1
         for (int lv = 0; lv < kLev; ++lv) {
-          uint32_t r[32];
-          tmem_ld32(tmem + ((uint32_t)(warp * 32) << 16) + h * (uint32_t)kWinCols + (uint32_t)(lv * kN), r);
+          uint32_t r[kH];
+          tmem_ld16(tmem + ((uint32_t)((warp & 3) * 32) << 16) + h * (uint32_t)kWinCols + (uint32_t)(lv * kN + cb), r);
 #pragma unroll
-          for (int c = 0; c < kN; ++c) {
+          for (int c = 0; c < kH; ++c) {
             const float pv = __uint_as_float(r[c]) * sc;
             const float s = ah[c] + pv;
             const float bp = s - ah[c];
@@ -410,23 +406,24 @@ __global__ void __launch_bounds__(kT, 1) tc_residual_kernel(
       }
       if (!ok) break;
       // E(i, q) = R(i, q) - (H Xhat)(i, q) + sigma Xhat(i, q) of the group's shifts
-      const int i = i0 + tid;
+      const int i = i0 + (tid & (kM - 1));
       const int Ei = i < n ? hexp[i] : 0;
 #pragma unroll
-      for (int l = 0; l < S; ++l) {
-        const int w = g * S + l;
+      for (int l = 0; l < SH; ++l) {
+        const int w = g * S + lb + l;
         if (w >= cnt) continue;
         const int sh = list[w];
         double e2 = 0.0, x2 = 0.0;
         if (i < n) {
           const cd sigma = shifts[sh];
-          const int* Ec = xexp + (size_t)g * kN + l * CS;
+          const int* Ec = xexp + (size_t)g * kN + cb + l * CL;
           const cd* Xh = X + (size_t)sh * m * ldx;
 #pragma unroll
-          for (int q = 0; q < CS / 2; ++q) {
+          for (int u = 0; u < CL / 2; ++u) {
+            const int q = cz / 2 + u;
             if (q < m) {
-              const int c = l * CS + 2 * q;
-              const int er_ = Ec[2 * q], ei_ = Ec[2 * q + 1];
+              const int c = l * CL + 2 * u;
+              const int er_ = Ec[2 * u], ei_ = Ec[2 * u + 1];
               const bool bad = Ei == kBadExp || er_ == kBadExp || ei_ == kBadExp;
               const double hxr = ldexp((double)ah[c] + (double)al[c], Ei + er_);
               const double hxi = ldexp((double)ah[c + 1] + (double)al[c + 1], Ei + ei_);
