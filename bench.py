@@ -414,13 +414,13 @@ def tensor_residual_roofline(n, m, s, mixed):
 
 def tcs_update_flops(n, m, s):
     """Executed BF16 flops of all tcs_update_kernel launches of one tensor-core sweep (the
-    loop of solve_tc): per item (128 rows above the block x one group of S = 64 / 2m shifts)
-    ceil(nbe / 32) stages of 35 digit pairs x 2 K-halves of 128 x 64 x 16, then per shift 28
-    pairs x 2 K-halves of 128 x 2m x 16 (Z2 P2).  Valid for 2m dividing 64."""
+    loop of solve_tc): per item (128 rows above the block x one group of S = 32 / 2m shifts)
+    ceil(nbe / 32) stages of 35 digit pairs x 2 K-halves of 128 x 32 x 16, then per shift 28
+    pairs x 2 K-halves of 128 x 2m x 16 (Z2 P2).  Valid for 2m dividing 32."""
     cs = 2 * m
-    if 64 % cs:
+    if 32 % cs:
         return None, 0
-    S = 64 // cs
+    S = 32 // cs
     G = -(-s // S)
     nbe_first = (n - m) % 128 or 128
     k, step, flops, launches = n, 0, 0.0, 0
@@ -430,7 +430,7 @@ def tcs_update_flops(n, m, s):
         hrows = k - nbe
         if hrows > 0:
             items = -(-hrows // 128) * G
-            per_item = -(-nbe // 32) * 70 * 2.0 * 128 * 64 * 16 + S * 56 * 2.0 * 128 * cs * 16
+            per_item = -(-nbe // 32) * 70 * 2.0 * 128 * 32 * 16 + S * 56 * 2.0 * 128 * cs * 16
             flops += items * per_item
             launches += 1
         k -= nbe

@@ -445,7 +445,9 @@ static __device__ __forceinline__ float pow2f(int e) { return __int_as_float((e 
 constexpr int kFastExp = 30;
 static __device__ __forceinline__ bool fast_exp(int e) { return e >= -kFastExp && e <= kFastExp; }
 
-constexpr int kUT = 2 * kUM + 64;  // update threads: two epilogue groups, the producer's and the issuer's warp
+constexpr int kUH = 16;              // columns of an epilogue thread
+constexpr int kUG = kUM * kUN / kUH;  // threads of an epilogue group
+constexpr int kUT = 2 * kUG + 64;    // update threads: two epilogue groups, the producer's and the issuer's warp
 
 // a bounded wait of one role: gives up at the poll limit or when another role
 // has (the block then leaves together)
@@ -458,6 +460,22 @@ static __device__ __forceinline__ bool role_wait(uint32_t mbar, uint32_t parity,
   return false;
 }
 
+// Item -> row block I of RT and group g of G.  All groups per row block, so that
+// the blocks running together share H's digit tiles; but where the groups' P1
+// digits (57 KB each) do not stay in L2, only as many groups at a time as blocks
+// run: theirs then stay while the rows go by.  2000 groups of 32 columns at n =
+// 5000: 93.3 ms in all one row block at a time, 87.8 in chunks; 250 groups at n =
+// 1000: a call of 7.97 ms one row block at a time, 8.25 in chunks.
+constexpr size_t kPGroupBytes = (size_t)kSD * kStages * kBT * 2;
+constexpr size_t kPKeep = (size_t)64 << 20;
+static __device__ __forceinline__ void item_of(long long item, int RT, int G, int& I, int& g) {
+  const int gb = (size_t)G * kPGroupBytes > kPKeep ? (int)gridDim.x : G;
+  const int q = (int)(item / ((long long)RT * gb));
+  const int rem = (int)(item - (long long)q * RT * gb), w = min(gb, G - q * gb);
+  I = rem / w;
+  g = q * gb + rem % w;
+}
+
 // The update of block step (k, nbe) for shifts of CS real columns (2m rounded
 // up to a power of two).  An item is 128 rows of H x one group of S = 32 / CS
 // shifts; a persistent block works on two at a time, in roles that only meet at
@@ -468,27 +486,31 @@ static __device__ __forceinline__ bool role_wait(uint32_t mbar, uint32_t parity,
 //   * an issuing thread multiplies: item v's Z1 P1 into the eight levels of TMEM
 //     window v mod 2, then, once these are read, its Z2 P2 into seven levels of
 //     the same window, one item behind;
-//   * two groups of four warps take alternate items (thread = row, 32 columns):
+//   * two groups of eight warps take alternate items (thread = row, 16 columns):
 //     levels into double-float sums, scaling, the shifted-diagonal correction,
 //     and the new rows: as FP32 pairs the 128 that the next panel (or the final
 //     block) reads, all others as the digit tiles of the next block step (CS <
 //     16: Z2 P2 in double-float here, and every row as pairs).
 //
 // What bounds it, per item at CS = 32: the copies from L2 (392 KB, about 6.5 k
-// clocks), the epilogue's instructions (5.3 k issue slots a scheduler) and the
-// products (5.5 k clocks), which run side by side.  One item at a time, each
-// phase after the other, took 6.0 ms a launch at the start of the sweep of 2000
-// shifts at n = 5000, m = 16 (114 ms for the 39 launches).
+// clocks), the epilogue's instructions (8.4 k issue slots a scheduler) and the
+// products (5.5 k clocks), which run side by side; DRAM 22 % busy.  Two epilogue
+// warps to a scheduler left it idle for 58 % of the clocks; with four, the update
+// of 600 shifts at n = 2500, m = 8 takes 4.29 ms (4.69), of 2000 at n = 1000, m = 4
+// 0.93 ms (1.30).  One item at a time, each phase after the other, took 6.0 ms a
+// launch at the start of the sweep of 2000 shifts at n = 5000, m = 16 (114 ms for
+// the 39 launches, now 87.8).
 template <int CS>
 __global__ void __launch_bounds__(kUT, 1) tcs_update_kernel(TcsArgs a, int k, int nbe) {
   constexpr bool TCZ = CS >= 16;
   constexpr int S = kUN / CS;             // shifts of a group
   extern __shared__ __align__(128) unsigned char smem[];
-  __shared__ __align__(8) unsigned long long mbar[14];
+  __shared__ __align__(8) unsigned long long mbar[22];
   __shared__ uint32_t tslot;
   __shared__ volatile int fail;
   // stages copied / multiplied, Z2 tiles copied / multiplied (read when a wait gave up)
   __shared__ int issued[4];
+  __shared__ unsigned char rowmax[2][2][kUM];  // CS = 32: FP32 exponent fields of the halves of a row
   const int n = a.n, m = a.m, p = a.p, ldz = p + n;
   const int hrows = k - nbe;              // H rows above the block
   const int j0 = k - m - nbe;             // first fresh column (a multiple of 32)
@@ -514,9 +536,11 @@ __global__ void __launch_bounds__(kUT, 1) tcs_update_kernel(TcsArgs a, int k, in
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;");
   }
   if (tid == 0) {
-    for (int q = 0; q < 14; ++q)  // pread and qread: one arrival per warp of the group
+    // pread and qread: one arrival per warp of the group; from 14 on: the warp
+    // pairs that share rows
+    for (int q = 0; q < 22; ++q)
       asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(full + 8u * q),
-                   "r"(q == 8 || q == 9 || q >= 12 ? kUM / 32 : 1));
+                   "r"(q >= 14 ? 2 : q == 8 || q == 9 || q >= 12 ? kUG / 32 : 1));
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     fail = 0;
     for (int q = 0; q < 4; ++q) issued[q] = 0;
@@ -531,14 +555,15 @@ __global__ void __launch_bounds__(kUT, 1) tcs_update_kernel(TcsArgs a, int k, in
   constexpr int kgz = CS >= 8 ? CS / 8 : 1;
   const long long mine = blockIdx.x < items ? (items - blockIdx.x + gridDim.x - 1) / gridDim.x : 0;
 
-  if (warp == 2 * kUM / 32) {
+  if (warp == 2 * kUG / 32) {
     if (lane == 0) {
       // ---- producer
       unsigned i = 0;
       bool ok = true;
       auto stages = [&](long long v) {
         const long long item = blockIdx.x + v * gridDim.x;
-        const int I = (int)(item / G), g = (int)(item % G);
+        int I, g;
+        item_of(item, RT, G, I, g);
         const size_t Pg0 = (size_t)g * kSD * kStages * kBT;
         for (int st = 0; st < nst && ok; ++st, ++i) {
           const uint32_t b = i & 1u;
@@ -561,7 +586,8 @@ __global__ void __launch_bounds__(kUT, 1) tcs_update_kernel(TcsArgs a, int k, in
       };
       auto ztiles = [&](long long v) {
         const long long item = blockIdx.x + v * gridDim.x;
-        const int I = (int)(item / G), g = (int)(item % G);
+        int I, g;
+        item_of(item, RT, G, I, g);
         if (!role_wait(zempty, ((unsigned)v & 1u) ^ 1u, &fail)) {
           ok = false;
           return;
@@ -585,7 +611,7 @@ __global__ void __launch_bounds__(kUT, 1) tcs_update_kernel(TcsArgs a, int k, in
         if (TCZ && v > 0 && ok) ztiles(v - 1);
       }
     }
-  } else if (warp == 2 * kUM / 32 + 1) {
+  } else if (warp == 2 * kUG / 32 + 1) {
     if (lane == 0) {
       // ---- issuer
       unsigned i = 0;
@@ -637,7 +663,9 @@ __global__ void __launch_bounds__(kUT, 1) tcs_update_kernel(TcsArgs a, int k, in
       auto z2p2 = [&](long long v) {
         const uint32_t h = (unsigned)v & 1u, u = (unsigned)(v >> 1);
         const uint32_t d = tmem + h * (uint32_t)kWinCols;
-        const int g = (int)((blockIdx.x + v * gridDim.x) % G), nsh = min(S, a.s - g * S);
+        int I, g;
+        item_of(blockIdx.x + v * gridDim.x, RT, G, I, g);
+        const int nsh = min(S, a.s - g * S);
         if (!role_wait(pread + 8u * h, u & 1u, &fail) || !role_wait(zfull, (unsigned)v & 1u, &fail)) {
           ok = false;
           return;
@@ -668,62 +696,64 @@ __global__ void __launch_bounds__(kUT, 1) tcs_update_kernel(TcsArgs a, int k, in
       }
     }
   } else {
-    // ---- epilogue: group h = warp / 4 takes items v = h, h + 2, ..
-    const uint32_t h = (uint32_t)(warp >> 2);
+    // ---- epilogue: group h takes items v = h, h + 2, ..; thread = (row, half of
+    // the columns): eight warps to a scheduler's two hide each other's latency
+    const uint32_t h = (uint32_t)(warp / (kUG / 32));
+    const int hf = (warp >> 2) & 1, cb = kUH * hf;  // its first column
     const int row = tid & (kUM - 1);
     const uint32_t tl = tmem + h * (uint32_t)kWinCols + ((uint32_t)((warp & 3) * 32) << 16);
+    // shifts of this half: lb .. lb + SH - 1 of the group
+    constexpr int SH = CS >= kUH ? 1 : kUH / CS, CL = CS < kUH ? CS : kUH;  // CL: columns of a shift here
+    const int lb = cb / CS, cz = cb % CS;  // cz: the first one's first column within its shift
     auto arrive = [&](uint32_t b) {
       fence_before();
       __syncwarp();
       if (lane == 0) asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(b) : "memory");
     };
+    [[maybe_unused]] int xn = 0;  // exchanges of row maxima so far
     for (long long v = h; v < mine; v += 2) {
       const uint32_t par = (unsigned)(v >> 1) & 1u;
       const long long item = blockIdx.x + v * gridDim.x;
-      const int I = (int)(item / G), g = (int)(item % G);
+      int I, g;
+      item_of(item, RT, G, I, g);
       const int ih = I * kUM + row;
       const bool live = ih < hrows;
       // exponents: of the row, of this lane's column (P1's, P2's), of the row's Z2
       const int Ei = live ? a.hexp[BCK(ih, a.npad)] : 0;
       int E1 = 0, E2 = 0;
       {
-        const int sh = g * S + lane / CS, c = lane % CS;
+        const int cg = cb + (lane & (kUH - 1)), sh = g * S + cg / CS, c = cg % CS;
         if (sh < a.s && c < 2 * m) {
           E1 = a.pexp[(size_t)sh * 2 * kMaxM + c];
           if (TCZ) E2 = a.p2exp[(size_t)sh * 2 * kMaxM + c];
         }
       }
-      int Ez[TCZ ? S : 1];
-      bool fast = fast_exp(Ei);
-      if constexpr (TCZ) {
-#pragma unroll
-        for (int l = 0; l < S; ++l) {
-          Ez[l] = (live && g * S + l < a.s) ? a.zexp[BCK((size_t)(g * S + l) * a.npad + ih, (size_t)a.s * a.npad)] : 0;
-          fast = fast && fast_exp(Ez[l]);
-        }
-      }
+      int ez = 0;
+      if constexpr (TCZ)
+        if (live && g * S + lb < a.s) ez = a.zexp[BCK((size_t)(g * S + lb) * a.npad + ih, (size_t)a.s * a.npad)];
       // the row exponents of a warp and the column exponents: one path per warp
-      fast = __all_sync(0xffffffffu, fast && fast_exp(E1) && fast_exp(E2));
+      const bool fast =
+          __all_sync(0xffffffffu, fast_exp(Ei) && fast_exp(ez) && fast_exp(E1) && fast_exp(E2));
       if (!__all_sync(0xffffffffu, role_wait(pfull + 8u * h, par, &fail))) break;
       fence_after();
-      // the new entries, 32 real columns of the row (Re, Im interleaved), as pairs
-      float ah[kUN], al[kUN];
+      // the new entries, 16 real columns of the row (Re, Im interleaved), as pairs
+      float ah[kUH], al[kUH];
 #pragma unroll
-      for (int c = 0; c < kUN; ++c) { ah[c] = 0.f; al[c] = 0.f; }
+      for (int c = 0; c < kUH; ++c) { ah[c] = 0.f; al[c] = 0.f; }
       {
         float sc = 0.0078125f * 0.0078125f;  // 2^{-7 (t + 2)}, t = 0
 #pragma unroll 1
         for (int lv = 0; lv < kLev; ++lv) {
-          uint32_t rr[32];
-          tmem_ld32(tl + (uint32_t)(lv * kUN), rr);
+          uint32_t rr[kUH];
+          tmem_ld16(tl + (uint32_t)(lv * kUN + cb), rr);
 #pragma unroll
-          for (int c = 0; c < kUN; ++c) add_f(ah[c], al[c], __uint_as_float(rr[c]) * sc);
+          for (int c = 0; c < kUH; ++c) add_f(ah[c], al[c], __uint_as_float(rr[c]) * sc);
           sc *= 0.0078125f;
         }
       }
       arrive(pread + 8u * h);
 #pragma unroll
-      for (int c = 0; c < kUN; ++c) {
+      for (int c = 0; c < kUH; ++c) {
         const int Ec = __shfl_sync(0xffffffffu, E1, c);
         if (fast) {
           const float f = pow2f(Ei + Ec);
@@ -740,48 +770,44 @@ __global__ void __launch_bounds__(kUT, 1) tcs_update_kernel(TcsArgs a, int k, in
       if constexpr (TCZ) {
         if (!__all_sync(0xffffffffu, role_wait(qfull + 8u * h, par, &fail))) break;
         fence_after();
-        // 16 columns at a time: shift l's levels start at column 7 CS l
+        // shift l's levels start at column 7 CS l
+        const uint32_t tz = tl + (uint32_t)(7 * CS * lb + cz);
+        if (fast) {
+          float f[kUH];
 #pragma unroll
-        for (int c0 = 0; c0 < kUN; c0 += 16) {
-          const uint32_t tz = tl + (uint32_t)(7 * CS * (c0 / CS) + c0 % CS);
-          const int ez = Ez[c0 / CS];
-          if (fast) {
-            float f[16];
-#pragma unroll
-            for (int c = 0; c < 16; ++c) f[c] = pow2f(ez + __shfl_sync(0xffffffffu, E2, c0 + c) - 14);
+          for (int c = 0; c < kUH; ++c) f[c] = pow2f(ez + __shfl_sync(0xffffffffu, E2, c) - 14);
 #pragma unroll 1
-            for (int lv = 0; lv < 7; ++lv) {
-              uint32_t rr[16];
-              tmem_ld16(tz + (uint32_t)(lv * CS), rr);
+          for (int lv = 0; lv < 7; ++lv) {
+            uint32_t rr[kUH];
+            tmem_ld16(tz + (uint32_t)(lv * CS), rr);
 #pragma unroll
-              for (int c = 0; c < 16; ++c) {
-                add_f(ah[c0 + c], al[c0 + c], __uint_as_float(rr[c]) * f[c]);
-                f[c] *= 0.0078125f;
-              }
+            for (int c = 0; c < kUH; ++c) {
+              add_f(ah[c], al[c], __uint_as_float(rr[c]) * f[c]);
+              f[c] *= 0.0078125f;
             }
-          } else {
-            float bh[16], bl[16];
+          }
+        } else {
+          float bh[kUH], bl[kUH];
 #pragma unroll
-            for (int c = 0; c < 16; ++c) { bh[c] = 0.f; bl[c] = 0.f; }
-            float sc = 0.0078125f * 0.0078125f;
+          for (int c = 0; c < kUH; ++c) { bh[c] = 0.f; bl[c] = 0.f; }
+          float sc = 0.0078125f * 0.0078125f;
 #pragma unroll 1
-            for (int lv = 0; lv < 7; ++lv) {
-              uint32_t rr[16];
-              tmem_ld16(tz + (uint32_t)(lv * CS), rr);
+          for (int lv = 0; lv < 7; ++lv) {
+            uint32_t rr[kUH];
+            tmem_ld16(tz + (uint32_t)(lv * CS), rr);
 #pragma unroll
-              for (int c = 0; c < 16; ++c) add_f(bh[c], bl[c], __uint_as_float(rr[c]) * sc);
-              sc *= 0.0078125f;
-            }
+            for (int c = 0; c < kUH; ++c) add_f(bh[c], bl[c], __uint_as_float(rr[c]) * sc);
+            sc *= 0.0078125f;
+          }
 #pragma unroll
-            for (int c = 0; c < 16; ++c) {
-              const int Ec = __shfl_sync(0xffffffffu, E2, c0 + c);
-              if (ez == kBadExp || Ec == kBadExp) {
-                ah[c0 + c] = __int_as_float(0x7fc00000);
-                al[c0 + c] = 0.f;
-              } else {
-                add_f(ah[c0 + c], al[c0 + c], ldexpf(bh[c], ez + Ec));
-                al[c0 + c] += ldexpf(bl[c], ez + Ec);
-              }
+          for (int c = 0; c < kUH; ++c) {
+            const int Ec = __shfl_sync(0xffffffffu, E2, c);
+            if (ez == kBadExp || Ec == kBadExp) {
+              ah[c] = __int_as_float(0x7fc00000);
+              al[c] = 0.f;
+            } else {
+              add_f(ah[c], al[c], ldexpf(bh[c], ez + Ec));
+              al[c] += ldexpf(bl[c], ez + Ec);
             }
           }
         }
@@ -791,10 +817,10 @@ __global__ void __launch_bounds__(kUT, 1) tcs_update_kernel(TcsArgs a, int k, in
         // old row of each shift
         constexpr int CC = CS / 2;  // complex columns of a shift
 #pragma unroll
-        for (int l = 0; l < S; ++l) {
-          if (g * S + l < a.s) {
-            const float4* z = a.Z2 + BCK((size_t)(g * S + l) * a.z2_stride + (p + ih), a.n_z2);
-            const float4* pc = a.pc + BCK((size_t)(g * S + l) * 2 * kMaxM * kMaxM, a.n_pc);
+        for (int l = 0; l < SH; ++l) {
+          if (g * S + lb + l < a.s) {
+            const float4* z = a.Z2 + BCK((size_t)(g * S + lb + l) * a.z2_stride + (p + ih), a.n_z2);
+            const float4* pc = a.pc + BCK((size_t)(g * S + lb + l) * 2 * kMaxM * kMaxM, a.n_pc);
             float4 zz[CC];
 #pragma unroll
             for (int qq = 0; qq < CC; ++qq) zz[qq] = qq < m ? z[(size_t)qq * ldz] : make_float4(0.f, 0.f, 0.f, 0.f);
@@ -819,8 +845,8 @@ __global__ void __launch_bounds__(kUT, 1) tcs_update_kernel(TcsArgs a, int k, in
       if (live && cdr >= 0 && cdr < nsig) {
         // - sigma P1(cdr, q)
 #pragma unroll
-        for (int c = 0; c < kUN; c += 2) {
-          const int l = c / CS, q = (c % CS) >> 1, sh = g * S + l;
+        for (int c = 0; c < kUH; c += 2) {
+          const int l = lb + c / CL, q = (cz + c % CL) >> 1, sh = g * S + l;
           if (q >= m || sh >= a.s) continue;
           const float4 sgf = df_split(a.shifts[sh]);
           const float4 w = a.pc[BCK((size_t)sh * 2 * kMaxM * kMaxM + m * m + cdr * m + q, a.n_pc)];
@@ -832,7 +858,7 @@ __global__ void __launch_bounds__(kUT, 1) tcs_update_kernel(TcsArgs a, int k, in
       }
       // normalised pairs
 #pragma unroll
-      for (int c = 0; c < kUN; ++c) {
+      for (int c = 0; c < kUH; ++c) {
         const float s = ah[c] + al[c];
         al[c] = al[c] - (s - ah[c]);
         ah[c] = s;
@@ -840,8 +866,8 @@ __global__ void __launch_bounds__(kUT, 1) tcs_update_kernel(TcsArgs a, int k, in
       // as pairs: the rows of the next panel or the final block
       if (live && (!TCZ || ih >= hrows - kNBT)) {
 #pragma unroll
-        for (int c = 0; c < kUN; c += 2) {
-          const int l = c / CS, q = (c % CS) >> 1;
+        for (int c = 0; c < kUH; c += 2) {
+          const int l = lb + c / CL, q = (cz + c % CL) >> 1;
           if (q >= m || g * S + l >= a.s) continue;
           a.Z2[BCK((size_t)(g * S + l) * a.z2_stride + (p + ih) + (size_t)q * ldz, a.n_z2)] =
               make_float4(ah[c], al[c], ah[c + 1], al[c + 1]);
@@ -849,33 +875,42 @@ __global__ void __launch_bounds__(kUT, 1) tcs_update_kernel(TcsArgs a, int k, in
       }
       // as digits: the rows above them (none of a tile that lies within the last 128 rows)
       if constexpr (TCZ) {
-        if (live && I * kUM < hrows - kNBT) {
+        if (I * kUM < hrows - kNBT) {
+          const int sh = g * S + lb;
+          // the row's digit exponent: the maximum over the shift's 2m entries, by
+          // FP32 exponent field (255: not finite)
+          int fe = 0;
 #pragma unroll
-          for (int l = 0; l < S; ++l) {
-            const int sh = g * S + l;
-            if (sh >= a.s) continue;
-            // the row's digit exponent: the maximum over the shift's 2m entries
-            float mx = 0.f;
-            bool bad = false;
-#pragma unroll
-            for (int c = l * CS; c < (l + 1) * CS; ++c) {
-              if (c % CS >= 2 * m) { ah[c] = 0.f; al[c] = 0.f; }
-              mx = fmaxf(mx, fabsf(ah[c]));
-              bad = bad || !(fabsf(ah[c]) <= 3.4e38f);
-            }
-            if (bad) mx = __int_as_float(0x7f800000);
-            const int E = col_exp(scale_exp_f(mx));
-            a.zexp[BCK((size_t)sh * a.npad + ih, (size_t)a.s * a.npad)] = E;
+          for (int c = 0; c < kUH; ++c) {
+            if (cz + c >= 2 * m) { ah[c] = 0.f; al[c] = 0.f; }
+            fe = max(fe, __float_as_int(ah[c]) & 0x7fffffff);
+          }
+          fe >>= 23;
+          if constexpr (CS > kUH) {
+            // the other half of the row is in the warp with the same rows: written
+            // in even phases of the pair's barrier, read in odd ones
+            const uint32_t xb = full + 8u * (14u + h * 4u + (uint32_t)(warp & 3));
+            if (xn > 0 && !__all_sync(0xffffffffu, role_wait(xb, 1u, &fail))) break;
+            rowmax[h][hf][row] = (unsigned char)fe;
+            arrive(xb);
+            if (!__all_sync(0xffffffffu, role_wait(xb, 0u, &fail))) break;
+            fe = max(fe, (int)rowmax[h][hf ^ 1][row]);
+            arrive(xb);
+            ++xn;
+          }
+          if (live && sh < a.s) {
+            const int E = col_exp(scale_exp_f(__int_as_float(fe << 23)));
+            if (cz == 0) a.zexp[BCK((size_t)sh * a.npad + ih, (size_t)a.s * a.npad)] = E;
             const float inv = digit_scale(E);
             const size_t T0 = ((size_t)sh * a.RB + I) * 7 * (128 * CS);
 #pragma unroll
-            for (int k8 = 0; k8 < CS; k8 += 8) {
+            for (int k8 = 0; k8 < kUH; k8 += 8) {
               float hi[8], lo[8];
 #pragma unroll
-              for (int e = 0; e < 8; ++e) { hi[e] = ah[l * CS + k8 + e]; lo[e] = al[l * CS + k8 + e]; }
+              for (int e = 0; e < 8; ++e) { hi[e] = ah[k8 + e]; lo[e] = al[k8 + e]; }
               uint4 dg[7];
               digits7_oct(hi, lo, inv, dg);
-              const int off = tile_off_kg(row, k8, kgz);
+              const int off = tile_off_kg(row, cz + k8, kgz);
 #pragma unroll
               for (int l2 = 0; l2 < 7; ++l2)
                 *reinterpret_cast<uint4*>(a.Zd + BCK(T0 + (size_t)l2 * (128 * CS) + off, a.n_zd)) = dg[l2];
