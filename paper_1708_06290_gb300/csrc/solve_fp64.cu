@@ -10,11 +10,11 @@ template <int MAXM, bool DF = false>
 __global__ void __launch_bounds__(sweep_threads<MAXM>(), sweep_per_sm(MAXM, DF)) solve_fp64_kernel(
     int n, int m, int p, int nb, const double* __restrict__ H, const double* __restrict__ Ct,
     int ldct, const double* __restrict__ R, int s, const cd* __restrict__ shifts, int mode,
-    cd* __restrict__ scratch, size_t slot_stride, cd* __restrict__ out, long long ldo,
+    cd* scratch, size_t slot_stride, cd* __restrict__ out, long long ldo,
     int* __restrict__ status, cd* __restrict__ xhat_copy, long long ldxc,
     const double* __restrict__ hnorm, const int* __restrict__ list,
     const int* __restrict__ count, const cd* __restrict__ bhat, long long ldb,
-    const float* __restrict__ Hhi, const float* __restrict__ Hlo) {
+    const float* __restrict__ Hhi, const float* __restrict__ Hlo, int team) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   __shared__ int s_piv;
   __shared__ int s_sing;
@@ -26,12 +26,14 @@ __global__ void __launch_bounds__(sweep_threads<MAXM>(), sweep_per_sm(MAXM, DF))
   d.Hhi = Hhi; d.Hlo = Hlo;
   d.gfull = GivensSched{nullptr, nullptr, 0};
   d.gtail = d.gfull;
-  cd* Z2 = scratch + (size_t)blockIdx.x * slot_stride;
-  // With a work list, the block takes list entries blockIdx.x, +gridDim.x, ...
+  // team: CTAs of a cluster per shift (fp64_shift)
+  const int rank = team > 1 ? cluster_rank() : 0, g = blockIdx.x / team, G = gridDim.x / team;
+  cd* Z2 = scratch + (size_t)g * slot_stride;
+  // With a work list, the team takes list entries g, g + G, ...
   const int nwork = list != nullptr ? *count : s;
-  for (int w = blockIdx.x; w < nwork; w += gridDim.x) {
+  for (int w = g; w < nwork; w += G) {
     const int sh = list != nullptr ? list[w] : w;
-    fp64_shift<MAXM, sweep_threads<MAXM>(), false, false, DF>(d, sh, Z2, smem_raw, &s_piv, &s_sing);
+    fp64_shift<MAXM, sweep_threads<MAXM>(), false, false, DF>(d, sh, Z2, smem_raw, &s_piv, &s_sing, team, rank);
   }
 }
 
@@ -55,12 +57,11 @@ int launch_solve(const Handle* h, int s, const double* shifts, int nb, int mode,
   int grid = std::min(s, num_sms() * per_sm);
   cd* scratch = nullptr;
   SSV_CUDA_TRY(pool_alloc((void**)&scratch, sizeof(cd) * slot * grid, st));
-  kern<<<grid, NT, L::bytes, st>>>(n, m, p, nb, h->H, h->Ct, p > 0 ? p : 1, h->R, s,
-                                         reinterpret_cast<const cd*>(shifts), mode, scratch, slot,
-                                         reinterpret_cast<cd*>(out), ldo, status, xhat_copy, ldxc,
-                                         h->hnorm2, list, count, bhat, ldb, h->Hhi, h->Hlo);
-  count_launch();
-  cudaError_t e = cudaGetLastError();
+  const int team = team_for(s, n, m);
+  cudaError_t e = launch_cluster(kern, grid * team, NT, team, L::bytes, st, n, m, p, nb, h->H, h->Ct, p > 0 ? p : 1,
+                                 h->R, s, reinterpret_cast<const cd*>(shifts), mode, scratch, slot,
+                                 reinterpret_cast<cd*>(out), ldo, status, xhat_copy, ldxc, h->hnorm2, list, count,
+                                 bhat, ldb, h->Hhi, h->Hlo, team);
   cudaError_t e2 = cudaFreeAsync(scratch, st);
   if (e == cudaSuccess) e = e2;
   if (e != cudaSuccess) {
@@ -284,7 +285,7 @@ int launch_solve_noalloc(const Handle* h, int s, const double* shifts, int nb, i
                                          reinterpret_cast<const cd*>(shifts), mode,
                                          reinterpret_cast<cd*>(base), slot,
                                          reinterpret_cast<cd*>(out), ldo, status, nullptr, 0,
-                                         h->hnorm2, nullptr, nullptr, nullptr, 0, nullptr, nullptr);
+                                         h->hnorm2, nullptr, nullptr, nullptr, 0, nullptr, nullptr, 1);
   count_launch();
   SSV_CUDA_TRY(cudaGetLastError());
   if (status != nullptr) {

@@ -22,13 +22,15 @@ __global__ void __launch_bounds__(kThreads) solve_fp64_givens_kernel(FpSys d, in
 // flipped form built by solve_fp64_trans); d.p == 0.
 template <int MAXM>
 __global__ void __launch_bounds__(sweep_threads<MAXM>(), sweep_per_sm(MAXM, false))
-    solve_fp64_rhs_kernel(FpSys d, int s, cd* __restrict__ scratch, size_t slot_stride) {
+    solve_fp64_rhs_kernel(FpSys d, int s, cd* scratch, size_t slot_stride, int team) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   __shared__ int s_piv;
   __shared__ int s_sing;
-  cd* Z2 = scratch + (size_t)blockIdx.x * slot_stride;
-  for (int w = blockIdx.x; w < s; w += gridDim.x)
-    fp64_shift<MAXM, sweep_threads<MAXM>(), true>(d, w, Z2, smem_raw, &s_piv, &s_sing);
+  // team: CTAs of a cluster per shift (fp64_shift)
+  const int rank = team > 1 ? cluster_rank() : 0, g = blockIdx.x / team, G = gridDim.x / team;
+  cd* Z2 = scratch + (size_t)g * slot_stride;
+  for (int w = g; w < s; w += G)
+    fp64_shift<MAXM, sweep_threads<MAXM>(), true>(d, w, Z2, smem_raw, &s_piv, &s_sing, team, rank);
 }
 
 // Ht(i, j) = H(n-1-j, n-1-i) on the structural part i <= j + m, zero below:
@@ -88,9 +90,8 @@ int launch_rhs(const FpSys& d, int s, cudaStream_t st) {
   const int grid = std::min(s, num_sms() * per_sm);
   cd* scratch = nullptr;
   SSV_CUDA_TRY(pool_alloc((void**)&scratch, sizeof(cd) * slot * grid, st));
-  kern<<<grid, NT, L::bytes, st>>>(d, s, scratch, slot);
-  count_launch();
-  cudaError_t e = cudaGetLastError();
+  const int team = team_for(s, d.n, d.m);
+  cudaError_t e = launch_cluster(kern, grid * team, NT, team, L::bytes, st, d, s, scratch, slot, team);
   cudaError_t e2 = cudaFreeAsync(scratch, st);
   if (e == cudaSuccess) e = e2;
   if (e != cudaSuccess) {

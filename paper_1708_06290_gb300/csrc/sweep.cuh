@@ -44,6 +44,7 @@
 #include <utility>
 #include <vector>
 
+#include "cluster.cuh"
 #include "dfloat.cuh"
 #include "panel.cuh"
 #include "ssv_internal.cuh"
@@ -80,6 +81,19 @@ constexpr int sweep_threads() {
   return MAXM <= 16 ? 256 : 512;
 }
 constexpr int sweep_per_sm(int maxm, bool df) { return maxm > 16 ? 1 : df && maxm <= 8 ? 3 : 2; }
+// CTAs that share a shift: a power of two up to 8 while every team's CTAs have SMs
+// of their own (clusters of four and eight do not tile all SMs of the chip: 19
+// teams of eight took 17.7 ms where 24 of four take 14.7), for windows with enough
+// rows to share (n = 256, m = 2: 0.54 ms either way).  FP64, n = 3000, m = 8: up to
+// 10 shifts 28.4 -> 12.4 ms, 24 shifts 14.7, 64 shifts 19.2; n = 600, m = 4, 64 shifts
+// 1.73 -> 1.60; double-float, n = 1500, m = 16, 24 shifts 9.1 -> 5.2.
+[[maybe_unused]] static int team_for(int s, int n, int m) {
+  if ((long long)n * m < 1024) return 1;
+  const long long sms = num_sms();
+  if (s * 8LL <= sms * 5 / 6) return 8;
+  if (s * 4LL <= sms * 5 / 6) return 4;
+  return s * 2LL <= sms ? 2 : 1;
+}
 constexpr int m_class(int m) { return m <= 1 ? 1 : m <= 2 ? 2 : m <= 4 ? 4 : m <= 8 ? 8 : m <= 16 ? 16 : 32; }
 
 // Givens-panel variant (Sec. 3.2, Algorithms 9/10): the whole window block
@@ -145,9 +159,14 @@ namespace {
 // as it is produced, bottom-up), the rows above the block through the
 // accumulated coefficients `coefr`; the solution is T(:, live) y - Tr with Tr
 // the T rows of sum_c (-f_c) F_c and y from the final m x m block.
+//
+// team > 1: the CTAs of a cluster share the shift and its window state.  Each runs
+// the panels (the same bits in all of them, so nothing is exchanged) and takes
+// its share of the other rows.
 template <int MAXM, int NT, bool RHS = false, bool GIVENS = false, bool DF = false>
-__device__ void fp64_shift(const FpSys& d, const int sh, cd* __restrict__ Z2,
-                           unsigned char* smem_raw, int* s_piv_p, int* s_sing_p) {
+__device__ void fp64_shift(const FpSys& d, const int sh, cd* Z2,
+                           unsigned char* smem_raw, int* s_piv_p, int* s_sing_p, const int team = 1,
+                           const int rank = 0) {
   using L = Layout<MAXM>;
   using GL = GivensLayout<MAXM>;
   constexpr int S = GIVENS ? GL::kSlots : L::kSlots;
@@ -180,6 +199,11 @@ __device__ void fp64_shift(const FpSys& d, const int sh, cd* __restrict__ Z2,
   cd* __restrict__ xhat_copy = d.xhat_copy;
   const double* __restrict__ hnorm = d.hnorm;
   const int tid = threadIdx.x;
+  const int gt = tid + rank * NT, GT = team * NT;  // thread of the team
+  auto team_sync = [&] {
+    if (!GIVENS && team > 1) cluster_sync_all();
+    else __syncthreads();
+  };
   const int ldz = p + n;
   const bool track_t = RHS || (mode == SSV_XHAT || mode == SSV_X || xhat_copy != nullptr);
   cd* ZT = Z2 + (size_t)ldz * m;  // n x m, valid when track_t
@@ -205,7 +229,7 @@ __device__ void fp64_shift(const FpSys& d, const int sh, cd* __restrict__ Z2,
   // (with double-float bulk updates the working precision is 2^-47)
   const double sing_tol = (double)n * (DF ? 7.105427357601002e-15 : 2.220446049250313e-16) * sqrt(mnorm2);
   // ---- shift setup: Z2 = last m columns of [Ct; H] - sigma on the diagonal
-  for (long long idx = tid; idx < (long long)ldz * m; idx += NT) {
+  for (long long idx = gt; idx < (long long)ldz * m; idx += GT) {
     int i = (int)(idx % ldz), q = (int)(idx / ldz);
     int j = n - m + q;
     double v = i < p ? Ct[i + (size_t)j * ldct] : H[(i - p) + (size_t)j * n];
@@ -214,20 +238,20 @@ __device__ void fp64_shift(const FpSys& d, const int sh, cd* __restrict__ Z2,
     z2st(idx, z);
   }
   if (track_t) {
-    for (long long idx = tid; idx < (long long)n * m; idx += NT) {
+    for (long long idx = gt; idx < (long long)n * m; idx += GT) {
       int i = (int)(idx % n), q = (int)(idx / n);
       ZT[idx] = mkcd(i == n - m + q ? 1.0 : 0.0, 0.0);
     }
   }
   if (RHS) {
     const cd* rin = d.rhs + (size_t)sh * d.ldr;
-    for (int i = tid; i < n; i += NT) {
+    for (int i = gt; i < n; i += GT) {
       Zr[i] = rin[i];
       Tr[i] = mkcd(0.0, 0.0);
     }
   }
   if (tid == 0) s_sing = 0;
-  __syncthreads();
+  team_sync();
 
   // Deferred T rows (X-hat output without per-step T updates).  The rows of
   // the accumulated column transform T set at block step b are P1_b, and
@@ -364,7 +388,7 @@ __device__ void fp64_shift(const FpSys& d, const int sh, cd* __restrict__ Z2,
     };
     // Row i takes G lanes, lane g the columns q = g, g + G, ..: the row's old
     // entries are read by all of them before any is written (__syncwarp).
-    for (int i0 = 0; i0 < r; i0 += RPP) {
+    for (int i0 = rank * RPP; i0 < r; i0 += team * RPP) {
       const int i = i0 + ln.row;
       const int cd_ = i - (r - m);  // diagonal correction of fresh column cd_
       const bool live = i < r, diag = live && cd_ >= 0 && cd_ < min(m, nbe);
@@ -472,7 +496,7 @@ __device__ void fp64_shift(const FpSys& d, const int sh, cd* __restrict__ Z2,
         }
       }
     }
-    if (defer_t) {
+    if (defer_t && rank == 0) {
       // rows j0 .. j0+nbe-1: ZT = P1; P2 parked in the output (see above)
       for (int idx = tid; idx < nbe * m; idx += NT) {
         const int i = j0 + idx % nbe, q = idx / nbe;
@@ -482,10 +506,10 @@ __device__ void fp64_shift(const FpSys& d, const int sh, cd* __restrict__ Z2,
         const int qq = idx % m, q = idx / m;
         tout[(n - nsteps * m + qq) + (size_t)q * tld] = coefd(LB + qq, q);
       }
-    } else if (track_t) {
+    } else if (track_t && !defer_t) {
       // rows k-m .. n-1: ZT <- ZT P2 ; rows j0 .. j0+nbe-1: ZT = P1
       const int lo = k - m;
-      for (int i0 = j0; i0 < n; i0 += RPP) {
+      for (int i0 = j0 + rank * RPP; i0 < n; i0 += team * RPP) {
         const int i = i0 + ln.row;
         const bool live = i < n;
         cd acc[NS];
@@ -541,7 +565,7 @@ __device__ void fp64_shift(const FpSys& d, const int sh, cd* __restrict__ Z2,
         }
       }
     }
-    __syncthreads();
+    team_sync();
     k -= nbe;
   }
 
@@ -620,7 +644,7 @@ __device__ void fp64_shift(const FpSys& d, const int sh, cd* __restrict__ Z2,
   const bool sing = s_sing != 0;
   const double nanv = __longlong_as_double(0x7ff8000000000000LL);
   // ---- outputs
-  if (mode == SSV_G || mode == SSV_TF) {
+  if ((mode == SSV_G || mode == SSV_TF) && rank == 0) {
     const double sg = mode == SSV_TF ? -1.0 : 1.0;
     cd* o = out + (size_t)sh * nr * ldo;
     for (int idx = tid; idx < p * nr; idx += NT) {
@@ -631,7 +655,7 @@ __device__ void fp64_shift(const FpSys& d, const int sh, cd* __restrict__ Z2,
       o[i + (size_t)q * ldo] = mkcd(sg * acc.x, sg * acc.y);
     }
   }
-  if (defer_t) {
+  if (defer_t && rank == 0) {
     // backward pass: z = Y; per step b = B .. 1: X-hat rows of b = P1_b z,
     // then z = P2_b z; finally the initial live rows n-m .. n-1 take z
     cd* zs = reinterpret_cast<cd*>(smem_raw);  // m x m (ld MAXM); the panel's arrays are done with
@@ -667,7 +691,7 @@ __device__ void fp64_shift(const FpSys& d, const int sh, cd* __restrict__ Z2,
       const int rr = e % m, q = e / m;
       tout[(n - m + rr) + (size_t)q * tld] = sing ? mkcd(nanv, nanv) : zs[rr + q * MAXM];
     }
-  } else if (track_t) {
+  } else if (track_t && !defer_t) {
     cd* o;
     long long ld;
     if (mode == SSV_XHAT || mode == SSV_X) {
@@ -677,7 +701,7 @@ __device__ void fp64_shift(const FpSys& d, const int sh, cd* __restrict__ Z2,
       o = xhat_copy + (size_t)sh * nr * ldxc;
       ld = ldxc;
     }
-    for (int idx = tid; idx < n * nr; idx += NT) {
+    for (int idx = gt; idx < n * nr; idx += GT) {
       int i = idx % n, q = idx / n;
       cd acc = mkcd(0.0, 0.0);
       if (RHS) acc = mkcd(-Tr[i].x, -Tr[i].y);
@@ -686,7 +710,7 @@ __device__ void fp64_shift(const FpSys& d, const int sh, cd* __restrict__ Z2,
       o[(d.flip_out ? n - 1 - i : i) + (size_t)q * ld] = acc;
     }
   }
-  if (status != nullptr && tid == 0) {
+  if (status != nullptr && tid == 0 && rank == 0) {
     // a non-finite solution (NaN / Inf in the inputs or an overflow) is reported
     // as such, also when no separate scan of the outputs follows
     bool fin = true;
@@ -696,7 +720,7 @@ __device__ void fp64_shift(const FpSys& d, const int sh, cd* __restrict__ Z2,
     }
     status[sh] = sing ? SSV_SHIFT_SINGULAR : (fin ? SSV_SHIFT_OK : SSV_SHIFT_NONFINITE);
   }
-  __syncthreads();
+  team_sync();
 }
 
 // Non-finite scan: status[sh] = NONFINITE if an output of an OK shift is not finite.
