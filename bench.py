@@ -404,7 +404,7 @@ def tensor_residual_roofline(n, m, s, mixed):
     ms = mixed["phase_ms_per_step"].get("mixed_residual", float("nan"))
     peak, src = bf16_peak_sustained()
     ach = flops / (ms * 1e-3) / 1e12
-    return {"kernel": "tc_residual2_kernel (two shifts per item, + digit split of Xhat)", "bound": "tensor",
+    return {"kernel": "tc_residual_kernel (+ digit split of Xhat)", "bound": "tensor",
             "unit": "TFLOP/s", "achieved": ach, "peak": peak, "frac": ach / peak,
             "peak_source": src,
             "flops_per_pass": flops, "pass_ms": ms,
@@ -688,7 +688,7 @@ def main():
     ach_ti = instr / (sweep0_ms * 1e-3) / 1e12
     peak_ti = fp32_peak / 2.0
     roof_first = {
-        "kernel": "tcs_panel_kernel + tcs_update_kernel<true> (tensor-core sweep, first solve of "
+        "kernel": "tcs_panel_kernel + tcs_update_kernel (tensor-core sweep, first solve of "
                   "the mixed path; %d launches each)" % (len(range(0, n - m, 128)) or 1),
         "bound": "alu", "unit": "T FP32-instr/s (double-float equivalent)", "achieved": ach_ti,
         "peak": peak_ti, "frac": ach_ti / peak_ti,
@@ -710,8 +710,8 @@ def main():
     red_flops = 10.0 / 3.0 * n ** 3 - 4.5 * n * n * m
     red_ach = red_flops / (red_ms * 1e-3) / 1e12
     roof_reduce = {
-        "kernel": ("tensor-core reduction (panel_kernel, tc_gemm_kernel<16,9> / <32,9> / <64,8>, "
-                   "digit splits; about 1400 launches)" if red_tc else
+        "kernel": ("tensor-core reduction (panel_update_kernel, panel_qr_kernel, tc_gemm_kernel<16,9> / <32,9> / <64,8>, "
+                   "digit splits; about 1900 launches)" if red_tc else
                    "reduce_blocked_kernel (FP64 controller-Hessenberg reduction, one launch)"),
         "bound": "alu", "unit": "TFLOP/s (FP64-equivalent)", "achieved": red_ach, "peak": fp64_peak,
         "frac": red_ach / fp64_peak,
@@ -734,7 +734,7 @@ def main():
         upd_ms = upd_tot / upd_calls
         ach_u = upd_flops / upd_launches / (upd_ms * 1e-3) / 1e12
         roof_update = {
-            "kernel": "tcs_update_kernel<true> (tensor-core sweep trailing update, %d launches "
+            "kernel": "tcs_update_kernel (tensor-core sweep trailing update, %d launches "
                       "per solve)" % upd_launches,
             "bound": "tensor", "unit": "TFLOP/s", "achieved": ach_u, "peak": bf16_peak,
             "frac": ach_u / bf16_peak, "peak_source": bf16_src, "launch_ms": upd_ms,
