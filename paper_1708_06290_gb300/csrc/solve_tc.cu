@@ -86,11 +86,11 @@ constexpr int kStages = kNBT / kKS;  // stages per block step
 constexpr int kAT = kUM * kKS;       // BF16 elements of one H digit tile
 constexpr int kBT = kUN * kKS;       // BF16 elements of one P1 digit tile
 constexpr uint32_t kStageBytes = (uint32_t)(kSDH * kAT + kSD * kBT) * 2;  // H and P1 digit tiles
-constexpr int kWinCols = kLev * kUN;  // TMEM columns of an item; two items in flight
+constexpr int kWinCols = kLev * kUN;  // TMEM columns of a window; there are two
 // polls of one mbarrier wait before the update gives up (a stage's copies and
 // products complete within microseconds)
 constexpr long long kUpdWait = 1LL << 22;
-static_assert(2 * kWinCols == 512, "TMEM columns of the two items");
+static_assert(2 * kWinCols == 512, "TMEM columns of the two windows");
 // shared memory of the update: two stage buffers, then the Z2 and P2 digit tiles
 // of one item (S shifts: 7 digits of 128 x cs and of cs x cs; S cs = kUN)
 constexpr size_t kOffZ = 2 * (size_t)kStageBytes;
@@ -464,7 +464,8 @@ static __device__ __forceinline__ bool role_wait(uint32_t mbar, uint32_t parity,
 // the blocks running together share H's digit tiles; but where the groups' P1
 // digits (57 KB each) do not stay in L2, only as many groups at a time as blocks
 // run: theirs then stay while the rows go by.  2000 groups of 32 columns at n =
-// 5000: 93.3 ms in all one row block at a time, 87.8 in chunks; 250 groups at n =
+// 5000: 93.3 ms in all one row block at a time, 87.8 in chunks (before each product
+// had a window of its own); 250 groups at n =
 // 1000: a call of 7.97 ms one row block at a time, 8.25 in chunks.
 constexpr size_t kPGroupBytes = (size_t)kSD * kStages * kBT * 2;
 constexpr size_t kPKeep = (size_t)64 << 20;
@@ -483,23 +484,24 @@ static __device__ __forceinline__ void item_of(long long item, int RT, int G, in
 //   * a producer thread copies the K stages of Z1 P1 (H digit tiles x P1 digit
 //     tiles) into two stage buffers and, CS >= 16, the group's Z2 and P2 digit
 //     tiles into a third;
-//   * an issuing thread multiplies: item v's Z1 P1 into the eight levels of TMEM
-//     window v mod 2, then, once these are read, its Z2 P2 into seven levels of
-//     the same window, one item behind;
+//   * an issuing thread multiplies: Z1 P1 into the eight levels of the first TMEM
+//     window, Z2 P2 into the seven of the second, so that each window is read
+//     under the other's products (CS < 16: item v's Z1 P1 into window v mod 2);
 //   * two groups of eight warps take alternate items (thread = row, 16 columns):
 //     levels into double-float sums, scaling, the shifted-diagonal correction,
 //     and the new rows: as FP32 pairs the 128 that the next panel (or the final
 //     block) reads, all others as the digit tiles of the next block step (CS <
 //     16: Z2 P2 in double-float here, and every row as pairs).
 //
-// What bounds it, per item at CS = 32: the copies from L2 (392 KB, about 6.5 k
-// clocks), the epilogue's instructions (8.4 k issue slots a scheduler) and the
-// products (5.5 k clocks), which run side by side; DRAM 22 % busy.  Two epilogue
-// warps to a scheduler left it idle for 58 % of the clocks; with four, the update
-// of 600 shifts at n = 2500, m = 8 takes 4.29 ms (4.69), of 2000 at n = 1000, m = 4
-// 0.93 ms (1.30).  One item at a time, each phase after the other, took 6.0 ms a
-// launch at the start of the sweep of 2000 shifts at n = 5000, m = 16 (114 ms for
-// the 39 launches, now 87.8).
+// What bounds it, per item at CS = 32: the products with their shared-memory
+// traffic (about 10 k clocks), the epilogue's instructions (8.4 k issue slots a
+// scheduler) and the copies from L2 (392 KB, 6.5 k clocks), which run side by side;
+// DRAM 28 % busy.  Measured steps, the sweep of 2000 shifts at n = 5000, m = 16 (39
+// launches) and of 600 at n = 2500, m = 8 (20): one item at a time, each phase after
+// the other 114 ms; roles, and the two products of an item in one window, which the
+// issuer waited 5 k of 18 k clocks an item to have read 93 and 4.7; sixteen epilogue
+// warps (eight left a scheduler idle for 58 % of the clocks) and the order of items
+// 87.8 and 4.29; a window for each product 79.5 and 3.55.
 template <int CS>
 __global__ void __launch_bounds__(kUT, 1) tcs_update_kernel(TcsArgs a, int k, int nbe) {
   constexpr bool TCZ = CS >= 16;
@@ -525,8 +527,8 @@ __global__ void __launch_bounds__(kUT, 1) tcs_update_kernel(TcsArgs a, int k, in
   const int nst = (nbe + kKS - 1) / kKS;
   const int JH0 = j0 / kKS;
   // full / empty[2]: a stage buffer copied / multiplied; zfull / zempty: the Z2
-  // buffer; pfull / pread[2]: window's Z1 P1 levels complete / read; qfull /
-  // qread[2]: its Z2 P2 levels
+  // buffer; pfull / pread[2]: the Z1 P1 levels of group h's item complete / read;
+  // qfull / qread[2]: its Z2 P2 levels
   const uint32_t full = smem_addr(mbar), empty = full + 16, zfull = full + 32, zempty = full + 40;
   const uint32_t pfull = full + 48, pread = full + 64, qfull = full + 80, qread = full + 96;
   const uint32_t sBase = smem_addr(smem), sZ = sBase + (uint32_t)kOffZ;
@@ -560,12 +562,12 @@ __global__ void __launch_bounds__(kUT, 1) tcs_update_kernel(TcsArgs a, int k, in
       // ---- producer
       unsigned i = 0;
       bool ok = true;
-      auto stages = [&](long long v) {
+      auto stages = [&](long long v, int s0, int s1) {
         const long long item = blockIdx.x + v * gridDim.x;
         int I, g;
         item_of(item, RT, G, I, g);
         const size_t Pg0 = (size_t)g * kSD * kStages * kBT;
-        for (int st = 0; st < nst && ok; ++st, ++i) {
+        for (int st = s0; st < s1 && ok; ++st, ++i) {
           const uint32_t b = i & 1u;
           if (!role_wait(empty + 8u * b, ((i >> 1) & 1u) ^ 1u, &fail)) {
             ok = false;
@@ -605,10 +607,12 @@ __global__ void __launch_bounds__(kUT, 1) tcs_update_kernel(TcsArgs a, int k, in
         }
         issued[2] = (int)(v + 1);
       };
-      // in the issuer's order: Z1 P1 of item v + 1 before Z2 P2 of item v
-      for (long long v = 0; v < mine + (TCZ ? 1 : 0) && ok; ++v) {
-        if (v < mine) stages(v);
-        if (TCZ && v > 0 && ok) ztiles(v - 1);
+      // both stage buffers first: they fill under the last item's Z2 P2
+      const int first = min(2, nst);
+      for (long long v = 0; v < mine && ok; ++v) {
+        stages(v, 0, first);
+        if (TCZ && ok) ztiles(v);
+        stages(v, first, nst);
       }
     }
   } else if (warp == 2 * kUG / 32 + 1) {
@@ -616,14 +620,18 @@ __global__ void __launch_bounds__(kUT, 1) tcs_update_kernel(TcsArgs a, int k, in
       // ---- issuer
       unsigned i = 0;
       bool ok = true;
+      // the group of item v has read its window
+      auto read_of = [&](uint32_t bars, long long v) {
+        return role_wait(bars + 8u * ((unsigned)v & 1u), (unsigned)(v >> 1) & 1u, &fail);
+      };
       // fused levels: the P1 digit tiles sit side by side (kUN rows each), so one
       // product of H digit kd against P1 digits 0 .. c - 1 (N = kUN c) lands digit
       // b in level kd + b.  The first products of an item open the levels: those
       // of kd = 0 levels 0 .. 6, digit 6 of kd = 1 level 7.
       auto z1p1 = [&](long long v) {
         const uint32_t h = (unsigned)v & 1u, u = (unsigned)(v >> 1);
-        const uint32_t d = tmem + h * (uint32_t)kWinCols;
-        if (!role_wait((TCZ ? qread : pread) + 8u * h, (u & 1u) ^ 1u, &fail)) ok = false;
+        const uint32_t d = tmem + (TCZ ? 0u : h * (uint32_t)kWinCols);
+        if (TCZ ? v > 0 && !read_of(pread, v - 1) : !role_wait(pread + 8u * h, (u & 1u) ^ 1u, &fail)) ok = false;
         for (int st = 0; st < nst && ok; ++st, ++i) {
           const uint32_t b = i & 1u;
           if (!role_wait(full + 8u * b, (i >> 1) & 1u, &fail)) {
@@ -661,12 +669,12 @@ __global__ void __launch_bounds__(kUT, 1) tcs_update_kernel(TcsArgs a, int k, in
       // P2 digit tiles (CS rows each) are stacked: one product of Z2 digit kd
       // against P2 digits 0 .. 6 - kd lands digit ld in level kd + ld
       auto z2p2 = [&](long long v) {
-        const uint32_t h = (unsigned)v & 1u, u = (unsigned)(v >> 1);
-        const uint32_t d = tmem + h * (uint32_t)kWinCols;
+        const uint32_t h = (unsigned)v & 1u;
+        const uint32_t d = tmem + (uint32_t)kWinCols;
         int I, g;
         item_of(blockIdx.x + v * gridDim.x, RT, G, I, g);
         const int nsh = min(S, a.s - g * S);
-        if (!role_wait(pread + 8u * h, u & 1u, &fail) || !role_wait(zfull, (unsigned)v & 1u, &fail)) {
+        if ((v > 0 && !read_of(qread, v - 1)) || !role_wait(zfull, (unsigned)v & 1u, &fail)) {
           ok = false;
           return;
         }
@@ -690,9 +698,9 @@ __global__ void __launch_bounds__(kUT, 1) tcs_update_kernel(TcsArgs a, int k, in
         mma_commit(qfull + 8u * h);
         issued[3] = (int)(v + 1);
       };
-      for (long long v = 0; v < mine + (TCZ ? 1 : 0) && ok; ++v) {
-        if (v < mine) z1p1(v);
-        if (TCZ && v > 0 && ok) z2p2(v - 1);
+      for (long long v = 0; v < mine && ok; ++v) {
+        z1p1(v);
+        if (TCZ && ok) z2p2(v);
       }
     }
   } else {
@@ -701,7 +709,7 @@ __global__ void __launch_bounds__(kUT, 1) tcs_update_kernel(TcsArgs a, int k, in
     const uint32_t h = (uint32_t)(warp / (kUG / 32));
     const int hf = (warp >> 2) & 1, cb = kUH * hf;  // its first column
     const int row = tid & (kUM - 1);
-    const uint32_t tl = tmem + h * (uint32_t)kWinCols + ((uint32_t)((warp & 3) * 32) << 16);
+    const uint32_t tl = tmem + (TCZ ? 0u : h * (uint32_t)kWinCols) + ((uint32_t)((warp & 3) * 32) << 16);
     // shifts of this half: lb .. lb + SH - 1 of the group
     constexpr int SH = CS >= kUH ? 1 : kUH / CS, CL = CS < kUH ? CS : kUH;  // CL: columns of a shift here
     const int lb = cb / CS, cz = cb % CS;  // cz: the first one's first column within its shift
@@ -771,7 +779,7 @@ __global__ void __launch_bounds__(kUT, 1) tcs_update_kernel(TcsArgs a, int k, in
         if (!__all_sync(0xffffffffu, role_wait(qfull + 8u * h, par, &fail))) break;
         fence_after();
         // shift l's levels start at column 7 CS l
-        const uint32_t tz = tl + (uint32_t)(7 * CS * lb + cz);
+        const uint32_t tz = tl + (uint32_t)(kWinCols + 7 * CS * lb + cz);
         if (fast) {
           float f[kUH];
 #pragma unroll
