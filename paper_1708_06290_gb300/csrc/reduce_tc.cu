@@ -1658,8 +1658,9 @@ size_t qtc_layout(int n, int nc, unsigned char* base, QtcScratch* Q) {
 }  // namespace
 
 // Where the digit products win over the FP64 pipe: that path grows with n^2 ncols,
-// this one up to some 256 columns with the number of blocks alone (2.1 us a
-// reflector before its sums were read in one trip).  FP64 / digit products measured
+// this one up to some 256 columns with the number of blocks alone.  Measured when a
+// block of 128 took 270 us (now some 170, so the line errs towards the FP64 pipe),
+// FP64 / digit products
 // at n ncols = 262144: n = 1024, 256 columns 1.99 / 2.09 ms; n = 2048, 128 columns
 // 5.1 / 4.2; n = 4096, 64 columns 13.2 / 8.9; below: n = 1536, 128 columns 3.0 / 3.2;
 // n = 384, 640 columns 0.96 / 0.99; far above, n = 4096, 640 columns 82.7 / 15.2.
