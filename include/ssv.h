@@ -362,7 +362,7 @@ int ssv_solve_noalloc(ssv_handle h, int s, const double* shifts, const ssv_opts*
 /*
  * ssv_apply_q -- X = Q Xhat (Sec. 2: X = Q Xhat in original coordinates).
  *   Xhat (device, complex) n x ncols, ldx >= n; X (device, complex) n x ncols,
- *   ldX >= n.  X may equal Xhat (in place).  Wide X (n ncols >= 275000) is
+ *   ldX >= n.  X may equal Xhat (in place).  Wide X (n ncols >= 180000) is
  *   formed by FP64-accurate digit products on the tensor cores, which take
  *   scratch from the pool; without room for it, and in ssv_solve's SSV_X with
  *   SSV_FP64, on the FP64 pipe.

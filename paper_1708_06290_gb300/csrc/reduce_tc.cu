@@ -1658,13 +1658,12 @@ size_t qtc_layout(int n, int nc, unsigned char* base, QtcScratch* Q) {
 }  // namespace
 
 // Where the digit products win over the FP64 pipe: that path grows with n^2 ncols,
-// this one up to some 256 columns with the number of blocks alone.  Measured when a
-// block of 128 took 270 us (now some 170, so the line errs towards the FP64 pipe),
-// FP64 / digit products
-// at n ncols = 262144: n = 1024, 256 columns 1.99 / 2.09 ms; n = 2048, 128 columns
-// 5.1 / 4.2; n = 4096, 64 columns 13.2 / 8.9; below: n = 1536, 128 columns 3.0 / 3.2;
-// n = 384, 640 columns 0.96 / 0.99; far above, n = 4096, 640 columns 82.7 / 15.2.
-bool apply_q_tc_supported(int n, int ncols) { return n >= 384 && (long long)n * ncols >= 275000; }
+// this one up to some 256 columns with the number of blocks alone (150 us each).
+// FP64 / digit products in ms, near the line: n = 256, 640 columns 0.51 / 0.45; n =
+// 384, 450 columns 0.52 / 0.53; n = 768, 256 columns 1.21 / 0.94; n = 2048, 64 columns
+// 2.98 / 2.42; below: n = 512, 256 columns 0.62 / 0.65; n = 256, 450 columns 0.28 / 0.39;
+// far above: n = 4096, 640 columns 82.1 / 8.9.
+bool apply_q_tc_supported(int n, int ncols) { return n >= 256 && (long long)n * ncols >= 180000; }
 
 size_t apply_q_tc_scratch_bytes(int n, int ncols) {
   return apply_q_tc_supported(n, ncols) ? qtc_layout(n, std::min(ncols, kQCols), nullptr, nullptr) : 0;

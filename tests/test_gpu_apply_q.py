@@ -22,7 +22,7 @@ pytestmark = pytest.mark.gpu
                                            (65, 40, 2, 3), (300, 5, 40, 0), (300, 3, 153, 0), (290, 16, 305, 7),
                                            (1100, 4, 24, 0), (2300, 2, 2, 5), (700, 8, 620, 0),
                                            # wide: digit products on the tensor cores
-                                           (384, 1, 720, 0), (769, 3, 365, 2), (1153, 130, 240, 0),
+                                           (256, 4, 704, 0), (384, 1, 720, 0), (769, 3, 365, 2), (1153, 130, 240, 0),
                                            (800, 2, 1100, 1), (1500, 16, 330, 0)])
 def test_apply_q_definition(n, m, ncols, pad):
     from paper_1708_06290_gb300 import ssv
