@@ -84,11 +84,11 @@ int launch_solve(const Handle* h, int s, const double* shifts, int nb, int mode,
 
 // Default block width of the FP64 sweep: n_b = 128 halves the per-shift
 // Z2 P2 work of n_b = 64 at the price of a longer panel (measured 9 % faster
-// at n = 5000, m = 16); small problems keep 64 (n = 1000, 64 / 128: m = 4 8.67 / 8.65
-// ms, m = 16 17.7 / 17.7).  Double-float, whose panel is cheaper beside its
-// updates, takes 128 from n = 256 on (n = 1000: m = 4 6.10 / 5.78, m = 16 7.27 / 6.68;
-// n = 256, m = 8 0.807 / 0.775).
-int default_nb(int n, int prec) { return n >= (prec == SSV_DFLOAT ? 256 : 1024) ? 128 : 64; }
+// at n = 5000, m = 16); small problems keep 64.
+int default_nb(int n, int m) {
+  (void)m;
+  return n >= 1024 ? 128 : 64;
+}
 
 // Work list of the shifts with mask[j] != 0 (single block, order preserved).
 __global__ void __launch_bounds__(1024) mask_to_list_kernel(int s, const int* __restrict__ mask,
@@ -118,7 +118,7 @@ int solve_fp64_masked(const Handle* h, int s, const double* shifts, int mode, in
                       double* out, long long ldo, int* status, const int* mask, void* xhat_copy,
                       long long ldxc, cudaStream_t st) {
   const int m = h->m;
-  if (nb <= 0) nb = default_nb(h->n, SSV_FP64);
+  if (nb <= 0) nb = default_nb(h->n, m);
   if (nb > kNB) return SSV_ENOTSUP;
   if (s == 0) return SSV_OK;
   int* list = nullptr;
@@ -343,7 +343,7 @@ std::map<TuneKey, int> g_tune;
 int tuned_nb(int n, int m, int p, int prec, int mode) {
   std::lock_guard<std::mutex> lk(g_tune_mu);
   auto it = g_tune.find(TuneKey{n, m, p, prec, mode});
-  return it == g_tune.end() ? default_nb(n, prec) : it->second;
+  return it == g_tune.end() ? default_nb(n, m) : it->second;
 }
 
 int autotune_nb(const Handle* h, int s, const double* shifts, const ssv_opts* o, double* out,
@@ -354,7 +354,7 @@ int autotune_nb(const Handle* h, int s, const double* shifts, const ssv_opts* o,
   cudaEvent_t e0, e1;
   SSV_CUDA_TRY(cudaEventCreate(&e0));
   SSV_CUDA_TRY(cudaEventCreate(&e1));
-  int best = default_nb(h->n, o->precision);
+  int best = default_nb(h->n, h->m);
   float bms = 1e30f;
   int rc = SSV_OK;
   for (int ci = 0; ci < 5; ++ci) {

@@ -200,7 +200,7 @@ int solve_fp64_noalloc(const Handle* h, int s, const double* shifts, const ssv_o
                        double* out, long long ldo, int* status, cudaStream_t st);
 size_t noalloc_scratch_bytes();
 
-int default_nb(int n, int prec);
+int default_nb(int n, int m);
 int num_sms();
 
 // batched multi-system FP64 solve (solve_fp64.cu)
