@@ -28,12 +28,12 @@
 //     BF16 x BF16 -> FP32, M = 128, K = 16) of H digit a against Xhat digits
 //     0 .. 7 - a (N = 32 (8 - a) columns) lands digit b in level a + b; every
 //     fourth stage completes a window;
-//   * four warps read a finished window's levels back (tcgen05.ld) and add
+//   * eight warps read a finished window's levels back (tcgen05.ld) and add
 //     them, scaled by 2^{-7t}, into double-float sums while the other window
 //     multiplies; after an item's last window they form E in FP64.
-// What bounds it: the stage copies from L2 (80 KB a stage) and the products
-// (36 x 32 columns) take about the same time, 1.2 k clocks a stage; the readout
-// of a window (2.2 k clocks of FP32) hides under the next one's products.
+// What bounds it: shared memory, which takes a stage's 80 KB and gives 138 KB to
+// the products (1.7 k clocks of its bandwidth; the products themselves 1.2 k, 2.6 k
+// measured); the readout of a window hides under the next one's products.
 #include <algorithm>
 
 #include "cluster.cuh"

@@ -84,7 +84,11 @@ int launch_solve(const Handle* h, int s, const double* shifts, int nb, int mode,
 
 // Default block width of the FP64 sweep: n_b = 128 halves the per-shift
 // Z2 P2 work of n_b = 64 at the price of a longer panel (measured 9 % faster
-// at n = 5000, m = 16); small problems keep 64.
+// at n = 5000, m = 16); small problems keep 64 (n = 1000, FP64, 64 / 128: m = 4 8.67
+// / 8.65 ms, m = 16 17.7 / 17.7).  Double-float sweeps keep it too: 128 rows are 3 to
+// 8 % faster at n = 256 .. 1000, but sum twice as many products per update, and the
+// error of Xhat grows from 1.9e-14 to 3.4e-14 at n = 600, m = 4 and from 2.4e-14 to
+// 4.0e-14 at m = 8 (geometric mean over 120 shifts).
 int default_nb(int n, int m) {
   (void)m;
   return n >= 1024 ? 128 : 64;
