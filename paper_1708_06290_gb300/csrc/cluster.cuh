@@ -34,15 +34,21 @@ static __device__ __forceinline__ void cluster_st(double* p, int rank, double v)
   asm volatile("st.shared::cluster.f64 [%0], %1;" ::"r"(cluster_map(p, rank)), "d"(v) : "memory");
 }
 
-// launch `grid` blocks in clusters of R (grid a multiple of R;
-// R > 8 needs cudaFuncAttributeNonPortableClusterSizeAllowed set on the kernel)
+// The most dynamic shared memory a kernel is ever launched with.  The limit belongs
+// to the kernel on the device, not to a launch, and is shared by all host threads:
+// set to the size of one launch, it can fall below the size of another thread's
+// launch before that one is made.  So always the same value for a kernel.
+template <typename... KArgs>
+cudaError_t allow_smem(void (*kern)(KArgs...), size_t most) {
+  return cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)most);
+}
+
+// launch `grid` blocks in clusters of R (grid a multiple of R; R > 8 needs
+// cudaFuncAttributeNonPortableClusterSizeAllowed set on the kernel, smem beyond
+// 48 KB allow_smem)
 template <typename... KArgs, typename... Args>
 cudaError_t launch_cluster(void (*kern)(KArgs...), int grid, int threads, int R, size_t smem, cudaStream_t st,
                            Args... args) {
-  cudaError_t e = cudaSuccess;
-  if (smem > 48 * 1024)
-    e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-  if (e != cudaSuccess) return e;
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3((unsigned)grid);
   cfg.blockDim = dim3((unsigned)threads);
@@ -55,7 +61,7 @@ cudaError_t launch_cluster(void (*kern)(KArgs...), int grid, int threads, int R,
   at[0].val.clusterDim.z = 1;
   cfg.attrs = at;
   cfg.numAttrs = 1;
-  e = cudaLaunchKernelEx(&cfg, kern, args...);
+  const cudaError_t e = cudaLaunchKernelEx(&cfg, kern, args...);
   if (e == cudaSuccess) count_launch();
   return e;
 }

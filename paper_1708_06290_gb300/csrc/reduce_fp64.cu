@@ -295,7 +295,8 @@ template <int CC>
 cudaError_t launch_apply_q(const QSrc& q, int R, const double* T, cd* X, long long ldx, int ncols,
                            cudaStream_t st) {
   const int grid = (ncols + CC - 1) / CC * R;
-  return launch_cluster(apply_q_kernel<CC>, grid, kQT, R, q_apply_smem<CC>(), st, q, R, T, X, ldx, ncols);
+  const cudaError_t e = allow_smem(apply_q_kernel<CC>, q_apply_smem<CC>());
+  return e != cudaSuccess ? e : launch_cluster(apply_q_kernel<CC>, grid, kQT, R, q_apply_smem<CC>(), st, q, R, T, X, ldx, ncols);
 }
 
 __global__ void copy_masked_kernel(const double* __restrict__ src, long long lds, int rows, int cols,
@@ -359,6 +360,7 @@ static int make_q_t(Handle* h, cudaStream_t st) {
   const int nblk = q_blocks(h->kb) + q_blocks(h->ka);
   if (nblk == 0) return SSV_OK;
   constexpr int kR = 4;
+  SSV_CUDA_TRY(allow_smem(q_t_kernel, kQTSmem));
   SSV_CUDA_TRY(launch_cluster(q_t_kernel, nblk * kR, kQT, kR, kQTSmem, st, q_src(h), kR, h->Tq));
   return SSV_OK;
 }

@@ -582,6 +582,7 @@ constexpr int kRedZ = 4096;              // Z = T^T W
 constexpr int kRedTotal = 8192;
 constexpr size_t kPanFixed = 4096 + 4096;  // doubles besides the panel
 constexpr size_t kPanSmem = 200 * 1024;  // with the staged rows of V and Y at most
+static_assert(sizeof(double) * (kPanRowsW + kPanFixed) <= kPanSmem, "a panel without the staged rows");
 
 struct PanArgs {
   double* P;          // panel column t, matrix row r: P[r + t * ldp]
@@ -957,6 +958,7 @@ struct YfixArgs {
   int* err;
 };
 __host__ __device__ constexpr int yfix_rows(int wp) { return wp <= 16 ? 16 : 256 / wp; }
+constexpr size_t kYfixSmem = sizeof(double) * ((size_t)kBmax * kMaxW + 256);
 
 __global__ void __launch_bounds__(256) yfix_kernel(YfixArgs a) {
   extern __shared__ double ysm[];
@@ -1261,7 +1263,7 @@ int run_panel(RtcScratch& S, int n, int p, double* P, size_t np, long long ldp, 
     const size_t rows = sizeof(double) * 2 * (size_t)rpc * j;
     a.staged = smem + rows <= kPanSmem ? 1 : 0;
     if (a.staged) smem += rows;
-    SSV_CUDA_TRY(cudaFuncSetAttribute(panel_update_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    SSV_CUDA_TRY(allow_smem(panel_update_kernel, kPanSmem));
     void* args[] = {&a};
     SSV_CUDA_TRY(cudaLaunchCooperativeKernel((const void*)panel_update_kernel, dim3(G), dim3(kPT), args, smem, st));
     count_launch();
@@ -1289,6 +1291,7 @@ int run_panel(RtcScratch& S, int n, int p, double* P, size_t np, long long ldp, 
     a.np = np;
     a.nv = S.nV;
     a.ntau = ntau;
+    SSV_CUDA_TRY(allow_smem(panel_qr_kernel, kQrSmem));
     SSV_CUDA_TRY(launch_cluster(panel_qr_kernel, a.cs, kQrT, a.cs, sizeof(double) * kQrFixed + (a.insm ? rows : 0),
                                 st, a));
   }
@@ -1326,7 +1329,7 @@ int run_panel(RtcScratch& S, int n, int p, double* P, size_t np, long long ldp, 
   y.err = err;
   const int R = yfix_rows(wp);
   const size_t ysm = sizeof(double) * ((size_t)(j + wp) * wp + 256);
-  SSV_CUDA_TRY(cudaFuncSetAttribute(yfix_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)ysm));
+  SSV_CUDA_TRY(allow_smem(yfix_kernel, kYfixSmem));
   yfix_kernel<<<(rowsE + R - 1) / R + (j + wp + R - 1) / R, 256, ysm, st>>>(y);
   count_launch();
   SSV_CUDA_TRY(cudaGetLastError());
@@ -1392,7 +1395,7 @@ int qr_cluster() {
   cfg.dynamicSmemBytes = kQrSmem;
   cfg.attrs = at;
   cfg.numAttrs = 1;
-  if (cudaFuncSetAttribute(panel_qr_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kQrSmem) == cudaSuccess &&
+  if (allow_smem(panel_qr_kernel, kQrSmem) == cudaSuccess &&
       cudaFuncSetAttribute(panel_qr_kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) == cudaSuccess &&
       cudaOccupancyMaxActiveClusters(&nc, panel_qr_kernel, &cfg) == cudaSuccess && nc > 0)
     return kQrC;
