@@ -86,7 +86,14 @@ extern "C" {
 #define SSV_G 0    /* out(p x m) = C X = Ct Xhat                             */
 #define SSV_TF 1   /* out(p x m) = C (sigma I - A)^{-1} B = -Ct Xhat (Sec. 2) */
 #define SSV_XHAT 2 /* out(n x m) = Xhat = (H - sigma I)^{-1} R                */
-#define SSV_X 3    /* out(n x m) = X = Q Xhat = (A - sigma I)^{-1} B          */
+#define SSV_X 3    /* out(n x m) = X = Q Xhat = (A - sigma I)^{-1} B.  The
+                      product is formed in FP64 with SSV_FP64.  With the other
+                      precisions wide X (n >= 256, n s m >= 180000) is formed by
+                      digit products on the tensor cores that hold 56 bits below
+                      the largest entry of a column: FP64-accurate in the norm of
+                      each column, not entry by entry where a column is graded
+                      and Q couples its parts weakly.  Without room for their
+                      scratch (ssv_footprint counts it) in FP64. */
 
 /* first solve of the mixed path (ssv_opts.first) */
 #define SSV_FIRST_DFLOAT 0 /* double-float sweep (about 48 bits): refinement usually
@@ -362,10 +369,8 @@ int ssv_solve_noalloc(ssv_handle h, int s, const double* shifts, const ssv_opts*
 /*
  * ssv_apply_q -- X = Q Xhat (Sec. 2: X = Q Xhat in original coordinates).
  *   Xhat (device, complex) n x ncols, ldx >= n; X (device, complex) n x ncols,
- *   ldX >= n.  X may equal Xhat (in place).  Wide X (n ncols >= 180000) is
- *   formed by FP64-accurate digit products on the tensor cores, which take
- *   scratch from the pool; without room for it, and in ssv_solve's SSV_X with
- *   SSV_FP64, on the FP64 pipe.
+ *   ldX >= n.  X may equal Xhat (in place).  Formed in FP64, on the FP64 pipe,
+ *   without scratch.
  */
 int ssv_apply_q(ssv_handle h, int ncols, const double* Xhat, long long ldx, double* X,
                 long long ldX, void* stream);

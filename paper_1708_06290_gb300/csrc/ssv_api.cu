@@ -489,7 +489,9 @@ int ssv_apply_q(ssv_handle hh, int ncols, const double* Xhat, long long ldx, dou
   if (ncols == 0) return SSV_OK;
   if (!Xhat || !X || ldx < h->n || ldX < h->n) return SSV_EINVAL;
   if (!h->has_q) return SSV_ENOTSUP;
-  return apply_q(h, ncols, Xhat, ldx, X, ldX, true, (cudaStream_t)stream);
+  // FP64 throughout: the digit products hold a column relative to its largest entry,
+  // which a caller of this function cannot choose (of ssv_solve's precisions, it can)
+  return apply_q(h, ncols, Xhat, ldx, X, ldX, false, (cudaStream_t)stream);
 }
 
 int ssv_get_reduced(ssv_handle hh, double* H, long long ldh, double* R, long long ldr, double* Ct,

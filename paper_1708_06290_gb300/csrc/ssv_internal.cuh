@@ -111,7 +111,8 @@ int reduce_fp64(Handle* h, const double* A, long long lda, const double* B, long
                 const double* C, long long ldc, int arith, cudaStream_t st);
 // back-transform X = Q Xhat (reduce_fp64.cu)
 size_t q_t_count(int n, int m);
-// X = Q Xhat; digits: many columns may go through apply_q_tc
+// X = Q Xhat; digits: many columns may go through apply_q_tc, which keeps the norm of
+// a column to FP64 accuracy, not its small entries
 int apply_q(const Handle* h, int ncols, const double* Xhat, long long ldx, double* X, long long ldX,
             bool digits, cudaStream_t st);
 // the same for many columns, with digit products on the tensor cores (reduce_tc.cu)
