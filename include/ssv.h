@@ -184,6 +184,8 @@ int ssv_reduce_arith(int n, int m, int p, const double* A, long long lda, const 
  *   resid (device, may be NULL): s doubles, the normwise backward error
  *     ||(H - sigma I) Xhat - R||_F / (||H - sigma I||_F ||Xhat||_F + ||R||_F)
  *     of each shift's computed Xhat.
+ * A bounded wait for the tensor cores that gives up makes the results it concerns
+ * NaN: their shifts are reported SSV_SHIFT_NONFINITE, their backward errors NaN.
  * The handle is read only; concurrent calls on one handle from different
  * streams are safe (each call allocates its own stream-ordered scratch).
  * Errors: SSV_EINVAL, SSV_ENOTSUP, SSV_ENOMEM, SSV_ECUDA.
@@ -464,6 +466,16 @@ int ssv_trace_read(int max, char* names, int name_len, float* total_ms, int* cal
  * SSV_ETIMEOUT when the timeout path works (the device stays usable), SSV_OK
  * if it did not trigger, SSV_EINVAL / SSV_ECUDA on errors.  Synchronises. */
 int ssv_selftest_barrier(long long spin_limit, void* stream);
+
+/* Self-test of the wide back-transform's failure report (the paper has no
+ * counterpart): X = Q X in place for s shifts of m columns by the digit products
+ * of SSV_X, with the error word that a wait for the tensor cores raises when it
+ * gives up set beforehand if gave_up != 0: then every entry of X is NaN, statuses
+ * SSV_SHIFT_OK become SSV_SHIFT_NONFINITE and backward errors NaN (either may be
+ * NULL), as ssv_solve reports it.  Errors: SSV_EINVAL, SSV_ENOTSUP (no Q, or X
+ * too narrow for that path), SSV_ENOMEM, SSV_ECUDA. */
+int ssv_selftest_backtransform(ssv_handle h, int s, int gave_up, double* X, long long ldX, int* status,
+                               double* resid, void* stream);
 
 /* Arithmetic peak probe (measurement aid; the paper has no counterpart):
  * runs independent fused multiply-add chains on every SM of the current

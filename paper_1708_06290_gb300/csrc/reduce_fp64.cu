@@ -392,7 +392,7 @@ int reduce_fp64(Handle* h, const double* A, long long lda, const double* B, long
 }
 
 int apply_q(const Handle* h, int ncols, const double* Xhat, long long ldx, double* X, long long ldX,
-            bool digits, cudaStream_t st) {
+            bool digits, cudaStream_t st, int* status, double* resid) {
   const int n = h->n;
   if (ncols == 0) return SSV_OK;
   cd* Xc = reinterpret_cast<cd*>(X);
@@ -406,7 +406,7 @@ int apply_q(const Handle* h, int ncols, const double* Xhat, long long ldx, doubl
   const int nblk = q_blocks(h->kb) + q_blocks(h->ka);
   if (nblk == 0) return SSV_OK;
   if (digits && apply_q_tc_supported(h->n, ncols)) {
-    const int rc = apply_q_tc(h, ncols, Xc, ldX, st);
+    const int rc = apply_q_tc(h, ncols, Xc, ldX, st, status, resid);
     if (rc != SSV_ENOMEM) return rc;
     cudaGetLastError();  // no room for its scratch (nothing written yet): the FP64 path needs none
   }

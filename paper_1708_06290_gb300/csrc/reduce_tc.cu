@@ -1606,10 +1606,15 @@ __global__ void __launch_bounds__(256) qz_kernel(const double* __restrict__ Wp, 
   }
 }
 
-// every entry NaN when a wait gave up
-__global__ void q_fail_kernel(const int* err, cd* X, long long ldx, int n, int ncols) {
+// when a wait gave up: every entry NaN, and the shifts (m columns each) so reported
+__global__ void q_fail_kernel(const int* err, cd* X, long long ldx, int n, int ncols, int m, int* status,
+                              double* resid) {
   if (*err == 0) return;
   const double nanv = __longlong_as_double(0x7ff8000000000000LL);
+  for (int sh = blockIdx.x * blockDim.x + threadIdx.x; sh < ncols / m; sh += gridDim.x * blockDim.x) {
+    if (status != nullptr && status[sh] == SSV_SHIFT_OK) status[sh] = SSV_SHIFT_NONFINITE;
+    if (resid != nullptr) resid[sh] = nanv;
+  }
   for (long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x; e < (long long)n * ncols;
        e += (long long)gridDim.x * blockDim.x)
     X[e % n + (size_t)(e / n) * ldx] = mkcd(nanv, nanv);
@@ -1672,7 +1677,8 @@ size_t apply_q_tc_scratch_bytes(int n, int ncols) {
   return apply_q_tc_supported(n, ncols) ? qtc_layout(n, std::min(ncols, kQCols), nullptr, nullptr) : 0;
 }
 
-int apply_q_tc(const Handle* h, int ncols, cd* X, long long ldX, cudaStream_t st) {
+int apply_q_tc(const Handle* h, int ncols, cd* X, long long ldX, cudaStream_t st, int* status, double* resid,
+               int err0) {
   const int n = h->n, m = h->m, sms = std::max(1, num_sms());
   const int ncm = std::min(ncols, kQCols);
   unsigned char* base = nullptr;
@@ -1690,7 +1696,7 @@ int apply_q_tc(const Handle* h, int ncols, cd* X, long long ldX, cudaStream_t st
       rc = SSV_ECUDA;
     }
   };
-  cu(cudaMemsetAsync(Q.err, 0, sizeof(int), st));
+  cu(cudaMemsetAsync(Q.err, err0, sizeof(int), st));
   cu(cudaFuncSetAttribute(qz_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
                           (int)(sizeof(double) * kBmax * kBmax)));
   const int nbA = (h->ka + kBmax - 1) / kBmax, nbB = (h->kb + kBmax - 1) / kBmax;
@@ -1751,7 +1757,7 @@ int apply_q_tc(const Handle* h, int ncols, cd* X, long long ldX, cudaStream_t st
     }
   }
   if (rc == SSV_OK) {
-    q_fail_kernel<<<256, 256, 0, st>>>(Q.err, X, ldX, n, ncols);
+    q_fail_kernel<<<256, 256, 0, st>>>(Q.err, X, ldX, n, ncols, m, status, resid);
     count_launch();
     cu(cudaGetLastError());
   }

@@ -264,7 +264,8 @@ int ssv_solve(ssv_handle hh, int s, const double* shifts, const ssv_opts* o_in, 
     rc = solve_fp64(h, s, shifts, &o, out, ldo, status, resid, st);
     trace_end(tr, st);
   }
-  if (rc == SSV_OK && o.mode == SSV_X) rc = apply_q(h, s * h->m, out, ldo, out, ldo, o.precision != SSV_FP64, st);
+  if (rc == SSV_OK && o.mode == SSV_X)
+    rc = apply_q(h, s * h->m, out, ldo, out, ldo, o.precision != SSV_FP64, st, status, resid);
   return rc;
 }
 
@@ -579,6 +580,15 @@ long long ssv_kernel_launches(void) { return g_launches.load(std::memory_order_r
 int ssv_selftest_barrier(long long spin_limit, void* stream) {
   if (spin_limit < 1) return SSV_EINVAL;
   return barrier_selftest(spin_limit, (cudaStream_t)stream);
+}
+
+int ssv_selftest_backtransform(ssv_handle hh, int s, int gave_up, double* X, long long ldX, int* status,
+                               double* resid, void* stream) {
+  Handle* h = reinterpret_cast<Handle*>(hh);
+  if (!h || s < 1 || !X || ldX < h->n) return SSV_EINVAL;
+  if (!h->has_q || !apply_q_tc_supported(h->n, s * h->m)) return SSV_ENOTSUP;
+  return apply_q_tc(h, s * h->m, reinterpret_cast<cd*>(X), ldX, (cudaStream_t)stream, status, resid,
+                    gave_up != 0 ? 1 : 0);
 }
 
 int ssv_peak_probe(int kind, void* stream, double* tflops) {

@@ -113,12 +113,18 @@ int reduce_fp64(Handle* h, const double* A, long long lda, const double* B, long
 size_t q_t_count(int n, int m);
 // X = Q Xhat; digits: many columns may go through apply_q_tc, which keeps the norm of
 // a column to FP64 accuracy, not its small entries
+// (status, resid: see apply_q_tc)
 int apply_q(const Handle* h, int ncols, const double* Xhat, long long ldx, double* X, long long ldX,
-            bool digits, cudaStream_t st);
+            bool digits, cudaStream_t st, int* status = nullptr, double* resid = nullptr);
 // the same for many columns, with digit products on the tensor cores (reduce_tc.cu)
 bool apply_q_tc_supported(int n, int ncols);
 size_t apply_q_tc_scratch_bytes(int n, int ncols);
-int apply_q_tc(const Handle* h, int ncols, cd* X, long long ldX, cudaStream_t st);
+// when a bounded wait gives up every entry of X is NaN, and with status / resid (one
+// entry per h->m columns, or null) the shifts reported SSV_SHIFT_OK become
+// SSV_SHIFT_NONFINITE and their backward errors NaN; err0: the error word's value
+// before the first product (the self-test's)
+int apply_q_tc(const Handle* h, int ncols, cd* X, long long ldX, cudaStream_t st, int* status = nullptr,
+               double* resid = nullptr, int err0 = 0);
 // load a stored reduced triple with explicit zeros (reduce_fp64.cu)
 int load_reduced(Handle* h, const double* H, long long ldh, const double* R, long long ldr,
                  const double* Ct, long long ldc, cudaStream_t st);

@@ -62,7 +62,8 @@ EXPORTS = ("ssv_default_opts", "ssv_reduce", "ssv_solve", "ssv_apply_q", "ssv_ge
            "ssv_batch_create", "ssv_batch_run", "ssv_batch_destroy", "ssv_autotune",
            "ssv_trace_enable", "ssv_trace_reset", "ssv_trace_read", "ssv_selftest_barrier",
            "ssv_solve_rhs", "ssv_solve_trans", "ssv_givens_schedule", "ssv_tf_norm2",
-           "ssv_backward_error", "ssv_refine_counts", "ssv_pool_trim", "ssv_reduce_arith")
+           "ssv_backward_error", "ssv_refine_counts", "ssv_pool_trim", "ssv_reduce_arith",
+           "ssv_selftest_backtransform")
 
 _lib = None
 
@@ -114,6 +115,8 @@ def load(build_if_missing=True):
                                ctypes.POINTER(ctypes.c_float)]
     L.ssv_selftest_barrier.argtypes = [LL, P]
     L.ssv_selftest_barrier.restype = I
+    L.ssv_selftest_backtransform.argtypes = [P, I, I, P, LL, P, P, P]
+    L.ssv_selftest_backtransform.restype = I
     L.ssv_trace_enable.argtypes = [I]
     L.ssv_trace_reset.argtypes = []
     L.ssv_trace_read.argtypes = [I, ctypes.c_char_p, I, ctypes.POINTER(ctypes.c_float),
@@ -585,3 +588,13 @@ def selftest_barrier(spin_limit=100000, stream=None):
     """Run the bounded-barrier timeout self-test; returns the library's return code
     (SSV_ETIMEOUT when the timeout path works)."""
     return load().ssv_selftest_barrier(int(spin_limit), _stream_ptr(stream))
+
+
+def selftest_backtransform(handle, x, status=None, resid=None, gave_up=False, stream=None):
+    """X = Q X in place by the digit products of mode "x" (x: complex128 (n, s m), wide
+    enough for them), as if a bounded wait had given up when gave_up is set."""
+    _need_cuda(x, torch.complex128, "x")
+    ptr = lambda t: ctypes.c_void_p(t.data_ptr()) if t is not None else None  # noqa: E731
+    _check(load().ssv_selftest_backtransform(handle.ptr, x.shape[1] // handle.m, 1 if gave_up else 0, ptr(x),
+                                             _ld(x, handle.n), ptr(status), ptr(resid), _stream_ptr(stream)),
+           "ssv_selftest_backtransform")
