@@ -73,7 +73,7 @@ constexpr unsigned long long kSpin = 1ull << 26;  // grid barrier naps before gi
 // Debug builds (-DSSV_BOUNDS_CHECK): every global index of these kernels is
 // checked against its buffer's extent; one out of range is clamped to 0 (a
 // bulk copy then stays inside its buffer) and sets bit 2 of the error word,
-// so the reduction fails.  The scratch is filled with NaN before use and a
+// so the reduction fails (the back-transform reports NaN).  The scratch is filled with NaN before use and a
 // canary after it is verified at the end.  In normal builds RBCK(i, n, e) is i.
 #ifdef SSV_BOUNDS_CHECK
 __device__ __forceinline__ size_t rbck(long long i, size_t n, int* err) {
@@ -1526,11 +1526,14 @@ namespace {
 // V(r, k), explicit zeros and unit pivots, of reflectors 0 .. cnt - 1 with pivot
 // rows pv + k, from their packed storage; rows r0 .. n - 1, columns 0 .. kBmax - 1
 __global__ void __launch_bounds__(256) qv_kernel(const double* __restrict__ src, int n, int r0, int pv, int cnt,
-                                                 double* __restrict__ V, long long ldv) {
+                                                 double* __restrict__ V, long long ldv, size_t nsrc, size_t nv,
+                                                 int* err) {
   const int r = r0 + blockIdx.x * 256 + threadIdx.x, k = blockIdx.y;
   if (r >= n) return;
   const int d = r - pv - k;
-  V[r + (size_t)k * ldv] = (k >= cnt || d < 0) ? 0.0 : d == 0 ? 1.0 : src[r + (size_t)k * n];
+  V[RBCK(r + (size_t)k * ldv, nv, err)] = (k >= cnt || d < 0) ? 0.0
+                                          : d == 0            ? 1.0
+                                                              : src[RBCK(r + (size_t)k * n, nsrc, err)];
 }
 
 constexpr int kQCols = 1024;  // complex columns at a time (bounds the digit scratch)
@@ -1539,14 +1542,15 @@ constexpr int kQSplit = 7;    // partial sums of V^T V at most
 // S = V^T V from its partial sums, row i scaled by tau_i: a step of the back
 // substitution is then a broadcast and a multiply-add
 __global__ void __launch_bounds__(256) qs_kernel(const double* __restrict__ Sp, int kss, int cnt,
-                                                 const double* __restrict__ tau, double* __restrict__ S) {
+                                                 const double* __restrict__ tau, double* __restrict__ S, size_t ns,
+                                                 size_t ntau, int* err) {
   const int e = blockIdx.x * 256 + threadIdx.x, i = e % kBmax;
   double v[kQSplit];
 #pragma unroll
-  for (int q = 0; q < kQSplit; ++q) v[q] = q < kss ? Sp[(size_t)q * kBmax * kBmax + e] : 0.0;
+  for (int q = 0; q < kQSplit; ++q) v[q] = q < kss ? Sp[RBCK((size_t)q * kBmax * kBmax + e, ns, err)] : 0.0;
 #pragma unroll
   for (int q = 1; q < kQSplit; ++q) v[0] += v[q];
-  S[e] = i < cnt ? v[0] * __ldg(tau + i) : 0.0;
+  S[RBCK(e, (size_t)kBmax * kBmax, err)] = i < cnt ? v[0] * __ldg(tau + RBCK(i, ntau, err)) : 0.0;
 }
 
 // Z = T W for 8 real columns per CTA, a warp each: lane l holds the rows l, l +
@@ -1556,7 +1560,8 @@ __global__ void __launch_bounds__(256) qs_kernel(const double* __restrict__ Sp, 
 // columns: 27 us; with every CTA adding S's partial sums itself 69).
 __global__ void __launch_bounds__(256) qz_kernel(const double* __restrict__ Wp, int ksw, long long wstride,
                                                  const double* __restrict__ Sg, int cnt, int ncol,
-                                                 const double* __restrict__ tau, DigitMat Z) {
+                                                 const double* __restrict__ tau, DigitMat Z, size_t nw, size_t ntau,
+                                                 int* err) {
   extern __shared__ double S[];  // kBmax x kBmax
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
 #pragma unroll 8
@@ -1571,8 +1576,8 @@ __global__ void __launch_bounds__(256) qz_kernel(const double* __restrict__ Wp, 
     const int i = lane + 32 * u;
     double v = 0.0;
     if (i < cnt) {
-      for (int q = 0; q < ksw; ++q) v += Wp[(size_t)q * wstride + i + (size_t)c * kBmax];
-      v *= __ldg(tau + i);
+      for (int q = 0; q < ksw; ++q) v += Wp[RBCK((size_t)q * wstride + i + (size_t)c * kBmax, nw, err)];
+      v *= __ldg(tau + RBCK(i, ntau, err));
     }
     w[u] = v;
   }
@@ -1595,14 +1600,14 @@ __global__ void __launch_bounds__(256) qz_kernel(const double* __restrict__ Wp, 
   for (int u = 0; u < kBmax / 32; ++u) mx = max(mx, abs_hi(w[u]));
   mx = __reduce_max_sync(0xffffffffu, mx);
   const int E = scale_exp_hi(mx);
-  if (lane == 0) Z.ex[c] = E;
+  if (lane == 0) Z.ex[RBCK(c, (size_t)Z.RT * kTR, err)] = E;
 #pragma unroll
   for (int u = 0; u < kBmax / 32; ++u) {
     unsigned short d[kD];
     digits_of(w[u], E, d);
     const size_t off = (size_t)tile_off_kg(c % kTR, lane, kTK / 8);
 #pragma unroll
-    for (int l = 0; l < kD; ++l) Z.d[tile_index(Z, l, u, c / kTR) + off] = d[l];
+    for (int l = 0; l < kD; ++l) Z.d[RBCK(tile_index(Z, l, u, c / kTR) + off, Z.nd, err)] = d[l];
   }
 }
 
@@ -1683,7 +1688,12 @@ int apply_q_tc(const Handle* h, int ncols, cd* X, long long ldX, cudaStream_t st
   const int ncm = std::min(ncols, kQCols);
   unsigned char* base = nullptr;
   const size_t bytes = qtc_layout(n, ncm, nullptr, nullptr);
-  SSV_CUDA_TRY(pool_alloc((void**)&base, bytes, st));
+#ifdef SSV_BOUNDS_CHECK
+  constexpr size_t kCanary = 256;  // checked at the end
+#else
+  constexpr size_t kCanary = 0;
+#endif
+  SSV_CUDA_TRY(pool_alloc((void**)&base, bytes + kCanary, st));
   QtcScratch Q;
   qtc_layout(n, ncm, base, &Q);
   int rc = SSV_OK;
@@ -1696,6 +1706,10 @@ int apply_q_tc(const Handle* h, int ncols, cd* X, long long ldX, cudaStream_t st
       rc = SSV_ECUDA;
     }
   };
+#ifdef SSV_BOUNDS_CHECK
+  cu(cudaMemsetAsync(base, 0xFF, bytes, st));
+  cu(cudaMemsetAsync(base + bytes, 0xA5, kCanary, st));
+#endif
   cu(cudaMemsetAsync(Q.err, err0, sizeof(int), st));
   cu(cudaFuncSetAttribute(qz_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
                           (int)(sizeof(double) * kBmax * kBmax)));
@@ -1718,7 +1732,9 @@ int apply_q_tc(const Handle* h, int ncols, cd* X, long long ldX, cudaStream_t st
     const int cnt = std::min(kBmax, (isA ? h->ka : h->kb) - j), pv = isA ? m + j : j;
     const double* src = isA ? h->H + (size_t)j * n : h->R + (size_t)j * n;
     const double* tau = isA ? h->tauA + j : h->tauB + j;
-    qv_kernel<<<dim3((unsigned)((n - pv + 255) / 256), kBmax), 256, 0, st>>>(src, n, pv, pv, cnt, Q.V, Q.ldv);
+    const size_t nsrc = (size_t)n * ((isA ? n : m) - j), ntau = (size_t)(isA ? n : m) - j;
+    qv_kernel<<<dim3((unsigned)((n - pv + 255) / 256), kBmax), 256, 0, st>>>(src, n, pv, pv, cnt, Q.V, Q.ldv,
+                                                                                      nsrc, Q.nV, Q.err);
     count_launch();
     cu(cudaGetLastError());
     step(split_into(Q.V, 1, Q.ldv, pv, n, 0, cnt, Q.vrow, Q.nV, Q.err, st));
@@ -1730,7 +1746,8 @@ int apply_q_tc(const Handle* h, int ncols, cd* X, long long ldX, cudaStream_t st
     gs.kstride = (long long)kBmax * kBmax;
     if (rc == SSV_OK) step(gemm_launch<32, 9>(gs, st));
     double* S1 = Q.S + (size_t)kQSplit * kBmax * kBmax;
-    qs_kernel<<<kBmax * kBmax / 256, 256, 0, st>>>(Q.S, gs.ksplit, cnt, tau, S1);
+    qs_kernel<<<kBmax * kBmax / 256, 256, 0, st>>>(Q.S, gs.ksplit, cnt, tau, S1, (size_t)8 * kBmax * kBmax,
+                                                         ntau, Q.err);
     count_launch();
     cu(cudaGetLastError());
     for (int c0 = 0; c0 < ncols && rc == SSV_OK; c0 += ncm) {
@@ -1744,7 +1761,7 @@ int apply_q_tc(const Handle* h, int ncols, cd* X, long long ldX, cudaStream_t st
       gw.kstride = (long long)kBmax * 2 * nc;
       if (rc == SSV_OK) step(gemm_launch<32, 9>(gw, st));
       qz_kernel<<<(2 * nc + 7) / 8, 256, sizeof(double) * kBmax * kBmax, st>>>(
-          Q.W, gw.ksplit, gw.kstride, S1, cnt, 2 * nc, tau, Q.zcol);
+          Q.W, gw.ksplit, gw.kstride, S1, cnt, 2 * nc, tau, Q.zcol, Q.nW, ntau, Q.err);
       count_launch();
       cu(cudaGetLastError());
       GArgs gx = args(Q.vrow, Q.zcol, 0, (cnt + kTK - 1) / kTK, pv, n, 2 * nc, Xd, nX, 2 * ldX);
@@ -1756,6 +1773,13 @@ int apply_q_tc(const Handle* h, int ncols, cd* X, long long ldX, cudaStream_t st
       if (rc == SSV_OK) step(gemm_launch<32, 9>(gx, st));
     }
   }
+#ifdef SSV_BOUNDS_CHECK
+  if (rc == SSV_OK) {
+    rtc_canary_kernel<<<1, 256, 0, st>>>(base + bytes, kCanary, Q.err);
+    count_launch();
+    cu(cudaGetLastError());
+  }
+#endif
   if (rc == SSV_OK) {
     q_fail_kernel<<<256, 256, 0, st>>>(Q.err, X, ldX, n, ncols, m, status, resid);
     count_launch();

@@ -54,11 +54,11 @@ namespace {
 
 using namespace tcg;
 
-// Debug builds (-DSSV_BOUNDS_CHECK): every global index of the sweep's kernels
-// is checked against its buffer; an index out of range sets bit 1 of the
-// solve's error word (every shift of the solve then reports a non-finite
-// result) and is replaced by 0, so the access stays inside the buffer.  In
-// normal builds BCK(i, n) is i.
+// Debug builds (-DSSV_BOUNDS_CHECK): the indices into the sweep's scratch, its
+// digit tiles, the panels' H and X-hat are checked against their buffers; an
+// index out of range sets bit 2 of the solve's error word (every shift of the
+// solve then reports a non-finite result) and is replaced by 0, so the access
+// stays inside the buffer.  In normal builds BCK(i, n) is i.
 #ifdef SSV_BOUNDS_CHECK
 __device__ __forceinline__ size_t bck(long long i, size_t n, int* err) {
   if (i < 0 || (size_t)i >= n) {
@@ -256,7 +256,12 @@ __global__ void __launch_bounds__(panel_threads<MAXM, FEW>(), panel_per_sm<MAXM,
     const int row = e % nbe, q = e / nbe;
     coef4[row * S + q] = Z2f[BCK((r + row) + (size_t)q * ldz, a.z2_stride)];
   }
-  pan::run<pan::DF32, MAXM, kNBT, T, false>(pan::DF32::H{a.Hhi, a.Hlo, n}, k - nbe, j0, sigma, nbe, m, sm.p,
+  pan::DF32::H hm{a.Hhi, a.Hlo, n, {}};
+#ifdef SSV_BOUNDS_CHECK
+  hm.bound.count = (size_t)n * n;
+  hm.bound.err = a.err;
+#endif
+  pan::run<pan::DF32, MAXM, kNBT, T, false>(hm, k - nbe, j0, sigma, nbe, m, sm.p,
                                             (pan::SmemR<pan::DF32, MAXM, kNBT>*)nullptr, sing_tol, &sm.sing);
   // coef rows c < nbe hold P1(c, :), rows kNBT + qq hold P2(qq, :) (slots 0..m-1)
 

@@ -372,8 +372,8 @@ __device__ void fp64_shift(const FpSys& d, const int sh, cd* Z2,
         for (int t = tid; t < nbe; t += NT) psr->r[t] = Zr[r + t];
       }
       typename A::H hm;
-      if constexpr (DF) hm = {d.Hhi, d.Hlo, n};
-      else hm = {H, n};
+      if constexpr (DF) hm = {d.Hhi, d.Hlo, n, {}};
+      else hm = {H, n, {}};
       pan::run<A, MAXM, kNB, NT, RHS>(hm, k - nbe, j0, sigma, nbe, m, psm, psr, sing_tol, &s_sing);
     }
 
