@@ -1,5 +1,5 @@
 // Double-word and double-float arithmetic on the FP32 pipe, shared by the
-// double-float sweeps (solve_fp64.cu) and the tensor-core sweep (solve_tc.cu).
+// double-float sweeps (sweep.cuh) and the tensor-core sweep (solve_tc.cu).
 #pragma once
 #include "ssv_internal.cuh"
 
@@ -7,8 +7,7 @@ namespace ssv {
 
 // Double-word scalars (hi + lo, |lo| <= ulp(hi) / 2) on the FP32 pipe, for the
 // few per-row reflector quantities of the double-float panel: Knuth's two-sum,
-// Dekker's fast two-sum, FMA-exact products, one correction step for the
-// quotient and for the square root (Newton on s^2 = x).  About 44 bits each.
+// Dekker's fast two-sum, FMA-exact products (root and reciprocal: panel.cuh).
 struct dw {
   float hi, lo;
 };
@@ -26,18 +25,6 @@ static __device__ __forceinline__ dw dw_mul(dw x, dw y) {
   const float p = __fmul_rn(x.hi, y.hi);  // not contracted into the sum below
   const float e = fmaf(x.hi, y.lo, fmaf(x.lo, y.hi, fmaf(x.hi, y.hi, -p)));
   return dw_fast(p, e);
-}
-static __device__ __forceinline__ dw dw_div(dw x, dw y) {
-  const float q1 = x.hi / y.hi;
-  // x - q1 y: the leading part is exact by FMA
-  const float r = fmaf(-q1, y.hi, x.hi) + fmaf(-q1, y.lo, x.lo);
-  return dw_fast(q1, r / y.hi);
-}
-static __device__ __forceinline__ dw dw_sqrt(dw x) {
-  if (!(x.hi > 0.f)) return dw{0.f, 0.f};
-  const float s = sqrtf(x.hi);
-  const float e = fmaf(-s, s, x.hi) + x.lo;
-  return dw_fast(s, e / (2.f * s));
 }
 // complex128 <-> double-float (re_hi, re_lo, im_hi, im_lo)
 static __device__ __forceinline__ float4 df_split(cd z) {

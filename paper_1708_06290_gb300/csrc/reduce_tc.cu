@@ -1670,12 +1670,15 @@ size_t qtc_layout(int n, int nc, unsigned char* base, QtcScratch* Q) {
 
 }  // namespace
 
-// Where the digit products win over the FP64 pipe: that path grows with n^2 ncols,
-// this one up to some 256 columns with the number of blocks alone (150 us each).
-// FP64 / digit products in ms, near the line: n = 256, 640 columns 0.51 / 0.45; n =
-// 384, 450 columns 0.52 / 0.53; n = 768, 256 columns 1.21 / 0.94; n = 2048, 64 columns
-// 2.98 / 2.42; below: n = 512, 256 columns 0.62 / 0.65; n = 256, 450 columns 0.28 / 0.39;
-// far above: n = 4096, 640 columns 82.1 / 8.9.
+// Where the digit products take over from the FP64 pipe (mode X of the precisions
+// below FP64): that path grows with n^2 ncols, this one up to some 256 columns with
+// the number of blocks alone (150 us each).  FP64 / digit products in ms, along the
+// line (n ncols = 180000): n = 256 0.50 / 0.44, 384 0.61 / 0.52, 768 1.20 / 0.92, 1200
+// 2.00 / 1.58, 2048 5.09 / 2.44, 4096 12.5 / 5.12; far above it: n = 4096, 640 columns
+// 80.7 / 8.9.  Below it the sides cross: n = 512, 256 columns 0.62 / 0.65 and n = 256,
+// 450 columns 0.28 / 0.39, but n = 2048, 64 columns 2.98 / 2.42, so the product of the
+// two does not part them there; such X stays on the FP64 pipe, which keeps every
+// entry's accuracy.
 bool apply_q_tc_supported(int n, int ncols) { return n >= 256 && (long long)n * ncols >= 180000; }
 
 size_t apply_q_tc_scratch_bytes(int n, int ncols) {

@@ -7,8 +7,9 @@
 // transform, Z2 <- Z1 P1 + Z2 P2 - sigma E P1) multiplies a tile of H that is
 // staged once for a group of shifts.  Per block step:
 //
-//   1. panel (one thread block per shift, three per SM): the n_b x (n_b + m) window block is
-//      triangularised bottom-up by one complex Householder reflector per row
+//   1. panel (one thread block per shift; five, three, two or one per SM by m and
+//      the number of shifts): the n_b x (n_b + m) window block is triangularised
+//      bottom-up by one complex Householder reflector per row
 //      over the m + 1 candidate columns (double-word reflector scalars,
 //      double-float application, as in the double-float sweep), giving the
 //      coefficients P1 (n_b x m) and P2 (m x m).  The panel also updates the p
@@ -24,12 +25,13 @@
 //      35 digit products H_k P_l with k + l <= 7 run as tcgen05.mma (BF16 x
 //      BF16 -> FP32, M = 128, K = 16, seven digits of P1 per product) into eight TMEM accumulators, one
 //      per level k + l, where every partial sum is an integer below
-//      7 * 128 * 127^2 < 2^24 and therefore exact.  The
+//      128 * 127 * (128 + 6 * 80) < 2^24 and therefore exact (H's digits are up to
+//      127, a column's first up to 128 and the others up to 80 in modulus).  The
 //      digit tiles reach shared memory by 1-D TMA bulk copies on an mbarrier,
 //      two stages in flight.  The epilogue reads the levels back (tcgen05.ld),
 //      adds them scaled by 2^{-7 t} into double-float sums, scales by the row
-//      and column exponents, and adds Z2 P2 and the shifted-diagonal
-//      correction in double-float on the FP32 pipe;
+//      and column exponents, and adds Z2 P2 (m >= 5: digit products too) and the
+//      shifted-diagonal correction in double-float on the FP32 pipe;
 //   3. after the last block: the final m x m block, G = Ct Xhat or X-hat by the
 //      backward pass over the stored block transforms.
 //

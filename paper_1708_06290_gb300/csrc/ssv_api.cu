@@ -1,6 +1,7 @@
 // C ABI entry points (include/ssv.h): argument checks, handle lifetime and
 // dispatch to the FP64 reduction and the solvers.
 #include <atomic>
+#include <climits>
 #include <mutex>
 #include <cstdlib>
 #include <cstring>
@@ -526,7 +527,7 @@ int ssv_footprint(int n, int m, int p, int s, const ssv_opts* o_in, size_t* byte
                                       : solve_fp64_scratch_bytes(n, m, p, s, &o);
   // the back-transform runs once the solve's scratch has gone back
   if (o.mode == SSV_X && o.precision != SSV_FP64)
-    *bytes = std::max(*bytes, apply_q_tc_scratch_bytes(n, s * m));
+    *bytes = std::max(*bytes, apply_q_tc_scratch_bytes(n, (int)std::min<long long>((long long)s * m, INT_MAX)));
   return SSV_OK;
 }
 

@@ -70,7 +70,7 @@ struct Handle {
   double* Ct;     // max(p,1) x n, ld max(p,1)
   double* tauB;   // m
   double* tauA;   // n
-  double* Tq;     // T factors of Q's compact WY blocks (q_t_count doubles; empty without Q)
+  double* Tq;     // T factors of Q's compact WY blocks (q_t_count doubles; unset without Q)
   double* hnorm2; // 2: ||H||_F^2 and trace(H) of the structural part
   float* Hhi;     // n x n: fl32(H) on and above the m-th subdiagonal, 0 below
   float* Hlo;     // n x n: fl32(H - Hhi), 0 below (Hhi + Hlo carries 48 bits of H)
@@ -141,6 +141,7 @@ int solve_fp64_rhs(const Handle* h, int s, const double* shifts, const double* b
                    long long ldb, const ssv_opts* o, double* out, long long ldo, int* status,
                    cudaStream_t st);
 // transposed systems (A - sigma_l I)^T x_l = C^T chat_l (Sec. 3.3); out = Q^T x_l (n x s)
+// (solve_trans.cu, with the Givens panel)
 int solve_fp64_trans(const Handle* h, int s, const double* shifts, const double* chat,
                      long long ldc, const ssv_opts* o, double* out, long long ldo, int* status,
                      cudaStream_t st);
@@ -210,7 +211,7 @@ size_t noalloc_scratch_bytes();
 int default_nb(int n, int m);
 int num_sms();
 
-// batched multi-system FP64 solve (solve_fp64.cu)
+// many systems in one launch, FP64 and double-float (solve_batch.cu)
 struct BatchPlan;
 // stream_ordered != nullptr: stream-ordered buffers on that stream (freed by
 // batch_destroy on it, no device-wide synchronisation); else cudaMalloc.

@@ -13,16 +13,8 @@ constexpr int kDigits = 8;               // 7-bit digits per value (56 bits)
 constexpr int kBadExp = 0x40000000;      // exponent marker of a non-finite row / column
 constexpr long long kWaitLimit = 1LL << 26;
 
-// 2^E > |x| for the largest |x| of a row / column: E from the exponent field
-static __device__ __forceinline__ int scale_exp(double maxabs) {
-  if (!(maxabs <= 1.7976931348623157e308)) return kBadExp;  // Inf or NaN
-  const unsigned long long b = (unsigned long long)__double_as_longlong(maxabs);
-  const int ef = (int)((b >> 52) & 0x7ff);
-  return ef == 0 ? -1022 : ef - 1022;
-}
-
-// |x|'s high word, ordered as |x| is (NaN above Inf above all), and the same
-// exponent from the largest one
+// |x|'s high word, ordered as |x| is (NaN above Inf above all), and from the largest
+// one of a row / column the exponent E with 2^E > |x|
 static __device__ __forceinline__ int abs_hi(double x) { return __double2hiint(x) & 0x7fffffff; }
 static __device__ __forceinline__ int scale_exp_hi(int hi) {
   const int ef = hi >> 20;
@@ -173,9 +165,6 @@ static __device__ __forceinline__ void bulk_copy(uint32_t dst, const void* src, 
   asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(dst),
                "l"(src), "r"(bytes), "r"(mbar)
                : "memory");
-}
-static __device__ __forceinline__ void cp16(uint32_t dst, const void* src) {
-  asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst), "l"(src) : "memory");
 }
 static __device__ __forceinline__ void tmem_ld8(uint32_t taddr, uint32_t (&r)[8]) {
   asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
