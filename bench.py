@@ -32,11 +32,11 @@ import workloads as W  # noqa: E402
 
 METRIC = "shift-solves/s at n=5000,m=16 (mixed vs FP64, resid<=1e-12); p50/p99 latency"
 # DRAM bytes of one reduce_blocked_kernel launch at n = 5000, m = p = 16 (ncu), or None
-REDUCE_TRAFFIC_N5000_M16 = 130381078528 + 90573036032
+REDUCE_TRAFFIC_N5000_M16 = 131546424320 + 90723151872
 # dram__bytes_read.sum + dram__bytes_write.sum of all tcs_update_kernel launches of one
 # 304-shift sweep of this workload, per shift (profiles/tcs_sweep_n5000_m16_304shifts.md);
 # the window state it streams is per shift, so traffic scales with the shifts
-TCS_UPDATE_TRAFFIC_PER_SHIFT = (17579877120 + 18607825408) / 304.0
+TCS_UPDATE_TRAFFIC_PER_SHIFT = (16930213376 + 12008796160) / 304.0
 UNIT = "shift-solves/s"
 
 
@@ -676,10 +676,10 @@ def main():
         "peak_source": "FP64 DFMA probe measured in this run (nominal GB300 FP64 1.25 TFLOP/s)",
         "launch_ms": fp64_ms,
         "flops_definition": "2 n^2 m + 4 n m p per shift (trailing update Z1 P1 + Ct rows)",
-        # ncu dram__bytes_read.sum + dram__bytes_write.sum of one launch on 152 shifts of
+        # ncu's DRAM bytes of one launch on 152 shifts of
         # this workload (profiles/solve_fp64_kernel_n5000_m16_152shifts.md), scaled by shifts:
         # each shift streams its own Z2 state
-        "traffic": (3.002227e9 + 3.462814e9) * s / 152.0 if args.nb in (0, 128) else None,
+        "traffic": 6.5116e9 * s / 152.0 if args.nb in (0, 128) else None,
     }
     sweep0_ms = res["mixed"]["phase_ms_per_step"].get("mixed_sweep0", float("nan"))
     # the double-float equivalent of the first solve: each double-float multiply-add issues
