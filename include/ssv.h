@@ -77,8 +77,8 @@ extern "C" {
                        columns of H, most of the work) on the tensor cores as
                        error-free BF16 digit products (H and the block transforms
                        split into seven 7-bit digits, exact FP32 accumulation per
-                       level, about 48 significant bits) and the panels and Z2 P2
-                       in double-float as in SSV_DFLOAT; no refinement.
+                       level, about 48 significant bits), Z2 P2 too for m >= 5,
+                       and the rest in double-float as in SSV_DFLOAT; no refinement.
                        m <= 16, n > m, n_b = 128, Householder panel; ssv_solve and
                        ssv_tf_norm2 (ssv_solve_many solves the systems one after
                        another).  Singularity threshold as SSV_DFLOAT. */

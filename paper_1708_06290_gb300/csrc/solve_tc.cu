@@ -228,7 +228,7 @@ struct PanelSmem {
 };
 // Threads and resident panels per SM.  FEW (no more shifts than SMs, m > 8): one
 // panel per SM with twice the threads for the update of the sub-block's other
-// rows (m = 16: 183 us per block of 128 rows against 191); else two with 256.
+// rows (m = 16: 180 us per block of 128 rows against 188); else two with 256.
 template <int MAXM, bool FEW>
 constexpr int panel_threads() { return MAXM <= 4 ? 128 : MAXM <= 8 || !FEW ? 256 : 512; }
 template <int MAXM, bool FEW>
