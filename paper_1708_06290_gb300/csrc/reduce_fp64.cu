@@ -285,6 +285,48 @@ __global__ void __launch_bounds__(kQT) apply_q_kernel(QSrc q, int R, const doubl
   if (R > 1) cluster_sync_all();  // no CTA leaves while its sums may still be read
 }
 
+// n <= 32 NR: a warp per column, lane l the rows l, l + 32, .., one reflector after
+// another.  Bound by the FP64 pipe (10 + 4 NR instructions of 64 clocks a column and
+// reflector).
+constexpr int kQSmall = 64;
+template <int NR>
+__global__ void __launch_bounds__(256) apply_q_small_kernel(QSrc q, cd* __restrict__ X, long long ldx, int ncols) {
+  const int lane = threadIdx.x & 31, c = (int)((blockIdx.x * 256ll + threadIdx.x) >> 5);
+  if (c >= ncols) return;  // the whole warp
+  cd x[NR];
+#pragma unroll
+  for (int u = 0; u < NR; ++u) {
+    const int r = lane + 32 * u;
+    x[u] = r < q.n ? X[r + (size_t)c * ldx] : mkcd(0.0, 0.0);
+  }
+  auto reflect = [&](const double* v, double tau, int pv) {
+    double vr[NR], wr = 0.0, wi = 0.0;
+#pragma unroll
+    for (int u = 0; u < NR; ++u) {
+      const int r = lane + 32 * u;
+      vr[u] = r < pv || r >= q.n ? 0.0 : r == pv ? 1.0 : v[r];
+      wr = fma(vr[u], x[u].x, wr);
+      wi = fma(vr[u], x[u].y, wi);
+    }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+      wr += __shfl_xor_sync(0xffffffffu, wr, o);
+      wi += __shfl_xor_sync(0xffffffffu, wi, o);
+    }
+    wr *= -tau;
+    wi *= -tau;
+#pragma unroll
+    for (int u = 0; u < NR; ++u) x[u] = mkcd(fma(wr, vr[u], x[u].x), fma(wi, vr[u], x[u].y));
+  };
+  for (int j = q.ka - 1; j >= 0; --j) reflect(q.A + (size_t)j * q.n, __ldg(q.tauA + j), q.m + j);
+  for (int j = q.kb - 1; j >= 0; --j) reflect(q.B + (size_t)j * q.n, __ldg(q.tauB + j), j);
+#pragma unroll
+  for (int u = 0; u < NR; ++u) {
+    const int r = lane + 32 * u;
+    if (r < q.n) X[r + (size_t)c * ldx] = x[u];
+  }
+}
+
 constexpr size_t kQTSmem = sizeof(double) * (size_t)(kQW * kQB * kQLd + kQB * kQB);
 template <int CC>
 constexpr size_t q_apply_smem() {
@@ -411,21 +453,28 @@ int apply_q(const Handle* h, int ncols, const double* Xhat, long long ldx, doubl
     cudaGetLastError();  // no room for its scratch (nothing written yet): the FP64 path needs none
   }
   const QSrc q = q_src(h);
-  const double* T = h->Tq;
-  // Columns per cluster: the fewest columns on the busiest SM, then the widest
-  // (V is read once per cluster); CTAs per cluster: as many as the SMs allow
-  // when there are fewer columns than SMs.
-  const int sms = num_sms();
-  int cc = 1;
-  long long best = -1;
-  for (int c = 1; c <= 4; ++c) {
-    const long long groups = (ncols + c - 1) / c;
-    const long long load = (groups + sms - 1) / sms * c;
-    if (best < 0 || load <= best) {
-      best = load;
-      cc = c;
-    }
+  // Small systems: the blocked kernel spends 20 us a wave of CTAs whatever n is, this
+  // one 1.3 us a reflector and wave.  One launch per reflector / blocks / this, us: n =
+  // 8, 700 columns 41 / 71 / 24; n = 32, 8000 columns 394 / 560 / 269; n = 64, 700
+  // columns 337 / 118 / 113 and 8000 859 / 882 / 646.  With fewer columns the blocks
+  // are the faster ones from n = 17 on (n = 33, 64 columns 40 / 63; n = 64 55 / 114).
+  if (n <= kQSmall && (n <= 16 || ncols >= 512)) {
+    auto kern = n <= 32 ? apply_q_small_kernel<1> : apply_q_small_kernel<2>;
+    kern<<<(unsigned)((ncols + 7) / 8), 256, 0, st>>>(q, Xc, ldX, ncols);
+    count_launch();
+    SSV_CUDA_TRY(cudaGetLastError());
+    return SSV_OK;
   }
+  const double* T = h->Tq;
+  // Columns per cluster: the widest (V is read once per cluster) with at most a tenth
+  // more columns on the busiest SM than the best width gives (8000 columns: four
+  // rather than one, whose SM has 56 instead of 53: n = 200, 3.67 -> 2.50 ms); CTAs per
+  // cluster: as many as the SMs allow when there are fewer columns than SMs.
+  const int sms = num_sms();
+  auto load = [&](int c) { return ((ncols + c - 1) / c + sms - 1) / sms * (long long)c; };
+  const long long best = std::min({load(1), load(2), load(3), load(4)});
+  int cc = 4;
+  while (10 * load(cc) > 11 * best) --cc;
   const int groups = (ncols + cc - 1) / cc;
   int R = 1;
   while (R < 8 && (long long)groups * R * 2 <= sms && n > 32 * kQW * R) R *= 2;
