@@ -260,6 +260,67 @@ __device__ void panel_qr(double* P, size_t ld, int L, int wp, int wc, int wg, do
   __syncthreads();
 }
 
+// A panel of one column (m = 1): the reflector of x(0:L) in place, V's column and T;
+// the first kPC rows of a thread stay in registers between norm and scaling.
+constexpr int kPC = 8;
+__device__ void panel_col(double* x, int L, double* tau, double* Vout, int ldv, double* Tout, double* sm) {
+  double* red = sm;             // kWarps
+  double* misc = red + kWarps;  // scal, tau, beta
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  double xr[kPC], ss = 0.0;
+#pragma unroll
+  for (int u = 0; u < kPC; ++u) {
+    const int i = 1 + tid + u * kT;
+    xr[u] = i < L ? __ldcg(x + i) : 0.0;
+  }
+  const double alpha = tid == 0 ? __ldcg(x) : 0.0;
+#pragma unroll
+  for (int u = 0; u < kPC; ++u)
+    if (1 + warp * 32 + u * kT < L) ss = fma(xr[u], xr[u], ss);
+  for (int i = 1 + tid + kPC * kT; i < L; i += kT) {
+    const double v = __ldcg(x + i);
+    ss = fma(v, v, ss);
+  }
+  for (int o = 16; o > 0; o >>= 1) ss += __shfl_xor_sync(0xffffffffu, ss, o);
+  if (lane == 0) red[warp] = ss;
+  __syncthreads();
+  if (warp == 0) {
+    double t = lane < kWarps ? red[lane] : 0.0;
+    for (int o = kWarps / 2; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
+    if (lane == 0) {
+      double tk = 0.0, scal = 0.0, beta = alpha;
+      if (t != 0.0) {
+        const double nrm = sqrt(fma(alpha, alpha, t));
+        beta = alpha >= 0.0 ? -nrm : nrm;
+        tk = (beta - alpha) / beta;
+        scal = 1.0 / (alpha - beta);
+      }
+      misc[0] = scal;
+      misc[1] = tk;
+      x[0] = beta;
+      tau[0] = tk;
+      Vout[0] = 1.0;
+    }
+  }
+  __syncthreads();
+  const double scal = misc[0], tk = misc[1];
+  if (tid < kSmT) Tout[tid] = tid == 0 ? tk : 0.0;
+  auto put = [&](int i, double v) {
+    if (tk != 0.0) {
+      v *= scal;
+      x[i] = v;
+    }
+    Vout[(size_t)i * ldv] = v;
+  };
+#pragma unroll
+  for (int u = 0; u < kPC; ++u) {
+    const int i = 1 + tid + u * kT;
+    if (i < L) put(i, xr[u]);
+  }
+  for (int i = 1 + tid + kPC * kT; i < L; i += kT) put(i, __ldcg(x + i));
+  __syncthreads();
+}
+
 // The same on a panel in global memory, staged in shared memory when it fits.
 __device__ void panel_qr_any(double* P, size_t ld, int L, int wp, int wc, int wg, double* tau,
                              double* Vout, int ldv, double* Tout, double* sm, double* pan) {
@@ -284,6 +345,12 @@ __device__ __forceinline__ double* ext_row(const RedArgs& a, int i, size_t* ld) 
   return a.Ct + (i - a.n);
 }
 
+// Lanes of a block that share one of `cnt` <= kW * kW sums: a warp where there are
+// enough, else eight.
+__device__ __forceinline__ int sum_lanes(int cnt) { return cnt * 32 <= kT ? 32 : 8; }
+static_assert(kW * kW * 8 <= kT, "eight lanes a sum");
+static_assert(kRS * kW <= kT && 2 * kRS * kW + kW * kW <= kSmPart, "one entry of a panel's rows per thread");
+
 // Phase B, rows [i0, i1) of A_ext: Y = A_ext(rows, r0:n) V T.  W >= w is the
 // compile-time width (V and T are zero beyond w).  For the columns pc .. pc +
 // wn - 1 of the next panel (rows r0 .. n - 1) also the right update, and this
@@ -299,7 +366,9 @@ __device__ void phase_b(const RedArgs& a, int r0, int w, const double* __restric
   const int tid = threadIdx.x;
   const int i0 = (int)(((long long)np * blockIdx.x) / gridDim.x);
   const int i1 = (int)(((long long)np * (blockIdx.x + 1)) / gridDim.x);
-  double wpart = 0.0;  // thread k * wn + q < w * wn: entry (k, q) of this block's part of W
+  // ln lanes share entry ew = k * wn + q of this block's part of W
+  const int ln = sum_lanes(w * wn), ew = tid / ln;
+  double wpart = 0.0;
   for (int rs0 = i0; rs0 < i1; rs0 += kRS) {
     const int RS = min(kRS, i1 - rs0);
     const int CG = kT / RS;
@@ -307,6 +376,15 @@ __device__ void phase_b(const RedArgs& a, int r0, int w, const double* __restric
     const bool act = g < CG;
     size_t ld = 0;
     const double* base = ext_row(a, rs0 + r, &ld);
+    // for the next panel: its entry, V's entry of the row, V's row of its column; their
+    // latency under the product's loads (n = 1000, m = 2: 16.25 -> 15.94 ms)
+    double rx = 0.0, rv = 0.0, rc = 0.0;
+    if (wn > 0) {
+      const int ix = rs0 + tid % RS, iv = rs0 + tid / W, cc = pc + tid / W;
+      if (tid < RS * wn && ix >= r0 && ix < n) rx = __ldcg(a.H + ix + (size_t)(pc + tid / RS) * n);
+      if (tid < RS * W && iv >= r0 && iv < n && tid % W < w) rv = __ldcg(V + (size_t)(iv - r0) * ldv + tid % W);
+      if (tid < wn * W && cc >= r0 && tid % W < w) rc = __ldcg(V + (size_t)(cc - r0) * ldv + tid % W);
+    }
     double acc[W];
 #pragma unroll
     for (int k = 0; k < W; ++k) acc[k] = 0.0;
@@ -346,47 +424,40 @@ __device__ void phase_b(const RedArgs& a, int r0, int w, const double* __restric
       a.Y[(size_t)(rs0 + rr) * kW + k] = s;
       part[rr * W + k] = s;
     }
+    double* vs = part + kRS * kW;    // RS x W: the rows of V
+    double* vc = vs + kRS * kW;      // wn x W: V's rows of the panel's columns
+    if (wn > 0) {
+      if (tid < RS * W) vs[tid] = rv;
+      if (tid < wn * W) vc[tid] = rc;
+    }
     __syncthreads();
     if (wn > 0) {
       // the next panel's columns: rows r0 .. n - 1 of this sub-strip
       double* xs = AV;                 // RS x wn (wn <= kW = the width AV is sized for)
-      double* vs = part + kRS * kW;    // RS x W: the rows of V
-      for (int e = tid; e < RS * W; e += kT) {
-        const int i = rs0 + e / W, k = e % W;
-        vs[e] = (i >= r0 && i < n && k < w) ? __ldcg(V + (size_t)(i - r0) * ldv + k) : 0.0;
-      }
-      for (int e = tid; e < RS * wn; e += kT) {
-        const int rr = e % RS, q = e / RS;
+      if (tid < RS * wn) {
+        const int rr = tid % RS, q = tid / RS;
         const int i = rs0 + rr, c = pc + q;
-        double x = 0.0;
-        if (i >= r0 && i < n) {
-          double* px = a.H + i + (size_t)c * n;
-          x = __ldcg(px);
-          if (c >= r0) {
-            const double* vc = V + (size_t)(c - r0) * ldv;
+        double x = rx;
+        if (i >= r0 && i < n && c >= r0) {
 #pragma unroll
-            for (int k = 0; k < W; ++k)
-              if (k < w) x = fma(-part[rr * W + k], __ldcg(vc + k), x);
-            *px = x;
-          }
+          for (int k = 0; k < W; ++k)
+            if (k < w) x = fma(-part[rr * W + k], vc[q * W + k], x);
+          a.H[i + (size_t)c * n] = x;
         }
         xs[rr * wn + q] = x;
       }
       __syncthreads();
-      if (tid < w * wn) {
-        const int k = tid / wn, q = tid % wn;
-        double s0 = 0.0, s1 = 0.0;
-        for (int rr = 0; rr + 1 < RS; rr += 2) {
-          s0 = fma(vs[rr * W + k], xs[rr * wn + q], s0);
-          s1 = fma(vs[(rr + 1) * W + k], xs[(rr + 1) * wn + q], s1);
-        }
-        if (RS & 1) s0 = fma(vs[(RS - 1) * W + k], xs[(RS - 1) * wn + q], s0);
-        wpart += s0 + s1;
+      if (ew < w * wn) {
+        const int k = ew / wn, q = ew % wn;
+        for (int rr = tid % ln; rr < RS; rr += ln) wpart = fma(vs[rr * W + k], xs[rr * wn + q], wpart);
       }
       __syncthreads();
     }
   }
-  if (wn > 0 && tid < w * wn) a.WP[(size_t)blockIdx.x * kW * kW + tid] = wpart;
+  if (wn > 0) {
+    for (int o = ln / 2; o > 0; o >>= 1) wpart += __shfl_xor_sync(0xffffffffu, wpart, o);
+    if (ew < w * wn && tid % ln == 0) a.WP[(size_t)blockIdx.x * kW * kW + ew] = wpart;
+  }
 }
 
 // The next panel after phase B (block 0): W from the blocks' parts, the left
@@ -399,12 +470,17 @@ __device__ void panel_step(const RedArgs& a, int r0, int w, const double* __rest
   double* Zs = Ws + kW * kW;
   const int tid = threadIdx.x;
   {
-    // eight lanes a sum, in a fixed order
-    const int e = tid / 8, sub = tid % 8;
+    // in a fixed order, eight loads in flight
+    const int ln = sum_lanes(w * wn), e = tid / ln, sub = tid % ln, G = (int)gridDim.x;
     double s = 0.0;
     if (e < w * wn)
-      for (int g = sub; g < (int)gridDim.x; g += 8) s += __ldcg(a.WP + (size_t)g * kW * kW + e);
-    for (int o = 4; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+      for (int g = sub; g < G; g += 8 * ln) {
+        double v[8];
+#pragma unroll
+        for (int u = 0; u < 8; ++u) v[u] = g + u * ln < G ? __ldcg(a.WP + (size_t)(g + u * ln) * kW * kW + e) : 0.0;
+        s += ((v[0] + v[1]) + (v[2] + v[3])) + ((v[4] + v[5]) + (v[6] + v[7]));
+      }
+    for (int o = ln / 2; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
     if (e < w * wn && sub == 0) Ws[e] = s;
   }
   __syncthreads();
@@ -634,11 +710,24 @@ template <int W>
 __device__ void block_step(const RedArgs& a, int r0, int lc, int w, const double* V, int ldv,
                            const double* Ts, int wn, int tn, double* work, bool* ok) {
   const int n = a.n, p = a.p;
-  phase_b<W>(a, r0, w, V, ldv, Ts, lc, wn, work);
+  // One reflector and one column: block 0 updates the panel alone, under the others'
+  // phase C, which is longer; sharing it lengthens phase B for everyone.  Shared /
+  // alone, ms: m = 1, n = 1000 26.9 / 25.7, n = 3000 258 / 251; m = 2, n = 1000 16.1 /
+  // 20.9, n = 3000 161 / 160.
+  const bool alone = W == 1 && wn == 1;
+  phase_b<W>(a, r0, w, V, ldv, Ts, lc, alone ? 0 : wn, work);
   if (!grid_barrier(a.bar, a.err, kBarrierSpins)) { *ok = false; return; }
   if (blockIdx.x == 0) {
     // look-ahead: the next panel's columns (rows r0 .. n-1), then its QR
-    if (wn > 0) panel_step<W>(a, r0, w, V, ldv, Ts, lc, wn, tn, work, work + kSmDoubles - kSmT);
+    if (alone) {
+      phase_c_bottom<W>(a, r0, w, V, ldv, Ts, lc, lc + wn, work);
+      __syncthreads();
+      const int rn = lc + a.m;
+      panel_col(a.H + rn + (size_t)lc * n, n - rn, a.tauA + lc, a.VA + (size_t)(tn & 1) * n * kW, kW,
+                a.TA + (size_t)(tn & 1) * kSmT, work);
+    } else if (wn > 0) {
+      panel_step<W>(a, r0, w, V, ldv, Ts, lc, wn, tn, work, work + kSmDoubles - kSmT);
+    }
   } else {
     // the other blocks split, by multiply-add count, the bottom columns
     // [lc + wn, n) (3 (n - r0) w each) followed by the top tiles
