@@ -129,29 +129,35 @@ __global__ void __launch_bounds__(kQT) q_t_kernel(QSrc q, int R, double* __restr
   const int rank = cluster_rank();
   const int b = blockIdx.x / R;
   const QBlock qb = q_block(q, b);
-  for (int e = tid; e < kQB * kQB; e += kQT) Sp[e] = 0.0;
-  __syncthreads();
-  double acc[kQB];
+  // The tiles of kQW row groups are staged at a time, each by its warp; every warp then
+  // adds up its kQB / kQW columns of S over all of them, a tile at a time (a warp that
+  // kept a tile to itself had 1024 multiply-adds of 64 clocks on its scheduler, 30 us,
+  // where a small system has one tile).
+  constexpr int NJ = kQB / kQW;
+  double acc[NJ];
 #pragma unroll
-  for (int j = 0; j < kQB; ++j) acc[j] = 0.0;
-  double* Vw = Vs + warp * kQB * kQLd;
-  const int step = kQW * R;
-  for (int g = qb.pv / 32 + warp * R + rank; g * 32 < q.n; g += step) {
-    __syncwarp();
-    q_stage(qb, q.n, g * 32, Vw);
-    __syncwarp();
-#pragma unroll 2
-    for (int rr = 0; rr < 32; ++rr) {
-      const double v = Vw[rr * kQLd + lane];
+  for (int u = 0; u < NJ; ++u) acc[u] = 0.0;
+  for (int g0 = qb.pv / 32 + rank; g0 * 32 < q.n; g0 += kQW * R) {
+    __syncthreads();
+    if ((g0 + warp * R) * 32 < q.n) q_stage(qb, q.n, (g0 + warp * R) * 32, Vs + warp * kQB * kQLd);
+    __syncthreads();
+    for (int t = 0; t < kQW && (g0 + t * R) * 32 < q.n; ++t) {
+      const double* Vt = Vs + t * kQB * kQLd;
+      double s[NJ];
 #pragma unroll
-      for (int j = 0; j < kQB; ++j) acc[j] = fma(v, Vw[rr * kQLd + j], acc[j]);
+      for (int u = 0; u < NJ; ++u) s[u] = 0.0;
+#pragma unroll 8
+      for (int rr = 0; rr < 32; ++rr) {
+        const double v = Vt[rr * kQLd + lane];
+#pragma unroll
+        for (int u = 0; u < NJ; ++u) s[u] = fma(v, Vt[rr * kQLd + warp * NJ + u], s[u]);
+      }
+#pragma unroll
+      for (int u = 0; u < NJ; ++u) acc[u] += s[u];
     }
   }
-  for (int w = 0; w < kQW; ++w) {  // fixed order: the same bits on every call
-    if (w == warp)
-      for (int j = 0; j < kQB; ++j) Sp[j * kQB + lane] += acc[j];
-    __syncthreads();
-  }
+#pragma unroll
+  for (int u = 0; u < NJ; ++u) Sp[(warp * NJ + u) * kQB + lane] = acc[u];
   cluster_sync_all();
   if (rank == 0) {
     double* S = Vs;                  // summed over the cluster
@@ -289,6 +295,7 @@ __global__ void __launch_bounds__(kQT) apply_q_kernel(QSrc q, int R, const doubl
 // another.  Bound by the FP64 pipe (10 + 4 NR instructions of 64 clocks a column and
 // reflector).
 constexpr int kQSmall = 64;
+constexpr int kQTiny = 16;  // up to here this kernel alone (no T factors)
 template <int NR>
 __global__ void __launch_bounds__(256) apply_q_small_kernel(QSrc q, cd* __restrict__ X, long long ldx, int ncols) {
   const int lane = threadIdx.x & 31, c = (int)((blockIdx.x * 256ll + threadIdx.x) >> 5);
@@ -397,10 +404,12 @@ QSrc q_src(const Handle* h) {
 
 size_t q_t_count(int n, int m) { return (size_t)(q_blocks(n) + q_blocks(m)) * kQB * kQB; }
 
-// the T factors of Q's blocks, kept in the handle
+// the T factors of Q's blocks, kept in the handle; none where apply_q needs none (with
+// that, and S spread over all warps, reductions of n = 2, 8 and 30 take 0.27, 0.38 and
+// 1.22 ms instead of 0.34, 0.45 and 1.29)
 static int make_q_t(Handle* h, cudaStream_t st) {
   const int nblk = q_blocks(h->kb) + q_blocks(h->ka);
-  if (nblk == 0) return SSV_OK;
+  if (nblk == 0 || h->n <= kQTiny) return SSV_OK;
   constexpr int kR = 4;
   SSV_CUDA_TRY(allow_smem(q_t_kernel, kQTSmem));
   SSV_CUDA_TRY(launch_cluster(q_t_kernel, nblk * kR, kQT, kR, kQTSmem, st, q_src(h), kR, h->Tq));
@@ -458,7 +467,7 @@ int apply_q(const Handle* h, int ncols, const double* Xhat, long long ldx, doubl
   // 8, 700 columns 41 / 71 / 24; n = 32, 8000 columns 394 / 560 / 269; n = 64, 700
   // columns 337 / 118 / 113 and 8000 859 / 882 / 646.  With fewer columns the blocks
   // are the faster ones from n = 17 on (n = 33, 64 columns 40 / 63; n = 64 55 / 114).
-  if (n <= kQSmall && (n <= 16 || ncols >= 512)) {
+  if (n <= kQTiny || (n <= kQSmall && ncols >= 512)) {
     auto kern = n <= 32 ? apply_q_small_kernel<1> : apply_q_small_kernel<2>;
     kern<<<(unsigned)((ncols + 7) / 8), 256, 0, st>>>(q, Xc, ldX, ncols);
     count_launch();

@@ -79,10 +79,7 @@ static void free_handle_buffers(Handle* h) {
   cudaFree(h->H);
   cudaFree(h->R);
   cudaFree(h->Ct);
-  cudaFree(h->tauB);
-  cudaFree(h->tauA);
-  cudaFree(h->Tq);
-  cudaFree(h->hnorm2);
+  cudaFree(h->tauB);  // with tauA, Tq and hnorm2 behind it
   cudaFree(h->Hhi);
   cudaFree(h->Hlo);
 }
@@ -161,10 +158,16 @@ static int make_handle(int n, int m, int p, cudaStream_t st, Handle** out) {
   alloc(&h->H, (size_t)n * n);
   alloc(&h->R, (size_t)n * m);
   alloc(&h->Ct, (size_t)ldct * n);
-  alloc(&h->tauB, (size_t)m);
-  alloc(&h->tauA, (size_t)n);
-  alloc(&h->Tq, q_t_count(n, m));
-  alloc(&h->hnorm2, 2);
+  // the small arrays in one allocation (a small system's reduction is mostly
+  // allocations and launches)
+  auto pad = [](size_t c) { return (c + 31) / 32 * 32; };
+  const size_t oA = pad(m), oT = oA + pad(n), oN = oT + pad(q_t_count(n, m));
+  alloc(&h->tauB, oN + 2);
+  if (e == cudaSuccess) {
+    h->tauA = h->tauB + oA;
+    h->Tq = h->tauB + oT;
+    h->hnorm2 = h->tauB + oN;
+  }
   if (e == cudaSuccess) e = cudaMalloc((void**)&h->Hhi, sizeof(float) * (size_t)n * n);
   if (e == cudaSuccess) e = cudaMalloc((void**)&h->Hlo, sizeof(float) * (size_t)n * n);
   if (e == cudaSuccess && p == 0) e = cudaMemsetAsync(h->Ct, 0, sizeof(double) * n, st);
